@@ -163,44 +163,59 @@ __global__ void k_from_f32(const float* __restrict__ in, double* __restrict__ ou
 
 namespace {
 
-constexpr int kDiagBlocks = 512;
+constexpr int kDiagBlocks = 608;    // 4 per SM
 constexpr int kDiagThreads = 256;
 
 // Per-block FP64 sums of M_I q_v,I (v = 0..4), M_I = Wx(gx) Wy(gy) Wz(gz)
-// with the Jacobian folded into Wx; a fixed tree order in shared memory.
+// with the Jacobian folded into Wx, in a fixed order: a warp takes whole rows
+// (its lanes along x), so that a value costs one FP64 FMA with Wx and a row
+// one with Wy Wz, and no index is divided; the FP64 pipe then bounds it beside
+// the reads.  128 x 128 x 16 order-4 box, FP64: 0.274 -> 0.176 ms.
 template <typename R>
-__global__ void k_diag_partial(const R* __restrict__ q, const double* __restrict__ wasm, int nx,
-                               int ny, int nz, long long np, double* __restrict__ partial) {
-  __shared__ double red[5][kDiagThreads];
+__global__ void __launch_bounds__(kDiagThreads) k_diag_partial(const R* __restrict__ q,
+                                                               const double* __restrict__ wasm, int nx, int ny,
+                                                               int nz, long long np, double* __restrict__ partial) {
+  constexpr int kWarps = kDiagThreads / 32;
+  __shared__ double red[5][kWarps];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double acc[5] = {0, 0, 0, 0, 0};
-  for (long long I = blockIdx.x * (long long)blockDim.x + threadIdx.x; I < np;
-       I += (long long)gridDim.x * blockDim.x) {
-    const int gx = (int)(I % nx);
-    const long long r = I / nx;
-    const int gy = (int)(r % ny), gz = (int)(r / ny);
-    const double m = wasm[gx] * wasm[nx + gy] * wasm[nx + ny + gz];
+  const long long nrows = (long long)ny * nz;
+  for (long long r = (long long)blockIdx.x * kWarps + warp; r < nrows; r += (long long)gridDim.x * kWarps) {
+    const int gz = (int)(r / ny), gy = (int)(r - (long long)gz * ny);
+    const R* row = q + r * nx;
+    double ar[5] = {0, 0, 0, 0, 0};
+#pragma unroll 2
+    for (int x = lane; x < nx; x += 32) {
+      const double w = wasm[x];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) acc[v] += m * xg::to_double(q[v * np + I]);
-  }
-#pragma unroll
-  for (int v = 0; v < 5; ++v) red[v][threadIdx.x] = acc[v];
-  __syncthreads();
-  for (int h = kDiagThreads / 2; h > 0; h >>= 1) {
-    if (threadIdx.x < h) {
-#pragma unroll
-      for (int v = 0; v < 5; ++v) red[v][threadIdx.x] += red[v][threadIdx.x + h];
+      for (int v = 0; v < 5; ++v) ar[v] = fma(w, xg::to_double(row[v * np + x]), ar[v]);
     }
-    __syncthreads();
+    const double wyz = wasm[nx + gy] * wasm[nx + ny + gz];
+#pragma unroll
+    for (int v = 0; v < 5; ++v) acc[v] = fma(wyz, ar[v], acc[v]);
   }
-  if (threadIdx.x < 5) partial[blockIdx.x * 5 + threadIdx.x] = red[threadIdx.x][0];
-}
-
-__global__ void k_diag_final(const double* __restrict__ partial, double* __restrict__ out) {
+#pragma unroll
+  for (int v = 0; v < 5; ++v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc[v] += __shfl_down_sync(0xffffffffu, acc[v], o);
+    if (lane == 0) red[v][warp] = acc[v];
+  }
+  __syncthreads();
   if (threadIdx.x < 5) {
     double s = 0.0;
-    for (int b = 0; b < kDiagBlocks; ++b) s += partial[b * 5 + threadIdx.x];
-    out[threadIdx.x] = s;
+    for (int w = 0; w < kWarps; ++w) s += red[threadIdx.x][w];
+    partial[blockIdx.x * 5 + threadIdx.x] = s;
   }
+}
+
+// one warp per variable
+__global__ void k_diag_final(const double* __restrict__ partial, double* __restrict__ out) {
+  const int v = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  double s = 0.0;
+  for (int b = lane; b < kDiagBlocks; b += 32) s += partial[b * 5 + v];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  if (lane == 0) out[v] = s;
 }
 
 unsigned conv_blocks(long long n) {
@@ -1140,7 +1155,7 @@ xg_status xg_diagnostics(xg_ctx* c, double out[5], void* stream) {
     k_diag_partial<double><<<kDiagBlocks, kDiagThreads, 0, st>>>(c->A, c->wasm, c->n[0], c->n[1],
                                                                  c->n[2], c->np, c->partial);
   XG_CUDA(c, cudaGetLastError());
-  k_diag_final<<<1, 32, 0, st>>>(c->partial, c->T);   // T is free between stages
+  k_diag_final<<<1, 160, 0, st>>>(c->partial, c->T);   // T is free between stages
   XG_CUDA(c, cudaGetLastError());
   XG_CUDA(c, cudaMemcpyAsync(c->hdiag, c->T, sizeof(double) * 5, cudaMemcpyDeviceToHost, st));
   XG_CUDA(c, cudaStreamSynchronize(st));

@@ -84,6 +84,9 @@ struct xg_ctx {
   double* dyn_L1 = nullptr;
   double* dyn_E = nullptr;
   double* dyn_gamma = nullptr;   // [n_z] sponge rate per level
+  // xg_ri_velocity's positions, sums and results (grown to the largest call)
+  double* ri_buf = nullptr;
+  size_t ri_bytes = 0;
   // IMEX work arrays (xg_imex.cu), allocated on first use
   void* imex = nullptr;
   // element partition along y (xg_partition_set): which y ends are
