@@ -598,6 +598,7 @@ xg_status xg_mesh_create(const xg_mesh_desc* d, xg_ctx** out) {
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev);
   if (sms <= 0) sms = 1;
+  c->sms = sms;
 
   xg::fill_line_params(d, geo, &c->P);
   c->dfm = d->precision == XG_DF64;

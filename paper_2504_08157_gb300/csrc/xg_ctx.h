@@ -19,6 +19,7 @@ struct xg_ctx {
   int n[3];
   long long np;
   int dev;
+  int sms = 1;           // the device's SM count
   xg::LineParams P;
   xg::DfParams Pdf;      // launch constants of the double-float kernels
   xg::FParams Pf;        // launch constants of the FP32 kernels

@@ -25,6 +25,7 @@
 
 #include "../../include/xg_dynamics.h"
 #include "xg_ctx.h"
+#include "xg_fixed.cuh"
 #include "xg_setup.h"
 
 namespace xg {
@@ -33,6 +34,7 @@ struct LapParams {
   int n[3], nseg[3], per[3];
   long long np;
   double Km[3][kMaxOrder + 1][kMaxOrder + 1];
+  FixRows Kf[3];   // Km in fixed point; x and y share their scale
 };
 
 template <int N>
@@ -67,32 +69,115 @@ __device__ __forceinline__ double line_apply(const LapParams& P, int d, const do
   return acc;
 }
 
-// out = Laplacian(in) (FIRST), or out = -Laplacian(in) - gamma(z) rho w
-// (second pass: in = the first pass's result, q = the state)
-template <int N, bool SECOND>
-__global__ void __launch_bounds__(128) k_laplace(const LapParams P, const double* __restrict__ in,
-                                                 const double* __restrict__ q,
-                                                 const double* __restrict__ gamma,
-                                                 double* __restrict__ out) {
-  const long long I = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (I >= P.np) return;
-  const long long np = P.np;
+// The Laplacian runs in two passes, the x and y parts over plane tiles and the
+// z part along columns, with the contractions in 64-bit fixed point
+// (xg_fixed.cuh): one thread per node with FP64 FMAs spent 3 (N + 1) (1 + 1/N)
+// of them a value, at the FP64 pipe's rate.  Grid of the plane pass: tiles, n_z,
+// 5 variables; out gets the x and y parts.  One Laplacian of the 64 x 64 x 16
+// order-4 box: 0.93-1.02 -> 0.22 + 0.12-0.16 ms; the plane pass is bound by
+// instruction issue (67 % busy, IMAD pipe 68 %), the z pass by the FP64 pipe
+// (3 instructions a value: conversion, scale-and-add, face sum).
+template <int N>
+__global__ void __launch_bounds__(kFixThreads) k_lap_plane(const LapParams P, const double* __restrict__ in,
+                                                          double* __restrict__ out) {
+  using L = FixPlane<N>;
+  __shared__ fix2 V[L::V];
+  __shared__ long long RA[2][L::RA], RB[2][L::RB];
+  __shared__ int emax;
+  const int z = blockIdx.y, var = blockIdx.z;
+  const int tilesx = (P.nseg[0] + L::E - 1) / L::E;
   const int nx = P.n[0], ny = P.n[1];
-  const int gx = (int)(I % nx);
-  const long long r = I / nx;
-  const int gy = (int)(r % ny), gz = (int)(r / ny);
-  const long long bx = I - gx, by = I - (long long)gy * nx, bz = I - (long long)gz * nx * ny;
-#pragma unroll 1
-  for (int v = 0; v < 5; ++v) {
-    const double* f = in + v * np;
-    double L = line_apply<N>(P, 0, f, bx, 1, gx);
-    L += line_apply<N>(P, 1, f, by, nx, gy);
-    L += line_apply<N>(P, 2, f, bz, (long long)nx * ny, gz);
-    if (SECOND) {
-      L = -L;
-      if (v == 3 && gamma) L = fma(-gamma[gz], q[3 * np + I], L);
+  const long long off = var * P.np + (long long)nx * ny * z;
+  FixTile T;
+  T.init<N>(P, blockIdx.x % tilesx, blockIdx.x / tilesx);
+  if (threadIdx.x == 0) emax = 0;
+  __syncthreads();
+  double v[L::kLoads];
+  fix_plane_load<N, true, true>(in + off, T, nx, ny, v, &emax);
+  __syncthreads();
+  const int E = emax == kFixNonfinite ? emax : fix_block_exp(emax, P.Kf[0].sc);
+  if (E != kFixNonfinite) {
+    fix_plane_convert<N>(v, E, V);
+    __syncthreads();
+    fix_plane_rows<N, 0>(P.Kf[0], T, V, RA[0], RB[0]);
+    fix_plane_rows<N, 1>(P.Kf[1], T, V, RA[1], RB[1]);
+    __syncthreads();
+  }
+  const double unit = fix_unit<N>(E, P.Kf[0].sc);
+  fix_plane_nodes<N>(T, [&](int i, int j) {
+    const long long I = T.x0 + i + (long long)nx * (T.y0 + j);
+    if (E != kFixNonfinite) {
+      const long long r = fix_plane_node<N, 0>(T, RA[0], RB[0], i, j) + fix_plane_node<N, 1>(T, RA[1], RB[1], j, i);
+      out[off + I] = (double)r * unit;
+    } else {   // an infinity or NaN in the tile: FP64, node by node
+      double s = line_apply<N>(P, 0, in + off, (long long)nx * (T.y0 + j), 1, T.x0 + i);
+      s += line_apply<N>(P, 1, in + off, T.x0 + i, nx, T.y0 + j);
+      out[off + I] = s;
     }
-    out[v * np + I] = L;
+  });
+}
+
+// out += the z part (FIRST: the x and y parts are in out), or out = -(out + z
+// part) - gamma(z) rho w.  One thread per column of one variable (blockIdx.z),
+// marching the segments of its chunk (blockIdx.y).
+template <int N, bool SECOND>
+__global__ void __launch_bounds__(128) k_lap_z(const LapParams P, const double* __restrict__ in, double* out,
+                                               const double* __restrict__ q, const double* __restrict__ gamma,
+                                               int chunk) {
+  const long long nxy = (long long)P.n[0] * P.n[1];
+  const long long col = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (col >= nxy) return;
+  const int var = blockIdx.z, nz = P.n[2], nseg = P.nseg[2];
+  const int s0 = blockIdx.y * chunk, s1 = min(nseg, s0 + chunk);
+  const double* __restrict__ f = in + var * P.np + col;
+  double* o = out + var * P.np + col;
+  const FixRows& K = P.Kf[2];
+  auto at = [&](int g) -> double { return f[nxy * (g == nz ? 0 : g)]; };
+  auto put = [&](int g, double s) {   // the FP64 pipe bounds this pass: signs ride in the operands
+    if (SECOND && var == 3 && gamma) s = fma(-gamma[g], q[3 * P.np + col + nxy * g], s);
+    o[nxy * g] = s;
+  };
+  double v[N + 1], next[N], carry = 0.0;
+  fix2 w[N + 1];
+  bool left = s0 > 0 || P.per[2];
+  if (left) {
+    const int sp = s0 > 0 ? s0 - 1 : nseg - 1;
+#pragma unroll
+    for (int l = 0; l <= N; ++l) v[l] = at(sp * N + l);
+    const int E = fix_segment<N>(v, K.sc, w);
+    carry = (double)fix_row<N>(K, N, w) * (SECOND ? -fix_unit<N>(E, K.sc) : fix_unit<N>(E, K.sc));
+  }
+  v[0] = at(s0 * N);
+#pragma unroll
+  for (int l = 0; l < N; ++l) next[l] = at(s0 * N + l + 1);
+  for (int s = s0; s < s1; ++s) {
+    double part[N];
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+      part[a] = o[nxy * (s * N + a)];
+      v[a + 1] = next[a];
+    }
+    if (s + 1 < s1) {   // the next segment's values while this one is computed
+#pragma unroll
+      for (int l = 0; l < N; ++l) next[l] = at((s + 1) * N + l + 1);
+    }
+    const int E = fix_segment<N>(v, K.sc, w);
+    const double unit = SECOND ? -fix_unit<N>(E, K.sc) : fix_unit<N>(E, K.sc);
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+      long long r = fix_row<N>(K, a, w);
+      if (a == 0 && !left) r += r;          // a wall's first node: its row twice
+      double x = fma((double)r, unit, SECOND ? -part[a] : part[a]);
+      if (a == 0 && left) x += carry;
+      put(s * N + a, x);
+    }
+    carry = (double)fix_row<N>(K, N, w) * unit;
+    v[0] = v[N];
+    left = true;
+  }
+  if (!P.per[2] && s1 == nseg) {
+    const double part = o[nxy * (nseg * N)];
+    put(nseg * N, fma(2.0, carry, SECOND ? -part : part));
   }
 }
 
@@ -360,15 +445,20 @@ std::vector<double> axis_positions(const xg_ctx* c, int d) {
 
 template <int N>
 void launch_lap(const LapParams& P, const double* q, double* L1, const double* gamma, double* E,
-                bool hyper, cudaStream_t st) {
-  const unsigned blocks = (unsigned)((P.np + 127) / 128);
+                bool hyper, int sms, cudaStream_t st) {
+  const long long nxy = (long long)P.n[0] * P.n[1];
   if (hyper) {
-    xg::k_laplace<N, false><<<blocks, 128, 0, st>>>(P, q, nullptr, nullptr, L1);
-    xg::k_laplace<N, true><<<blocks, 128, 0, st>>>(P, L1, q, gamma, E);
+    constexpr int TE = xg::fix_plane_elems(N);
+    const dim3 gp(((P.nseg[0] + TE - 1) / TE) * ((P.nseg[1] + TE - 1) / TE), P.n[2], 5);
+    const int chunk = xg::fix_z_chunk(P.nseg[2], 5 * nxy, sms);
+    const dim3 gz((unsigned)((nxy + 127) / 128), (P.nseg[2] + chunk - 1) / chunk, 5);
+    xg::k_lap_plane<N><<<gp, xg::kFixThreads, 0, st>>>(P, q, L1);
+    xg::k_lap_z<N, false><<<gz, 128, 0, st>>>(P, q, L1, nullptr, nullptr, chunk);
+    xg::k_lap_plane<N><<<gp, xg::kFixThreads, 0, st>>>(P, L1, E);
+    xg::k_lap_z<N, true><<<gz, 128, 0, st>>>(P, L1, E, q, gamma, chunk);
   } else {
-    const int nxy = P.n[0] * P.n[1];
     xg::k_sponge_only<<<(unsigned)std::min<long long>((5 * P.np + 255) / 256, 65535), 256, 0, st>>>(
-        P.np, nxy, q, gamma, E);
+        P.np, (int)nxy, q, gamma, E);
   }
 }
 
@@ -379,14 +469,14 @@ cudaError_t dynamics_launch(xg_ctx* c, const double* q, cudaStream_t st) {
   const LapParams& P = *static_cast<const LapParams*>(c->dyn_params);
   const bool hyper = c->dyn_hyper;
   switch (c->d.order) {
-    case 1: launch_lap<1>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, st); break;
-    case 2: launch_lap<2>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, st); break;
-    case 3: launch_lap<3>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, st); break;
-    case 4: launch_lap<4>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, st); break;
-    case 5: launch_lap<5>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, st); break;
-    case 6: launch_lap<6>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, st); break;
-    case 7: launch_lap<7>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, st); break;
-    case 8: launch_lap<8>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, st); break;
+    case 1: launch_lap<1>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, c->sms, st); break;
+    case 2: launch_lap<2>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, c->sms, st); break;
+    case 3: launch_lap<3>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, c->sms, st); break;
+    case 4: launch_lap<4>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, c->sms, st); break;
+    case 5: launch_lap<5>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, c->sms, st); break;
+    case 6: launch_lap<6>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, c->sms, st); break;
+    case 7: launch_lap<7>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, c->sms, st); break;
+    case 8: launch_lap<8>(P, q, c->dyn_L1, c->dyn_gamma, c->dyn_E, hyper, c->sms, st); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -452,20 +542,26 @@ xg_status xg_set_dynamics(xg_ctx* c, const xg_dynamics* dyn) {
     const double dx = h[d] / N;
     nu[d] = hyper ? std::sqrt(dyn->hyper_c[i]) * dx * dx / std::sqrt(dyn->hyper_dt) : 0.0;
   }
-  double D[xg::kMaxOrder + 1][xg::kMaxOrder + 1], w[xg::kMaxOrder + 1];
+  long double D[xg::kMaxOrder + 1][xg::kMaxOrder + 1], w[xg::kMaxOrder + 1];
   xg::lgl_derivative(N, D);
   xg::lgl_weights(N, w);
+  xg::FixMatrix Kl[3];
+  double most[3];
   for (int d = 0; d < 3; ++d) {
-    const double s = -nu[d] * (2.0 / h[d]) * (2.0 / h[d]);
+    const long double s = -(long double)nu[d] * (2.0L / h[d]) * (2.0L / h[d]);
     for (int a = 0; a <= N; ++a) {
-      const double wa = (a == 0 || a == N) ? 2.0 * w[0] : w[a];
+      const long double wa = (a == 0 || a == N) ? 2.0L * w[0] : w[a];
       for (int l = 0; l <= N; ++l) {
         long double K = 0.0L;
-        for (int k = 0; k <= N; ++k) K += (long double)w[k] * D[k][a] * D[k][l];
-        P->Km[d][a][l] = (double)(s * (double)K / wa);
+        for (int k = 0; k <= N; ++k) K += w[k] * D[k][a] * D[k][l];
+        Kl[d][a][l] = s * K / wa;
+        P->Km[d][a][l] = (double)Kl[d][a][l];
       }
     }
+    most[d] = xg::fix_row_sum(N, Kl[d]);
   }
+  for (int d = 0; d < 3; ++d)   // x and y sums are added as integers: one scale
+    xg::fix_rows(N, Kl[d], xg::fix_scale_of(d < 2 ? std::max(most[0], most[1]) : most[2]), &P->Kf[d]);
   cudaError_t e = cudaSuccess;
   const size_t vec = sizeof(double) * 5 * (size_t)c->np;
   if (!c->dyn_L1) e = cudaMalloc((void**)&c->dyn_L1, vec);

@@ -1,22 +1,20 @@
 // xg_imex.cu -- IMEX ARK2 time integration with matrix-free GMRES
 // (include/xg_imex.h).
 //
-// The linear operator is evaluated node by node: for each node the
-// assembled derivatives it needs (rho u along x, rho v along y, rho w and
-// theta_0 rho w along z, Theta' along x and y, p'_lin along z) are sums of
-// the pre-scaled derivative rows Dm over the node's segments (a face node
-// adds the segment before, a wall node doubles its row), exactly the
-// structure of the right-hand side's contractions.  One kernel returns
-// c0 v + c1 L(v), so a GMRES product (I - dt g L) v is a single pass.
+// The linear operator needs seven assembled derivatives (rho u along x, rho v
+// along y, rho w and theta_0 rho w along z, Theta' along x and y, p'_lin along
+// z): sums of the pre-scaled derivative rows Dm over a node's segments (a face
+// node adds the segment before, a wall node doubles its row), exactly the
+// structure of the right-hand side's contractions.  Two kernels return
+// c0 v + c1 L(v), their sums in 64-bit fixed point.
 //
 // GMRES (restarted; one classical Gram-Schmidt pass, a second only where the
 // first cancels severely) runs on the host with the device vectors; the
 // inner products are deterministic (fixed grid, per-block and per-variable
 // partial sums added on the host in block order) and weight variable v by
 // 1/rms(b_v)^2.  The explicit part is the context's own stage in
-// right-hand-side mode (FP64, or the mixed XG_DF64 stage); L, the inner
-// products and the combinations are FP64, and all of them are bound by
-// GB300's FP64 pipe.
+// right-hand-side mode (FP64, or the mixed XG_DF64 stage); the inner
+// products and the combinations are FP64 and bound by GB300's FP64 pipe.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -28,6 +26,7 @@
 
 #include "../../include/xg_imex.h"
 #include "xg_ctx.h"
+#include "xg_fixed.cuh"
 #include "xg_setup.h"
 
 namespace xg {
@@ -37,92 +36,229 @@ constexpr int kDotThreads = 256;
 constexpr int kDotBatch = 16;   // vectors per multi-dot launch
 constexpr int kCombMax = 17;    // terms per combination launch
 
+// The matrices of the linear operator in fixed point: Dm per direction.
+struct LinParams {
+  LineParams P;
+  FixRows D[3];
+};
+
 // sum over the node's segment(s) along d of Dm rows times f: -d/dx_d of the
-// assembled field.  With tab (z only) the coefficients are tab's, the rows
-// of Dm already multiplied by a per-level factor of the loaded node:
-// tab[(s (N + 1) + a) (N + 1) + l] = Dm[2][a][l] lev[s N + l] (k_lin_tables).
+// assembled field (FP64; the plane pass takes it where a tile holds an
+// infinity or NaN, which has no fixed-point form).
 template <int N>
 __device__ __forceinline__ double line_sum(const LineParams& P, int d, const double* __restrict__ f,
-                                           long long base, long long sd, int g,
-                                           const double* __restrict__ tab) {
+                                           long long base, long long sd, int g) {
   const int nd = P.n[d], nseg = P.nseg[d];
-  int s = g / N;
-  if (s >= nseg) s = nseg - 1;
-  const int a = g - s * N;
-  const double* t = tab ? tab + (s * (N + 1) + a) * (N + 1) : nullptr;
-  double acc = 0.0;
-#pragma unroll
+  const int s = min(g / N, nseg - 1), a = g - s * N;
+  const bool left = a == 0 && (s > 0 || P.per[d]);
+  const int s2 = s > 0 ? s - 1 : nseg - 1;
+  double acc = 0.0, accl = 0.0;
   for (int l = 0; l <= N; ++l) {
-    int k = s * N + l;
-    if (k >= nd) k -= nd;
-    acc = fma(t ? t[l] : P.Dm[d][a][l], f[base + sd * k], acc);
+    const int k = s * N + l, k2 = s2 * N + l;
+    acc = fma(P.Dm[d][a][l], f[base + sd * (k >= nd ? k - nd : k)], acc);
+    if (left) accl = fma(P.Dm[d][N][l], f[base + sd * (k2 >= nd ? k2 - nd : k2)], accl);
   }
-  if (a == 0) {
-    if (s > 0 || P.per[d]) {
-      const int s2 = s > 0 ? s - 1 : nseg - 1;
-      const double* t2 = tab ? tab + (s2 * (N + 1) + N) * (N + 1) : nullptr;
-#pragma unroll
-      for (int l = 0; l <= N; ++l) {
-        int k = s2 * N + l;
-        if (k >= nd) k -= nd;
-        acc = fma(t2 ? t2[l] : P.Dm[d][N][l], f[base + sd * k], acc);
-      }
-    } else {
-      acc = acc + acc;
-    }
-  } else if (a == N) {
-    acc = acc + acc;
-  }
-  return acc;
+  if (left) return acc + accl;
+  return a == 0 || a == N ? acc + acc : acc;
 }
 
-// out = c0 v + c1 L(v) (out = L(v) for c0 = 0, c1 = 1); cpl = gamma p0 /
-// Theta0 per level, tw and tp the z rows times theta0 = Theta0 / rho0 and
-// times cpl (k_lin_tables).  FP64 work per node: the seven line sums' FMAs
-// (N + 1 each, twice at a face node) and the assembly; the per-level factors
-// of the z sums ride in their coefficients.
-template <int N>
-__global__ void __launch_bounds__(128) k_linear(const LineParams P, const double* __restrict__ v,
-                                                const double* __restrict__ cpl,
-                                                const double* __restrict__ th0,
-                                                const double* __restrict__ tw,
-                                                const double* __restrict__ tp, double c0, double c1,
-                                                double* __restrict__ out) {
-  const long long I = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (I >= P.np) return;
-  const long long np = P.np;
-  const int nx = P.n[0], ny = P.n[1];
-  const long long nxy = (long long)nx * ny;
-  const int gx = (int)(I % nx);
-  const long long r = I / nx;
-  const int gy = (int)(r % ny), gz = (int)(r / ny);
-  const long long bx = I - gx, by = I - (long long)gy * nx, bz = I - (long long)gz * nxy;
-  const double* ru = v + np;
-  const double* rv = v + 2 * np;
-  const double* rw = v + 3 * np;
-  const double* th = v + 4 * np;
-  const double dxu = line_sum<N>(P, 0, ru, bx, 1, gx, nullptr);
-  const double dyv = line_sum<N>(P, 1, rv, by, nx, gy, nullptr);
-  const double dzw = line_sum<N>(P, 2, rw, bz, nxy, gz, nullptr);
-  const double dzwt = line_sum<N>(P, 2, rw, bz, nxy, gz, tw);
-  const double dxp = cpl[gz] * line_sum<N>(P, 0, th, bx, 1, gx, nullptr);
-  const double dyp = cpl[gz] * line_sum<N>(P, 1, th, by, nx, gy, nullptr);
-  const double dzp = line_sum<N>(P, 2, th, bz, nxy, gz, tp);
-  double L[5];
-  L[0] = dxu + dyv + dzw;
-  L[1] = dxp;
-  L[2] = dyp;
-  L[3] = fma(-P.g, v[I], dzp);
-  L[4] = fma(th0[gz], dxu + dyv, dzwt);
-  if (!P.per[0] && (gx == 0 || gx == nx - 1)) L[1] = 0.0;
-  if (!P.per[1] && (gy == 0 || gy == ny - 1)) L[2] = 0.0;
-  if (!P.per[2] && (gz == 0 || gz == P.n[2] - 1)) L[3] = 0.0;
-  if (c0 == 0.0 && c1 == 1.0) {
-#pragma unroll
-    for (int c = 0; c < 5; ++c) out[c * np + I] = L[c];
+// out = c0 v + c1 L(v) (out = L(v) for c0 = 0, c1 = 1) in two passes with the
+// line sums in 64-bit fixed point (xg_fixed.cuh).  One thread per node with
+// FP64 FMAs spent 7 (N + 1) (1 + 1/N) of them a node and ran at the FP64
+// pipe's rate, 8 times the time of the bytes.  Here the FP64 pipe is left with the
+// conversions of the sums and the assembly, about 20 instructions a node.
+// 80 x 80 x 24 order-5 box: 2.39 -> 0.61 + 0.51 ms (issue-bound; FP64 pipe 71 %
+// busy in the z pass).
+//
+// Plane pass: x and y sums over the tiles of a level (blockIdx.x), level
+// blockIdx.y; blockIdx.z = 0 puts A = dx(rho u) + dy(rho v) into out[0] for
+// the z pass, blockIdx.z = 1 finishes rho u and rho v from Theta' (cpl = gamma
+// p0 / Theta0 per level).
+template <int N, bool PLAIN>
+__global__ void __launch_bounds__(kFixThreads) k_lin_plane(const LinParams Q, const double* __restrict__ v,
+                                                          const double* __restrict__ cpl, double c0, double c1,
+                                                          double* __restrict__ out) {
+  using L = FixPlane<N>;
+  __shared__ fix2 V[2][L::V];
+  __shared__ long long RA[2][L::RA], RB[2][L::RB];
+  __shared__ int emax;
+  const LineParams& P = Q.P;
+  const int z = blockIdx.y, nx = P.n[0], ny = P.n[1], sc = Q.D[0].sc;
+  const int tilesx = (P.nseg[0] + L::E - 1) / L::E;
+  const long long np = P.np, off = (long long)nx * ny * z;
+  FixTile T;
+  T.init<N>(P, blockIdx.x % tilesx, blockIdx.x / tilesx);
+  if (threadIdx.x == 0) emax = 0;
+  __syncthreads();
+  const bool theta = blockIdx.z == 1;
+  const double* fx = v + (theta ? 4 : 1) * np + off;
+  const double* fy = v + (theta ? 4 : 2) * np + off;
+  const fix2* Vy = theta ? V[0] : V[1];
+  int E;
+  if (theta) {
+    double a[L::kLoads];
+    fix_plane_load<N, true, true>(fx, T, nx, ny, a, &emax);
+    __syncthreads();
+    E = emax == kFixNonfinite ? emax : fix_block_exp(emax, sc);
+    if (E != kFixNonfinite) fix_plane_convert<N>(a, E, V[0]);
   } else {
+    // one exponent for both momenta: A is a sum of integers, exact where the
+    // two parts nearly cancel (a vortex)
+    double a[L::kLoads], b[L::kLoads];
+    fix_plane_load<N, true, false>(fx, T, nx, ny, a, &emax);
+    fix_plane_load<N, false, true>(fy, T, nx, ny, b, &emax);
+    __syncthreads();
+    E = emax == kFixNonfinite ? emax : fix_block_exp(emax, sc);
+    if (E != kFixNonfinite) {
+      fix_plane_convert<N>(a, E, V[0]);
+      fix_plane_convert<N>(b, E, V[1]);
+    }
+  }
+  __syncthreads();
+  if (E != kFixNonfinite) {
+    fix_plane_rows<N, 0>(Q.D[0], T, V[0], RA[0], RB[0]);
+    fix_plane_rows<N, 1>(Q.D[1], T, Vy, RA[1], RB[1]);
+    __syncthreads();
+  }
+  const double cp = theta ? cpl[z] : 1.0, unit = fix_unit<N>(E, sc) * cp;
+  fix_plane_nodes<N>(T, [&](int i, int j) {
+    const int gx = T.x0 + i, gy = T.y0 + j;
+    const long long I = off + gx + (long long)nx * gy;
+    double dx, dy = 0.0;
+    if (E != kFixNonfinite) {
+      const long long rx = fix_plane_node<N, 0>(T, RA[0], RB[0], i, j), ry = fix_plane_node<N, 1>(T, RA[1], RB[1], j, i);
+      if (!theta) {
+        out[I] = (double)(rx + ry) * unit;
+        return;
+      }
+      dx = (double)rx * unit;
+      dy = (double)ry * unit;
+    } else {
+      dx = cp * line_sum<N>(P, 0, fx, (long long)nx * gy, 1, gx);
+      dy = cp * line_sum<N>(P, 1, fy, gx, nx, gy);
+      if (!theta) {
+        out[I] = dx + dy;
+        return;
+      }
+    }
+    if (!P.per[0] && (gx == 0 || gx == nx - 1)) dx = 0.0;
+    if (!P.per[1] && (gy == 0 || gy == ny - 1)) dy = 0.0;
+    if (PLAIN) {
+      out[np + I] = dx;
+      out[2 * np + I] = dy;
+    } else {
+      out[np + I] = fma(c1, dx, c0 * v[np + I]);
+      out[2 * np + I] = fma(c1, dy, c0 * v[2 * np + I]);
+    }
+  });
+}
+
+// z pass: one thread per column, marching the segments of its chunk
+// (blockIdx.y): rho' = A + dz(rho w), rho w = dz(p'_lin) - g rho', Theta' =
+// theta0 A + dz(theta0 rho w), A from out[0].
+template <int N, bool PLAIN>
+__global__ void __launch_bounds__(128) k_lin_z(const LinParams Q, const double* __restrict__ v,
+                                               const double* __restrict__ cpl, const double* __restrict__ th0,
+                                               double c0, double c1, double* out, int chunk) {
+  const LineParams& P = Q.P;
+  const FixRows& D = Q.D[2];
+  const long long np = P.np, nxy = (long long)P.n[0] * P.n[1];
+  const long long col = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (col >= nxy) return;
+  const int nz = P.n[2], nseg = P.nseg[2];
+  const int s0 = blockIdx.y * chunk, s1 = min(nseg, s0 + chunk);
+  const double* __restrict__ rw = v + 3 * np + col;
+  const double* __restrict__ th = v + 4 * np + col;
+  auto lev = [&](int g) -> int { return g == nz ? 0 : g; };
+  double w[N + 1], t[N + 1], carry[3] = {0.0, 0.0, 0.0};   // rows N of dz w, dz (theta0 w), dz p'
+  fix2 f[N + 1];
+  // rows 0..N of field u, added to add[.] (rows 0..N-1), row N in last; a
+  // line's wall end (twice: 2) counts row 0 twice
+  auto rows = [&](const double (&u)[N + 1], const double (&add)[N], double (&r)[N], double& last, bool twice) {
+    const int E = fix_segment<N>(u, D.sc, f);
+    const double unit = fix_unit<N>(E, D.sc);
 #pragma unroll
-    for (int c = 0; c < 5; ++c) out[c * np + I] = c0 == 0.0 ? c1 * L[c] : fma(c1, L[c], c0 * v[c * np + I]);
+    for (int a = 0; a < N; ++a) {
+      long long x = fix_row<N>(D, a, f);
+      if (a == 0 && twice) x += x;
+      r[a] = fma((double)x, unit, add[a]);
+    }
+    last = (double)fix_row<N>(D, N, f) * unit;
+  };
+  auto row_last = [&](const double (&u)[N + 1]) -> double {
+    const int E = fix_segment<N>(u, D.sc, f);
+    return (double)fix_row<N>(D, N, f) * fix_unit<N>(E, D.sc);
+  };
+  auto put = [&](int g, double rp, double L0, double L4, double L3) {
+    const long long I = col + nxy * g;
+    if (!P.per[2] && (g == 0 || g == nz - 1)) L3 = 0.0;
+    if (!PLAIN) {
+      L0 = fma(c1, L0, c0 * rp);
+      L3 = fma(c1, L3, c0 * rw[nxy * g]);
+      L4 = fma(c1, L4, c0 * th[nxy * g]);
+    }
+    out[I] = L0;
+    out[3 * np + I] = L3;
+    out[4 * np + I] = L4;
+  };
+  bool left = s0 > 0 || P.per[2];
+  if (left) {
+    const int sp = s0 > 0 ? s0 - 1 : nseg - 1;
+    double x[N + 1];
+#pragma unroll
+    for (int l = 0; l <= N; ++l) {
+      const int g = lev(sp * N + l);
+      w[l] = rw[nxy * g];
+      x[l] = w[l] * th0[g];
+      t[l] = th[nxy * g] * cpl[g];
+    }
+    carry[0] = row_last(w);
+    carry[1] = row_last(x);
+    carry[2] = row_last(t);
+  }
+  w[0] = rw[nxy * (s0 * N)];
+  t[0] = th[nxy * (s0 * N)] * cpl[s0 * N];
+  for (int s = s0; s < s1; ++s) {
+    double A[N], rp[N], x[N + 1], r0[N], r1[N], r2[N];
+#pragma unroll
+    for (int l = 1; l <= N; ++l) {
+      const int g = lev(s * N + l);
+      w[l] = rw[nxy * g];
+      t[l] = th[nxy * g];
+    }
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+      A[a] = out[col + nxy * (s * N + a)];
+      rp[a] = v[col + nxy * (s * N + a)];
+    }
+#pragma unroll
+    for (int l = 1; l <= N; ++l) t[l] *= cpl[lev(s * N + l)];
+#pragma unroll
+    for (int l = 0; l <= N; ++l) x[l] = w[l] * th0[lev(s * N + l)];
+    double before[3] = {carry[0], carry[1], carry[2]}, tA[N], gr[N];
+#pragma unroll
+    for (int a = 0; a < N; ++a) {
+      tA[a] = th0[s * N + a] * A[a];
+      gr[a] = -P.g * rp[a];
+    }
+    rows(w, A, r0, carry[0], !left);
+    rows(x, tA, r1, carry[1], !left);
+    rows(t, gr, r2, carry[2], !left);
+    if (left) {
+      r0[0] += before[0];
+      r1[0] += before[1];
+      r2[0] += before[2];
+    }
+#pragma unroll
+    for (int a = 0; a < N; ++a) put(s * N + a, rp[a], r0[a], r1[a], r2[a]);
+    w[0] = w[N];
+    t[0] = t[N];
+    left = true;
+  }
+  if (!P.per[2] && s1 == nseg) {
+    const int g = nseg * N;
+    const double A = out[col + nxy * g], rp = v[col + nxy * g];
+    put(g, rp, fma(2.0, carry[0], A), fma(2.0, carry[1], th0[g] * A), 0.0);
   }
 }
 
@@ -210,22 +346,6 @@ __global__ void __launch_bounds__(kDotThreads, 4) k_wdots(const double* __restri
   }
 }
 
-// tw[(s (N + 1) + a) (N + 1) + l] = Dm[2][a][l] theta0[k] and tp the same
-// with cpl[k], k = s N + l (wrapped when z is periodic): the z rows of the
-// linear operator with their per-level factor
-template <int N>
-__global__ void k_lin_tables(const LineParams P, const double* __restrict__ cpl, const double* __restrict__ th0,
-                             double* __restrict__ tw, double* __restrict__ tp) {
-  const int nseg = P.nseg[2], nd = P.n[2];
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nseg * (N + 1) * (N + 1)) return;
-  const int l = e % (N + 1), a = (e / (N + 1)) % (N + 1), s = e / ((N + 1) * (N + 1));
-  int k = s * N + l;
-  if (k >= nd) k -= nd;
-  tw[e] = P.Dm[2][a][l] * th0[k];
-  tp[e] = P.Dm[2][a][l] * cpl[k];
-}
-
 __global__ void k_lin_levels(const double* __restrict__ base, int nz, double gamma, double* __restrict__ cpl,
                              double* __restrict__ th0) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -253,8 +373,7 @@ struct Imex {
   double* q1 = nullptr;        // q^{n+1}
   double* cpl = nullptr;       // [nz]
   double* th0 = nullptr;       // [nz]
-  double* tw = nullptr;        // [nseg_z][N + 1][N + 1] z rows times theta0
-  double* tp = nullptr;        // [nseg_z][N + 1][N + 1] z rows times cpl
+  xg::LinParams lin;           // the operator's matrices in fixed point
   double wt[5] = {1.0, 1.0, 1.0, 1.0, 1.0};   // inner-product weights per variable
   double* partial = nullptr;   // [kDotBlocksMax][5][kDotBatch]
   int dot_blocks = 512;        // blocks of the reductions: 4 per SM
@@ -262,19 +381,34 @@ struct Imex {
   long long reorth = 0;        // Arnoldi steps that took a second Gram-Schmidt pass
 };
 
+template <int N>
+void launch_linear_n(xg_ctx* c, const Imex& X, const double* v, double c0, double c1, double* out, cudaStream_t st) {
+  constexpr int E = xg::fix_plane_elems(N);
+  const LineParams& P = X.lin.P;
+  const long long nxy = (long long)P.n[0] * P.n[1];
+  const dim3 gp(((P.nseg[0] + E - 1) / E) * ((P.nseg[1] + E - 1) / E), P.n[2], 2);
+  const int chunk = xg::fix_z_chunk(P.nseg[2], nxy, c->sms);
+  const dim3 gz((unsigned)((nxy + 127) / 128), (P.nseg[2] + chunk - 1) / chunk);
+  if (c0 == 0.0 && c1 == 1.0) {
+    xg::k_lin_plane<N, true><<<gp, xg::kFixThreads, 0, st>>>(X.lin, v, X.cpl, c0, c1, out);
+    xg::k_lin_z<N, true><<<gz, 128, 0, st>>>(X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
+  } else {
+    xg::k_lin_plane<N, false><<<gp, xg::kFixThreads, 0, st>>>(X.lin, v, X.cpl, c0, c1, out);
+    xg::k_lin_z<N, false><<<gz, 128, 0, st>>>(X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
+  }
+}
+
 cudaError_t launch_linear(xg_ctx* c, const Imex& X, const double* v, double c0, double c1, double* out,
                           cudaStream_t st) {
-  const LineParams& P = c->P;
-  const unsigned blocks = (unsigned)((c->np + 127) / 128);
   switch (c->d.order) {
-    case 1: xg::k_linear<1><<<blocks, 128, 0, st>>>(P, v, X.cpl, X.th0, X.tw, X.tp, c0, c1, out); break;
-    case 2: xg::k_linear<2><<<blocks, 128, 0, st>>>(P, v, X.cpl, X.th0, X.tw, X.tp, c0, c1, out); break;
-    case 3: xg::k_linear<3><<<blocks, 128, 0, st>>>(P, v, X.cpl, X.th0, X.tw, X.tp, c0, c1, out); break;
-    case 4: xg::k_linear<4><<<blocks, 128, 0, st>>>(P, v, X.cpl, X.th0, X.tw, X.tp, c0, c1, out); break;
-    case 5: xg::k_linear<5><<<blocks, 128, 0, st>>>(P, v, X.cpl, X.th0, X.tw, X.tp, c0, c1, out); break;
-    case 6: xg::k_linear<6><<<blocks, 128, 0, st>>>(P, v, X.cpl, X.th0, X.tw, X.tp, c0, c1, out); break;
-    case 7: xg::k_linear<7><<<blocks, 128, 0, st>>>(P, v, X.cpl, X.th0, X.tw, X.tp, c0, c1, out); break;
-    case 8: xg::k_linear<8><<<blocks, 128, 0, st>>>(P, v, X.cpl, X.th0, X.tw, X.tp, c0, c1, out); break;
+    case 1: launch_linear_n<1>(c, X, v, c0, c1, out, st); break;
+    case 2: launch_linear_n<2>(c, X, v, c0, c1, out, st); break;
+    case 3: launch_linear_n<3>(c, X, v, c0, c1, out, st); break;
+    case 4: launch_linear_n<4>(c, X, v, c0, c1, out, st); break;
+    case 5: launch_linear_n<5>(c, X, v, c0, c1, out, st); break;
+    case 6: launch_linear_n<6>(c, X, v, c0, c1, out, st); break;
+    case 7: launch_linear_n<7>(c, X, v, c0, c1, out, st); break;
+    case 8: launch_linear_n<8>(c, X, v, c0, c1, out, st); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
@@ -530,8 +664,6 @@ void imex_free_buffers(Imex* X) {
   cudaFree(X->q1);
   cudaFree(X->cpl);
   cudaFree(X->th0);
-  cudaFree(X->tw);
-  cudaFree(X->tp);
   cudaFree(X->partial);
 }
 
@@ -560,6 +692,20 @@ cudaError_t prepare(xg_ctx* c, int m, cudaStream_t st) {
     c->imex = X;
     X->m = m;
     X->n = n;
+    X->lin.P = c->P;
+    const int N = c->d.order;
+    long double D[xg::kMaxOrder + 1][xg::kMaxOrder + 1];
+    xg::FixMatrix Dl[3];
+    double most[3];
+    xg::lgl_derivative(N, D);
+    for (int d = 0; d < 3; ++d) {   // -(2/h) D, rows 0 and N halved
+      const long double h = ((long double)c->d.hi[d] - c->d.lo[d]) / c->d.nel[d];
+      for (int a = 0; a <= N; ++a)
+        for (int l = 0; l <= N; ++l) Dl[d][a][l] = -(2.0L / h) * (a == 0 || a == N ? 0.5L : 1.0L) * D[a][l];
+      most[d] = xg::fix_row_sum(N, Dl[d]);
+    }
+    for (int d = 0; d < 3; ++d)     // x and y sums are added as integers: one scale
+      xg::fix_rows(N, Dl[d], xg::fix_scale_of(d < 2 ? std::max(most[0], most[1]) : most[2]), &X->lin.D[d]);
     X->hpart.resize((size_t)xg::kDotBlocksMax * 5 * xg::kDotBatch);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev);
@@ -571,9 +717,6 @@ cudaError_t prepare(xg_ctx* c, int m, cudaStream_t st) {
       if (e == cudaSuccess) e = cudaMalloc((void**)p, vb);
     if (e == cudaSuccess) e = cudaMalloc((void**)&X->cpl, sizeof(double) * c->n[2]);
     if (e == cudaSuccess) e = cudaMalloc((void**)&X->th0, sizeof(double) * c->n[2]);
-    const size_t tb = sizeof(double) * (size_t)c->P.nseg[2] * (c->d.order + 1) * (c->d.order + 1);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&X->tw, tb);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&X->tp, tb);
     if (e == cudaSuccess)
       e = cudaMalloc((void**)&X->partial, sizeof(double) * xg::kDotBlocksMax * 5 * xg::kDotBatch);
     if (e != cudaSuccess) {
@@ -584,16 +727,6 @@ cudaError_t prepare(xg_ctx* c, int m, cudaStream_t st) {
     }
   }
   xg::k_lin_levels<<<(c->n[2] + 127) / 128, 128, 0, st>>>(c->base64, c->n[2], c->P.gamma, X->cpl, X->th0);
-  const int ne = c->P.nseg[2] * (c->d.order + 1) * (c->d.order + 1);
-  const unsigned tblocks = (unsigned)((ne + 127) / 128);
-  switch (c->d.order) {
-#define XG_TABLES_CASE(N) \
-  case N: xg::k_lin_tables<N><<<tblocks, 128, 0, st>>>(c->P, X->cpl, X->th0, X->tw, X->tp); break;
-    XG_TABLES_CASE(1) XG_TABLES_CASE(2) XG_TABLES_CASE(3) XG_TABLES_CASE(4)
-    XG_TABLES_CASE(5) XG_TABLES_CASE(6) XG_TABLES_CASE(7) XG_TABLES_CASE(8)
-#undef XG_TABLES_CASE
-    default: return cudaErrorInvalidValue;
-  }
   return cudaGetLastError();
 }
 

@@ -55,7 +55,8 @@ inline void lgl_nodes(int N, long double* x) {
   x[N] = 1.0L;
 }
 
-inline void lgl_derivative(int N, double D[kMaxOrder + 1][kMaxOrder + 1]) {
+template <typename T>
+inline void lgl_derivative(int N, T D[kMaxOrder + 1][kMaxOrder + 1]) {
   long double x[kMaxOrder + 1], PN[kMaxOrder + 1];
   lgl_nodes(N, x);
   for (int j = 0; j <= N; ++j) {
@@ -69,12 +70,13 @@ inline void lgl_derivative(int N, double D[kMaxOrder + 1][kMaxOrder + 1]) {
       else if (i == 0) v = -(long double)N * (N + 1) / 4.0L;
       else if (i == N) v = (long double)N * (N + 1) / 4.0L;
       else v = 0.0L;
-      D[i][j] = (double)v;
+      D[i][j] = (T)v;
     }
 }
 
 // LGL weights w_j = 2 / (N (N+1) P_N(x_j)^2) at the points of lgl_derivative.
-inline void lgl_weights(int N, double* w) {
+template <typename T>
+inline void lgl_weights(int N, T* w) {
   const long double pi = 3.14159265358979323846264338327950288L;
   for (int j = 0; j <= N; ++j) {
     long double xj = -cosl(pi * j / N);
@@ -89,7 +91,7 @@ inline void lgl_weights(int N, double* w) {
     if (j == N) xj = 1.0L;
     long double pn, pn1;
     legendre2(N, xj, &pn, &pn1);
-    w[j] = (double)(2.0L / ((long double)N * (N + 1) * pn * pn));
+    w[j] = (T)(2.0L / ((long double)N * (N + 1) * pn * pn));
   }
 }
 
