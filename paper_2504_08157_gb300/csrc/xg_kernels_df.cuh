@@ -76,18 +76,17 @@ struct DfBufs {
 __device__ __forceinline__ df df_of_double(double x) {
   const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
   const int e = (int)((hi >> 20) & 0x7ffu);
-  const unsigned sign = hi & 0x80000000u;
-  if (e < 1023 - 100) return {__uint_as_float(sign), 0.0f};
-  if (e > 1023 + 127) return {__uint_as_float(sign | 0x7f800000u), 0.0f};
-  const unsigned top = ((hi & 0xfffffu) << 3) | (lo >> 29);
-  const float h = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | top);
-  float l = 0.0f;
-  if (e >= 949) {   // the remainder's scale 2^(e - 1075) is a normal float
-    l = __fmul_rn(__uint2float_rn(lo & 0x1fffffffu), __uint_as_float((unsigned)(e - 948) << 23));
-    if (sign) l = -l;
+  // the exponent's low 8 bits and 23 of the significand, moved to a float's
+  // places: its field is e - 896, which flips their top bit
+  const unsigned hb = ((__funnelshift_l(lo, hi, 3) ^ 0x40000000u) & 0x7fffffffu) | (hi & 0x80000000u);
+  if ((unsigned)(e - 949) > 1150u - 949u) {
+    if (e < 1023 - 100) return {__uint_as_float(hi & 0x80000000u), 0.0f};
+    if (e > 1023 + 127) return {__uint_as_float((hi & 0x80000000u) | 0x7f800000u), 0.0f};
+    return {__uint_as_float(hb), 0.0f};   // the remainder's scale is no normal float
   }
+  const float l = __fmul_rn(__uint2float_rn(lo & 0x1fffffffu), __uint_as_float((hb & 0xff800000u) - (52u << 23)));
   float s, t;
-  fast_two_sum(h, l, s, t);
+  fast_two_sum(__uint_as_float(hb), l, s, t);
   return {s, t};
 }
 
@@ -108,7 +107,7 @@ __device__ __forceinline__ double dbl_of_float(float f) {
 // unit in the last place of the double, far below the pair's own 2^-48).
 // Expects a normalised pair (|l| <= ulp(h)/2, as every double-float
 // operation returns).
-__device__ __forceinline__ double dbl_of_df(df a) {
+static __device__ __noinline__ double dbl_of_df_edge(df a) {
   const unsigned uh = __float_as_uint(a.h), ul = __float_as_uint(a.l);
   const int eh = (int)((uh >> 23) & 0xffu), el = (int)((ul >> 23) & 0xffu);
   if (eh == 0 || eh == 255 || el == 0) return dbl_of_float(a.h);
@@ -127,6 +126,21 @@ __device__ __forceinline__ double dbl_of_df(df a) {
   const unsigned long long bits = ((unsigned long long)(uh & 0x80000000u) << 32) |
                                   ((unsigned long long)(e + 896) << 52) | (M & ((1ull << 52) - 1));
   return __longlong_as_double((long long)bits);
+}
+
+// Away from the float range's ends, and but for a power of two less something,
+// the double of h plus or minus l's units is one 64-bit addition.
+__device__ __forceinline__ double dbl_of_df(df a) {
+  const unsigned uh = __float_as_uint(a.h), ul = __float_as_uint(a.l);
+  const int eh = (int)((uh >> 23) & 0xffu);
+  if ((unsigned)(eh - 56) >= 199u || ((uh & 0x7fffffu) == 0 && (int)(uh ^ ul) < 0)) return dbl_of_df_edge(a);
+  const int el = (int)((ul >> 23) & 0xffu);
+  unsigned L;   // l in units of the double's last place (0 for a shift above 31)
+  asm("shr.u32 %0, %1, %2;" : "=r"(L) : "r"(((ul & 0x7fffffu) | 0x800000u) << 5), "r"((unsigned)(eh - el - 24)));
+  const int s = (int)(uh ^ ul) >> 31;
+  const unsigned hi = (uh & 0x80000000u) | (((uh & 0x7fffffffu) >> 3) + (896u << 20));
+  const long long b = ((long long)hi << 32 | (long long)(unsigned long long)(uh << 29)) + (int)((L ^ (unsigned)s) - (unsigned)s);
+  return __longlong_as_double(b);
 }
 
 // (1+x)^gamma - 1 = x (c1 + x (c2 + x (c3 + x g(x)))), g = c4 + ... + c8 x^4
