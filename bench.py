@@ -51,11 +51,10 @@ TRAFFIC_FILE = os.path.join(ROOT, "profiles", "ncu_traffic.txt")
 KERNEL_SRCS = [os.path.join(ROOT, "paper_2504_08157_gb300", "csrc", f)
                for f in ("xg_kernels.cuh", "xg_kernels_df.cuh", "xg_df.cuh", "xg_kernels_f32.cuh",
                          "xg_plane_f32.cuh", "xg_batch.cu", "xg_closure.cu", "xg_tc.cuh", "xg_plane_tc.cuh",
-                         "xg_plane_h16.cuh", "xg_column_f32.cuh", "xg_tma.cuh")]
-KERNELS = ("k_line_x", "k_line_y", "k_line_z")
-# the kernels behind the three timing slots in each precision (the FP32 form
-# fuses the x and y passes into one plane kernel; slot 1 stays empty)
-KERNEL_NAMES = {0: ("k_line_x", "k_line_y", "k_line_z"),
+                         "xg_plane_h16.cuh", "xg_column_f32.cuh", "xg_tma.cuh", "xg_fixed.cuh", "xg_plane64.cuh")]
+# the kernels behind the three timing slots in each precision (FP64 and FP32
+# fuse the x and y passes into one plane kernel; slot 1 stays empty)
+KERNEL_NAMES = {0: ("k_plane_xy", "-", "k_tile_z"),
                 2: ("k_df_line_x", "k_df_tline_y", "k_df_tline_z"),
                 1: ("k_f_plane_xy", "-", "k_f_tline")}
 # the FP32 plane kernel of each tensor-core contraction mode (by --contraction
@@ -86,30 +85,19 @@ FP64_PIPE_PEAK_GINSTR = 152 * 2 * 2.07e9 / 1e9
 
 
 def flops_per_node(kernel, N):
-    """Algorithmic FP64 flops per unique node of each kernel (FMA = 2), from
-    the arithmetic each performs for N-th order elements (one segment of
-    N+1 nodes covers N unique nodes):
+    """Algorithmic flops on the FP64 pipe per unique node of each kernel (FMA =
+    2; the contractions run on the integer pipe):
 
-    * x: the even/odd contraction of one flux component over a segment,
-      2P adds + P (4P + 2e) + e (2P - 1) with P = (N+1)//2, e = [N even];
-      face sums 5/N; pointwise rho (1), 1/rho (4 fma), u v w (3),
-      Theta'/Theta0 (1), 8-term series (7 fma + 1 mul), p0 * (1), Theta (1),
-      x-fluxes (1 fma + 3 mul).
-    * y, z: N rows of N+1 fma started from the running tendency, row N
-      (1 mul + N fma) and the face addition: 2N^2 + 4N + 2 per component and
-      segment; fluxes (3 mul + 1 fma + 1 add).  z adds the sources (3 fma,
-      1 add, 1 fma) and the stage update (5 fma in stage 1, 5 x (2 fma +
-      1 mul) in stages 2-3, averaged)."""
-    P, e = (N + 1) // 2, 1 if N % 2 == 0 else 0
-    eo = 2 * P + P * (4 * P + 2 * e) + e * (2 * P - 1)
-    folded = 2 * N * N + 4 * N + 2
-    if kernel == "k_line_x":
-        pointwise = 1 + 8 + 3 + 1 + 15 + 1 + 1 + 1 + 5
-        return pointwise + 5.0 * eo / N + 5.0 / N
-    if kernel == "k_line_y":
-        return 6 + 5.0 * folded / N
-    if kernel == "k_line_z":
-        return 6 + 5.0 * folded / N + 9 + (10 + 25 + 25) / 3.0
+    * k_plane_xy: rho (1), 1/rho (4 fma), u v w (3), Theta'/Theta0 (1), 8-term
+      series (7 fma + 1 mul), p0 * (1), Theta (1), theta (1), fluxes (2 fma +
+      3 mul), y face sums 5/N.
+    * k_tile_z: fluxes (2 mul + 1 fma), T + rows (5) and face sums 5/N, sources
+      (4 fma + 1 add) and the stage update (5 fma in stage 1, 5 x (2 fma + 1 mul)
+      in stages 2-3, averaged)."""
+    if kernel == "k_plane_xy":
+        return 1 + 8 + 3 + 1 + 15 + 1 + 1 + 1 + 7 + 5.0 / N
+    if kernel == "k_tile_z":
+        return 4 + 5 + 5.0 / N + 9 + (10 + 25 + 25) / 3.0
     raise KeyError(kernel)
 
 
@@ -494,7 +482,9 @@ def make_ctx(xg, torch, wl, dev, precision=0):
 # stage output (5).  The FP32 plane pass (x and y fused) reads q and writes
 # W (3) and T; its z pass reads w and p' (no theta).
 _Z_VALUES = 5 + 3 + 5 + 1 + 5 * 2 / 3 + 5
-KERNEL_VALUES_PER_NODE = {"k_line_x": 14, "k_line_y": 16, "k_line_z": _Z_VALUES,
+KERNEL_VALUES_PER_NODE = {"k_line_x": 14, "k_line_y": 16, "k_line_z": _Z_VALUES,   # three split passes
+                          # the FP64 tiles also hand a plane of face rows on a y tile (8 lines at N = 4)
+                          "k_plane_xy": 13 + 5 / 8, "k_tile_z": _Z_VALUES + 5 / 8,
                           # the mixed path's y pass also writes, and its z pass reads, the rows of
                           # the y faces (5 values at one plane in N = 4, the bench order)
                           "k_df_line_x": 14, "k_df_tline_y": 16 + 5 / 4, "k_df_tline_z": _Z_VALUES + 5 / 4,
@@ -569,7 +559,6 @@ def run_xg(args, world, rank, local):
     # figure belongs to.  kernel_frac: the dominant kernel's own compulsory
     # bytes (its inputs and outputs, intermediates included) over its time.
     k = int(np.argmax(kms))
-    name = KERNELS[k]
     kname = knames[k]
     avg_ms = kms[k] / max(klaunch[k], 1)
     peaks = json.load(open(PEAKS_FILE)) if os.path.exists(PEAKS_FILE) else {}
@@ -594,7 +583,7 @@ def run_xg(args, world, rank, local):
             "kernel_bytes_per_node": round(KERNEL_VALUES_PER_NODE[kname] * vb, 2),
             "kernel_ms_per_launch": per_launch}
     if prec == xg.XG_FP64:
-        flops = flops_per_node(name, wl["N"]) * cfg["nodes"]
+        flops = flops_per_node(kname, wl["N"]) * cfg["nodes"]
         fach = flops / (avg_ms / 1e3) / 1e12
         roof["alu"] = {"kernel": kname, "achieved": round(fach, 4), "peak": round(FP64_PEAK_TFLOPS, 4),
                        "unit": "TFLOP/s", "frac": round(fach / FP64_PEAK_TFLOPS, 4),

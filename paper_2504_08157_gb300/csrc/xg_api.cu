@@ -105,7 +105,7 @@ __global__ void k_eos_check_f32(const xg::FParams P, const xg::df* __restrict__ 
 // Partition faces (values of 8 bytes: FP64 or double-float pairs).  Face
 // arrays are [5][n_z][n_x].  pack: the slab's first y plane of T (x part
 // plus row 0 of the first y segment) into out.  combine: the first plane
-// gets the left neighbour's row N (t0 + carry, the order of k_line_y at a
+// gets the left neighbour's row N (t0 + row N, the order of k_plane_xy at a
 // shared face), the last plane the right neighbour's t0 plus this slab's own
 // row N -- so both slabs hold bit for bit the value a single domain has.
 template <typename V>
@@ -265,32 +265,65 @@ void prof_fold(xg_ctx* c) {
   c->ev_used = 0;
 }
 
-// parts: bit 0 the x and y passes, bit 1 the z pass (a partitioned stage
-// exchanges the partition faces' rows in between)
+// The x-y pass of an FP64-state stage.
+template <int N, typename Params, typename Bufs>
+void launch_plane_n(xg_ctx* c, const Params& P, const Bufs& B, cudaStream_t st) {
+  using L = xg::XYTile<N>;
+  const dim3 g((c->d.nel[0] + L::EX - 1) / L::EX, B.nty, c->n[2]);
+  prof_mark(c, 0, false, st);
+  xg::k_plane_xy<N><<<g, L::threads(c->tile_ey), L::bytes, st>>>(P, B, c->tile_ey);
+  prof_mark(c, 0, true, st);
+}
+
+// parts: bit 0 the x-y pass, bit 1 the z pass (a partitioned stage exchanges
+// the partition faces' rows in between)
 template <int N>
 void launch_stage_n(xg_ctx* c, const StageBufs& B, cudaStream_t st, int parts) {
-  if (parts & 1) {
-    dim3 gx(c->n[1], c->n[2]);
-    prof_mark(c, 0, false, st);
-    xg::k_line_x<N><<<gx, xg::kXThreads, c->xsmem, st>>>(c->P, B);
-    prof_mark(c, 0, true, st);
-    dim3 gy((c->n[0] + 127) / 128, c->nchunk_y, c->n[2]);
-    prof_mark(c, 1, false, st);
-    xg::k_line_y<N><<<gy, 128, 0, st>>>(c->P, B, c->chunk_y);
-    prof_mark(c, 1, true, st);
+  if (parts & 1) launch_plane_n<N>(c, c->P64, B, st);
+  if (parts & 2) {
+    constexpr int K = xg::z_tile_segments(N);
+    const dim3 gz((c->n[0] + xg::kTileCols - 1) / xg::kTileCols, (c->d.nel[2] + K - 1) / K, c->n[1]);
+    prof_mark(c, 2, false, st);
+    xg::k_tile_z<N><<<gz, dim3(xg::kTileCols, K * N + 1), 0, st>>>(c->P64, B);
+    prof_mark(c, 2, true, st);
+  }
+}
+
+template <int N>
+void launch_stage_n(xg_ctx* c, const DfBufs& B, cudaStream_t st, int parts) {
+  const unsigned xb = (c->n[0] + xg::kTileCols - 1) / xg::kTileCols;
+  if ((parts & 1) && c->df_plane) {
+    launch_plane_n<N>(c, c->Ptile, B, st);
+  } else if (parts & 1) {
+    if constexpr (N <= xg::kDfLineOrder) {
+      dim3 gx(c->n[1], c->n[2]);
+      prof_mark(c, 0, false, st);
+      xg::k_df_line_x<N><<<gx, xg::kXThreads, xg::df_x_smem(c->n[0], c->d.nel[0]), st>>>(c->Pdf, B);
+      prof_mark(c, 0, true, st);
+      constexpr int K = xg::df_tile_segments(N, 1);
+      const dim3 blk(xg::kTileCols, K * N + 1);
+      dim3 gy(xb, (c->d.nel[1] + K - 1) / K, c->n[2]);
+      prof_mark(c, 1, false, st);
+      xg::k_df_tline<N, 1><<<gy, blk, 0, st>>>(c->Pdf, B);
+      prof_mark(c, 1, true, st);
+    }
   }
   if (parts & 2) {
-    dim3 gz((c->n[0] + 127) / 128, c->nchunk_z, c->n[1]);
+    constexpr int K = xg::df_tile_segments(N, 2);
+    const dim3 blk(xg::kTileCols, K * N + 1);
+    dim3 gz(xb, (c->d.nel[2] + K - 1) / K, c->n[1]);
     prof_mark(c, 2, false, st);
-    xg::k_line_z<N><<<gz, 128, 0, st>>>(c->P, B, c->chunk_z);
+    xg::k_df_tline<N, 2><<<gz, blk, 0, st>>>(c->Pdf, B);
     prof_mark(c, 2, true, st);
   }
 }
 
 template <int N>
 cudaError_t configure_n(xg_ctx* c) {
-  cudaError_t e = xg::raise_dynamic_smem(xg::k_line_x<N>, c->xsmem);
-  if (e == cudaSuccess) e = xg::raise_dynamic_smem(xg::k_df_line_x<N>, c->xsmem);
+  cudaError_t e = xg::raise_dynamic_smem(xg::k_plane_xy<N, xg::F64Params>, xg::XYTile<N>::bytes);
+  if (e == cudaSuccess) e = xg::raise_dynamic_smem(xg::k_plane_xy<N, xg::DfTileParams>, xg::XYTile<N>::bytes);
+  if constexpr (N <= xg::kDfLineOrder)
+    if (e == cudaSuccess) e = xg::raise_dynamic_smem(xg::k_df_line_x<N>, xg::df_x_smem(c->n[0], c->d.nel[0]));
   if (e == cudaSuccess) e = xg::raise_dynamic_smem(xg::k_f_plane_xy<N>, xg::PlaneLayoutF<N>::bytes);
   if (N == xg::PlaneTcLayout::N && e == cudaSuccess)
     e = xg::raise_dynamic_smem(xg::k_f_plane_xy_tc, xg::PlaneTcLayout::bytes);
@@ -304,32 +337,6 @@ cudaError_t configure_n(xg_ctx* c) {
                                100);
   }
   return e;
-}
-
-template <int N>
-void launch_df_stage_n(xg_ctx* c, const DfBufs& B, cudaStream_t st, int parts) {
-  if (parts & 1) {
-    dim3 gx(c->n[1], c->n[2]);
-    prof_mark(c, 0, false, st);
-    xg::k_df_line_x<N><<<gx, xg::kXThreads, c->xsmem, st>>>(c->Pdf, B);
-    prof_mark(c, 0, true, st);
-    constexpr int K = xg::df_tile_segments(N, 1);
-    const dim3 blk(xg::kTileCols, K * N + 1);
-    const unsigned xb = (c->n[0] + xg::kTileCols - 1) / xg::kTileCols;
-    dim3 gy(xb, (c->d.nel[1] + K - 1) / K, c->n[2]);
-    prof_mark(c, 1, false, st);
-    xg::k_df_tline<N, 1><<<gy, blk, 0, st>>>(c->Pdf, B);
-    prof_mark(c, 1, true, st);
-  }
-  if (parts & 2) {
-    constexpr int K = xg::df_tile_segments(N, 2);
-    const dim3 blk(xg::kTileCols, K * N + 1);
-    const unsigned xb = (c->n[0] + xg::kTileCols - 1) / xg::kTileCols;
-    dim3 gz(xb, (c->d.nel[2] + K - 1) / K, c->n[1]);
-    prof_mark(c, 2, false, st);
-    xg::k_df_tline<N, 2><<<gz, blk, 0, st>>>(c->Pdf, B);
-    prof_mark(c, 2, true, st);
-  }
 }
 
 // The fused column pass applies: FP32 form, order 4, the CUDA-core
@@ -409,22 +416,8 @@ cudaError_t launch_f32_stage(xg_ctx* c, const xg::FBufs& B, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_df_stage(xg_ctx* c, const DfBufs& B, cudaStream_t st, int parts) {
-  switch (c->d.order) {
-    case 1: launch_df_stage_n<1>(c, B, st, parts); break;
-    case 2: launch_df_stage_n<2>(c, B, st, parts); break;
-    case 3: launch_df_stage_n<3>(c, B, st, parts); break;
-    case 4: launch_df_stage_n<4>(c, B, st, parts); break;
-    case 5: launch_df_stage_n<5>(c, B, st, parts); break;
-    case 6: launch_df_stage_n<6>(c, B, st, parts); break;
-    case 7: launch_df_stage_n<7>(c, B, st, parts); break;
-    case 8: launch_df_stage_n<8>(c, B, st, parts); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_stage(xg_ctx* c, const StageBufs& B, cudaStream_t st, int parts) {
+template <typename Bufs>
+cudaError_t launch_stage(xg_ctx* c, const Bufs& B, cudaStream_t st, int parts) {
   switch (c->d.order) {
     case 1: launch_stage_n<1>(c, B, st, parts); break;
     case 2: launch_stage_n<2>(c, B, st, parts); break;
@@ -469,6 +462,9 @@ StageBufs make_bufs(xg_ctx* c, const double* q, const double* qn, double* out, d
   B.beta = beta;
   B.rhs_only = rhs_only;
   B.face_hi = c->part_send[1];
+  B.Fy = c->Fy;
+  B.fy = c->fy;
+  B.nty = c->nty;
   return B;
 }
 
@@ -533,7 +529,9 @@ cudaError_t run_stage(xg_ctx* c, const void* q, const void* qn, void* out, doubl
   B.rhs_only = rhs_only;
   B.face_hi = c->part_send[1];
   B.Fy = c->Fy;
-  return launch_df_stage(c, B, st, parts);
+  B.fy = c->fy;
+  B.nty = c->nty;
+  return launch_stage(c, B, st, parts);
 }
 
 // Device FP64 array -> the context's device representation (n values; FP64
@@ -585,14 +583,12 @@ xg_status xg_mesh_create(const xg_mesh_desc* d, xg_ctx** out) {
   if (st != XG_OK) return st;
   const int* n = geo.n;
   const long long np = geo.np;
-  const size_t xsmem = geo.xsmem;
 
   xg_ctx* c = new (std::nothrow) xg_ctx();
   if (!c) return XG_ERR_OOM;
   c->d = *d;
   c->n[0] = n[0]; c->n[1] = n[1]; c->n[2] = n[2];
   c->np = np;
-  c->xsmem = xsmem;
   cudaError_t e = cudaGetDevice(&c->dev);
   if (e != cudaSuccess) { fail_cuda(c, e, "cudaGetDevice"); delete c; return XG_ERR_CUDA; }
   int sms = 0;
@@ -603,9 +599,21 @@ xg_status xg_mesh_create(const xg_mesh_desc* d, xg_ctx** out) {
   xg::fill_line_params(d, geo, &c->P);
   c->dfm = d->precision == XG_DF64;
   c->f32 = d->precision == XG_FP32;
-  if (c->dfm) xg::fill_df_params(c->P, &c->Pdf);
+  c->P64.P64 = c->P;
+  xg::fill_fix_params(d, c->P64.F);
+  if (c->dfm) {
+    xg::fill_df_params(c->P, &c->Pdf);
+    c->Ptile.D = c->Pdf;
+    for (int k = 0; k < 2; ++k) c->Ptile.F[k] = c->P64.F[k];
+  }
   if (c->f32) xg::fill_f32_params(c->P, &c->Pf);
-  xg::plan_marches(d, geo, sms, &c->chunk_y, &c->nchunk_y, &c->chunk_z, &c->nchunk_z);
+  c->tile_ey = xg::xy_tile_rows(d->order, d->nel, n[2], sms);
+  c->df_plane = xg::df_uses_plane(d->order, geo.n);
+  const int ey = c->dfm && !c->df_plane ? xg::df_tile_segments(d->order, 1) : c->tile_ey;
+  c->fy = ey * d->order;
+  // (y tiles of the line kernels hand their row N on by way of Fy also where
+  // one tile closes on itself, which a count above 1 says)
+  c->nty = (d->nel[1] + ey - 1) / ey + (c->dfm && !c->df_plane ? 1 : 0);
 
   const size_t vec = sizeof(double) * (size_t)np;
   struct { double** p; size_t bytes; } allocs[] = {
@@ -621,8 +629,8 @@ xg_status xg_mesh_create(const xg_mesh_desc* d, xg_ctx** out) {
     }
   }
   e = cudaMalloc((void**)&c->flag, sizeof(int));
-  if (e == cudaSuccess && c->dfm)
-    e = cudaMalloc((void**)&c->Fy, sizeof(double) * 5 * (size_t)c->P.nseg[1] * (size_t)n[2] * (size_t)n[0]);
+  if (e == cudaSuccess && !c->f32)
+    e = cudaMalloc((void**)&c->Fy, sizeof(double) * 5 * (size_t)c->nty * (size_t)n[2] * (size_t)n[0]);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hflag, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->wasm, sizeof(double) * (size_t)(n[0] + n[1] + n[2]));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->partial, sizeof(double) * 5 * kDiagBlocks);
@@ -1061,8 +1069,9 @@ xg_status xg_partition_set(xg_ctx* c, int open_lo, int open_hi, double* send_lo,
   c->part_recv[0] = open_lo ? recv_lo : nullptr;
   c->part_send[1] = open_hi ? send_hi : nullptr;
   c->part_recv[1] = open_hi ? recv_hi : nullptr;
-  c->P.open_y[0] = c->Pdf.open_y[0] = c->Pdf.P64.open_y[0] = open_lo;
-  c->P.open_y[1] = c->Pdf.open_y[1] = c->Pdf.P64.open_y[1] = open_hi;
+  c->P.open_y[0] = c->P64.P64.open_y[0] = c->Pdf.open_y[0] = c->Pdf.P64.open_y[0] = open_lo;
+  c->P.open_y[1] = c->P64.P64.open_y[1] = c->Pdf.open_y[1] = c->Pdf.P64.open_y[1] = open_hi;
+  c->Ptile.D = c->Pdf;
   return XG_OK;
 }
 

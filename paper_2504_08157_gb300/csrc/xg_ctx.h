@@ -13,6 +13,7 @@
 #include "xg_kernels.cuh"
 #include "xg_kernels_df.cuh"
 #include "xg_kernels_f32.cuh"
+#include "xg_plane64.cuh"
 
 struct xg_ctx {
   xg_mesh_desc d;
@@ -21,7 +22,9 @@ struct xg_ctx {
   int dev;
   int sms = 1;           // the device's SM count
   xg::LineParams P;
+  xg::F64Params P64;     // launch constants of the FP64 stage kernels
   xg::DfParams Pdf;      // launch constants of the double-float kernels
+  xg::DfTileParams Ptile;  // and of the mixed x-y tiles
   xg::FParams Pf;        // launch constants of the FP32 kernels
   bool dfm = false;      // precision XG_DF64: FP64 arrays, mixed FP64 / double-float kernels
   bool f32 = false;      // precision XG_FP32: device arrays hold floats
@@ -47,9 +50,9 @@ struct xg_ctx {
   double* Bq = nullptr;  // stage buffer
   double* Cq = nullptr;  // stage buffer
   double* Dq = nullptr;  // q^{n+1}; swapped with A after every step
-  double* W = nullptr;   // [4][np] primitives v, w, p', theta (FP32: [3][np])
+  double* W = nullptr;   // [4][np] primitives: w, p', theta in rows 1..3 (FP32: v, w, p' in [3][np])
   double* T = nullptr;   // [5][np] partial tendency
-  double* Fy = nullptr;  // XG_DF64: [5][nseg_y][nz][nx] y-face rows between the y and z passes
+  double* Fy = nullptr;  // FP64 states: [5][y tiles][nz][nx] y-face rows between the x-y and z passes
   double* S = nullptr;   // [np] heating
   double* base = nullptr;  // [4][nz] (double-float pairs for XG_DF64 and XG_FP32)
   double* base64 = nullptr;  // [4][nz] the same table in FP64
@@ -62,8 +65,9 @@ struct xg_ctx {
   bool has_base = false;
   bool has_forcing = false;
   bool failed = false;
-  int chunk_y = 1, nchunk_y = 1, chunk_z = 1, nchunk_z = 1;
-  size_t xsmem = 0;
+  int tile_ey = 1;       // element rows of the FP64 states' x-y tiles
+  bool df_plane = false; // XG_DF64: the x-y tiles instead of the x and y lines
+  int fy = 1, nty = 1;   // lines of a y tile, tiles (Fy)
   // profiling: event pairs recorded around launches since the last fold
   bool profiling = false;
   std::vector<cudaEvent_t> events;

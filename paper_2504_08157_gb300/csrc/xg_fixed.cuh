@@ -325,6 +325,83 @@ inline int fix_z_chunk(int nseg, long long columns, int sms) {
   return (int)((nseg + chunks - 1) / chunks);
 }
 
+// ---------------------------------------------------------------- fluxes
+// exponent field of v, 0 for an infinity or NaN
+__device__ __forceinline__ int fix_exp_finite(double v, bool& bad) {
+  const int e = fix_exp(v);
+  const bool b = e == kFixNonfinite;
+  bad |= b;
+  return b ? 0 : e;
+}
+
+__device__ __forceinline__ bool fix_bad(double v) { return fix_exp(v) == kFixNonfinite; }
+
+constexpr int kFixMark = (int)0x80000000;   // high limb of a value without an exponent: |h| < 2^31 for all others
+
+__device__ __forceinline__ unsigned long long fix_shr(unsigned long long m, unsigned s) {
+  unsigned long long v;
+  asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(s));   // clamps: 0 for s >= 64
+  return v;
+}
+
+__device__ __forceinline__ fix2 fix_limbs(unsigned long long V, int sg) {
+  return {(int)(V >> 30) * sg, (int)((unsigned)V & 0x3fffffffu) * sg};
+}
+
+// a b in limbs of a block whose exponent fields of a and b add up to G at
+// most: |a b| 2^(B - 2 - (G - 2046)) cut to an integer (values below 2^-1022
+// count as zero).
+template <int N>
+__device__ __forceinline__ fix2 fix_prod(double a, double b, int G) {
+  const unsigned ah = (unsigned)__double2hiint(a), al = (unsigned)__double2loint(a);
+  const unsigned bh = (unsigned)__double2hiint(b), bl = (unsigned)__double2loint(b);
+  const unsigned ea = (ah >> 20) & 0x7ffu, eb = (bh >> 20) & 0x7ffu;
+  // mantissas with their leading bit at 2^63
+  const unsigned A1 = __funnelshift_l(al, (ah & 0xfffffu) | 0x100000u, 11), A0 = al << 11;
+  const unsigned B1 = __funnelshift_l(bl, (bh & 0xfffffu) | 0x100000u, 11), B0 = bl << 11;
+  unsigned long long P = (unsigned long long)A1 * B1 + __umulhi(A1, B0) + __umulhi(A0, B1);
+  if (ea == 0 || eb == 0) P = 0;
+  return fix_limbs(fix_shr(P, (unsigned)(64 - fix_bits(N) + G) - (ea + eb)), ((int)(ah ^ bh) >> 31) | 1);
+}
+
+// Block exponents usable with rows of scale sc (for fix_prod's sums of two
+// fields), and the exponent field of the unit 2^(60 - sc - sv) of its rows.
+template <int N>
+__device__ __forceinline__ int fix_prod_exp(int G, int sc) { return max(G, 962 + fix_bits(N) + sc); }
+template <int N>
+__device__ __forceinline__ int fix_field(int E, int sc) { return E + 61 - fix_bits(N) - sc; }
+template <int N>
+__device__ __forceinline__ int fix_prod_field(int G, int sc) { return G - 961 - fix_bits(N) - sc; }
+
+// r 2^(u - 1023) as an FP64 value, rounded to nearest, in integer operations
+// (I2F.F64 and the scaling product would cost two at the FP64 rate); u >= 1,
+// |r| < 2^63.
+__device__ __forceinline__ void fix_value(long long r, int u, double& out) {
+  const int sg = (int)(r >> 63);
+  const unsigned long long m = (unsigned long long)((r ^ sg) - sg);
+  const int n = __clzll((long long)m);
+  const unsigned long long a = m << (n & 63);
+  const unsigned long long b = (a >> 11) + ((a >> 10) & 1ull);      // 2^52 .. 2^53
+  const int e = u + 62 - n;
+  unsigned long long bits = ((unsigned long long)(unsigned)e << 52) + b;
+  if (e >= 2046) bits = 0x7ff0000000000000ull;
+  if (m == 0) bits = 0;
+  out = __hiloint2double((int)((unsigned)(bits >> 32) | ((unsigned)sg & 0x80000000u)), (int)(unsigned)bits);
+}
+
+__device__ __forceinline__ double xg_nan(double) { return __hiloint2double(0x7ff80000, 0); }
+
+// r 2^(u - 1023) for the form at hand: the FP64 form, bound by the FP64 pipe,
+// converts in integer operations; the mixed one, bound by issue slots, spends
+// two FP64 operations.
+template <bool MIXED>
+__device__ __forceinline__ double fix_out(long long r, int u) {
+  double v;
+  if (MIXED) v = (double)r * __hiloint2double(min(u, 2046) << 20, 0);
+  else fix_value(r, u, v);
+  return v;
+}
+
 #endif  // __CUDACC__
 
 }  // namespace xg

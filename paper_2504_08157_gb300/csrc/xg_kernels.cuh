@@ -1,4 +1,6 @@
-// xg_kernels.cuh -- FP64 line kernels of the explicit CG Euler path (sm_103a).
+// xg_kernels.cuh -- what the FP64-state kernels of the explicit CG Euler path share
+// (sm_103a): launch constants, the equation of state, the FP64 contractions, and
+// the completion of a node.
 //
 // The right-hand side of Sec. 2.1 (Eq. 1 restated for q = (rho', rho u,
 // rho v, rho w, Theta'), pressure from Eq. 3) is evaluated by the collocated
@@ -14,30 +16,26 @@
 // cancel against M.  This is the paper's gather/assembly/scatter of
 // Alg. 1-3, reached without element-local storage and without atomics.
 //
-// One stage = three kernels over the SoA state:
-//   k_line_x  one CTA per x-line: pointwise primitives (u, v, w, p') of every
-//             node, x-fluxes staged in shared memory, one thread per element
-//             segment for the 1-D contraction (Alg. 2), face averaging;
-//             writes the x part of the tendency to T and (v, w, p', theta =
-//             Theta/rho) to W.
-//   k_line_y  one thread per (x, z) column marching along y over a chunk of
-//             element segments, carrying the shared face node's flux and
-//             one-sided derivative; adds the y part into T.
-//   k_line_z  one thread per (x, y) column marching along z; adds the z part,
-//             the sources (-rho' g k, -f k x rho u, rho S_theta), applies
-//             no-flux walls and either stores dq/dt or the fused SSP-RK
-//             stage combination out = alpha q^n + beta (q + dt L(q)) into a
-//             buffer distinct from every input.
+// A stage of an XG_FP64 context is two kernels over the SoA state
+// (xg_plane64.cuh), with the contractions in 64-bit fixed point:
+//   k_plane_xy  tiles of a level: pointwise primitives (w, p', theta =
+//               Theta/rho to W), x and y fluxes, the x + y part of the tendency
+//               to T;
+//   k_tile_z    32 columns by a few element segments: z fluxes, the z part,
+//               the sources (-rho' g k, -f k x rho u, rho S_theta), no-flux
+//               walls, and either dq/dt or the fused SSP-RK stage combination
+//               out = alpha q^n + beta (q + dt L(q)) into a buffer distinct from
+//               every input.
+// XG_DF64 contexts have kernels of their own (xg_kernels_df.cuh) or the first
+// of these in mixed arithmetic.
 //
-// Every arithmetic step is FP64.  The derivative matrices come pre-scaled by
-// -2/h_d (chain rule of the affine map, sign of the divergence) with rows 0
-// and N halved for the face average; wall nodes undo the halving.  The FP64
-// pipe (2 DFMA/clk/SM on GB300) bounds these kernels, so the arithmetic is
-// arranged to spend few FP64 instructions: the running tendency is the
-// starting value of each contraction's FMA chain (no separate additions), the
-// x contraction uses the even/odd split of the centro-antisymmetric LGL
-// derivative matrix, 1/rho is one hardware reciprocal estimate refined by
-// two Newton steps, and the equation of state is a short binomial series.
+// The derivative matrices come pre-scaled by -2/h_d (chain rule of the affine
+// map, sign of the divergence) with rows 0 and N halved for the face average;
+// wall nodes undo the halving.  The FP64 pipe (2 DFMA/clk/SM on GB300) bounds
+// what runs on it, so the arithmetic is arranged to spend few FP64 instructions:
+// 1/rho is one hardware reciprocal estimate refined by two Newton steps, the
+// equation of state is a short binomial series, and the FP64 contraction of the
+// mixed x pass uses the even/odd split of the centro-antisymmetric LGL matrix.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -47,6 +45,7 @@ namespace xg {
 
 constexpr int kMaxOrder = 8;
 constexpr int kMaxPairs = (kMaxOrder + 1) / 2;
+constexpr int kXThreads = 128;
 constexpr int kEosTerms = 8;
 
 // Launch-time constants of one mesh (passed by value as a kernel parameter).
@@ -83,7 +82,7 @@ struct StageBufs {
   const double* q;      // [5][np] state the tendency is taken of
   const double* qn;     // [5][np] q^n of the RK combination (alpha != 0)
   double* out;          // [5][np] new state, or dq/dt when rhs_only
-  double* W;            // [4][np] v, w, p', theta = Theta/rho (written by k_line_x)
+  double* W;            // [4][np]: w, p', theta = Theta/rho in rows 1..3 (written by k_plane_xy)
   double* T;            // [5][np] x + y parts of the tendency
   const double* S;      // [np] heating S_theta (K/s)
   const double* base;   // [4][nz]: rho0, Theta0, p0, 1/Theta0 per level
@@ -92,9 +91,13 @@ struct StageBufs {
   int rhs_only;
   const double* E = nullptr;  // [5][np] extra tendency (hyper-diffusion, sponge) or null
   // open_y[1]: the one-sided row N of the slab's last y segment at every
-  // (x, z) of the end face, [5][n_z][n_x] (written by k_line_y instead of the
+  // (x, z) of the end face, [5][n_z][n_x] (written by k_plane_xy instead of the
   // wall's doubled row)
   double* face_hi = nullptr;
+  // row N of the y segment that ends at each y tile's first line, written by
+  // the x-y pass and added by the z pass: [5][nty][n_z][n_x], fy lines a tile
+  double* Fy = nullptr;
+  int fy = 1, nty = 1;
 };
 
 // (1 + x)^gamma - 1: the binomial series (Horner) for small |x|, where the
@@ -160,24 +163,6 @@ __device__ __forceinline__ void contract_eo(const LineParams& P, const double (&
   }
 }
 
-// start + sum_l Dm[d][a][l] f[l] as one FMA chain (N+1 operations).
-template <int N, int D>
-__device__ __forceinline__ double row_from(const LineParams& P, int a, const double (&f)[N + 1],
-                                           double start) {
-  double acc = start;
-#pragma unroll
-  for (int l = 0; l <= N; ++l) acc = fma(P.Dm[D][a][l], f[l], acc);
-  return acc;
-}
-
-template <int N, int D>
-__device__ __forceinline__ double row_N(const LineParams& P, const double (&f)[N + 1]) {
-  double acc = P.Dm[D][N][0] * f[0];
-#pragma unroll
-  for (int l = 1; l <= N; ++l) acc = fma(P.Dm[D][N][l], f[l], acc);
-  return acc;
-}
-
 // ---------------------------------------------------------------- difference form
 // The rho' and Theta' tendencies are residuals of cancelling flux
 // derivatives where the flow is nearly non-divergent (in a vortex the x and
@@ -226,398 +211,47 @@ __device__ __forceinline__ double drow_N(const LineParams& P, const double (&d)[
   return acc;
 }
 
-// ---------------------------------------------------------------- x lines
-// grid (n_y, n_z), block kXThreads, dynamic shared memory
-// 8 * (5 (n_x + 1) + 5 nseg_x) bytes.
-constexpr int kXThreads = 128;
-
-template <int N>
-__global__ void __launch_bounds__(kXThreads) k_line_x(const LineParams P, const StageBufs B) {
-  extern __shared__ double sm[];
-  const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
-  const int nseg = P.nseg[0];
-  const int y = blockIdx.x, z = blockIdx.y;
-  const long long np = P.np;
-  const long long row = (long long)nx * (y + (long long)ny * z);
-  const int ld = nx + 1;
-  // F [5][ld]: x-fluxes of the line's nodes (+ periodic wrap slot); later
-  // each segment's one-sided rows 0..N-1 in place.  RN [5][nseg]: row N.
-  double* F = sm;
-  double* RN = sm + 5 * ld;
-  const double rho0 = __ldg(B.base + z);
-  const double Th0 = __ldg(B.base + nz + z);
-  const double p0 = __ldg(B.base + 2 * nz + z);
-  const double iTh0 = __ldg(B.base + 3 * nz + z);
-  const double* __restrict__ q = B.q;
-  double* __restrict__ Wo = B.W;
-  double* __restrict__ To = B.T;
-
-  // pointwise primitives and x-fluxes, one node per thread (coalesced)
-  for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-    const long long I = row + i;
-    const double rp = q[I], mu = q[np + I], mv = q[2 * np + I], mw = q[3 * np + I];
-    const double tp = q[4 * np + I];
-    const double ir = rcp_newton(rho0 + rp);
-    const double u = mu * ir, v = mv * ir, w = mw * ir;
-    const double pp = p0 * eos_phi(P, tp * iTh0);
-    const double Th = Th0 + tp;
-    const double th = Th * ir;
-    Wo[I] = v;
-    Wo[np + I] = w;
-    Wo[2 * np + I] = pp;
-    Wo[3 * np + I] = th;
-    F[i] = mu;
-    F[ld + i] = fma(mu, u, pp);
-    F[2 * ld + i] = mv * u;
-    F[3 * ld + i] = mw * u;
-    F[4 * ld + i] = th;              // theta: the Theta' flux is theta (rho u)
-    if (P.per[0] && i == 0) {
-      F[nx] = F[0];
-      F[ld + nx] = F[ld];
-      F[2 * ld + nx] = F[2 * ld];
-      F[3 * ld + nx] = F[3 * ld];
-      F[4 * ld + nx] = F[4 * ld];
-    }
-  }
-  __syncthreads();
-
-  // one element segment per thread: even/odd contraction per flux component;
-  // every segment is read before any is overwritten (the loop below keeps
-  // each thread's segments in registers when nseg <= blockDim, the usual
-  // case; otherwise segments are processed in rounds with a barrier)
-  for (int s0 = 0; s0 < nseg; s0 += blockDim.x) {
-    const int s = s0 + threadIdx.x;
-    double rows[5][N + 1];
-    if (s < nseg) {
-      {   // rho' and Theta' in difference form
-        double m[N + 1], th[N + 1], dm[N + 1], dF[N + 1];
-#pragma unroll
-        for (int l = 0; l <= N; ++l) {
-          m[l] = F[s * N + l];
-          th[l] = F[4 * ld + s * N + l];
-        }
-        seg_diffs<N>(m, th, dm, dF);
-        contract_eo<N, 0>(P, dm, rows[0]);
-        contract_eo<N, 0>(P, dF, rows[4]);
-      }
-#pragma unroll
-      for (int c = 1; c < 4; ++c) {
-        double f[N + 1];
-#pragma unroll
-        for (int l = 0; l <= N; ++l) f[l] = F[c * ld + s * N + l];
-        contract_eo<N, 0>(P, f, rows[c]);
-      }
-    }
-    __syncthreads();
-    if (s < nseg) {
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-#pragma unroll
-        for (int a = 0; a < N; ++a) F[c * ld + s * N + a] = rows[c][a];
-        RN[c * nseg + s] = rows[c][N];
-      }
-    }
-    __syncthreads();
-  }
-
-  // assemble: face nodes add both one-sided halves, wall nodes double theirs
-  for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-    const int s = i / N, a = i - s * N;
-    const long long I = row + i;
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      double v;
-      if (s == nseg) {                     // last wall node
-        v = RN[c * nseg + nseg - 1];
-        v = v + v;
-      } else if (a != 0) {
-        v = F[c * ld + i];
-      } else {
-        const double r0 = F[c * ld + i];
-        const int left = s > 0 ? s - 1 : (P.per[0] ? nseg - 1 : -1);
-        v = r0 + (left >= 0 ? RN[c * nseg + left] : r0);
-      }
-      To[c * np + I] = v;
-    }
-  }
-}
-
-// ---------------------------------------------------------------- y lines
-// grid (ceil(n_x / blockDim), nchunk, n_z); each thread marches `chunk`
-// element segments along y at its (x, z).
-// y-fluxes at one node; slot 4 holds theta (the Theta' flux theta (rho v)
-// is taken in difference form with slot 0)
-__device__ __forceinline__ void flux_y(const double* __restrict__ q, const double* __restrict__ W,
-                                       long long np, long long I, double (&f)[5]) {
-  const double mu = q[np + I], mv = q[2 * np + I], mw = q[3 * np + I];
-  const double v = W[I], pp = W[2 * np + I];
-  f[0] = mv;
-  f[1] = mu * v;
-  f[2] = fma(mv, v, pp);
-  f[3] = mw * v;
-  f[4] = W[3 * np + I];
-}
-
-template <int N>
-__global__ void __launch_bounds__(128) k_line_y(const LineParams P, const StageBufs B, int chunk) {
-  const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
-  const int nseg = P.nseg[1];
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= nx) return;
-  const int z = blockIdx.z;
-  const int s0 = blockIdx.y * chunk;
-  const int s1 = min(nseg, s0 + chunk);
-  if (s0 >= s1) return;
-  const long long np = P.np;
-  const long long col = x + (long long)nx * ny * z;
-  const double* __restrict__ q = B.q;
-  const double* __restrict__ W = B.W;
-  auto nodeI = [&](int gy) -> long long { return col + (long long)nx * (gy == ny ? 0 : gy); };
-
-  double carry[5];
-  bool has_left = (s0 > 0) || P.per[1];
-  if (has_left) {
-    const int sp = s0 > 0 ? s0 - 1 : nseg - 1;
-    double fl[5][N + 1];
-#pragma unroll
-    for (int l = 0; l <= N; ++l) {
-      double f[5];
-      flux_y(q, W, np, nodeI(sp * N + l), f);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) fl[c][l] = f[c];
-    }
-    double dm[N + 1], dF[N + 1];
-    seg_diffs<N>(fl[0], fl[4], dm, dF);
-    carry[0] = drow_N<N, 1>(P, dm);
-    carry[4] = drow_N<N, 1>(P, dF);
-#pragma unroll
-    for (int c = 1; c < 4; ++c) carry[c] = row_N<N, 1>(P, fl[c]);
-  }
-
-  double fc[5][N + 1];
-  {
-    double f[5];
-    flux_y(q, W, np, nodeI(s0 * N), f);
-#pragma unroll
-    for (int c = 0; c < 5; ++c) fc[c][0] = f[c];
-  }
-  double* __restrict__ T = B.T;
-  for (int s = s0; s < s1; ++s) {
-#pragma unroll
-    for (int l = 1; l <= N; ++l) {
-      double f[5];
-      flux_y(q, W, np, nodeI(s * N + l), f);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) fc[c][l] = f[c];
-    }
-    double dm[N + 1], dF[N + 1];
-    seg_diffs<N>(fc[0], fc[4], dm, dF);
-    // row a of variable c from start (rho' and Theta' in difference form)
-    auto rowc = [&](int c, int a, double start) -> double {
-      if (c == 0) return drow_from<N, 1>(P, a, dm, start);
-      if (c == 4) return drow_from<N, 1>(P, a, dF, start);
-      return row_from<N, 1>(P, a, fc[c], start);
-    };
-    // the segment's running x parts, all loaded before any store
-    double tv[5][N];
-#pragma unroll
-    for (int a = 0; a < N; ++a) {
-      const long long I = nodeI(s * N + a);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) tv[c][a] = T[c * np + I];
-    }
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      // the running x part is the start of each row's FMA chain
-      double t0 = tv[c][0];
-      if (!has_left && !P.open_y[0]) t0 = rowc(c, 0, t0);   // wall: the row counts twice
-      t0 = rowc(c, 0, t0);
-      T[c * np + nodeI(s * N)] = has_left ? t0 + carry[c] : t0;
-#pragma unroll
-      for (int a = 1; a < N; ++a) T[c * np + nodeI(s * N + a)] = rowc(c, a, tv[c][a]);
-      carry[c] = c == 0 ? drow_N<N, 1>(P, dm) : (c == 4 ? drow_N<N, 1>(P, dF) : row_N<N, 1>(P, fc[c]));
-    }
-#pragma unroll
-    for (int c = 0; c < 5; ++c) fc[c][0] = fc[c][N];
-    has_left = true;
-  }
-  if (!P.per[1] && s1 == nseg) {
-    const long long I = nodeI(nseg * N);
-    if (P.open_y[1]) {   // partition face: the row goes to the neighbour
-      const long long Fo = x + (long long)nx * z;
-#pragma unroll
-      for (int c = 0; c < 5; ++c) B.face_hi[c * (long long)nx * nz + Fo] = carry[c];
-    } else {
-#pragma unroll
-      for (int c = 0; c < 5; ++c) T[c * np + I] += carry[c] + carry[c];
-    }
-  }
+// Row N of the y segment before a y tile, for the tile's first line (written by
+// the y or x-y pass): its offset in one variable of Fy, or -1 where the node at line
+// y has none.  fy: lines of a tile, nty: tiles.
+__device__ __forceinline__ long long xy_face_at(const LineParams& P, int fy, int nty, int x, int y, int z) {
+  if (nty == 1 || !(P.per[1] || (y > 0 && y < P.n[1] - 1))) return -1;
+  // y / fy without an integer division (exact: y < 2^16, so the float quotient
+  // of y + 1/2 is nearer to it than 1 / (2 fy))
+  const int t = (int)__fdividef((float)y + 0.5f, (float)fy);
+  if (y != t * fy) return -1;
+  return ((long long)t * P.n[2] + z) * P.n[0] + x;
 }
 
 // ---------------------------------------------------------------- z lines + sources + stage
-// z-fluxes at one node; slot 4 holds theta (see flux_y)
-__device__ __forceinline__ void flux_z(const double* __restrict__ q, const double* __restrict__ W,
-                                       long long np, long long I, double (&f)[5]) {
-  const double mu = q[np + I], mv = q[2 * np + I], mw = q[3 * np + I];
-  const double w = W[np + I], pp = W[2 * np + I];
-  f[0] = mw;
-  f[1] = mu * w;
-  f[2] = mv * w;
-  f[3] = fma(mw, w, pp);
-  f[4] = W[3 * np + I];
-}
-
-// Completes node I at level gz given L[5] = T + z part (the assembled flux
-// divergence): sources, no-flux walls, then the stage store.  Every array of
-// a launch is distinct (the stage output never overwrites an input), which
-// the __restrict__ qualifiers state so loads can be issued ahead of stores.
-__device__ __forceinline__ void finish_node(const LineParams& P, const StageBufs& B,
-                                            const double* __restrict__ q,
-                                            const double* __restrict__ qn,
-                                            double* __restrict__ out, long long I, int x, int y,
-                                            int gz, double (&L)[5], bool& bad) {
+// Completes node I at level gz given its state qv and L[5] = T + z part (the
+// assembled flux divergence): sources, no-flux walls, then the stage store.
+// Every array of a launch is distinct (the stage output never overwrites an
+// input).
+__device__ __forceinline__ void finish_node(const LineParams& P, const StageBufs& B, const double (&qv)[5],
+                                            long long I, int x, int y, int gz, double (&L)[5], bool& bad) {
   const long long np = P.np;
-  const double rp = q[I], mu = q[np + I], mv = q[2 * np + I];
   if (B.E) {
 #pragma unroll
     for (int c = 0; c < 5; ++c) L[c] += B.E[c * np + I];
   }
-  L[1] = fma(P.f, mv, L[1]);                     // -f k x (rho u): +f rho v
-  L[2] = fma(-P.f, mu, L[2]);                    //                 -f rho u
-  L[3] = fma(-P.g, rp, L[3]);                    // -rho' g
-  if (B.S) L[4] = fma(__ldg(B.base + gz) + rp, __ldg(B.S + I), L[4]);  // rho S_theta
+  L[1] = fma(P.f, qv[2], L[1]);                  // -f k x (rho u): +f rho v
+  L[2] = fma(-P.f, qv[1], L[2]);                 //                 -f rho u
+  L[3] = fma(-P.g, qv[0], L[3]);                 // -rho' g
+  if (B.S) L[4] = fma(__ldg(B.base + gz) + qv[0], __ldg(B.S + I), L[4]);  // rho S_theta
   if (!P.per[0] && (x == 0 || x == P.n[0] - 1)) L[1] = 0.0;
   if (!P.per[1] && ((y == 0 && !P.open_y[0]) || (y == P.n[1] - 1 && !P.open_y[1]))) L[2] = 0.0;
   if (!P.per[2] && (gz == 0 || gz == P.n[2] - 1)) L[3] = 0.0;
-  if (B.rhs_only) {
 #pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      out[c * np + I] = L[c];
-      bad |= is_nonfinite(L[c]);
+  for (int c = 0; c < 5; ++c) {
+    double o = L[c];
+    if (!B.rhs_only) {
+      o = fma(B.dt, L[c], qv[c]);
+      if (B.alpha != 0.0) o = fma(B.alpha, B.qn[c * np + I], B.beta * o);
     }
-  } else if (B.alpha == 0.0) {
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      const double o = fma(B.dt, L[c], q[c * np + I]);
-      out[c * np + I] = o;
-      bad |= is_nonfinite(o);
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < 5; ++c) {
-      const double o = fma(B.alpha, qn[c * np + I], B.beta * fma(B.dt, L[c], q[c * np + I]));
-      out[c * np + I] = o;
-      bad |= is_nonfinite(o);
-    }
+    B.out[c * np + I] = o;
+    bad |= is_nonfinite(o);
   }
-}
-
-// grid (ceil(n_x / blockDim), nchunk, n_y); each thread marches `chunk`
-// element segments along z at its (x, y).
-template <int N>
-__global__ void __launch_bounds__(128) k_line_z(const LineParams P, const StageBufs B, int chunk) {
-  const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
-  const int nseg = P.nseg[2];
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= nx) return;
-  const int y = blockIdx.z;
-  const int s0 = blockIdx.y * chunk;
-  const int s1 = min(nseg, s0 + chunk);
-  if (s0 >= s1) return;
-  const long long np = P.np;
-  const long long nxy = (long long)nx * ny;
-  const long long col = x + (long long)nx * y;
-  const double* __restrict__ q = B.q;
-  const double* __restrict__ W = B.W;
-  const double* __restrict__ T = B.T;
-  const double* __restrict__ qn = B.qn;
-  double* __restrict__ out = B.out;
-  auto lev = [&](int gz) -> int { return gz == nz ? 0 : gz; };
-  bool bad = false;
-
-  double carry[5];
-  bool has_left = (s0 > 0) || P.per[2];
-  if (has_left) {
-    const int sp = s0 > 0 ? s0 - 1 : nseg - 1;
-    double fl[5][N + 1];
-#pragma unroll
-    for (int l = 0; l <= N; ++l) {
-      const int gz = lev(sp * N + l);
-      double f[5];
-      flux_z(q, W, np, col + nxy * gz, f);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) fl[c][l] = f[c];
-    }
-    double dm[N + 1], dF[N + 1];
-    seg_diffs<N>(fl[0], fl[4], dm, dF);
-    carry[0] = drow_N<N, 2>(P, dm);
-    carry[4] = drow_N<N, 2>(P, dF);
-#pragma unroll
-    for (int c = 1; c < 4; ++c) carry[c] = row_N<N, 2>(P, fl[c]);
-  }
-
-  double fc[5][N + 1];
-  {
-    const int gz = s0 * N;
-    double f[5];
-    flux_z(q, W, np, col + nxy * gz, f);
-#pragma unroll
-    for (int c = 0; c < 5; ++c) fc[c][0] = f[c];
-  }
-  for (int s = s0; s < s1; ++s) {
-#pragma unroll
-    for (int l = 1; l <= N; ++l) {
-      const int gz = lev(s * N + l);
-      double f[5];
-      flux_z(q, W, np, col + nxy * gz, f);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) fc[c][l] = f[c];
-    }
-    double dm[N + 1], dF[N + 1];
-    seg_diffs<N>(fc[0], fc[4], dm, dF);
-    auto rowc = [&](int c, int a, double start) -> double {
-      if (c == 0) return drow_from<N, 2>(P, a, dm, start);
-      if (c == 4) return drow_from<N, 2>(P, a, dF, start);
-      return row_from<N, 2>(P, a, fc[c], start);
-    };
-    // the segment's x + y parts, all loaded before any store
-    double tv[5][N];
-#pragma unroll
-    for (int a = 0; a < N; ++a) {
-      const long long I = col + nxy * (s * N + a);
-#pragma unroll
-      for (int c = 0; c < 5; ++c) tv[c][a] = T[c * np + I];
-    }
-#pragma unroll
-    for (int a = 0; a < N; ++a) {
-      const int gz = s * N + a;
-      const long long I = col + nxy * gz;
-      double L[5];
-#pragma unroll
-      for (int c = 0; c < 5; ++c) {
-        double t = tv[c][a];
-        if (a == 0 && !has_left) t = rowc(c, 0, t);  // wall: the row counts twice
-        t = rowc(c, a, t);
-        L[c] = (a == 0 && has_left) ? t + carry[c] : t;
-      }
-      finish_node(P, B, q, qn, out, I, x, y, gz, L, bad);
-    }
-#pragma unroll
-    for (int c = 0; c < 5; ++c)
-      carry[c] = c == 0 ? drow_N<N, 2>(P, dm) : (c == 4 ? drow_N<N, 2>(P, dF) : row_N<N, 2>(P, fc[c]));
-#pragma unroll
-    for (int c = 0; c < 5; ++c) fc[c][0] = fc[c][N];
-    has_left = true;
-  }
-  if (!P.per[2] && s1 == nseg) {
-    const int gz = nseg * N;
-    const long long I = col + nxy * gz;
-    double L[5];
-#pragma unroll
-    for (int c = 0; c < 5; ++c) L[c] = T[c * np + I] + (carry[c] + carry[c]);
-    finish_node(P, B, q, qn, out, I, x, y, gz, L, bad);
-  }
-  if (bad) *B.flag = 1;
 }
 
 }  // namespace xg

@@ -62,9 +62,11 @@ struct DfBufs {
   double dt64, alpha64, beta64; // rho' and Theta' stage coefficients
   int rhs_only;
   double* face_hi;  // [5][n_z][n_x] row N at an open y end (slot types as T)
-  // [5][nseg_y][n_z][n_x] row N of the y segment that ends at each y face,
-  // written by the y pass and added by the z pass (slot types as T)
+  // row N of the y segment that ends at each y tile's first line, written by
+  // the y (or x-y) pass and added by the z pass (slot types as T):
+  // [5][nty][n_z][n_x], fy lines a tile
   double* Fy;
+  int fy, nty;
 };
 
 // ---------------------------------------------------------------- FP64 <-> pairs
@@ -177,6 +179,11 @@ __device__ __forceinline__ df df_row(const DfParams& P, int a, const df (&f)[N +
 }
 
 // ---------------------------------------------------------------- x lines
+// Orders whose x and y lines this file takes (above them df_uses_plane holds).
+constexpr int kDfLineOrder = 5;
+
+// Dynamic shared memory of the x pass: a line's fluxes and its segments' rows N.
+inline size_t df_x_smem(int nx, int nseg) { return sizeof(double) * (5 * (size_t)(nx + 1) + 5 * (size_t)nseg); }
 // Orders up to 4 at 8 CTAs per SM (64 registers): 0.691 against 0.722 ms per
 // launch with no bound (71 registers, 7 CTAs) and 0.706 at 10 (spilling), on
 // the 128 x 128 x 16 order-4 box; higher orders would spill at 8
@@ -519,11 +526,12 @@ __global__ void __launch_bounds__(df_tile_threads(N, DIR), df_tile_min_blocks(N,
   if (main_plane && (ty > 0 || (H > 0 && has_left))) diff_slot(H + ty);   // slot N closes the halo
   if (halo && ty > 0) diff_slot(ty);
   __syncthreads();
-  const long long nfy = (long long)P.nseg[1] * P.n[2] * P.n[0];   // one variable of Fy
+  const long long nfy = (long long)B.nty * P.n[2] * P.n[0];   // one variable of Fy
   if (DIR == 1 && xin && ty == kc * N && !owns && B.Fy) {
     // the end face, owned by the next tile (or, periodic, the first): row N
     // of this tile's last segment for it
-    const long long Io = ((s0 + kc) % nseg) * (long long)P.n[2] * P.n[0] + (long long)P.n[0] * other + x;
+    const long long Io =
+        ((long long)((s0 + kc) % nseg / K) * P.n[2] + other) * P.n[0] + x;
 #pragma unroll
     for (int e = 0; e < 2; ++e) {
       double d[N + 1];
@@ -541,15 +549,12 @@ __global__ void __launch_bounds__(df_tile_threads(N, DIR), df_tile_min_blocks(N,
     }
   }
   if (!owns) return;
-  if (DIR == 2 && B.Fy) {   // the first node of a y tile: t0 + row N of the tile before
-    constexpr int KY = df_tile_segments(N, 1);
-    if (other % (KY * N) == 0 && (P.per[1] || (other > 0 && other < ny - 1))) {
-      const long long If = (other / N) * (long long)P.n[2] * P.n[0] + (long long)P.n[0] * g + x;
-      t64[0] = t64[0] + B.Fy[If];
-      t64[1] = t64[1] + B.Fy[4 * nfy + If];
+  const long long If = DIR == 2 ? xy_face_at(P64, B.fy, B.nty, x, other, g) : -1;
+  if (If >= 0) {   // the first node of a y tile: t0 + row N of the tile before
+    t64[0] = t64[0] + B.Fy[If];
+    t64[1] = t64[1] + B.Fy[4 * nfy + If];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) tm[c] = df_add(tm[c], reinterpret_cast<const df*>(B.Fy)[(c + 1) * nfy + If]);
-    }
+    for (int c = 0; c < 3; ++c) tm[c] = df_add(tm[c], reinterpret_cast<const df*>(B.Fy)[(c + 1) * nfy + If]);
   }
 
   // the node's segment k and local index a; the wall node is row N of the last

@@ -1,8 +1,8 @@
 // xg_noalloc.cu -- the right-hand side for callers that must not allocate
 // device memory (see xg_rhs_noalloc in include/xg.h).
 //
-// The line kernels need scratch beyond their inputs and outputs: W (v, w, p',
-// theta per node), T (x + y parts of the tendency), the per-level reference table
+// The stage kernels need scratch beyond their inputs and outputs: W (w, p',
+// theta per node, and the y faces' rows), T (x + y parts of the tendency), the per-level reference table
 // and the non-finite flag.  A context allocates those with cudaMalloc.  Here
 // they live in one file-scope __device__ array of fixed size instead, so a
 // call allocates nothing: no cudaMalloc, no cudaFree, no allocating library
@@ -72,16 +72,21 @@ __global__ void k_base_table(const double* __restrict__ rho0, const double* __re
 }
 
 template <int N>
-cudaError_t launch_rhs(const xg::LineParams& P, const xg::StageBufs& B, size_t xsmem,
-                       int chunk_y, int nchunk_y, int chunk_z, int nchunk_z, cudaStream_t st) {
-  cudaError_t e = xg::raise_dynamic_smem(xg::k_line_x<N>, xsmem);
+cudaError_t launch_rhs(const xg::F64Params& P, xg::StageBufs B, cudaStream_t st) {
+  using L = xg::XYTile<N>;
+  cudaError_t e = xg::raise_dynamic_smem(xg::k_plane_xy<N, xg::F64Params>, L::bytes);
   if (e != cudaSuccess) return e;
-  dim3 gx(P.n[1], P.n[2]);
-  xg::k_line_x<N><<<gx, xg::kXThreads, xsmem, st>>>(P, B);
-  dim3 gy((P.n[0] + 127) / 128, nchunk_y, P.n[2]);
-  xg::k_line_y<N><<<gy, 128, 0, st>>>(P, B, chunk_y);
-  dim3 gz((P.n[0] + 127) / 128, nchunk_z, P.n[1]);
-  xg::k_line_z<N><<<gz, 128, 0, st>>>(P, B, chunk_z);
+  // tiles of EY element rows: their faces' rows, 5 values a tile and column,
+  // fit the np doubles of W's unused first row (at least two tiles: 5 tiles
+  // <= n_y lines for every order; a single tile closes on itself)
+  B.fy = L::TY;
+  B.nty = (P.P64.nseg[1] + L::EY - 1) / L::EY;
+  B.Fy = B.W;
+  const dim3 gx((P.P64.nseg[0] + L::EX - 1) / L::EX, B.nty, P.P64.n[2]);
+  xg::k_plane_xy<N><<<gx, L::threads(L::EY), L::bytes, st>>>(P, B, L::EY);
+  constexpr int K = xg::z_tile_segments(N);
+  const dim3 gz((P.P64.n[0] + xg::kTileCols - 1) / xg::kTileCols, (P.P64.nseg[2] + K - 1) / K, P.P64.n[1]);
+  xg::k_tile_z<N><<<gz, dim3(xg::kTileCols, K * N + 1), 0, st>>>(P, B);
   return cudaGetLastError();
 }
 
@@ -120,14 +125,9 @@ extern "C" xg_status xg_rhs_noalloc(const xg_mesh_desc* d, const double* q, cons
   xg_status s = scratch_address(&scratch);
   if (s != XG_OK) return s;
 
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (sms <= 0) sms = 1;
-  xg::LineParams P;
-  xg::fill_line_params(d, geo, &P);
-  int chunk_y, nchunk_y, chunk_z, nchunk_z;
-  xg::plan_marches(d, geo, sms, &chunk_y, &nchunk_y, &chunk_z, &nchunk_z);
+  xg::F64Params P;
+  xg::fill_line_params(d, geo, &P.P64);
+  xg::fill_fix_params(d, P.F);
 
   xg::StageBufs B;
   B.q = q;
@@ -153,14 +153,14 @@ extern "C" xg_status xg_rhs_noalloc(const xg_mesh_desc* d, const double* q, cons
   }
   if (e == cudaSuccess) {
     switch (d->order) {
-      case 1: e = launch_rhs<1>(P, B, geo.xsmem, chunk_y, nchunk_y, chunk_z, nchunk_z, cs); break;
-      case 2: e = launch_rhs<2>(P, B, geo.xsmem, chunk_y, nchunk_y, chunk_z, nchunk_z, cs); break;
-      case 3: e = launch_rhs<3>(P, B, geo.xsmem, chunk_y, nchunk_y, chunk_z, nchunk_z, cs); break;
-      case 4: e = launch_rhs<4>(P, B, geo.xsmem, chunk_y, nchunk_y, chunk_z, nchunk_z, cs); break;
-      case 5: e = launch_rhs<5>(P, B, geo.xsmem, chunk_y, nchunk_y, chunk_z, nchunk_z, cs); break;
-      case 6: e = launch_rhs<6>(P, B, geo.xsmem, chunk_y, nchunk_y, chunk_z, nchunk_z, cs); break;
-      case 7: e = launch_rhs<7>(P, B, geo.xsmem, chunk_y, nchunk_y, chunk_z, nchunk_z, cs); break;
-      case 8: e = launch_rhs<8>(P, B, geo.xsmem, chunk_y, nchunk_y, chunk_z, nchunk_z, cs); break;
+      case 1: e = launch_rhs<1>(P, B, cs); break;
+      case 2: e = launch_rhs<2>(P, B, cs); break;
+      case 3: e = launch_rhs<3>(P, B, cs); break;
+      case 4: e = launch_rhs<4>(P, B, cs); break;
+      case 5: e = launch_rhs<5>(P, B, cs); break;
+      case 6: e = launch_rhs<6>(P, B, cs); break;
+      case 7: e = launch_rhs<7>(P, B, cs); break;
+      case 8: e = launch_rhs<8>(P, B, cs); break;
       default: e = cudaErrorInvalidValue;
     }
   }

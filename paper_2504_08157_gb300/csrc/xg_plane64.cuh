@@ -1,0 +1,641 @@
+// xg_plane64.cuh -- the x and y passes of the FP64-accurate paths (XG_FP64 and
+// XG_DF64) as one kernel over plane tiles.
+//
+// A CTA takes E_x x E_y elements of one level: the pointwise primitives of the
+// tile's nodes (FP64, or the mixed arithmetic of xg_kernels_df.cuh), the x and
+// y fluxes of the five equations, and the x + y part of each node's tendency
+// by 1-D contractions in 64-bit fixed point (xg_fixed.cuh): GB300 issues 1.9
+// FP64 FMAs a clock and SM against 60 IMAD.WIDE, and an order-4 row is 15 of
+// those.  The kernel writes T (the x + y part) and W (w, p', theta), which the
+// z pass reads; v and the x part never leave the chip.
+//
+// Fixed point needs an exponent.  Every (x tile, y segment) has its own, per
+// group of fluxes that are summed together (rho' with Theta' apart, the two
+// horizontal momenta, the vertical one): the maximum over the segment's N + 1
+// lines, so it does not depend on which segments share a CTA, and a domain cut
+// into y-slabs gets the same bits as the whole.  x and y rows of a node are
+// then integers of one scale and are added exactly; a shared y face adds the
+// row N of the segment before it in the format of T (t0 + row N, the order in
+// which a partition face is completed).  The Theta' flux theta (rho u_d) is
+// formed as an integer product of 62 bits, so only theta's own rounding is in
+// it; the difference form of the FP64 chains is not needed.
+//
+// XG_FP64, a stage on the 128 x 128 x 16 order-4 box (17.0 M nodes): three line
+// kernels with FP64 chains 1.87 + 1.44 + 2.02 ms; tiles 1.57 + 1.41 ms (FP64
+// pipe 61 and 70 % busy, 38 and 28 FP64 instructions a node; 2,020 and 1,150
+// instructions a node in all).  33^3 nodes: 66 -> 27 us.
+#pragma once
+
+#include <type_traits>
+
+#include <cuda_runtime.h>
+
+#include "xg_fixed.cuh"
+#include "xg_kernels.cuh"
+#include "xg_kernels_df.cuh"
+
+namespace xg {
+
+// FP64 launch constants with the fixed-point matrices of the three directions
+// (x and y share their scale).
+struct F64Params {
+  LineParams P64;
+  FixRows F[3];
+};
+
+// Launch constants of the mixed x-y tiles.
+struct DfTileParams {
+  DfParams D;
+  FixRows F[2];
+};
+
+// Segments of a z tile and its launch bounds: two segments (of order 4) at 4
+// CTAs per SM (56 registers).
+__host__ __device__ constexpr int z_tile_segments(int N) { return N >= 8 ? 1 : 8 / N; }
+__host__ __device__ constexpr int z_tile_threads(int N) { return kTileCols * (z_tile_segments(N) * N + 1); }
+__host__ __device__ constexpr int z_tile_min_blocks(int N) { return 1152 / z_tile_threads(N); }
+
+// Element rows of a tile: about 8 nodes, so that the N + 1 columns before and
+// after a tile and its closing line are a quarter of its nodes.
+__host__ __device__ constexpr int xy_elems_y(int N) { return N == 1 ? 9 : (N == 3 ? 3 : (N >= 5 ? 1 : 8 / N)); }
+
+template <int N>
+struct XYTile {
+  static constexpr int EX = 32 / N, EY = xy_elems_y(N);
+  static constexpr int TX = EX * N, TY = EY * N;
+  static constexpr int CX = TX == 32 ? N + 1 : N;       // columns beside the 32 that a warp's lanes take
+  static constexpr int PX = (N + TX + 1) | 1;           // V: columns -N .. TX
+  static constexpr int PR = TX | 1;                     // x rows
+  static constexpr int LY = TY + 1, LX = TX + 1;
+  static constexpr int V = EY * (N + 1) * PX;           // one flux
+  static constexpr int RX = LY * PR, RNX = LY * (EX + 1);
+  static constexpr int RY = TY * LX, RNY = EY * LX;
+  static constexpr size_t bytes = 8 * (size_t)(9 * V + 5 * (RX + RNX + RY + RNY));
+  static constexpr int side_warps(int ey) { return ((ey * N + 1) * CX + 31) / 32; }
+  static constexpr int threads(int ey) { return 32 * (ey * N + 1 + side_warps(ey)); }
+};
+
+#ifdef __CUDACC__
+
+// x and y fluxes of one node (M: the momentum's type)
+template <typename M>
+struct XYFlux {
+  double mu, mv, th;     // rho u, rho v, theta: the rho' fluxes and the factors of the Theta' ones
+  M xx, xy, xz, yy, yz;  // rho u u + p', rho u v, rho u w, rho v v + p', rho v w
+};
+
+// FP64: primitives and fluxes of the node I of level z; w, p', theta to W
+// where the tile owns the node.
+__device__ __forceinline__ void xy_point(const F64Params& Q, const StageBufs& B, long long I, int z, bool own,
+                                         XYFlux<double>& f) {
+  const LineParams& P = Q.P64;
+  const long long np = P.np;
+  const int nz = P.n[2];
+  const double* __restrict__ q = B.q;
+  const double rp = q[I], mu = q[np + I], mv = q[2 * np + I], mw = q[3 * np + I], tp = q[4 * np + I];
+  const double ir = rcp_newton(__ldg(B.base + z) + rp);
+  const double u = mu * ir, v = mv * ir;
+  const double pp = __ldg(B.base + 2 * nz + z) * eos_phi(P, tp * __ldg(B.base + 3 * nz + z));
+  f.mu = mu;
+  f.mv = mv;
+  f.th = (__ldg(B.base + nz + z) + tp) * ir;
+  f.xx = fma(mu, u, pp);
+  f.xy = mv * u;
+  f.xz = mw * u;
+  f.yy = fma(mv, v, pp);
+  f.yz = mw * v;
+  if (own) {
+    B.W[np + I] = mw * ir;
+    B.W[2 * np + I] = pp;
+    B.W[3 * np + I] = f.th;
+  }
+}
+
+// Mixed: theta in FP64 from a double-float estimate and one Newton correction
+// (t1 = t0 + (Theta - t0 rho) / rho: the estimate's 2^-47 error squares away),
+// two FP64 additions and two FMAs; everything else in double-float.
+__device__ __forceinline__ void xy_point(const DfTileParams& Q, const DfBufs& B, long long I, int z, bool own,
+                                         XYFlux<df>& f) {
+  const DfParams& P = Q.D;
+  const long long np = P.np;
+  const int nz = P.n[2];
+  const double* __restrict__ q = B.q;
+  const double rp = q[I], mu = q[np + I], mv = q[2 * np + I], mw = q[3 * np + I], tp = q[4 * np + I];
+  const double rho = B.base64[z] + rp, Th = B.base64[nz + z] + tp;
+  const df ir = df_rcp(df_of_double(rho));
+  const double t0 = dbl_of_df(df_mul(df_of_double(Th), ir));
+  f.th = fma(fma(-t0, rho, Th), dbl_of_df(ir), t0);
+  f.mu = mu;
+  f.mv = mv;
+  const df muD = df_of_double(mu), mvD = df_of_double(mv), mwD = df_of_double(mw);
+  const df u = df_mul(muD, ir), v = df_mul(mvD, ir);
+  const df pp = df_mul(B.base[2 * nz + z], df_eos_phi(P, df_mul(df_of_double(tp), B.base[3 * nz + z])));
+  f.xx = df_add(df_mul(muD, u), pp);
+  f.xy = df_mul(mvD, u);
+  f.xz = df_mul(mwD, u);
+  f.yy = df_add(df_mul(mvD, v), pp);
+  f.yz = df_mul(mwD, v);
+  if (own) {
+    B.W[np + I] = df_mul(mwD, ir);
+    B.W[2 * np + I] = pp;
+    B.W64[I] = f.th;
+  }
+}
+
+template <typename Params>
+struct XYTypes;
+template <>
+struct XYTypes<F64Params> {
+  using Bufs = StageBufs;
+  using M = double;
+  static constexpr bool mixed = false;
+  static __device__ __forceinline__ const LineParams& line(const F64Params& P) { return P.P64; }
+};
+template <>
+struct XYTypes<DfTileParams> {
+  using Bufs = DfBufs;
+  using M = df;
+  static constexpr bool mixed = true;
+  static __device__ __forceinline__ const LineParams& line(const DfTileParams& P) { return P.D.P64; }
+};
+
+// grid (x tiles, y tiles, n_z), block XYTile<N>::threads(ey), dynamic shared
+// memory XYTile<N>::bytes; ey <= EY element rows a tile.  Fy [5][y tiles][n_z]
+// [n_x] gets row N of the segment that ends at each tile's first line, which
+// the z pass adds.
+template <int N, typename Params>
+__global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTile<N>::threads(XYTile<N>::EY))
+    k_plane_xy(const __grid_constant__ Params P, const __grid_constant__ typename XYTypes<Params>::Bufs B, int ey) {
+  using L = XYTile<N>;
+  using M = typename XYTypes<Params>::M;
+  constexpr bool MIXED = XYTypes<Params>::mixed;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  fix2* V = reinterpret_cast<fix2*>(smem_raw);
+  long long* RX = reinterpret_cast<long long*>(V + 9 * L::V);
+  long long* RNX = RX + 5 * L::RX;
+  long long* RY = RNX + 5 * L::RNX;
+  long long* RNY = RY + 5 * L::RY;
+  __shared__ int Es[4][L::EY];
+  __shared__ int nonfinite;
+
+  const LineParams& G = XYTypes<Params>::line(P);
+  const int nx = G.n[0], ny = G.n[1];
+  const long long np = G.np;
+  const int z = blockIdx.z;
+  const int ekx = min(L::EX, G.nseg[0] - (int)blockIdx.x * L::EX), eky = min(ey, G.nseg[1] - (int)blockIdx.y * ey);
+  const int x0 = blockIdx.x * L::TX, y0 = blockIdx.y * ey * N;
+  const bool endx = !G.per[0] && (int)blockIdx.x * L::EX + ekx == G.nseg[0];
+  const bool endy = !G.per[1] && (int)blockIdx.y * ey + eky == G.nseg[1];
+  const bool open_lo = G.open_y[0] && blockIdx.y == 0, open_hi = endy && G.open_y[1];
+  const int fx = ekx * N, fy = eky * N;                    // the closing column and line
+  const int ox = fx + (endx ? 1 : 0), oy = fy + (endy ? 1 : 0);   // owned columns and lines
+  const int oyx = fy + (endy && !open_hi ? 1 : 0);         // lines with x rows
+  const bool hxl = blockIdx.x > 0 || G.per[0], hyl = blockIdx.y > 0 || G.per[1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warps = blockDim.x >> 5;
+  const int lines = ey * N + 1;                            // warps that take a line each
+
+  if (threadIdx.x < 4 * L::EY) (&Es[0][0])[threadIdx.x] = 0;
+  if (threadIdx.x == 0) nonfinite = 0;
+  __syncthreads();
+
+  // this thread's node (i, j) of the tile: a warp takes a line, the warps
+  // after them the N columns before the tile and its 33rd
+  int i, j;
+  if (warp < lines) {
+    j = warp;
+    i = lane;
+  } else {
+    const int t = (int)threadIdx.x - 32 * lines;
+    j = t / L::CX;
+    const int k = t - j * L::CX;
+    i = k == N ? 32 : k - N;
+  }
+  const bool inside = i >= 0 && i < ox && j <= fy;         // takes part in y rows
+  const bool need = inside || (j < oyx && i <= fx && (i >= 0 || hxl));
+  // the y segment of the node (its own), and the one it closes
+  const int sj = j < fy ? j / N : eky - 1, aj = j - sj * N;
+  const bool closes = aj == 0 && sj > 0 && inside;
+
+  // exponents: of rho u and rho v, of theta's products with them, and (FP64
+  // form) of the horizontal momenta's fluxes and the vertical one's
+  constexpr int kE = MIXED ? 2 : 4;
+  XYFlux<M> f;
+  int e[kE];
+#pragma unroll
+  for (int k = 0; k < kE; ++k) e[k] = 0;
+  if (need) {
+    int gx = x0 + i, gy = y0 + j;
+    if (gx < 0) gx += nx;
+    if (gx >= nx) gx -= nx;
+    if (gy >= ny) gy -= ny;
+    xy_point(P, B, gx + (long long)nx * (gy + (long long)ny * z), z, i >= 0 && i < ox && j < oy, f);
+    bool bad = false;
+    e[0] = max(fix_exp_finite(f.mu, bad), fix_exp_finite(f.mv, bad));
+    e[1] = e[0] + fix_exp_finite(f.th, bad);
+    if constexpr (!MIXED) {
+      e[2] = max(max(fix_exp_finite(f.xx, bad), fix_exp_finite(f.xy, bad)), fix_exp_finite(f.yy, bad));
+      e[3] = max(fix_exp_finite(f.xz, bad), fix_exp_finite(f.yz, bad));
+    }
+    if (bad) nonfinite = 1;
+  }
+  if (warp < lines) {
+    // a line that closes segment sj - 1 counts for it by its `inside` columns
+    // alone; only the closing column of an inner tile can be among the lanes
+    // without being inside
+    const bool two = aj == 0 && sj > 0 && j <= fy, differ = two && ox <= 31;
+#pragma unroll
+    for (int k = 0; k < kE; ++k) {
+      const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)e[k]);
+      const int mc = differ ? (int)__reduce_max_sync(0xffffffffu, inside ? (unsigned)e[k] : 0u) : m;
+      if (lane == k && j <= fy) {
+        atomicMax(&Es[k][sj], m);
+        if (two) atomicMax(&Es[k][sj - 1], mc);
+      }
+    }
+  } else {
+    for (int s = 0; s < eky; ++s) {
+      const bool in = need && (s == sj || (closes && s == sj - 1));
+#pragma unroll
+      for (int k = 0; k < kE; ++k) {
+        const int m = (int)__reduce_max_sync(0xffffffffu, in ? (unsigned)e[k] : 0u);
+        if (lane == k) atomicMax(&Es[k][s], m);
+      }
+    }
+  }
+  __syncthreads();
+
+  const int sc = P.F[0].sc;
+  if (need) {
+    auto put = [&](int s, int a) {
+      fix2* v = V + (s * (N + 1) + a) * L::PX + i + N;
+      const int E0 = fix_block_exp(Es[0][s], sc), E4 = fix_prod_exp<N>(Es[1][s], sc);
+      v[0] = fix_of<N>(f.mu, E0);
+      v[L::V] = fix_of<N>(f.mv, E0);
+      v[2 * L::V] = fix_prod<N>(f.th, f.mu, E4);
+      v[3 * L::V] = fix_prod<N>(f.th, f.mv, E4);
+      if constexpr (MIXED) {
+        df* p = reinterpret_cast<df*>(v);
+        p[4 * L::V] = f.xx;
+        p[5 * L::V] = f.xy;
+        p[6 * L::V] = f.xz;
+        p[7 * L::V] = f.yy;
+        p[8 * L::V] = f.yz;
+      } else {
+        const int E1 = fix_block_exp(Es[2][s], sc), E3 = fix_block_exp(Es[3][s], sc);
+        v[4 * L::V] = fix_of<N>(f.xx, E1);
+        v[5 * L::V] = fix_of<N>(f.xy, E1);
+        v[6 * L::V] = fix_of<N>(f.xz, E3);
+        v[7 * L::V] = fix_of<N>(f.yy, E1);
+        v[8 * L::V] = fix_of<N>(f.yz, E3);
+      }
+      if (nonfinite) {
+        const fix2 mark = {kFixMark, 0};
+        const bool bth = fix_bad(f.th);
+        if (fix_bad(f.mu)) v[0] = mark;
+        if (fix_bad(f.mv)) v[L::V] = mark;
+        if (fix_bad(f.mu) || bth) v[2 * L::V] = mark;
+        if (fix_bad(f.mv) || bth) v[3 * L::V] = mark;
+        if constexpr (!MIXED) {
+          if (fix_bad(f.xx)) v[4 * L::V] = mark;
+          if (fix_bad(f.xy)) v[5 * L::V] = mark;
+          if (fix_bad(f.xz)) v[6 * L::V] = mark;
+          if (fix_bad(f.yy)) v[7 * L::V] = mark;
+          if (fix_bad(f.yz)) v[8 * L::V] = mark;
+        }
+      }
+    };
+    put(sj, aj);
+    if (closes) put(sj - 1, N);
+  }
+  __syncthreads();
+
+  // one thread per segment, variable and direction; a warp's tasks are of one
+  // kind.  fluxes of variable c along x: mu, xx, xy, xz, theta mu; along y:
+  // mv, xy, yy, yz, theta mv
+  constexpr unsigned kFx = 0x26540u, kFy = 0x38751u;
+  // row A .. B - 1 of the segment at p (stride sp) in direction D to r (stride
+  // sr), row N to rn; mixed momentum in double-float, the rest in fixed point
+  auto rows = [&](auto dir, int c, const fix2* p, int sp, long long* r, int sr, long long* rn, bool all) {
+    constexpr int D = decltype(dir)::value;
+    if (MIXED && c != 0 && c != 4) {
+      if constexpr (MIXED) {
+        df v[N + 1];
+#pragma unroll
+        for (int l = 0; l <= N; ++l) v[l] = reinterpret_cast<const df*>(p)[l * sp];
+        if (all) {
+#pragma unroll
+          for (int a = 0; a < N; ++a) reinterpret_cast<df*>(r)[a * sr] = df_row<N, D>(P.D, a, v);
+        }
+        *reinterpret_cast<df*>(rn) = df_row<N, D>(P.D, N, v);
+      }
+    } else {
+      fix2 v[N + 1];
+#pragma unroll
+      for (int l = 0; l <= N; ++l) v[l] = p[l * sp];
+      if (all) {
+#pragma unroll
+        for (int a = 0; a < N; ++a) r[a * sr] = fix_row<N>(P.F[D], a, v);
+      }
+      *rn = fix_row<N>(P.F[D], N, v);
+    }
+  };
+  const int cy = ox > L::TX ? L::LX : L::TX;              // columns of the y tasks
+  const int wx = (oyx * L::EX + 31) / 32, wy = (eky * cy + 31) / 32;
+  const int wl = hxl ? (oyx + 31) / 32 : 0;
+  for (int w = warp; w < 5 * (wx + wy + wl); w += warps) {
+    if (w < 5 * wx) {
+      const int c = w / wx, t = (w - c * wx) * 32 + lane;
+      const int o = t / L::EX, s = t - o * L::EX;
+      if (o < oyx && s < ekx) {
+        const int so = o < fy ? o / N : eky - 1;
+        rows(std::integral_constant<int, 0>(), c,
+             V + ((kFx >> (4 * c)) & 15u) * L::V + (so * (N + 1) + o - so * N) * L::PX + N + s * N, 1,
+             RX + c * L::RX + o * L::PR + s * N, 1, RNX + c * L::RNX + o * (L::EX + 1) + s + 1, true);
+      }
+    } else if (w < 5 * (wx + wy)) {
+      const int c = (w - 5 * wx) / wy, t = (w - 5 * wx - c * wy) * 32 + lane;
+      const int s = ox > L::TX ? t / L::LX : t / L::TX, k = t - s * cy;
+      if (s < eky && k < ox)
+        rows(std::integral_constant<int, 1>(), c, V + ((kFy >> (4 * c)) & 15u) * L::V + s * (N + 1) * L::PX + N + k,
+             L::PX, RY + c * L::RY + s * N * L::LX + k, L::LX, RNY + c * L::RNY + s * L::LX + k, true);
+    } else {   // row N of the x segment before the tile
+      const int c = (w - 5 * (wx + wy)) / wl, o = (w - 5 * (wx + wy) - c * wl) * 32 + lane;
+      if (o < oyx) {
+        const int so = o < fy ? o / N : eky - 1;
+        rows(std::integral_constant<int, 0>(), c, V + ((kFx >> (4 * c)) & 15u) * L::V + (so * (N + 1) + o - so * N) * L::PX,
+             1, nullptr, 1, RNX + c * L::RNX + o * (L::EX + 1), false);
+      }
+    }
+  }
+  __syncthreads();
+
+  if (i < 0 || i >= ox || j > fy) return;
+  const bool closing = j == fy && (!endy || open_hi);     // row N alone: the next tile's, or the neighbour's
+  if (closing && !open_hi && gridDim.y == 1) return;
+  double* faces = nullptr;
+  long long fstride = 0, fat = 0;
+  if (closing) {
+    if (open_hi) {
+      faces = B.face_hi;
+      fstride = (long long)nx * G.n[2];
+      fat = (long long)nx * z + x0 + i;
+    } else {
+      const int next = (int)blockIdx.y + 1 < (int)gridDim.y ? blockIdx.y + 1 : 0;
+      faces = B.Fy;
+      fstride = (long long)gridDim.y * G.n[2] * nx;
+      fat = ((long long)next * G.n[2] + z) * nx + x0 + i;
+    }
+  }
+  const int si = i / N;
+  const bool wraps = j == 0 && hyl && gridDim.y == 1;     // one tile around: its own closing row
+  const int sl = wraps ? eky - 1 : sj - 1;                // the y segment that ends at this line
+  const long long I = x0 + i + (long long)nx * (y0 + j + (long long)ny * z);
+  auto marked = [&](const fix2* p, int stride) {
+    bool m = false;
+    for (int l = 0; l <= N; ++l) m |= p[l * stride].h == kFixMark;
+    return m;
+  };
+  // a variable in fixed point
+  auto node = [&](int c) {
+    const fix2* vy = V + ((kFy >> (4 * c)) & 15u) * L::V + N + i;
+    const int k = c == 0 ? 0 : (c == 4 ? 1 : (c == 3 ? 3 : 2));
+    auto field = [&](int s) {
+      return c == 4 ? fix_prod_field<N>(fix_prod_exp<N>(Es[k][s], sc), sc) : fix_field<N>(fix_block_exp(Es[k][s], sc), sc);
+    };
+    if (closing) {
+      double r = fix_out<MIXED>(RNY[c * L::RNY + (eky - 1) * L::LX + i], field(eky - 1));
+      if (nonfinite && marked(vy + (eky - 1) * (N + 1) * L::PX, L::PX)) r = xg_nan(0.0);
+      faces[c * fstride + fat] = r;
+      return;
+    }
+    long long r;
+    const long long* rn = RNX + c * L::RNX + j * (L::EX + 1);
+    if (i == fx) {
+      r = 2 * rn[ekx];                                    // a wall's last node: its row twice
+    } else {
+      r = RX[c * L::RX + j * L::PR + i];
+      if (i == si * N) r += (si > 0 || hxl) ? rn[si] : r;
+    }
+    if (j == fy) {
+      r += 2 * RNY[c * L::RNY + (eky - 1) * L::LX + i];
+    } else {
+      const long long t = RY[c * L::RY + j * L::LX + i];
+      r += t;
+      if (j == 0 && !hyl && !open_lo) r += t;
+    }
+    double v = fix_out<MIXED>(r, field(sj));
+    if (closes || wraps) v = v + fix_out<MIXED>(RNY[c * L::RNY + sl * L::LX + i], field(sl));
+    if (nonfinite) {
+      const fix2* vx = V + ((kFx >> (4 * c)) & 15u) * L::V + (sj * (N + 1) + aj) * L::PX + N;
+      bool m = marked(vy + sj * (N + 1) * L::PX, L::PX);
+      if (closes || wraps) m |= marked(vy + sl * (N + 1) * L::PX, L::PX);
+      if (i < fx) m |= marked(vx + si * N, 1);
+      if (i == si * N && (si > 0 || hxl)) m |= marked(vx + (si - 1) * N, 1);
+      if (m) v = xg_nan(0.0);
+    }
+    B.T[c * np + I] = v;
+  };
+  node(0);
+  node(4);
+  if constexpr (!MIXED) {
+    node(1);
+    node(2);
+    node(3);
+  } else {
+    const df* RXm = reinterpret_cast<const df*>(RX);
+    const df* RNXm = reinterpret_cast<const df*>(RNX);
+    const df* RYm = reinterpret_cast<const df*>(RY);
+    const df* RNYm = reinterpret_cast<const df*>(RNY);
+#pragma unroll
+    for (int c = 1; c < 4; ++c) {
+      if (closing) {
+        reinterpret_cast<df*>(faces)[c * fstride + fat] = RNYm[c * L::RNY + (eky - 1) * L::LX + i];
+        continue;
+      }
+      df r;
+      const df* rn = RNXm + c * L::RNX + j * (L::EX + 1);
+      if (i == fx) {
+        r = df_scale2(rn[ekx], 2.0f);
+      } else {
+        r = RXm[c * L::RX + j * L::PR + i];
+        if (i == si * N) r = (si > 0 || hxl) ? df_add(r, rn[si]) : df_scale2(r, 2.0f);
+      }
+      if (j == fy) {
+        r = df_add(r, df_scale2(RNYm[c * L::RNY + (eky - 1) * L::LX + i], 2.0f));
+      } else {
+        df t = RYm[c * L::RY + j * L::LX + i];
+        if (j == 0 && !hyl && !open_lo) t = df_scale2(t, 2.0f);
+        r = df_add(r, t);
+      }
+      if (closes || wraps) r = df_add(r, RNYm[c * L::RNY + sl * L::LX + i]);
+      B.Tm[c * np + I] = r;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- z lines + sources + stage, FP64
+// One CTA per (32 x-columns) x (K element segments along z) x y, one thread per
+// node: block (32, K N + 1), a warp a level.  The loads of the fluxes come
+// first; fluxes go to shared memory with those of the N levels of the segment
+// before the tile (Theta' as rho w and theta); then one thread per (column,
+// segment) and variable takes its rows in fixed point, with an exponent of its
+// own; after a barrier each thread assembles its node: sources, walls, stage.
+template <int N>
+__global__ void __launch_bounds__(z_tile_threads(N), z_tile_min_blocks(N))
+    k_tile_z(const __grid_constant__ F64Params P, const __grid_constant__ StageBufs B) {
+  constexpr int K = z_tile_segments(N);
+  constexpr int NS = K * N + N + 1;            // flux slots: N halo levels + K N + 1
+  __shared__ double Fm[3][NS][kTileCols];           // momentum fluxes
+  __shared__ double Fs[2][NS][kTileCols];      // rho w and theta
+  __shared__ double Rz[5][K * N][kTileCols];  // rows 0..N-1 of every segment, in the order 0, 4, 1, 2, 3
+  __shared__ double RN[5][K + 1][kTileCols];  // row N, from the segment before the tile on
+  const LineParams& G = P.P64;
+  const int nx = G.n[0], ny = G.n[1], nz = G.n[2];
+  const int nseg = G.nseg[2];
+  const bool per = G.per[2] != 0;
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  const int x = blockIdx.x * kTileCols + tx;
+  const bool xin = x < nx;
+  const int s0 = blockIdx.y * K;
+  const int kc = min(K, nseg - s0);             // segments in this tile
+  const int y = blockIdx.z;
+  const long long np = G.np;
+  const long long sd = (long long)nx * ny;
+  const long long base = x + (long long)nx * y;
+  const bool has_left = s0 > 0 || per;
+  auto level = [&](int g) -> int { return g >= nz ? g - nz : (g < 0 ? g + nz : g); };
+
+  const int own = s0 * N + ty;
+  const bool owns = xin && (ty < kc * N || (ty == kc * N && s0 + kc == nseg && !per));
+  const bool main_level = xin && ty <= kc * N;   // the extra row fills the end face
+  const bool halo = xin && has_left && ty < N;   // the N levels before the tile
+  const int g = level(own);
+  const int gh = level((s0 - 1) * N + ty);
+  const long long I = base + sd * (main_level ? g : 0);
+  const long long Ih = base + sd * (halo ? gh : 0);
+  const double* __restrict__ W = B.W;
+
+  // the global loads the fluxes and rows need first (one memory round trip);
+  // q^n and S, needed only by the stage at the end, are loaded there
+  double qv[5], hq[3], th = 0.0, hth = 0.0, vel, pp, hvel, hpp;
+  if (main_level) {
+#pragma unroll
+    for (int c = 0; c < 5; ++c) qv[c] = B.q[c * np + I];
+    vel = W[np + I];
+    pp = W[2 * np + I];
+    th = W[3 * np + I];
+  }
+  if (halo) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) hq[c] = B.q[(c + 1) * np + Ih];
+    hvel = W[np + Ih];
+    hpp = W[2 * np + Ih];
+    hth = W[3 * np + Ih];
+  }
+  if (main_level) {
+    Fm[0][N + ty][tx] = qv[1] * vel;
+    Fm[1][N + ty][tx] = qv[2] * vel;
+    Fm[2][N + ty][tx] = fma(qv[3], vel, pp);
+    Fs[0][N + ty][tx] = qv[3];
+    Fs[1][N + ty][tx] = th;
+  }
+  if (halo) {
+    Fm[0][ty][tx] = hq[0] * hvel;
+    Fm[1][ty][tx] = hq[1] * hvel;
+    Fm[2][ty][tx] = fma(hq[2], hvel, hpp);
+    Fs[0][ty][tx] = hq[2];
+    Fs[1][ty][tx] = hth;
+  }
+  __syncthreads();
+
+  // a warp takes one variable of one segment (the segment before the tile, of
+  // which only row N is needed, last)
+  if (xin) {
+    const int sc = P.F[2].sc;
+    for (int w = ty; w < 5 * (kc + (has_left ? 1 : 0)); w += K * N + 1) {
+      const int k = w < 5 * kc ? w / 5 + 1 : 0, e = w % 5;      // segment k - 1 of the tile
+      const double* src = e < 2 ? &Fs[0][k * N][tx] : &Fm[e >= 2 ? e - 2 : 0][k * N][tx];
+      bool b = false;
+      int E = 0, u;
+      fix2 v[N + 1];
+      double a[N + 1];
+#pragma unroll
+      for (int l = 0; l <= N; ++l) a[l] = src[l * kTileCols];
+      if (e == 1) {
+        double t[N + 1];
+#pragma unroll
+        for (int l = 0; l <= N; ++l) {
+          t[l] = src[(NS + l) * kTileCols];
+          E = max(E, fix_exp_finite(a[l], b) + fix_exp_finite(t[l], b));
+        }
+        E = fix_prod_exp<N>(E, sc);
+#pragma unroll
+        for (int l = 0; l <= N; ++l) v[l] = fix_prod<N>(t[l], a[l], E);
+        u = fix_prod_field<N>(E, sc);
+      } else {
+#pragma unroll
+        for (int l = 0; l <= N; ++l) E = max(E, fix_exp_finite(a[l], b));
+        E = fix_block_exp(E, sc);
+#pragma unroll
+        for (int l = 0; l <= N; ++l) v[l] = fix_of<N>(a[l], E);
+        u = fix_field<N>(E, sc);
+      }
+      if (k > 0) {
+#pragma unroll
+        for (int r = 0; r < N; ++r)
+          Rz[e][(k - 1) * N + r][tx] = b ? xg_nan(0.0) : fix_out<false>(fix_row<N>(P.F[2], r, v), u);
+      }
+      RN[e][k][tx] = b ? xg_nan(0.0) : fix_out<false>(fix_row<N>(P.F[2], N, v), u);
+    }
+  }
+
+  __syncthreads();
+  if (!owns) return;
+
+  // the node's segment k and local index a; the wall node is row N of the last
+  const int k = ty < kc * N ? ty / N : kc - 1;
+  const int a = ty < kc * N ? ty - k * N : N;
+  const long long fat = xy_face_at(G, B.fy, B.nty, x, y, g), nf = (long long)B.nty * nz * nx;
+  double L[5];
+#pragma unroll
+  for (int c = 0; c < 5; ++c) {
+    const int e = c == 0 ? 0 : (c == 4 ? 1 : c + 1);
+    double t = B.T[c * np + I];
+    if (fat >= 0) t = t + B.Fy[c * nf + fat];           // the y face's row N: t0 + row N
+    if (a == N) {                                       // wall node: its one-sided row counts twice
+      const double r = RN[e][kc][tx];
+      L[c] = t + (r + r);
+    } else {
+      const double r = Rz[e][ty][tx];
+      t = t + r;
+      L[c] = a == 0 ? t + (k > 0 || has_left ? RN[e][k][tx] : r) : t;
+    }
+  }
+  bool bad = false;
+  finish_node(G, B, qv, I, x, y, g, L, bad);
+  if (bad) *B.flag = 1;
+}
+
+#endif  // __CUDACC__
+
+// Element rows of the x-y tiles of a mesh: the most, EY, unless fewer give the
+// chip blocks that it would lack.
+inline int xy_tile_rows(int N, const int (&nseg)[3], int levels, int sms) {
+  const int most = xy_elems_y(N), ex = 32 / N;
+  const long long columns = (long long)((nseg[0] + ex - 1) / ex) * levels;
+  int ey = most;
+  while (ey > 1 && columns * ((nseg[1] + ey - 1) / ey) < 3ll * sms) --ey;
+  return ey;
+}
+
+// Whether the mixed form takes the x-y tiles instead of the x and y line
+// kernels.  The tiles do the pointwise work 1.4 times and the rho' and Theta'
+// rows without the FP64 pipe; the lines need a second launch and an x line's
+// segments to fill a CTA.  Measured a stage, tiles against lines: order 7, 4.1 M
+// nodes 0.94 / 1.20 ms; order 5 0.80 / 0.78; order 4, 17 M nodes 2.69 / 2.26;
+// order 4, 33^3 nodes 22 / 29 us.  The rule leaves n_y out, so that a y-slab of
+// a domain takes the path of the whole.
+inline bool df_uses_plane(int N, const int (&n)[3]) { return N > kDfLineOrder || (long long)n[0] * n[2] <= 4096; }
+
+}  // namespace xg

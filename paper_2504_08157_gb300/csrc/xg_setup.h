@@ -1,7 +1,7 @@
 // xg_setup.h -- host-side mesh checks and launch constants shared by the
 // entry points: the LGL derivative matrix (Sec. 2.2, Eq. 5), the binomial
 // series of the equation of state (Eq. 3), the pre-scaled per-direction
-// derivative matrices, and the marching-chunk choice of the line kernels.
+// derivative matrices.
 #pragma once
 
 #include <cmath>
@@ -14,6 +14,7 @@
 #include "xg_kernels.cuh"
 #include "xg_kernels_df.cuh"
 #include "xg_kernels_f32.cuh"
+#include "xg_plane64.cuh"
 #include "xg_plane_f32.cuh"
 
 namespace xg {
@@ -116,7 +117,6 @@ inline void eos_series(double gamma, double* c, double* xmax) {
 struct MeshGeom {
   int n[3];        // global nodes per direction
   long long np;    // n[0] n[1] n[2]
-  size_t xsmem;    // dynamic shared memory of k_line_x
 };
 
 // Host-side checks of a mesh description (no GPU work).  XG_ERR_ARG for
@@ -142,9 +142,8 @@ inline xg_status check_desc(const xg_mesh_desc* d, MeshGeom* g) {
     g->n[k] = (int)nk;
   }
   g->np = (long long)g->n[0] * g->n[1] * g->n[2];
-  // one x-line per CTA: its fluxes and segment derivatives in shared memory
-  g->xsmem = sizeof(double) * (5 * (size_t)(g->n[0] + 1) + 5 * (size_t)d->nel[0]);
-  if (g->xsmem > 220 * 1024) return XG_ERR_UNSUPPORTED;
+  // one x line per CTA of the mixed form's x pass
+  if (sizeof(double) * (5 * (size_t)(g->n[0] + 1) + 5 * (size_t)d->nel[0]) > 220 * 1024) return XG_ERR_UNSUPPORTED;
   if (g->n[1] > 65535 || g->n[2] > 65535) return XG_ERR_UNSUPPORTED;  // grid y/z limits
   return XG_OK;
 }
@@ -182,6 +181,23 @@ inline void fill_line_params(const xg_mesh_desc* d, const MeshGeom& g, LineParam
   P->gamma = gamma;
   P->f = d->f_coriolis;
   P->g = d->g;
+}
+
+// The same matrices -(2/h_d) D (rows 0 and N halved) in fixed point.
+inline void fill_fix_params(const xg_mesh_desc* d, FixRows (&F)[3]) {
+  const int N = d->order;
+  long double D[kMaxOrder + 1][kMaxOrder + 1];
+  lgl_derivative(N, D);
+  FixMatrix M[3];
+  for (int k = 0; k < 3; ++k) {
+    const long double h = ((long double)d->hi[k] - d->lo[k]) / d->nel[k];
+    for (int a = 0; a <= N; ++a)
+      for (int l = 0; l <= N; ++l) M[k][a][l] = -(2.0L / h) * ((a == 0 || a == N) ? 0.5L : 1.0L) * D[a][l];
+  }
+  const int sxy = fix_scale_of(std::fmax(fix_row_sum(N, M[0]), fix_row_sum(N, M[1])));
+  fix_rows(N, M[0], sxy, &F[0]);
+  fix_rows(N, M[1], sxy, &F[1]);
+  fix_rows(N, M[2], fix_scale_of(fix_row_sum(N, M[2])), &F[2]);
 }
 
 // A double split into a double-float pair (host).
@@ -227,41 +243,6 @@ inline void fill_f32_params(const LineParams& P, FParams* Q) {
   Q->gamma = P.gamma;
   Q->f = (float)P.f;
   Q->g = (float)P.g;
-}
-
-// Element segments per marching thread of k_line_y / k_line_z.  A launch
-// has items_per_chunk CTAs for every chunk of the line.  The kernels are
-// bound by the FP64 pipe of each SM, which its resident CTAs share, so the
-// launch lasts about as long as the SM given the most CTAs: ceil(items /
-// SMs) chunks, each one chunk of segments plus the halo segment a chunk
-// start recomputes (about a fifth of a segment's work).  The chunk count with
-// the smallest such makespan wins.
-inline void choose_chunks(int nseg, long long items_per_chunk, long long sms, bool periodic,
-                          int* chunk, int* nchunk) {
-  if (sms < 1) sms = 1;
-  double best = 1e300;
-  *chunk = nseg;
-  *nchunk = 1;
-  for (int k = 1; k <= nseg; ++k) {
-    const int c = (nseg + k - 1) / k;
-    const int nk = (nseg + c - 1) / c;
-    if (nk != k) continue;
-    const long long per_sm = (items_per_chunk * nk + sms - 1) / sms;
-    const double cost = (double)per_sm * (c + ((nk > 1 || periodic) ? 0.2 : 0.0));
-    if (cost < best - 1e-9) {
-      best = cost;
-      *chunk = c;
-      *nchunk = nk;
-    }
-  }
-}
-
-// Chunking of both marching kernels for a mesh on a device with `sms` SMs.
-inline void plan_marches(const xg_mesh_desc* d, const MeshGeom& g, int sms, int* chunk_y,
-                         int* nchunk_y, int* chunk_z, int* nchunk_z) {
-  const long long xblocks = (g.n[0] + 127) / 128;
-  choose_chunks(d->nel[1], xblocks * g.n[2], sms, d->periodic[1] != 0, chunk_y, nchunk_y);
-  choose_chunks(d->nel[2], xblocks * g.n[1], sms, d->periodic[2] != 0, chunk_z, nchunk_z);
 }
 
 // Raise a kernel's dynamic shared-memory limit to at least `bytes`.  The
