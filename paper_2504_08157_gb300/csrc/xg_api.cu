@@ -298,7 +298,7 @@ void launch_stage_n(xg_ctx* c, const DfBufs& B, cudaStream_t st, int parts) {
     if constexpr (N <= xg::kDfLineOrder) {
       dim3 gx(c->n[1], c->n[2]);
       prof_mark(c, 0, false, st);
-      xg::k_df_line_x<N><<<gx, xg::kXThreads, xg::df_x_smem(c->n[0], c->d.nel[0]), st>>>(c->Pdf, B);
+      xg::k_df_line_x<N><<<gx, xg::kXThreads, xg::df_x_smem(N, c->d.nel[0]), st>>>(c->Pdf, c->P64.F[0], B);
       prof_mark(c, 0, true, st);
       constexpr int K = xg::df_tile_segments(N, 1);
       const dim3 blk(xg::kTileCols, K * N + 1);
@@ -323,7 +323,7 @@ cudaError_t configure_n(xg_ctx* c) {
   cudaError_t e = xg::raise_dynamic_smem(xg::k_plane_xy<N, xg::F64Params>, xg::XYTile<N>::bytes);
   if (e == cudaSuccess) e = xg::raise_dynamic_smem(xg::k_plane_xy<N, xg::DfTileParams>, xg::XYTile<N>::bytes);
   if constexpr (N <= xg::kDfLineOrder)
-    if (e == cudaSuccess) e = xg::raise_dynamic_smem(xg::k_df_line_x<N>, xg::df_x_smem(c->n[0], c->d.nel[0]));
+    if (e == cudaSuccess) e = xg::raise_dynamic_smem(xg::k_df_line_x<N>, xg::df_x_smem(N, c->d.nel[0]));
   if (e == cudaSuccess) e = xg::raise_dynamic_smem(xg::k_f_plane_xy<N>, xg::PlaneLayoutF<N>::bytes);
   if (N == xg::PlaneTcLayout::N && e == cudaSuccess)
     e = xg::raise_dynamic_smem(xg::k_f_plane_xy_tc, xg::PlaneTcLayout::bytes);

@@ -402,6 +402,34 @@ __device__ __forceinline__ double fix_out(long long r, int u) {
   return v;
 }
 
+// Rows of the rho' and Theta' fluxes m and theta m of one segment, with an
+// exponent each, handed to put0(a, row) and put4 (a value that is not finite
+// makes its rows NaN); MIXED as fix_out.
+template <int N, typename Put0, typename Put4>
+__device__ __forceinline__ void fix_flux_rows(const FixRows& F, const double (&m)[N + 1], const double (&th)[N + 1],
+                                              Put0 put0, Put4 put4) {
+  bool b0 = false, b4 = false;
+  int e0 = 0, e4 = 0;
+#pragma unroll
+  for (int l = 0; l <= N; ++l) {
+    const int em = fix_exp_finite(m[l], b0);
+    e0 = max(e0, em);
+    e4 = max(e4, em + fix_exp_finite(th[l], b4));
+  }
+  b4 |= b0;
+  fix2 v[N + 1];
+  const int E0 = fix_block_exp(e0, F.sc), E4 = fix_prod_exp<N>(e4, F.sc);
+#pragma unroll
+  for (int l = 0; l <= N; ++l) v[l] = fix_of<N>(m[l], E0);
+#pragma unroll
+  for (int a = 0; a <= N; ++a) put0(a, b0 ? xg_nan(0.0) : fix_out<true>(fix_row<N>(F, a, v), fix_field<N>(E0, F.sc)));
+#pragma unroll
+  for (int l = 0; l <= N; ++l) v[l] = fix_prod<N>(th[l], m[l], E4);
+#pragma unroll
+  for (int a = 0; a <= N; ++a)
+    put4(a, b4 ? xg_nan(0.0) : fix_out<true>(fix_row<N>(F, a, v), fix_prod_field<N>(E4, F.sc)));
+}
+
 #endif  // __CUDACC__
 
 }  // namespace xg

@@ -33,9 +33,8 @@
 // map, sign of the divergence) with rows 0 and N halved for the face average;
 // wall nodes undo the halving.  The FP64 pipe (2 DFMA/clk/SM on GB300) bounds
 // what runs on it, so the arithmetic is arranged to spend few FP64 instructions:
-// 1/rho is one hardware reciprocal estimate refined by two Newton steps, the
-// equation of state is a short binomial series, and the FP64 contraction of the
-// mixed x pass uses the even/odd split of the centro-antisymmetric LGL matrix.
+// 1/rho is one hardware reciprocal estimate refined by two Newton steps and the
+// equation of state is a short binomial series.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -44,7 +43,6 @@
 namespace xg {
 
 constexpr int kMaxOrder = 8;
-constexpr int kMaxPairs = (kMaxOrder + 1) / 2;
 constexpr int kXThreads = 128;
 constexpr int kEosTerms = 8;
 
@@ -61,15 +59,6 @@ struct LineParams {
   long long np;   // n[0] n[1] n[2]
   // Dm[d][a][l] = -(2/h_d) D[a][l] (x 1/2 for a = 0 and a = N)
   double Dm[3][kMaxOrder + 1][kMaxOrder + 1];
-  // even/odd split of Dm (pairs l < N-l):  for i < (N+1)/2
-  //   (Dm f)_i   = sum_l EA[i][l] o_l + (sum_l EB[i][l] e_l + EBm[i] f_mid)
-  //   (Dm f)_N-i = sum_l EA[i][l] o_l - (...)
-  // with e_l = f_l + f_{N-l}, o_l = f_l - f_{N-l}; for even N the middle row
-  //   (Dm f)_{N/2} = sum_l EM[l] o_l.
-  double EA[3][kMaxPairs][kMaxPairs];
-  double EB[3][kMaxPairs][kMaxPairs];
-  double EBm[3][kMaxPairs];
-  double EM[3][kMaxPairs];
   // (1 + x)^gamma - 1 = sum_{k=1..8} eos_c[k-1] x^k for |x| < eos_xmax
   double eos_c[kEosTerms];
   double eos_xmax;
@@ -130,39 +119,6 @@ __device__ __forceinline__ bool is_nonfinite(double v) {
   return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000;
 }
 
-// rows[a] = sum_l Dm[d][a][l] f[l], a = 0..N, by the even/odd split
-// (2P + P (2P + [N even] + 2) + [N even] P FP64 operations, P = (N+1)/2:
-// 20 instead of 25 at N = 4).
-template <int N, int D>
-__device__ __forceinline__ void contract_eo(const LineParams& P, const double (&f)[N + 1],
-                                            double (&rows)[N + 1]) {
-  constexpr int Pp = (N + 1) / 2;
-  double e[Pp], o[Pp];
-#pragma unroll
-  for (int l = 0; l < Pp; ++l) {
-    e[l] = f[l] + f[N - l];
-    o[l] = f[l] - f[N - l];
-  }
-#pragma unroll
-  for (int i = 0; i < Pp; ++i) {
-    double s = P.EA[D][i][0] * o[0];
-#pragma unroll
-    for (int l = 1; l < Pp; ++l) s = fma(P.EA[D][i][l], o[l], s);
-    double t = P.EB[D][i][0] * e[0];
-#pragma unroll
-    for (int l = 1; l < Pp; ++l) t = fma(P.EB[D][i][l], e[l], t);
-    if (N % 2 == 0) t = fma(P.EBm[D][i], f[N / 2], t);
-    rows[i] = s + t;
-    rows[N - i] = s - t;
-  }
-  if (N % 2 == 0) {
-    double m = P.EM[D][0] * o[0];
-#pragma unroll
-    for (int l = 1; l < Pp; ++l) m = fma(P.EM[D][l], o[l], m);
-    rows[N / 2] = m;
-  }
-}
-
 // ---------------------------------------------------------------- difference form
 // The rho' and Theta' tendencies are residuals of cancelling flux
 // derivatives where the flow is nearly non-divergent (in a vortex the x and
@@ -177,21 +133,6 @@ __device__ __forceinline__ void contract_eo(const LineParams& P, const double (&
 //     F_l - F_0 = theta_l (m_l - m_0) + (theta_l - theta_0) m_0,
 // so the product's rounding scales with the variation as well.  The exact
 // value is unchanged.
-//
-// diffs(m, th, dm, dF): dm[l] = m_l - m_0 and dF[l] = theta_l m_l - theta_0
-// m_0 in that form, l = 0..N (dm[0] = dF[0] = -0, the additive identity, so
-// the even/odd contraction's sums with them need no instruction).
-template <int N>
-__device__ __forceinline__ void seg_diffs(const double (&m)[N + 1], const double (&th)[N + 1],
-                                          double (&dm)[N + 1], double (&dF)[N + 1]) {
-  dm[0] = -0.0;
-  dF[0] = -0.0;
-#pragma unroll
-  for (int l = 1; l <= N; ++l) {
-    dm[l] = m[l] - m[0];
-    dF[l] = fma(th[l], dm[l], (th[l] - th[0]) * m[0]);
-  }
-}
 
 // start + sum_{l>=1} Dm[d][a][l] d[l] (d[0] = 0 is not used)
 template <int N, int D>

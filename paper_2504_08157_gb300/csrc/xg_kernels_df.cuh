@@ -7,11 +7,12 @@
 // each equation is computed in the arithmetic its conditioning needs:
 //   * rho' and Theta' (Eq. 1a, 1c) -- their tendencies are residuals of
 //     cancelling flux derivatives where the flow is nearly non-divergent, so
-//     their whole path is native FP64: theta = Theta/rho, the fluxes' segment
-//     differences (difference form, xg_kernels.cuh), the contractions, the
+//     they keep FP64's precision throughout: theta = Theta/rho, the x
+//     contractions in 64-bit fixed point (xg_fixed.cuh), the y and z ones on
+//     the fluxes' segment differences (difference form, xg_kernels.cuh), the
 //     face sums, the partial tendency T, the heating source and the stage
-//     update.  These are the only FP64 instructions of the stage (~60 per
-//     node), which bound it.
+//     update.  These are the only FP64 instructions of the stage (46 per node
+//     at N = 4).
 //   * the momentum (Eq. 1b) -- its tendency does not cancel; primitives,
 //     the equation of state, fluxes, contractions (compensated Dot2), face
 //     sums, Coriolis and gravity and the stage update run in double-float
@@ -27,6 +28,7 @@
 #include <cuda_runtime.h>
 
 #include "xg_df.cuh"
+#include "xg_fixed.cuh"
 #include "xg_kernels.cuh"
 
 namespace xg {
@@ -182,21 +184,29 @@ __device__ __forceinline__ df df_row(const DfParams& P, int a, const df (&f)[N +
 // Orders whose x and y lines this file takes (above them df_uses_plane holds).
 constexpr int kDfLineOrder = 5;
 
-// Dynamic shared memory of the x pass: a line's fluxes and its segments' rows N.
-inline size_t df_x_smem(int nx, int nseg) { return sizeof(double) * (5 * (size_t)(nx + 1) + 5 * (size_t)nseg); }
-// Orders up to 4 at 8 CTAs per SM (64 registers): 0.691 against 0.722 ms per
-// launch with no bound (71 registers, 7 CTAs) and 0.706 at 10 (spilling), on
-// the 128 x 128 x 16 order-4 box; higher orders would spill at 8
+// Dynamic shared memory of the x pass: a line's fluxes (the segment after the
+// last holds the end node) and its segments' rows N.
+inline size_t df_x_smem(int N, int nseg) { return sizeof(double) * (5 * (size_t)(nseg + 1) * N + 5 * (size_t)nseg); }
+// Slot of node l of segment s.  At N = 2 and 4 the segment's slots rotate with
+// s, or the 16 lanes that share a wavefront, a segment each, would meet in 2 N
+// banks.
+template <int N>
+__device__ __forceinline__ int df_x_slot(int s, int l) {
+  if (N == 2 || N == 4) return s * N + ((l + (N == 2 ? s >> 3 : s >> 2)) & (N - 1));
+  return s * N + l;
+}
+// Orders up to 4 at 8 CTAs per SM (64 registers); higher orders would spill
 __host__ __device__ constexpr int df_x_min_blocks(int N) { return N <= 4 ? 8 : 1; }
 template <int N>
-__global__ void __launch_bounds__(kXThreads, df_x_min_blocks(N)) k_df_line_x(const DfParams P, const DfBufs B) {
+__global__ void __launch_bounds__(kXThreads, df_x_min_blocks(N)) k_df_line_x(const DfParams P, const FixRows FX,
+                                                                             const DfBufs B) {
   extern __shared__ df smd[];
   const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
   const int nseg = P.nseg[0];
   const int y = blockIdx.x, z = blockIdx.y;
   const long long np = P.np;
   const long long row = (long long)nx * (y + (long long)ny * z);
-  const int ld = nx + 1;
+  const int ld = (nseg + 1) * N;
   // [5][ld] fluxes (slots 0 and 4 doubles: rho u and theta; 1..3 pairs), later
   // rows 0..N-1 of every segment in place; RN [5][nseg] row N (same types)
   df* F = smd;
@@ -225,66 +235,73 @@ __global__ void __launch_bounds__(kXThreads, df_x_min_blocks(N)) k_df_line_x(con
     B.W[np + I] = w;
     B.W[2 * np + I] = pp;
     B.W64[I] = th;
-    F64[i] = mu;
-    F[ld + i] = df_add(df_mul(muD, u), pp);
-    F[2 * ld + i] = df_mul(mvD, u);
-    F[3 * ld + i] = df_mul(mwD, u);
-    F64[4 * ld + i] = th;                 // the Theta' flux is theta (rho u)
+    const int at = df_x_slot<N>(i / N, i % N);
+    F64[at] = mu;
+    F[ld + at] = df_add(df_mul(muD, u), pp);
+    F[2 * ld + at] = df_mul(mvD, u);
+    F[3 * ld + at] = df_mul(mwD, u);
+    F64[4 * ld + at] = th;                 // the Theta' flux is theta (rho u)
     if (P.per[0] && i == 0) {
-      F64[nx] = mu;
+      const int end = df_x_slot<N>(nseg, 0);
+      F64[end] = mu;
 #pragma unroll
-      for (int c = 1; c < 4; ++c) F[c * ld + nx] = F[c * ld];
-      F64[4 * ld + nx] = th;
+      for (int c = 1; c < 4; ++c) F[c * ld + end] = F[c * ld];
+      F64[4 * ld + end] = th;
     }
   }
   __syncthreads();
 
+  // one segment per thread, in place: the end node's values, which the next
+  // segment's thread overwrites, are read before any row is written.  rho' and
+  // Theta' in fixed point: with FP64 difference forms and even/odd contractions
+  // (17.5 FP64 instructions a node, now 12) the FP64 pipe bounded the pass, 0.696
+  // against 0.598 ms a launch on the 128 x 128 x 16 order-4 box; issue slots do
+  // now.  (In the y and z passes, at 14 and 21 FP64 instructions a node beside
+  // 820 and 1,390 of all kinds, fixed point only moved the bound: z 1.02 -> 1.11.)
   for (int s0 = 0; s0 < nseg; s0 += blockDim.x) {
     const int s = s0 + threadIdx.x;
-    double r64[2][N + 1];
-    df rows[3][N + 1];
+    int at[N];
+    double me = 0.0, te = 0.0;
+    df fe[3];
     if (s < nseg) {
-      {   // rho' and Theta': FP64, difference form
-        double m[N + 1], th[N + 1], dm[N + 1], dF[N + 1];
 #pragma unroll
-        for (int l = 0; l <= N; ++l) {
-          m[l] = F64[s * N + l];
-          th[l] = F64[4 * ld + s * N + l];
+      for (int l = 0; l < N; ++l) at[l] = df_x_slot<N>(s, l);
+      const int end = df_x_slot<N>(s + 1, 0);
+      me = F64[end];
+      te = F64[4 * ld + end];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) fe[c] = F[(c + 1) * ld + end];
+    }
+    __syncthreads();
+    if (s < nseg) {
+      {   // rho' and Theta' in fixed point
+        double m[N + 1], th[N + 1];
+#pragma unroll
+        for (int l = 0; l < N; ++l) {
+          m[l] = F64[at[l]];
+          th[l] = F64[4 * ld + at[l]];
         }
-        seg_diffs<N>(m, th, dm, dF);
-        contract_eo<N, 0>(P.P64, dm, r64[0]);
-        contract_eo<N, 0>(P.P64, dF, r64[1]);
+        m[N] = me;
+        th[N] = te;
+        fix_flux_rows<N>(FX, m, th, [&](int a, double r) { (a < N ? F64[at[a < N ? a : 0]] : RN64[s]) = r; },
+                         [&](int a, double r) { (a < N ? F64[4 * ld + at[a < N ? a : 0]] : RN64[4 * nseg + s]) = r; });
       }
 #pragma unroll
       for (int c = 1; c < 4; ++c) {
         df f[N + 1];
 #pragma unroll
-        for (int l = 0; l <= N; ++l) f[l] = F[c * ld + s * N + l];
+        for (int l = 0; l < N; ++l) f[l] = F[c * ld + at[l]];
+        f[N] = fe[c - 1];
 #pragma unroll
-        for (int a = 0; a <= N; ++a) rows[c - 1][a] = df_row<N, 0>(P, a, f);
-      }
-    }
-    __syncthreads();
-    if (s < nseg) {
-#pragma unroll
-      for (int a = 0; a < N; ++a) {
-        F64[s * N + a] = r64[0][a];
-        F64[4 * ld + s * N + a] = r64[1][a];
-      }
-      RN64[s] = r64[0][N];
-      RN64[4 * nseg + s] = r64[1][N];
-#pragma unroll
-      for (int c = 1; c < 4; ++c) {
-#pragma unroll
-        for (int a = 0; a < N; ++a) F[c * ld + s * N + a] = rows[c - 1][a];
-        RN[c * nseg + s] = rows[c - 1][N];
+        for (int a = 0; a < N; ++a) F[c * ld + at[a]] = df_row<N, 0>(P, a, f);
+        RN[c * nseg + s] = df_row<N, 0>(P, N, f);
       }
     }
     __syncthreads();
   }
 
   for (int i = threadIdx.x; i < nx; i += blockDim.x) {
-    const int s = i / N, a = i - s * N;
+    const int s = i / N, a = i - s * N, at = df_x_slot<N>(s, a);
     const long long I = row + i;
     const int left = s > 0 ? s - 1 : (P.per[0] ? nseg - 1 : -1);
 #pragma unroll
@@ -294,9 +311,9 @@ __global__ void __launch_bounds__(kXThreads, df_x_min_blocks(N)) k_df_line_x(con
         v = RN64[c * nseg + nseg - 1];
         v = v + v;
       } else if (a != 0) {
-        v = F64[c * ld + i];
+        v = F64[c * ld + at];
       } else {
-        const double r0 = F64[c * ld + i];
+        const double r0 = F64[c * ld + at];
         v = r0 + (left >= 0 ? RN64[c * nseg + left] : r0);
       }
       B.T[c * np + I] = v;
@@ -307,9 +324,9 @@ __global__ void __launch_bounds__(kXThreads, df_x_min_blocks(N)) k_df_line_x(con
       if (s == nseg) {
         v = df_scale2(RN[c * nseg + nseg - 1], 2.0f);
       } else if (a != 0) {
-        v = F[c * ld + i];
+        v = F[c * ld + at];
       } else {
-        const df r0 = F[c * ld + i];
+        const df r0 = F[c * ld + at];
         v = left >= 0 ? df_add(r0, RN[c * nseg + left]) : df_scale2(r0, 2.0f);
       }
       B.Tm[c * np + I] = v;

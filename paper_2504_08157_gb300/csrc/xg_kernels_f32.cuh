@@ -85,7 +85,7 @@ __device__ __forceinline__ float f_row_from(const FParams& P, int a, const float
 // zero; the roundings scale with the fluxes' variation across the segment
 // instead of the fluxes themselves, which matters where the two tendencies
 // are residuals of cancelling x, y and z parts (the difference form is
-// described in full beside df_seg_diffs).
+// described in full in xg_kernels.cuh).
 template <int N, int D>
 __device__ __forceinline__ void f_drows(const FParams& P, int a, const float (&m)[N + 1],
                                         const float (&th)[N + 1], float& r0, float& r4) {

@@ -163,17 +163,6 @@ inline void fill_line_params(const xg_mesh_desc* d, const MeshGeom& g, LineParam
       const double face = (a == 0 || a == N) ? 0.5 : 1.0;
       for (int l = 0; l <= N; ++l) P->Dm[k][a][l] = -(2.0 / h) * face * D[a][l];
     }
-    // even/odd split (the LGL matrix is centro-antisymmetric,
-    // D[N-i][N-l] = -D[i][l]; the halved rows 0 and N keep that property)
-    const int Pp = (N + 1) / 2;
-    for (int i = 0; i < Pp; ++i) {
-      for (int l = 0; l < Pp; ++l) {
-        P->EA[k][i][l] = 0.5 * (P->Dm[k][i][l] - P->Dm[k][i][N - l]);
-        P->EB[k][i][l] = 0.5 * (P->Dm[k][i][l] + P->Dm[k][i][N - l]);
-      }
-      P->EBm[k][i] = (N % 2 == 0) ? P->Dm[k][i][N / 2] : 0.0;
-      P->EM[k][i] = (N % 2 == 0) ? P->Dm[k][N / 2][i] : 0.0;
-    }
   }
   P->np = g.np;
   const double gamma = d->cp / d->cv;
