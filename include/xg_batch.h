@@ -11,22 +11,24 @@
  * instance's results equal those of xg_step / xg_rhs on an XG_FP32 context
  * of the same description bit for bit.
  *
- * Execution: one cooperative launch of G = ctas_per_sm x (SM count) CTAs
- * per call runs every pass of every stage of every step of every instance.
- * A pass is a list of tiles (x-y plane tiles of E x E elements per level,
- * then z tiles of 32 columns x K elements); CTAs take tiles according to a
- * schedule (below) and meet at a grid barrier between passes.  Each barrier
- * wait is bounded: a CTA that waits longer than the spin limit records
- * XG_ERR_TIMEOUT and every CTA leaves the launch at its next barrier.  The
- * launch is captured once per step count into a CUDA graph and replayed.
+ * Execution: a pass is a list of tiles (x-y plane tiles of E x E elements per
+ * level, then z tiles of 32 columns x K elements).  With XG_SCHED_LPT every
+ * pass of every order is one launch with a CTA per tile, the orders on streams
+ * of their own between a fork and a join of the call's stream.  With the other
+ * schedules one cooperative launch of G = ctas_per_sm x (SM count) CTAs per
+ * call runs every pass of every stage of every step of every instance: CTAs
+ * take tiles according to the schedule and meet at a grid barrier between
+ * passes.  Each barrier wait is bounded: a CTA that waits longer than the spin
+ * limit records XG_ERR_TIMEOUT and every CTA leaves the launch at its next
+ * barrier.  Either way the call's launches are captured once per step count
+ * into a CUDA graph and replayed.
  *
- * Schedules (element-to-CTA assignment):
+ * Schedules (tile-to-CTA assignment):
  *   XG_SCHED_ROUND_ROBIN  tile t of a pass goes to CTA t mod G (tiles in
  *                         instance order);
- *   XG_SCHED_LPT          tiles are assigned ahead of time by longest
- *                         processing time first from a per-tile cost model
- *                         (owned nodes, halo nodes, order), each CTA a
- *                         contiguous range;
+ *   XG_SCHED_LPT          longest processing time first: tiles sorted by a
+ *                         cost model (owned nodes, halo nodes, order), each
+ *                         started where room comes free first;
  *   XG_SCHED_DYNAMIC      CTAs claim the next tile with an atomic counter.
  * plane_tile selects the x-y tile: 0 = 32/N elements per side (up to 32 x
  * 32 nodes), 1 = 16/N.  xg_batch_autotune times the candidate (schedule,
@@ -49,10 +51,11 @@ typedef struct xg_batch xg_batch;
 
 enum { XG_SCHED_ROUND_ROBIN = 0, XG_SCHED_LPT = 1, XG_SCHED_DYNAMIC = 2 };
 
-/* A launch configuration of the persistent kernel.
+/* A launch configuration.
  *   schedule      XG_SCHED_*
  *   plane_tile    0 or 1 (see above)
- *   ctas_per_sm   1 or 2 (clamped to what fits on an SM)
+ *   ctas_per_sm   1 or 2 (clamped to what fits on an SM; XG_SCHED_LPT: 1 keeps
+ *                 an SM to one CTA of a pass, 2 lets as many run as fit)
  *   ms_per_step   filled by xg_batch_autotune / xg_batch_get_tuning: the
  *                 measured milliseconds per SSP-RK3 step of the whole batch
  *                 with this configuration (0 when not measured) */
@@ -83,7 +86,7 @@ xg_status xg_batch_count(const xg_batch* b, int* count);
 xg_ctx* xg_batch_instance(xg_batch* b, int i);
 
 /* nsteps SSP-RK3 steps of every instance i with its own step dt[i] (host
- * array of `count` values), all in one persistent launch on `stream`.
+ * array of `count` values), on `stream`.
  * Every instance must have a state.  Waits for the GPU at the end.
  * Errors: XG_ERR_ARG (NULL, nsteps < 0, a dt not finite, an instance
  * without state), XG_ERR_UNSUPPORTED (an instance has a learned closure
@@ -92,8 +95,7 @@ xg_ctx* xg_batch_instance(xg_batch* b, int i);
  * XG_ERR_TIMEOUT, XG_ERR_CUDA. */
 xg_status xg_batch_step(xg_batch* b, const double* dt, int nsteps, void* stream);
 
-/* Right-hand sides of every instance for its current state, in one
- * persistent launch: dqdt[i] [5][Np_i] (an array of `count` pointers, each
+/* Right-hand sides of every instance for its current state: dqdt[i] [5][Np_i] (an array of `count` pointers, each
  * host or device memory as `where` says).  Does not modify any state.
  * Errors: XG_ERR_ARG, XG_ERR_TIMEOUT, XG_ERR_CUDA. */
 xg_status xg_batch_rhs(xg_batch* b, double* const* dqdt, int where, void* stream);

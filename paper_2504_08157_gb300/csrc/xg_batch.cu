@@ -1,15 +1,16 @@
 // xg_batch.cu -- the batched persistent form (include/xg_batch.h).
 //
 // Many independent XG_FP32 instances (own mesh, order, reference state and
-// forcing) advance in one cooperative launch of a persistent kernel.  Every
-// stage is two passes over all instances -- x-y plane tiles (f_plane_tile:
-// primitives, x and y parts) and z tiles (f_tline_tile: z part, sources,
-// walls, inverse mass, SSP-RK3 combination) -- separated by a grid barrier
-// with a bounded wait.  The per-node arithmetic is the single-context FP32
+// forcing) advance together.  Every stage is two passes over all instances --
+// x-y plane tiles (f_plane_tile: primitives, x and y parts) and z tiles
+// (f_tline_tile: z part, sources, walls, inverse mass, SSP-RK3 combination) --
+// as a launch per pass and order (XG_SCHED_LPT, the default) or inside one
+// cooperative launch of a persistent kernel, with a grid barrier of bounded wait
+// between the passes.  The per-node arithmetic is the single-context FP32
 // path's (the same device functions), so results are bitwise those of an
 // XG_FP32 context; what is batched is only the scheduling.
 //
-// Data written inside the launch (stage buffers, W, T) is read with
+// Data written inside the persistent launch (stage buffers, W, T) is read with
 // L2-only loads (the CG variants of the tile functions): L1 is not coherent
 // across SMs within a launch.
 #include <algorithm>
@@ -18,7 +19,6 @@
 #include <cstring>
 #include <map>
 #include <new>
-#include <queue>
 #include <utility>
 #include <vector>
 
@@ -61,12 +61,10 @@ constexpr int kGroups = kBatchMaxOrder - kBatchMinOrder + 1;   // tiles grouped 
 
 // Launch arguments.  Each pass's tile list is grouped by order (group g:
 // N = 3 + g) and, within a group, in instance order; goff/gcnt locate the
-// groups.  XG_SCHED_LPT permutes the list so that CTA c's tiles of group g
-// are lpt[pass][c (kGroups + 1) + g] .. lpt[pass][c (kGroups + 1) + g + 1] - 1.
+// groups.  XG_SCHED_LPT sorts each group by cost.
 struct BRun {
   const BInst* inst;
   const int4* items[2];   // pass 0 {inst, bx, by, z}; pass 1 {inst, bx, z-block, y}
-  const int* lpt[2];
   int goff[2][kGroups], gcnt[2][kGroups];
   int schedule;
   int plane_half;
@@ -147,17 +145,9 @@ __device__ __noinline__ void run_group(const BRun& R, int s, int st, int par, in
   const int4* items = R.items[PASS];
   BInst& I = *reinterpret_cast<BInst*>(smb);
   float* work = reinterpret_cast<float*>(smb + kInstBytes);
-  int k, kend, kstep;
-  if (R.schedule == XG_SCHED_LPT) {
-    const int* t = R.lpt[PASS] + blockIdx.x * (kGroups + 1) + g;
-    k = t[0];
-    kend = t[1];
-    kstep = 1;
-  } else {   // round robin over the whole pass list: position p goes to CTA p mod G
-    k = off + (int)((blockIdx.x + G - (unsigned)off % G) % G);
-    kend = off + n;
-    kstep = G;
-  }
+  // round robin over the whole pass list: position p goes to CTA p mod G
+  int k = off + (int)((blockIdx.x + G - (unsigned)off % G) % G);
+  const int kend = off + n, kstep = G;
   const unsigned long long cbase = (unsigned long long)s * (unsigned long long)(n + G);
   while (true) {
     if (R.schedule == XG_SCHED_DYNAMIC) {
@@ -226,6 +216,73 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch(const __grid_constan
   }
 }
 
+// ---------------------------------------------------------------- passes as launches (XG_SCHED_LPT)
+// One launch a pass and order, one CTA a tile, the tiles sorted by cost: the
+// hardware hands the longest tile left to the first SM with room, which is the
+// LPT rule itself with the true times, and the CTA shapes and occupancy are
+// the single context's (plane: 256 threads; z: K N + 1 <= 9 levels of 32)
+// instead of the 2 x 16 warps that have to serve every tile of the persistent
+// kernel.  The orders are chains of their own: no pass waits for another
+// order's tiles, and their tails overlap.  96 uneven boxes (15.6 M nodes), four
+// steps with the states' copies in and out: 20.9 -> 14.4 ms.
+template <int THREADS>
+__device__ __forceinline__ const BInst& load_instance(const BRun& R, int i, unsigned char* smb) {
+  const int4* src = reinterpret_cast<const int4*>(R.inst + i);
+  int4* dst = reinterpret_cast<int4*>(smb);
+  const int tid = threadIdx.x + 32 * threadIdx.y;
+  for (int t = tid; t < (int)(sizeof(BInst) / 16); t += THREADS) dst[t] = __ldg(src + t);
+  __syncthreads();
+  return *reinterpret_cast<const BInst*>(smb);
+}
+
+template <int N, int HALF>
+__global__ void __launch_bounds__(kPlaneThreads) k_batch_plane(const __grid_constant__ BRun R, int st, int par) {
+  extern __shared__ __align__(128) unsigned char smb[];
+  const int4 it = __ldg(R.items[0] + R.goff[0][N - kBatchMinOrder] + blockIdx.x);
+  const BInst& I = load_instance<kPlaneThreads>(R, it.x, smb);
+  f_plane_tile<N, batch_plane_elems(N, HALF), kPlaneBatch, false>(I.P, stage_bufs(R, I, st, par), it.y, it.z, it.w,
+                                                                  reinterpret_cast<float*>(smb + kInstBytes),
+                                                                  threadIdx.x, kPlaneThreads);
+}
+
+template <int N>
+__global__ void __launch_bounds__(kTileCols * (8 + 1), 4) k_batch_z(const __grid_constant__ BRun R, int st, int par) {
+  constexpr int K = f32_tile_segments(N);
+  extern __shared__ __align__(128) unsigned char smb[];
+  const int4 it = __ldg(R.items[1] + R.goff[1][N - kBatchMinOrder] + blockIdx.x);
+  const BInst& I = load_instance<kTileCols * (K * N + 1)>(R, it.x, smb);
+  f_tline_tile<N, 2, false, K>(I.P, stage_bufs(R, I, st, par), it.y, it.z, it.w, threadIdx.x, threadIdx.y,
+                               reinterpret_cast<float*>(smb + kInstBytes));
+}
+
+template <int N>
+size_t pass_smem(int pass, int half) {
+  if (pass == 1) return kInstBytes + sizeof(float) * (size_t)tline_smem_floats(N, f32_tile_segments(N));
+  return kInstBytes + (half ? PlaneLayoutF<N, batch_plane_elems(N, 1)>::bytes : PlaneLayoutF<N, batch_plane_elems(N, 0)>::bytes);
+}
+
+// The stages of order N's instances on stream st; ctas_per_sm = 1 leaves room
+// for one CTA of a pass per SM.
+template <int N>
+cudaError_t launch_order(const BRun& R, int one_cta, size_t sm_smem, cudaStream_t st) {
+  constexpr int g = N - kBatchMinOrder;
+  if (R.gcnt[0][g] == 0) return cudaSuccess;
+  size_t bytes[2];
+  for (int pass = 0; pass < 2; ++pass)
+    bytes[pass] = one_cta ? std::max(pass_smem<N>(pass, R.plane_half), sm_smem / 2 + 1024) : pass_smem<N>(pass, R.plane_half);
+  cudaError_t e = raise_dynamic_smem(k_batch_z<N>, bytes[1]);
+  if (e == cudaSuccess)
+    e = R.plane_half ? raise_dynamic_smem(k_batch_plane<N, 1>, bytes[0]) : raise_dynamic_smem(k_batch_plane<N, 0>, bytes[0]);
+  if (e != cudaSuccess) return e;
+  for (int s = 0; s < R.nstages; ++s) {
+    const int stage = R.rhs_only ? 0 : s % 3, par = R.rhs_only ? 0 : (s / 3) & 1;
+    if (R.plane_half) k_batch_plane<N, 1><<<R.gcnt[0][g], kPlaneThreads, bytes[0], st>>>(R, stage, par);
+    else k_batch_plane<N, 0><<<R.gcnt[0][g], kPlaneThreads, bytes[0], st>>>(R, stage, par);
+    k_batch_z<N><<<R.gcnt[1][g], dim3(kTileCols, f32_tile_segments(N) * N + 1), bytes[1], st>>>(R, stage, par);
+  }
+  return cudaGetLastError();
+}
+
 // Shared memory of one CTA for the orders lo..hi and a plane tile choice.
 size_t batch_smem(int lo, int hi, int half) {
   size_t m = 0;
@@ -244,6 +301,12 @@ size_t batch_smem(int lo, int hi, int half) {
 using xg::BInst;
 using xg::BRun;
 
+// Both passes' tiles on the device, grouped by order.
+struct TileList {
+  int4* items[2] = {nullptr, nullptr};
+  int off[2][xg::kGroups] = {}, cnt[2][xg::kGroups] = {};
+};
+
 struct xg_batch {
   std::vector<xg_ctx*> inst;
   int count = 0;
@@ -257,21 +320,19 @@ struct xg_batch {
   bool failed = false;
   BInst* dinst = nullptr;        // [count]
   BInst* hinst = nullptr;        // pinned [count]
-  // tile lists per plane-tile choice and pass, grouped by order, with the
-  // LPT permutation and per-CTA ranges for the grid they were built for
-  int4* ditems[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
-  int goff[2][2][xg::kGroups] = {}, gcnt[2][2][xg::kGroups] = {};
-  std::vector<int4> hitems[2][2];
-  std::vector<double> cost[2][2];
-  int4* dlpt[2] = {nullptr, nullptr};   // current configuration's LPT order, per pass
-  int* dtbl[2] = {nullptr, nullptr};    // [grid][kGroups + 1] range starts
-  int lpt_grid = 0, lpt_half = -1;
+  // tile lists per plane-tile choice, grouped by order: of the persistent
+  // kernel's schedules, and of the launches (sorted by cost)
+  TileList tiles[2], sorted[2];
   // launch bookkeeping: bar, err, flag, ctr[2][kGroups] (zeroed at every launch)
   unsigned char* dsync = nullptr;
   int* hsync = nullptr;          // pinned copy of err, flag
   cudaStream_t cap = nullptr;
   std::map<std::pair<int, int>, cudaGraphExec_t> graphs;   // (stages, rhs_only)
   cudaEvent_t ev[2] = {nullptr, nullptr};
+  // XG_SCHED_LPT: a stream and a join event an order, and the fork
+  cudaStream_t side[xg::kGroups] = {};
+  cudaEvent_t fork = nullptr, join[xg::kGroups] = {};
+  size_t sm_smem = 0;
 };
 
 namespace {
@@ -297,110 +358,63 @@ void drop_graphs(xg_batch* b) {
   b->graphs.clear();
 }
 
-// Tile lists of every instance for one plane-tile choice, grouped by
-// order, with a cost per tile for the LPT schedule: loaded and owned nodes
-// plus a fixed per-tile overhead (in node units).
-void build_items(xg_batch* b, int half) {
-  for (int pass = 0; pass < 2; ++pass) {
-    b->hitems[half][pass].clear();
-    b->cost[half][pass].clear();
-  }
+// Tile lists of every instance for one plane-tile choice, grouped by order;
+// z_segments: of a z tile.  by_cost: each pass and group longest first (equal
+// ones in instance order), by a cost per tile of loaded and owned nodes plus a
+// fixed overhead (in node units).
+cudaError_t build_tiles(const xg_batch* b, int half, int (*z_segments)(int), bool by_cost, TileList* out) {
   const double overhead = 256.0;
-  for (int g = 0; g < xg::kGroups; ++g) {
-    for (int pass = 0; pass < 2; ++pass) b->goff[half][pass][g] = (int)b->hitems[half][pass].size();
-    for (int i = 0; i < b->count; ++i) {
-      const xg_ctx* c = b->inst[i];
-      const int N = c->d.order;
-      if (N != xg::kBatchMinOrder + g) continue;
-      const int* nel = c->d.nel;
-      const int E = xg::batch_plane_elems(N, half);
-      for (int z = 0; z < c->n[2]; ++z)
-        for (int by = 0; by < (nel[1] + E - 1) / E; ++by)
-          for (int bx = 0; bx < (nel[0] + E - 1) / E; ++bx) {
-            b->hitems[half][0].push_back(make_int4(i, bx, by, z));
-            const int ex = std::min(E, nel[0] - bx * E), ey = std::min(E, nel[1] - by * E);
-            const double own = (double)(ex * N + 1) * (ey * N + 1);
-            const double halo = (double)N * ((ex + ey) * N + 2);
-            b->cost[half][0].push_back(2.0 * own + halo + overhead);
-          }
-      const int K = xg::batch_z_segments(N);
-      const int xb = (c->n[0] + xg::kTileCols - 1) / xg::kTileCols;
-      for (int y = 0; y < c->n[1]; ++y)
-        for (int zb = 0; zb < (nel[2] + K - 1) / K; ++zb)
-          for (int bx = 0; bx < xb; ++bx) {
-            b->hitems[half][1].push_back(make_int4(i, bx, zb, y));
-            const int cols = std::min(xg::kTileCols, c->n[0] - bx * xg::kTileCols);
-            const int kc = std::min(K, nel[2] - zb * K);
-            b->cost[half][1].push_back((double)cols * (kc * N + 1) * 2.5 + (double)cols * N + overhead);
-          }
-    }
-    for (int pass = 0; pass < 2; ++pass)
-      b->gcnt[half][pass][g] = (int)b->hitems[half][pass].size() - b->goff[half][pass][g];
-  }
-}
-
-cudaError_t upload_items(xg_batch* b, int half) {
-  for (int pass = 0; pass < 2; ++pass) {
-    const auto& h = b->hitems[half][pass];
-    cudaError_t e = cudaMalloc((void**)&b->ditems[half][pass], sizeof(int4) * std::max<size_t>(h.size(), 1));
-    if (e != cudaSuccess) return e;
-    e = cudaMemcpy(b->ditems[half][pass], h.data(), sizeof(int4) * h.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-// Longest-processing-time-first assignment of each pass's tiles to the
-// grid's CTAs; every CTA's tiles are then ordered by group and instance.
-cudaError_t build_lpt(xg_batch* b, int half, int grid) {
-  if (b->lpt_grid == grid && b->lpt_half == half) return cudaSuccess;
-  constexpr int NG = xg::kGroups;
-  for (int pass = 0; pass < 2; ++pass) {
-    const auto& items = b->hitems[half][pass];
-    const auto& cost = b->cost[half][pass];
-    const size_t n = items.size();
-    std::vector<int> order(n), group(n);
-    for (int g = 0; g < NG; ++g)
-      for (int k = 0; k < b->gcnt[half][pass][g]; ++k) group[b->goff[half][pass][g] + k] = g;
-    for (size_t k = 0; k < n; ++k) order[k] = (int)k;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int c) { return cost[a] > cost[c]; });
-    using Load = std::pair<double, int>;
-    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
-    for (int g = 0; g < grid; ++g) heap.push({0.0, g});
-    std::vector<int> owner(n);
-    for (int k : order) {
-      Load l = heap.top();
-      heap.pop();
-      owner[k] = l.second;
-      l.first += cost[k];
-      heap.push(l);
-    }
-    std::vector<int> tbl((size_t)grid * (NG + 1), 0), fill((size_t)grid * NG, 0);
-    for (size_t k = 0; k < n; ++k) ++fill[(size_t)owner[k] * NG + group[k]];
-    int pos = 0;
-    for (int c = 0; c < grid; ++c) {
-      for (int g = 0; g < NG; ++g) {
-        tbl[(size_t)c * (NG + 1) + g] = pos;
-        const int cnt = fill[(size_t)c * NG + g];
-        fill[(size_t)c * NG + g] = pos;
-        pos += cnt;
+  TileList t;
+  cudaError_t e = cudaSuccess;
+  for (int pass = 0; pass < 2 && e == cudaSuccess; ++pass) {
+    std::vector<int4> list;
+    for (int g = 0; g < xg::kGroups; ++g) {
+      const int N = xg::kBatchMinOrder + g;
+      std::vector<std::pair<double, int4>> tiles;
+      for (int i = 0; i < b->count; ++i) {
+        const xg_ctx* c = b->inst[i];
+        if (c->d.order != N) continue;
+        const int* nel = c->d.nel;
+        if (pass == 0) {
+          const int E = xg::batch_plane_elems(N, half);
+          for (int z = 0; z < c->n[2]; ++z)
+            for (int by = 0; by < (nel[1] + E - 1) / E; ++by)
+              for (int bx = 0; bx < (nel[0] + E - 1) / E; ++bx) {
+                const int ex = std::min(E, nel[0] - bx * E), ey = std::min(E, nel[1] - by * E);
+                const double own = (double)(ex * N + 1) * (ey * N + 1);
+                const double halo = (double)N * ((ex + ey) * N + 2);
+                tiles.push_back({2.0 * own + halo + overhead, make_int4(i, bx, by, z)});
+              }
+        } else {
+          const int K = z_segments(N);
+          const int xb = (c->n[0] + xg::kTileCols - 1) / xg::kTileCols;
+          for (int y = 0; y < c->n[1]; ++y)
+            for (int zb = 0; zb < (nel[2] + K - 1) / K; ++zb)
+              for (int bx = 0; bx < xb; ++bx) {
+                const int cols = std::min(xg::kTileCols, c->n[0] - bx * xg::kTileCols);
+                const int kc = std::min(K, nel[2] - zb * K);
+                tiles.push_back({(double)cols * (kc * N + 1) * 2.5 + (double)cols * N + overhead,
+                                 make_int4(i, bx, zb, y)});
+              }
+        }
       }
-      tbl[(size_t)c * (NG + 1) + NG] = pos;
+      if (by_cost)
+        std::stable_sort(tiles.begin(), tiles.end(), [](const std::pair<double, int4>& p, const std::pair<double, int4>& q) {
+          return p.first > q.first;
+        });
+      t.off[pass][g] = (int)list.size();
+      t.cnt[pass][g] = (int)tiles.size();
+      for (const auto& x : tiles) list.push_back(x.second);
     }
-    std::vector<int4> perm(std::max<size_t>(n, 1));
-    for (size_t k = 0; k < n; ++k) perm[fill[(size_t)owner[k] * NG + group[k]]++] = items[k];
-    cudaFree(b->dlpt[pass]);
-    cudaFree(b->dtbl[pass]);
-    b->dlpt[pass] = nullptr;
-    b->dtbl[pass] = nullptr;
-    cudaError_t e = cudaMalloc((void**)&b->dlpt[pass], sizeof(int4) * perm.size());
-    if (e == cudaSuccess) e = cudaMalloc((void**)&b->dtbl[pass], sizeof(int) * tbl.size());
-    if (e == cudaSuccess) e = cudaMemcpy(b->dlpt[pass], perm.data(), sizeof(int4) * perm.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(b->dtbl[pass], tbl.data(), sizeof(int) * tbl.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return e;
+    e = cudaMalloc((void**)&t.items[pass], sizeof(int4) * std::max<size_t>(list.size(), 1));
+    if (e == cudaSuccess)
+      e = cudaMemcpy(t.items[pass], list.data(), sizeof(int4) * list.size(), cudaMemcpyHostToDevice);
   }
-  b->lpt_grid = grid;
-  b->lpt_half = half;
+  if (e != cudaSuccess) {
+    for (int4* p : t.items) cudaFree(p);
+    return e;
+  }
+  *out = t;
   return cudaSuccess;
 }
 
@@ -409,9 +423,11 @@ cudaError_t build_lpt(xg_batch* b, int half, int grid) {
 cudaError_t apply_tuning(xg_batch* b) {
   const int half = b->tune.plane_tile;
   cudaError_t e = cudaSuccess;
-  if (!b->ditems[half][0]) {
-    build_items(b, half);
-    e = upload_items(b, half);
+  const bool lpt = b->tune.schedule == XG_SCHED_LPT;
+  TileList& t = lpt ? b->sorted[half] : b->tiles[half];
+  if (!t.items[0]) {
+    e = build_tiles(b, half, lpt ? [](int N) { return xg::f32_tile_segments(N); }
+                                 : [](int N) { return xg::batch_z_segments(N); }, lpt, &t);
     if (e != cudaSuccess) return e;
   }
   const size_t smem = xg::batch_smem(b->lo_order, b->hi_order, half);
@@ -420,10 +436,6 @@ cudaError_t apply_tuning(xg_batch* b) {
   if (e != cudaSuccess) return e;
   if (occ < 1) return cudaErrorInvalidConfiguration;
   const int grid = std::min(b->tune.ctas_per_sm, occ) * b->sms;
-  if (b->tune.schedule == XG_SCHED_LPT) {
-    e = build_lpt(b, half, grid);
-    if (e != cudaSuccess) return e;
-  }
   drop_graphs(b);   // a captured launch holds the old configuration's arguments
   b->grid = grid;
   b->smem = smem;
@@ -435,17 +447,12 @@ BRun make_run(xg_batch* b, int nstages, int rhs_only, int selftest, long long sp
   memset(&R, 0, sizeof(R));
   const int half = b->tune.plane_tile;
   R.inst = b->dinst;
+  const TileList& t = b->tune.schedule == XG_SCHED_LPT ? b->sorted[half] : b->tiles[half];
   for (int pass = 0; pass < 2; ++pass) {
+    R.items[pass] = t.items[pass];
     for (int g = 0; g < xg::kGroups; ++g) {
-      R.goff[pass][g] = b->goff[half][pass][g];
-      R.gcnt[pass][g] = b->gcnt[half][pass][g];
-    }
-    if (b->tune.schedule == XG_SCHED_LPT) {
-      R.items[pass] = b->dlpt[pass];
-      R.lpt[pass] = b->dtbl[pass];
-    } else {
-      R.items[pass] = b->ditems[half][pass];
-      R.lpt[pass] = nullptr;
+      R.goff[pass][g] = t.off[pass][g];
+      R.gcnt[pass][g] = t.cnt[pass][g];
     }
   }
   R.schedule = b->tune.schedule;
@@ -481,6 +488,26 @@ cudaError_t launch(xg_batch* b, const BRun& R, cudaStream_t st) {
   cfg.numAttrs = 1;
   cudaError_t e = cudaMemsetAsync(b->dsync, 0, kSyncBytes, st);
   if (e != cudaSuccess) return e;
+  if (R.schedule == XG_SCHED_LPT && !R.selftest) {
+    const int one = b->tune.ctas_per_sm == 1;
+    e = cudaEventRecord(b->fork, st);
+    for (int g = 0; g < xg::kGroups && e == cudaSuccess; ++g) {
+      if (R.gcnt[0][g] == 0) continue;
+      e = cudaStreamWaitEvent(b->side[g], b->fork, 0);
+      if (e == cudaSuccess) {
+        switch (xg::kBatchMinOrder + g) {
+          case 3: e = xg::launch_order<3>(R, one, b->sm_smem, b->side[g]); break;
+          case 4: e = xg::launch_order<4>(R, one, b->sm_smem, b->side[g]); break;
+          case 5: e = xg::launch_order<5>(R, one, b->sm_smem, b->side[g]); break;
+          default: e = xg::launch_order<6>(R, one, b->sm_smem, b->side[g]); break;
+        }
+      }
+      const cudaError_t ej = cudaEventRecord(b->join[g], b->side[g]);   // joined also after an error (a capture ends)
+      const cudaError_t ew = cudaStreamWaitEvent(st, b->join[g], 0);
+      if (e == cudaSuccess) e = ej != cudaSuccess ? ej : ew;
+    }
+    return e;
+  }
   return cudaLaunchKernelEx(&cfg, xg::k_batch, R);
 }
 
@@ -607,6 +634,14 @@ xg_status xg_batch_create(const xg_mesh_desc* d, int count, xg_batch** out) {
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreate(&b->ev[0]);
   if (e == cudaSuccess) e = cudaEventCreate(&b->ev[1]);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
+  for (int g = 0; g < xg::kGroups && e == cudaSuccess; ++g) {
+    e = cudaStreamCreateWithFlags(&b->side[g], cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join[g], cudaEventDisableTiming);
+  }
+  int per_sm = 0;
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, b->dev);
+  b->sm_smem = (size_t)per_sm;
   if (e == cudaSuccess) e = apply_tuning(b);
   if (e != cudaSuccess) {
     const bool oom = e == cudaErrorMemoryAllocation;
@@ -778,11 +813,10 @@ void xg_batch_destroy(xg_batch* b) {
   drop_graphs(b);
   for (xg_ctx* c : b->inst) xg_destroy(c);
   for (int h = 0; h < 2; ++h)
-    for (int p = 0; p < 2; ++p) cudaFree(b->ditems[h][p]);
-  for (int p = 0; p < 2; ++p) {
-    cudaFree(b->dlpt[p]);
-    cudaFree(b->dtbl[p]);
-  }
+    for (int p = 0; p < 2; ++p) {
+      cudaFree(b->tiles[h].items[p]);
+      cudaFree(b->sorted[h].items[p]);
+    }
   cudaFree(b->dinst);
   cudaFreeHost(b->hinst);
   cudaFree(b->dsync);
@@ -790,6 +824,11 @@ void xg_batch_destroy(xg_batch* b) {
   if (b->cap) cudaStreamDestroy(b->cap);
   for (auto& e : b->ev)
     if (e) cudaEventDestroy(e);
+  if (b->fork) cudaEventDestroy(b->fork);
+  for (int g = 0; g < xg::kGroups; ++g) {
+    if (b->side[g]) cudaStreamDestroy(b->side[g]);
+    if (b->join[g]) cudaEventDestroy(b->join[g]);
+  }
   cudaGetLastError();
   delete b;
 }
