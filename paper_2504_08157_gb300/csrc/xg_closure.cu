@@ -3,7 +3,7 @@
 // Kernels:
 //   * features of a state: q, assembled gradients, heating (k_features);
 //   * restriction of fine fields to coarse nodes, one axis at a time
-//     (k_interp_axis);
+//     (k_interp_z, k_interp_y, k_interp_x);
 //   * training in FP32 on the CUDA cores: forward and back-propagation over
 //     chunks of samples with the weights and activations in shared memory
 //     and the block's gradient sums in registers (k_mlp_grad, each gradient
@@ -22,6 +22,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -137,25 +138,119 @@ __global__ void __launch_bounds__(128) k_features(const FParams P, const float* 
 
 // ------------------------------------------------------------------ restriction
 
-// out[o][c][i] = sum_a w[c][a] in[o][(start[c] + a) mod n_in][i]
-__global__ void k_interp_axis(const double* __restrict__ in, double* __restrict__ out, long long outer,
-                              int n_in, int n_out, long long inner, const int* __restrict__ start,
-                              const double* __restrict__ w, int npts) {
-  const long long total = outer * n_out * inner;
-  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x) {
-    const long long i = t % inner;
-    const long long rest = t / inner;
-    const int c = (int)(rest % n_out);
-    const long long o = rest / n_out;
-    double acc = 0.0;
-    for (int a = 0; a < npts; ++a) {
-      int k = start[c] + a;
-      if (k >= n_in) k -= n_in;
-      acc = fma(w[c * npts + a], in[(o * n_in + k) * inner + i], acc);
+// One axis of the restriction: coarse node c takes the np_f = N_f + 1 values of
+// its fine element from fine node start[c] on, with weights w[c][.].  one[c]:
+// the point that the coarse node falls on (its weight is 1 and the others are
+// below 2^-60), or -1: half of the coarse nodes of a mesh refined by two, which
+// then cost no FP64 operation.
+struct InterpAxis {
+  const int* start;
+  const int* one;
+  const double* w;
+  int n_in, n_out, npts;
+};
+
+// One coarse node's weights and points, in registers.
+template <int NP>
+struct InterpNode {
+  int k[NP], one;   // one: the fine node it falls on, or -1
+  double w[NP];
+  __device__ __forceinline__ void load(const InterpAxis& A, int c) {
+    const int s = A.start[c], o = A.one[c];
+    one = o < 0 ? -1 : (s + o >= A.n_in ? s + o - A.n_in : s + o);
+#pragma unroll
+    for (int a = 0; a < NP; ++a) {
+      k[a] = s + a >= A.n_in ? s + a - A.n_in : s + a;
+      w[a] = A.w[c * NP + a];
     }
-    out[t] = acc;
   }
+  // at(k): the value of fine node k.  A value that is not finite counts with
+  // every weight, a zero among them.
+  template <typename At>
+  __device__ __forceinline__ double value(At at) const {
+    if (one >= 0) {
+      unsigned e = 0;
+#pragma unroll
+      for (int a = 0; a < NP; ++a)
+        if (k[a] != one) e = max(e, (unsigned)__double2hiint(at(k[a])) & 0x7ff00000u);
+      const double v = at(one);
+      return e == 0x7ff00000u ? __hiloint2double(0x7ff80000, 0) : v;
+    }
+    double r = 0.0;
+#pragma unroll
+    for (int a = 0; a < NP; ++a) r = fma(w[a], at(k[a]), r);
+    return r;
+  }
+};
+
+// The three passes, z, y, x, over the n planes from p0 on (of nvar n_zc
+// [variable][coarse level]) of one chunk: z reads src and writes out [plane]
+// [y_f][x_f], y writes [plane][y_c][x_f], x the result.  With z first every
+// pass runs along contiguous lines, no index is divided, and a chunk's
+// intermediates stay in L2.  A thread of the z and y passes walks along the
+// interpolated axis, so that the fine values that consecutive coarse nodes share
+// come from L1: one coarse node a thread read five values from L2 for each.
+template <int NP>
+__global__ void __launch_bounds__(256) k_interp_z(const double* __restrict__ in, double* __restrict__ out,
+                                                  const InterpAxis A, long long plane, int p0, int np) {
+  for (long long i = blockIdx.x * 256ll + threadIdx.x; i < plane; i += gridDim.x * 256ll) {
+    int v = p0 / A.n_out, c = p0 - v * A.n_out;
+    const double* f = in + (long long)v * A.n_in * plane + i;
+    double* o = out + i;
+    for (int p = 0; p < np; ++p) {
+      InterpNode<NP> n;
+      n.load(A, c);
+      *o = n.value([&](int k) { return f[k * plane]; });
+      o += plane;
+      if (++c == A.n_out) {
+        c = 0;
+        f += A.n_in * plane;
+      }
+    }
+  }
+}
+
+constexpr int kInterpRows = 16;   // coarse lines a thread of the y pass walks
+template <int NP>
+__global__ void __launch_bounds__(128) k_interp_y(const double* __restrict__ in, double* __restrict__ out,
+                                                  const InterpAxis A, int nx) {
+  const double* f = in + (long long)blockIdx.z * A.n_in * nx;
+  double* o = out + (long long)blockIdx.z * A.n_out * nx;
+  for (int c0 = blockIdx.y * kInterpRows; c0 < A.n_out; c0 += gridDim.y * kInterpRows)
+    for (int i = blockIdx.x * 128 + threadIdx.x; i < nx; i += gridDim.x * 128)
+      for (int c = c0; c < min(c0 + kInterpRows, A.n_out); ++c) {
+        InterpNode<NP> n;
+        n.load(A, c);
+        o[(long long)c * nx + i] = n.value([&](int k) { return f[(long long)k * nx + i]; });
+      }
+}
+
+// A thread keeps its coarse node and walks down the lines.
+template <int NP>
+__global__ void __launch_bounds__(128) k_interp_x(const double* __restrict__ in, double* __restrict__ out,
+                                                  const InterpAxis A, long long lines) {
+  const int c = blockIdx.x * 128 + threadIdx.x;
+  if (c >= A.n_out) return;
+  InterpNode<NP> n;
+  n.load(A, c);
+  for (long long j = blockIdx.y; j < lines; j += gridDim.y)
+    out[j * A.n_out + c] = n.value([&](int k) { return in[j * A.n_in + k]; });
+}
+
+// The passes of one chunk of n planes.
+template <int NP>
+cudaError_t interp_chunk(const double* src, double* t1, double* t2, double* dst, const InterpAxis (&A)[3], int p0,
+                         unsigned n, cudaStream_t st) {
+  const int nx = A[0].n_in, nyf = A[1].n_in, nyc = A[1].n_out;
+  const long long plane = (long long)nx * nyf;
+  const unsigned bz = (unsigned)std::min<long long>((plane + 255) / 256, 1 << 20);
+  k_interp_z<NP><<<bz, 256, 0, st>>>(src, t1, A[2], plane, p0, (int)n);
+  const unsigned by = (unsigned)std::min((nyc + kInterpRows - 1) / kInterpRows, 65535);
+  k_interp_y<NP><<<dim3((unsigned)((nx + 127) / 128), by, n), 128, 0, st>>>(t1, t2, A[1], nx);
+  const long long lines = (long long)nyc * n;
+  k_interp_x<NP><<<dim3((unsigned)((A[0].n_out + 127) / 128), (unsigned)std::min<long long>((lines + 3) / 4, 65535)),
+                   128, 0, st>>>(t2, dst, A[0], lines);
+  return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ training (FP32)
@@ -877,37 +972,51 @@ cudaError_t scratch_alloc(void** p, size_t bytes, int dev, cudaStream_t st) {
 }
 
 // 1-D restriction table: for each coarse node its fine element's first
-// global node and the N_f + 1 Lagrange weights of the fine element's LGL
-// points at the coarse node's position.
-void axis_table(const xg_ctx* f, const xg_ctx* c, int d, std::vector<int>& start, std::vector<double>& w) {
+// global node, the N_f + 1 Lagrange weights of the fine element's LGL points at
+// the coarse node's position, and the point it falls on (InterpAxis::one).
+// Coarse element e starts at fine element e nel_f / nel_c, in whole numbers and
+// a remainder, and elements of one remainder share their weights (a mesh
+// refined by a whole factor has one): long double is software arithmetic on
+// Arm, where weights for every node took more than a millisecond an axis.
+void axis_table(const xg_ctx* f, const xg_ctx* c, int d, std::vector<int>& start, std::vector<int>& one,
+                std::vector<double>& w) {
   const int Nf = f->d.order, Nc = c->d.order;
   long double xf[xg::kMaxOrder + 1], xc[xg::kMaxOrder + 1];
   xg::lgl_nodes(Nf, xf);
   xg::lgl_nodes(Nc, xc);
-  const double lo = f->d.lo[d], hi = f->d.hi[d];
   const int nelf = f->d.nel[d], nelc = c->d.nel[d];
   const int nf = f->n[d], ncn = c->n[d];
   start.assign(ncn, 0);
+  one.assign(ncn, -1);
   w.assign((size_t)ncn * (Nf + 1), 0.0);
+  struct Entry { int ef = -1, one = -1; double w[xg::kMaxOrder + 1]; };
+  std::map<std::pair<int, int>, Entry> seen;   // (remainder, local node)
   for (int g = 0; g < ncn; ++g) {
-    int e = std::min(g / Nc, nelc - 1);
+    const int e = std::min(g / Nc, nelc - 1);
     const int a = g - Nc * e;
-    // position as a fraction of the box, then in fine element units
-    const long double frac = ((long double)e + (xc[a] + 1.0L) / 2.0L) / nelc;
-    const long double sf = frac * nelf;
-    int ef = (int)floorl(sf);
-    ef = std::max(0, std::min(ef, nelf - 1));
-    const long double loc = 2.0L * (sf - ef) - 1.0L;
-    start[g] = (Nf * ef) % nf;
-    for (int l = 0; l <= Nf; ++l) {
-      long double L = 1.0L;
-      for (int k = 0; k <= Nf; ++k)
-        if (k != l) L *= (loc - xf[k]) / (xf[l] - xf[k]);
-      w[(size_t)g * (Nf + 1) + l] = (double)L;
+    const int whole = (int)((long long)e * nelf / nelc), rem = (int)((long long)e * nelf % nelc);
+    Entry& t = seen[{rem, a}];
+    if (t.ef < 0) {   // fine elements past `whole`, and the weights there
+      const long double sf = ((long double)rem + (xc[a] + 1.0L) / 2.0L * nelf) / nelc;
+      t.ef = std::max(0, (int)floorl(sf));
+      if (whole + t.ef >= nelf) t.ef = nelf - 1 - whole;   // the last node of the box
+      const long double loc = 2.0L * (sf - t.ef) - 1.0L;
+      int big = 0, small = 0;
+      for (int l = 0; l <= Nf; ++l) {
+        long double L = 1.0L;
+        for (int k = 0; k <= Nf; ++k)
+          if (k != l) L *= (loc - xf[k]) / (xf[l] - xf[k]);
+        t.w[l] = (double)L;
+        if (std::fabs(t.w[l]) > std::fabs(t.w[big])) big = l;
+      }
+      for (int l = 0; l <= Nf; ++l) small += l != big && std::fabs(t.w[l]) < 0x1p-60;
+      if (small == Nf && t.w[big] == 1.0) t.one = big;
     }
+    start[g] = (int)((long long)Nf * (whole + t.ef) % nf);
+    one[g] = t.one;
+    for (int l = 0; l <= Nf; ++l) w[(size_t)g * (Nf + 1) + l] = t.w[l];
+    if (whole + t.ef == nelf - 1) seen.erase({rem, a});    // (an entry made at the box's end is its own)
   }
-  (void)lo;
-  (void)hi;
 }
 
 }  // namespace
@@ -945,58 +1054,70 @@ xg_status xg_restrict(const xg_ctx* f, const xg_ctx* c, const double* src, int n
     if ((f->d.periodic[d] != 0) != (c->d.periodic[d] != 0)) return XG_ERR_ARG;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  const int Nf = f->d.order;
-  std::vector<int> start[3];
-  std::vector<double> w[3];
-  for (int d = 0; d < 3; ++d) axis_table(f, c, d, start[d], w[d]);
   const int* nf = f->n;
   const int* nc = c->n;
-  const long long s1 = (long long)nvar * nf[2] * nf[1] * nc[0];
-  const long long s2 = (long long)nvar * nf[2] * nc[1] * nc[0];
-  double *t1 = nullptr, *t2 = nullptr, *dw = nullptr;
-  int* ds = nullptr;
-  size_t nw = 0, ns = 0;
+  // the tables of the three axes in one buffer: weights, starts, points
+  const int npts = f->d.order + 1;
+  const size_t nodes = (size_t)nc[0] + nc[1] + nc[2];
+  std::vector<double> table(nodes * (npts + 1));
+  double* hw = table.data();
+  int* hs = reinterpret_cast<int*>(hw + nodes * npts);
+  int* ho = hs + nodes;
+  size_t off[3], at = 0;
   for (int d = 0; d < 3; ++d) {
-    nw += w[d].size();
-    ns += start[d].size();
+    std::vector<int> start, one;
+    std::vector<double> w;
+    axis_table(f, c, d, start, one, w);
+    std::copy(w.begin(), w.end(), hw + at * npts);
+    std::copy(start.begin(), start.end(), hs + at);
+    std::copy(one.begin(), one.end(), ho + at);
+    off[d] = at;
+    at += (size_t)nc[d];
   }
-  cudaError_t e = cudaMalloc((void**)&t1, sizeof(double) * s1);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&t2, sizeof(double) * s2);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&dw, sizeof(double) * nw);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&ds, sizeof(int) * ns);
-  size_t ow[3], os[3];
-  if (e == cudaSuccess) {
-    size_t a = 0, b = 0;
-    for (int d = 0; d < 3; ++d) {
-      ow[d] = a;
-      os[d] = b;
-      e = cudaMemcpy(dw + a, w[d].data(), sizeof(double) * w[d].size(), cudaMemcpyHostToDevice);
-      if (e == cudaSuccess)
-        e = cudaMemcpy(ds + b, start[d].data(), sizeof(int) * start[d].size(), cudaMemcpyHostToDevice);
-      if (e != cudaSuccess) break;
-      a += w[d].size();
-      b += start[d].size();
+  // chunks of planes whose intermediates fit half the scratch that the pool keeps
+  const long long plane = (long long)nf[0] * nf[1], mid = (long long)nf[0] * nc[1];
+  const long long planes = (long long)nvar * nc[2];
+  const long long per = 8 * (plane + mid);
+  int chunk = (int)std::max<long long>(1, std::min<long long>(planes, (long long)(kScratchKept / 2) / per));
+  chunk = std::min(chunk, 65535);
+  // a result over the source is written only once all of it is read
+  const size_t out_bytes = 8 * (size_t)planes * nc[0] * nc[1];
+  const uintptr_t s0 = (uintptr_t)src, d0 = (uintptr_t)dst;
+  const bool over = s0 < d0 + out_bytes && d0 < s0 + 8 * (size_t)nvar * f->np;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  const size_t tbytes = (8 * table.size() + 255) / 256 * 256;
+  double* scratch = nullptr;
+  if (e == cudaSuccess) e = scratch_alloc((void**)&scratch, tbytes + (size_t)per * chunk + (over ? out_bytes : 0), dev, st);
+  if (e != cudaSuccess) return cuda_status(e, "xg_restrict");
+  e = cudaMemcpyAsync(scratch, hw, 8 * table.size(), cudaMemcpyHostToDevice, st);
+  const int* ds = reinterpret_cast<const int*>(scratch + nodes * npts);
+  xg::InterpAxis A[3];
+  for (int d = 0; d < 3; ++d)
+    A[d] = {ds + off[d], ds + nodes + off[d], scratch + off[d] * npts, nf[d], nc[d], npts};
+  double* t1 = scratch + tbytes / 8;
+  double* t2 = t1 + plane * chunk;
+  double* res = over ? t2 + mid * chunk : dst;
+  for (long long p = 0; p < planes && e == cudaSuccess; p += chunk) {
+    const unsigned n = (unsigned)std::min<long long>(chunk, planes - p);
+    double* out = res + p * (long long)nc[0] * nc[1];
+    switch (npts) {
+      case 2: e = xg::interp_chunk<2>(src, t1, t2, out, A, (int)p, n, st); break;
+      case 3: e = xg::interp_chunk<3>(src, t1, t2, out, A, (int)p, n, st); break;
+      case 4: e = xg::interp_chunk<4>(src, t1, t2, out, A, (int)p, n, st); break;
+      case 5: e = xg::interp_chunk<5>(src, t1, t2, out, A, (int)p, n, st); break;
+      case 6: e = xg::interp_chunk<6>(src, t1, t2, out, A, (int)p, n, st); break;
+      case 7: e = xg::interp_chunk<7>(src, t1, t2, out, A, (int)p, n, st); break;
+      case 8: e = xg::interp_chunk<8>(src, t1, t2, out, A, (int)p, n, st); break;
+      case 9: e = xg::interp_chunk<9>(src, t1, t2, out, A, (int)p, n, st); break;
+      default: e = cudaErrorInvalidValue;
     }
   }
-  if (e == cudaSuccess) {
-    auto grid = [](long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 65535); };
-    // x: [v][z_f][y_f] x (x_f -> x_c)
-    xg::k_interp_axis<<<grid(s1), 256, 0, st>>>(src, t1, (long long)nvar * nf[2] * nf[1], nf[0], nc[0], 1,
-                                                ds + os[0], dw + ow[0], Nf + 1);
-    // y: [v][z_f] x (y_f -> y_c) x [x_c]
-    xg::k_interp_axis<<<grid(s2), 256, 0, st>>>(t1, t2, (long long)nvar * nf[2], nf[1], nc[1], nc[0],
-                                                ds + os[1], dw + ow[1], Nf + 1);
-    // z: [v] x (z_f -> z_c) x [y_c x_c]
-    const long long s3 = (long long)nvar * nc[2] * nc[1] * nc[0];
-    xg::k_interp_axis<<<grid(s3), 256, 0, st>>>(t2, dst, nvar, nf[2], nc[2], (long long)nc[1] * nc[0],
-                                                ds + os[2], dw + ow[2], Nf + 1);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  }
-  cudaFree(t1);
-  cudaFree(t2);
-  cudaFree(dw);
-  cudaFree(ds);
+  if (e == cudaSuccess && over) e = cudaMemcpyAsync(dst, res, out_bytes, cudaMemcpyDeviceToDevice, st);
+  const cudaError_t ef = cudaFreeAsync(scratch, st);
+  if (e == cudaSuccess) e = ef;
+  const cudaError_t es = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) e = es;
   return cuda_status(e, "xg_restrict");
 }
 
