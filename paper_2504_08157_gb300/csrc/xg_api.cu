@@ -150,11 +150,13 @@ __global__ void k_face_combine(double* __restrict__ T, const double* __restrict_
 
 namespace xg {
 __global__ void k_to_f32(const double* __restrict__ in, float* __restrict__ out, long long n) {
+  stage_kernel_begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     out[i] = __double2float_rn(in[i]);
 }
 __global__ void k_from_f32(const float* __restrict__ in, double* __restrict__ out, long long n) {
+  stage_kernel_begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x)
     out[i] = (double)in[i];
@@ -271,7 +273,7 @@ void launch_plane_n(xg_ctx* c, const Params& P, const Bufs& B, cudaStream_t st) 
   using L = xg::XYTile<N>;
   const dim3 g((c->d.nel[0] + L::EX - 1) / L::EX, B.nty, c->n[2]);
   prof_mark(c, 0, false, st);
-  xg::k_plane_xy<N><<<g, L::threads(c->tile_ey), L::bytes, st>>>(P, B, c->tile_ey);
+  xg::launch_stage_kernel(xg::k_plane_xy<N, Params>, g, L::threads(c->tile_ey), L::bytes, st, P, B, c->tile_ey);
   prof_mark(c, 0, true, st);
 }
 
@@ -284,7 +286,7 @@ void launch_stage_n(xg_ctx* c, const StageBufs& B, cudaStream_t st, int parts) {
     constexpr int K = xg::z_tile_segments(N);
     const dim3 gz((c->n[0] + xg::kTileCols - 1) / xg::kTileCols, (c->d.nel[2] + K - 1) / K, c->n[1]);
     prof_mark(c, 2, false, st);
-    xg::k_tile_z<N><<<gz, dim3(xg::kTileCols, K * N + 1), 0, st>>>(c->P64, B);
+    xg::launch_stage_kernel(xg::k_tile_z<N>, gz, dim3(xg::kTileCols, K * N + 1), 0, st, c->P64, B);
     prof_mark(c, 2, true, st);
   }
 }
@@ -298,13 +300,14 @@ void launch_stage_n(xg_ctx* c, const DfBufs& B, cudaStream_t st, int parts) {
     if constexpr (N <= xg::kDfLineOrder) {
       dim3 gx(c->n[1], c->n[2]);
       prof_mark(c, 0, false, st);
-      xg::k_df_line_x<N><<<gx, xg::kXThreads, xg::df_x_smem(N, c->d.nel[0]), st>>>(c->Pdf, c->P64.F[0], B);
+      xg::launch_stage_kernel(xg::k_df_line_x<N>, gx, xg::kXThreads, xg::df_x_smem(N, c->d.nel[0]), st, c->Pdf,
+                              c->P64.F[0], B);
       prof_mark(c, 0, true, st);
       constexpr int K = xg::df_tile_segments(N, 1);
       const dim3 blk(xg::kTileCols, K * N + 1);
       dim3 gy(xb, (c->d.nel[1] + K - 1) / K, c->n[2]);
       prof_mark(c, 1, false, st);
-      xg::k_df_tline<N, 1><<<gy, blk, 0, st>>>(c->Pdf, B);
+      xg::launch_stage_kernel(xg::k_df_tline<N, 1>, gy, blk, 0, st, c->Pdf, B);
       prof_mark(c, 1, true, st);
     }
   }
@@ -313,7 +316,7 @@ void launch_stage_n(xg_ctx* c, const DfBufs& B, cudaStream_t st, int parts) {
     const dim3 blk(xg::kTileCols, K * N + 1);
     dim3 gz(xb, (c->d.nel[2] + K - 1) / K, c->n[1]);
     prof_mark(c, 2, false, st);
-    xg::k_df_tline<N, 2><<<gz, blk, 0, st>>>(c->Pdf, B);
+    xg::launch_stage_kernel(xg::k_df_tline<N, 2>, gz, blk, 0, st, c->Pdf, B);
     prof_mark(c, 2, true, st);
   }
 }
@@ -389,7 +392,7 @@ void launch_f32_stage_n(xg_ctx* c, const xg::FBufs& B, cudaStream_t st) {
     static_assert(xg::plane_elems_f32(4) == xg::PlaneH16Layout::E, "same tiles");
     xg::k_f_plane_xy_h16<<<gp, xg::kPlaneH16Threads, xg::PlaneH16Layout::bytes, st>>>(c->Pf, B);
   } else {
-    xg::k_f_plane_xy<N><<<gp, xg::kPlaneThreads, xg::PlaneLayoutF<N>::bytes, st>>>(c->Pf, B);
+    xg::launch_stage_kernel(xg::k_f_plane_xy<N>, gp, xg::kPlaneThreads, xg::PlaneLayoutF<N>::bytes, st, c->Pf, B);
   }
   prof_mark(c, 0, true, st);
   constexpr int K = xg::f32_tile_segments(N);
@@ -397,7 +400,7 @@ void launch_f32_stage_n(xg_ctx* c, const xg::FBufs& B, cudaStream_t st) {
   const unsigned xb = (c->n[0] + xg::kTileCols - 1) / xg::kTileCols;
   dim3 gz(xb, (c->d.nel[2] + K - 1) / K, c->n[1]);
   prof_mark(c, 2, false, st);
-  xg::k_f_tline<N, 2><<<gz, blk, 0, st>>>(c->Pf, B);
+  xg::launch_stage_kernel(xg::k_f_tline<N, 2>, gz, blk, 0, st, c->Pf, B);
   prof_mark(c, 2, true, st);
 }
 
@@ -538,8 +541,7 @@ cudaError_t run_stage(xg_ctx* c, const void* q, const void* qn, void* out, doubl
 // and XG_DF64 contexts hold FP64 arrays).
 cudaError_t import_values(xg_ctx* c, const double* src, void* dst, long long n, cudaStream_t st) {
   if (c->f32) {
-    xg::k_to_f32<<<conv_blocks(n), 256, 0, st>>>(src, (float*)dst, n);
-    return cudaGetLastError();
+    return xg::launch_stage_kernel(xg::k_to_f32, conv_blocks(n), 256, 0, st, src, (float*)dst, n);
   }
   return cudaMemcpyAsync(dst, src, sizeof(double) * (size_t)n, cudaMemcpyDeviceToDevice, st);
 }
@@ -547,8 +549,7 @@ cudaError_t import_values(xg_ctx* c, const double* src, void* dst, long long n, 
 // The context's device representation -> device FP64 array.
 cudaError_t export_values(xg_ctx* c, const void* src, double* dst, long long n, cudaStream_t st) {
   if (c->f32) {
-    xg::k_from_f32<<<conv_blocks(n), 256, 0, st>>>((const float*)src, dst, n);
-    return cudaGetLastError();
+    return xg::launch_stage_kernel(xg::k_from_f32, conv_blocks(n), 256, 0, st, (const float*)src, dst, n);
   }
   return cudaMemcpyAsync(dst, src, sizeof(double) * (size_t)n, cudaMemcpyDeviceToDevice, st);
 }

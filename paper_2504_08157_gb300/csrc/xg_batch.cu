@@ -238,6 +238,7 @@ __device__ __forceinline__ const BInst& load_instance(const BRun& R, int i, unsi
 template <int N, int HALF>
 __global__ void __launch_bounds__(kPlaneThreads) k_batch_plane(const __grid_constant__ BRun R, int st, int par) {
   extern __shared__ __align__(128) unsigned char smb[];
+  stage_kernel_begin();
   const int4 it = __ldg(R.items[0] + R.goff[0][N - kBatchMinOrder] + blockIdx.x);
   const BInst& I = load_instance<kPlaneThreads>(R, it.x, smb);
   f_plane_tile<N, batch_plane_elems(N, HALF), kPlaneBatch, false>(I.P, stage_bufs(R, I, st, par), it.y, it.z, it.w,
@@ -249,6 +250,7 @@ template <int N>
 __global__ void __launch_bounds__(kTileCols * (8 + 1), 4) k_batch_z(const __grid_constant__ BRun R, int st, int par) {
   constexpr int K = f32_tile_segments(N);
   extern __shared__ __align__(128) unsigned char smb[];
+  stage_kernel_begin();
   const int4 it = __ldg(R.items[1] + R.goff[1][N - kBatchMinOrder] + blockIdx.x);
   const BInst& I = load_instance<kTileCols * (K * N + 1)>(R, it.x, smb);
   f_tline_tile<N, 2, false, K>(I.P, stage_bufs(R, I, st, par), it.y, it.z, it.w, threadIdx.x, threadIdx.y,
@@ -276,9 +278,12 @@ cudaError_t launch_order(const BRun& R, int one_cta, size_t sm_smem, cudaStream_
   if (e != cudaSuccess) return e;
   for (int s = 0; s < R.nstages; ++s) {
     const int stage = R.rhs_only ? 0 : s % 3, par = R.rhs_only ? 0 : (s / 3) & 1;
-    if (R.plane_half) k_batch_plane<N, 1><<<R.gcnt[0][g], kPlaneThreads, bytes[0], st>>>(R, stage, par);
-    else k_batch_plane<N, 0><<<R.gcnt[0][g], kPlaneThreads, bytes[0], st>>>(R, stage, par);
-    k_batch_z<N><<<R.gcnt[1][g], dim3(kTileCols, f32_tile_segments(N) * N + 1), bytes[1], st>>>(R, stage, par);
+    e = R.plane_half ? launch_stage_kernel(k_batch_plane<N, 1>, R.gcnt[0][g], kPlaneThreads, bytes[0], st, R, stage, par)
+                     : launch_stage_kernel(k_batch_plane<N, 0>, R.gcnt[0][g], kPlaneThreads, bytes[0], st, R, stage, par);
+    if (e == cudaSuccess)
+      e = launch_stage_kernel(k_batch_z<N>, R.gcnt[1][g], dim3(kTileCols, f32_tile_segments(N) * N + 1), bytes[1], st, R, stage,
+                              par);
+    if (e != cudaSuccess) return e;
   }
   return cudaGetLastError();
 }

@@ -831,6 +831,7 @@ __global__ void __launch_bounds__(kTcRows, kTcCtasPerSm)
     k_closure(const FParams P, const InferPack* __restrict__ pack, const float* __restrict__ q,
               const float* __restrict__ Sth, float* __restrict__ C, int* flag) {
   __shared__ __align__(128) TcSmem S;
+  stage_kernel_begin();
   tc_infer(S, pack, P.np, C, P.np, flag,
            [&](long long I, auto&& emit) { node_features<N>(P, q, Sth, I, emit); });
 }
@@ -888,7 +889,7 @@ cudaError_t closure_launch(xg_ctx* c, const float* q, cudaStream_t st) {
   case n: {                                                                                             \
     if (!c->cl_grid) c->cl_grid = xg::tc_grid(np);                                                      \
     const unsigned g = (unsigned)c->cl_grid;                                                            \
-    xg::k_closure<n><<<g, xg::kTcRows, 0, st>>>(c->Pf, K, q, S, c->cl_C, c->flag);                       \
+    xg::launch_stage_kernel(xg::k_closure<n>, g, xg::kTcRows, 0, st, c->Pf, K, q, S, c->cl_C, c->flag);   \
     break;                                                                                              \
   }
     XG_CLOSURE_CASE(1) XG_CLOSURE_CASE(2) XG_CLOSURE_CASE(3) XG_CLOSURE_CASE(4)

@@ -84,6 +84,7 @@ __global__ void __launch_bounds__(kFixThreads) k_lap_plane(const LapParams P, co
   __shared__ fix2 V[L::V];
   __shared__ long long RA[2][L::RA], RB[2][L::RB];
   __shared__ int emax;
+  stage_kernel_begin();
   const int z = blockIdx.y, var = blockIdx.z;
   const int tilesx = (P.nseg[0] + L::E - 1) / L::E;
   const int nx = P.n[0], ny = P.n[1];
@@ -124,6 +125,7 @@ template <int N, bool SECOND>
 __global__ void __launch_bounds__(128) k_lap_z(const LapParams P, const double* __restrict__ in, double* out,
                                                const double* __restrict__ q, const double* __restrict__ gamma,
                                                int chunk) {
+  stage_kernel_begin();
   const long long nxy = (long long)P.n[0] * P.n[1];
   const long long col = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (col >= nxy) return;
@@ -184,6 +186,7 @@ __global__ void __launch_bounds__(128) k_lap_z(const LapParams P, const double* 
 // E = sponge only (no hyper-diffusion)
 __global__ void k_sponge_only(long long np, int nxy, const double* __restrict__ q,
                               const double* __restrict__ gamma, double* __restrict__ out) {
+  stage_kernel_begin();
   for (long long I = blockIdx.x * (long long)blockDim.x + threadIdx.x; I < 5 * np;
        I += (long long)gridDim.x * blockDim.x) {
     const long long v = I / np, J = I - v * np;
@@ -452,13 +455,12 @@ void launch_lap(const LapParams& P, const double* q, double* L1, const double* g
     const dim3 gp(((P.nseg[0] + TE - 1) / TE) * ((P.nseg[1] + TE - 1) / TE), P.n[2], 5);
     const int chunk = xg::fix_z_chunk(P.nseg[2], 5 * nxy, sms);
     const dim3 gz((unsigned)((nxy + 127) / 128), (P.nseg[2] + chunk - 1) / chunk, 5);
-    xg::k_lap_plane<N><<<gp, xg::kFixThreads, 0, st>>>(P, q, L1);
-    xg::k_lap_z<N, false><<<gz, 128, 0, st>>>(P, q, L1, nullptr, nullptr, chunk);
-    xg::k_lap_plane<N><<<gp, xg::kFixThreads, 0, st>>>(P, L1, E);
-    xg::k_lap_z<N, true><<<gz, 128, 0, st>>>(P, L1, E, q, gamma, chunk);
+    xg::launch_stage_kernel(xg::k_lap_plane<N>, gp, xg::kFixThreads, 0, st, P, q, L1);
+    xg::launch_stage_kernel(xg::k_lap_z<N, false>, gz, 128, 0, st, P, q, L1, nullptr, nullptr, chunk);
+    xg::launch_stage_kernel(xg::k_lap_plane<N>, gp, xg::kFixThreads, 0, st, P, L1, E);
+    xg::launch_stage_kernel(xg::k_lap_z<N, true>, gz, 128, 0, st, P, L1, E, q, gamma, chunk);
   } else {
-    xg::k_sponge_only<<<(unsigned)std::min<long long>((5 * P.np + 255) / 256, 65535), 256, 0, st>>>(
-        P.np, (int)nxy, q, gamma, E);
+    xg::launch_stage_kernel(xg::k_sponge_only, (unsigned)std::min<long long>((5 * P.np + 255) / 256, 65535), 256, 0, st, P.np, (int)nxy, q, gamma, E);
   }
 }
 

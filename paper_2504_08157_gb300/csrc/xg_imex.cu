@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(kFixThreads) k_lin_plane(const LinParams Q, co
   __shared__ fix2 V[2][L::V];
   __shared__ long long RA[2][L::RA], RB[2][L::RB];
   __shared__ int emax;
+  stage_kernel_begin();
   const LineParams& P = Q.P;
   const int z = blockIdx.y, nx = P.n[0], ny = P.n[1], sc = Q.D[0].sc;
   const int tilesx = (P.nseg[0] + L::E - 1) / L::E;
@@ -160,6 +161,7 @@ template <int N, bool PLAIN>
 __global__ void __launch_bounds__(128) k_lin_z(const LinParams Q, const double* __restrict__ v,
                                                const double* __restrict__ cpl, const double* __restrict__ th0,
                                                double c0, double c1, double* out, int chunk) {
+  stage_kernel_begin();
   const LineParams& P = Q.P;
   const FixRows& D = Q.D[2];
   const long long np = P.np, nxy = (long long)P.n[0] * P.n[1];
@@ -273,6 +275,7 @@ struct Comb {
 // together.
 template <int K>
 __global__ void __launch_bounds__(256) k_comb(const Comb C, double* out, long long n) {
+  stage_kernel_begin();
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
        i += (long long)gridDim.x * blockDim.x) {
     double x[K];
@@ -302,6 +305,7 @@ __global__ void __launch_bounds__(kDotThreads, 4) k_wdots(const double* __restri
                                                        double* __restrict__ partial) {
   constexpr int U = K <= 8 ? 2 : 1;   // nodes per thread and iteration
   __shared__ double red[K][kDotThreads / 32];
+  stage_kernel_begin();
   const long long per = (np + gridDim.x - 1) / gridDim.x;
   const long long lo = blockIdx.x * per, hi = min(np, lo + per);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -390,11 +394,11 @@ void launch_linear_n(xg_ctx* c, const Imex& X, const double* v, double c0, doubl
   const int chunk = xg::fix_z_chunk(P.nseg[2], nxy, c->sms);
   const dim3 gz((unsigned)((nxy + 127) / 128), (P.nseg[2] + chunk - 1) / chunk);
   if (c0 == 0.0 && c1 == 1.0) {
-    xg::k_lin_plane<N, true><<<gp, xg::kFixThreads, 0, st>>>(X.lin, v, X.cpl, c0, c1, out);
-    xg::k_lin_z<N, true><<<gz, 128, 0, st>>>(X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
+    xg::launch_stage_kernel(xg::k_lin_plane<N, true>, gp, xg::kFixThreads, 0, st, X.lin, v, X.cpl, c0, c1, out);
+    xg::launch_stage_kernel(xg::k_lin_z<N, true>, gz, 128, 0, st, X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
   } else {
-    xg::k_lin_plane<N, false><<<gp, xg::kFixThreads, 0, st>>>(X.lin, v, X.cpl, c0, c1, out);
-    xg::k_lin_z<N, false><<<gz, 128, 0, st>>>(X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
+    xg::launch_stage_kernel(xg::k_lin_plane<N, false>, gp, xg::kFixThreads, 0, st, X.lin, v, X.cpl, c0, c1, out);
+    xg::launch_stage_kernel(xg::k_lin_z<N, false>, gz, 128, 0, st, X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
   }
 }
 
@@ -436,11 +440,11 @@ cudaError_t comb(const std::vector<std::pair<double, const double*>>& terms, dou
     const unsigned blocks = (unsigned)std::min<long long>((n + 255) / 256, 8192);
     switch (C.k) {
 #define XG_COMB_CASE(K) \
-  case K: xg::k_comb<K><<<blocks, 256, 0, st>>>(C, out, n); break;
+  case K: xg::launch_stage_kernel(xg::k_comb<K>, blocks, 256, 0, st, C, out, n); break;
       XG_COMB_CASE(1) XG_COMB_CASE(2) XG_COMB_CASE(3) XG_COMB_CASE(4) XG_COMB_CASE(5) XG_COMB_CASE(6)
       XG_COMB_CASE(7) XG_COMB_CASE(8) XG_COMB_CASE(9) XG_COMB_CASE(10) XG_COMB_CASE(11) XG_COMB_CASE(12)
       XG_COMB_CASE(13) XG_COMB_CASE(14) XG_COMB_CASE(15) XG_COMB_CASE(16)
-      default: xg::k_comb<xg::kCombMax><<<blocks, 256, 0, st>>>(C, out, n); break;
+      default: xg::launch_stage_kernel(xg::k_comb<xg::kCombMax>, blocks, 256, 0, st, C, out, n); break;
 #undef XG_COMB_CASE
     }
     first = false;
@@ -456,10 +460,10 @@ cudaError_t var_dots(Imex& X, long long np, const double* w, const double* const
   D.k = k;
   for (int i = 0; i < k; ++i) D.v[i] = vs[i];
   if (k == 1 && D.v[0] == w) {
-    xg::k_wdots<1, true><<<X.dot_blocks, xg::kDotThreads, 0, st>>>(w, D, np, X.partial);
+    xg::launch_stage_kernel(xg::k_wdots<1, true>, X.dot_blocks, xg::kDotThreads, 0, st, w, D, np, X.partial);
   } else switch (k) {
 #define XG_WDOTS_CASE(K) \
-  case K: xg::k_wdots<K><<<X.dot_blocks, xg::kDotThreads, 0, st>>>(w, D, np, X.partial); break;
+  case K: xg::launch_stage_kernel(xg::k_wdots<K>, X.dot_blocks, xg::kDotThreads, 0, st, w, D, np, X.partial); break;
     XG_WDOTS_CASE(1) XG_WDOTS_CASE(2) XG_WDOTS_CASE(3) XG_WDOTS_CASE(4) XG_WDOTS_CASE(5)
     XG_WDOTS_CASE(6) XG_WDOTS_CASE(7) XG_WDOTS_CASE(8) XG_WDOTS_CASE(9) XG_WDOTS_CASE(10)
     XG_WDOTS_CASE(11) XG_WDOTS_CASE(12) XG_WDOTS_CASE(13) XG_WDOTS_CASE(14) XG_WDOTS_CASE(15)

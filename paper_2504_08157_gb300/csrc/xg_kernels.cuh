@@ -89,6 +89,10 @@ struct StageBufs {
   int fy = 1, nty = 1;
 };
 
+// Start of a stage kernel (launched by launch_stage_kernel): waits for the end of
+// the kernel before it on the stream, all its writes included.
+__device__ __forceinline__ void stage_kernel_begin() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // (1 + x)^gamma - 1: the binomial series (Horner) for small |x|, where the
 // truncation error after 8 terms is below 2^-56 relative (bound checked on
 // the host), else expm1(gamma log1p(x)).

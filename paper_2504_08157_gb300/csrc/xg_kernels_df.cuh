@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(kXThreads, df_x_min_blocks(N)) k_df_line_x(con
   double* F64 = reinterpret_cast<double*>(smd);
   df* RN = smd + 5 * ld;
   double* RN64 = reinterpret_cast<double*>(RN);
+  stage_kernel_begin();
   const df p0 = B.base[2 * nz + z], iTh0 = B.base[3 * nz + z];
   const double rho0 = B.base64[z], Th0 = B.base64[nz + z];
   const double* __restrict__ q = B.q;
@@ -482,6 +483,7 @@ __global__ void __launch_bounds__(df_tile_threads(N, DIR), df_tile_min_blocks(N,
   const long long I = base + sd * (main_plane ? g : 0);
   const long long Ih = base + sd * (halo ? gh : 0);
 
+  stage_kernel_begin();
   // the global loads the fluxes and rows need first (one memory round trip);
   // q^n and S, needed only by the stage at the end, are loaded there: kept
   // live across the rows they spilled 56 bytes per thread, and z launches

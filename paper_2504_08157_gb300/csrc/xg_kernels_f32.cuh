@@ -331,6 +331,7 @@ template <int N, int DIR>
 __global__ void __launch_bounds__(kTileCols * (8 + 1), 4) k_f_tline(const FParams P, const FBufs B) {
   constexpr int K = f32_tile_segments(N);
   __shared__ float Fs[tline_smem_floats(N, K)];
+  stage_kernel_begin();
   f_tline_tile<N, DIR, false, K>(P, B, blockIdx.x, blockIdx.y, blockIdx.z, threadIdx.x, threadIdx.y, Fs);
 }
 

@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
 
   if (threadIdx.x < 4 * L::EY) (&Es[0][0])[threadIdx.x] = 0;
   if (threadIdx.x == 0) nonfinite = 0;
+  stage_kernel_begin();
   __syncthreads();
 
   // this thread's node (i, j) of the tile: a warp takes a line, the warps
@@ -516,6 +517,7 @@ __global__ void __launch_bounds__(z_tile_threads(N), z_tile_min_blocks(N))
   const long long Ih = base + sd * (halo ? gh : 0);
   const double* __restrict__ W = B.W;
 
+  stage_kernel_begin();
   // the global loads the fluxes and rows need first (one memory round trip);
   // q^n and S, needed only by the stage at the end, are loaded there
   double qv[5], hq[3], th = 0.0, hth = 0.0, vel, pp, hvel, hpp;

@@ -303,6 +303,7 @@ __device__ __forceinline__ void f_plane_tile(const FParams& P, const FBufs& B, i
 template <int N>
 __global__ void __launch_bounds__(kPlaneThreads) k_f_plane_xy(const FParams P, const FBufs B) {
   extern __shared__ float sm_plane[];
+  stage_kernel_begin();
   f_plane_tile<N, plane_elems_f32(N), kPlaneBatch, false>(P, B, blockIdx.x, blockIdx.y, blockIdx.z,
                                                            sm_plane, threadIdx.x, blockDim.x);
 }

@@ -250,4 +250,27 @@ inline cudaError_t raise_dynamic_smem(F* func, size_t bytes) {
   return cudaFuncSetAttribute((const void*)func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+// Launch of a kernel that begins with stage_kernel_begin: where the stream's last
+// work is a kernel, the launch is paid while that one runs, and the wait at the
+// kernel's start keeps the order (no kernel lets its successor in before its own
+// end: blocks that wait took room and issue slots from blocks that work, 24.1
+// against 16.4 us below).  A mixed stage on 33^3 nodes 20.9 -> 16.4 us, FP32 18.6
+// -> 13.3, FP64 26.5 -> 20.5.
+template <typename... P, typename... A>
+inline cudaError_t launch_stage_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                       const A&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 }  // namespace xg
