@@ -12,11 +12,12 @@
 //     entries, with sum_l |C_l| <= 2^60 over every assembled row (59 bits
 //     against FP64's 53); a row that sums to zero up to that rounding is made
 //     to sum to zero exactly, so constants have no derivative;
-//   * both are split into limbs of 30 bits, V = h 2^30 + l, and a product
-//     takes three IMAD.WIDE, hi += ch h and mid += ch l + cl h; the low
-//     product (below 2^-58 of sum |c| max |v|) is left out.  Nothing
-//     overflows: |hi| <= 2^61, |mid| <= 2^60 + (N + 1) 2^(B - 2) <= 2^63;
-//   * r = hi + mid 2^-30 is one FP64 value again by one conversion, times
+//   * both are split into limbs, X = h 2^30 + l with |l| <= 2^29 (so that what
+//     is left out has no bias), and a product takes three IMAD.WIDE, hi += ch h
+//     and mid += ch l + cl h; the low product (below 2^-60 of sum |c| max |v|) is
+//     left out.  Nothing overflows: |hi| <= 2^61, |mid| <= 2^60 + (N + 1)
+//     2^(B - 2) <= 2^63;
+//   * r = hi + mid 2^-30, rounded, is one FP64 value again by one conversion, times
 //     2^(60 - sc - sv).
 // The sums of a block are exact up to those cuts, about 2^-59 of
 // sum |c| max |v|, where an FP64 FMA chain rounds at 2^-53 of its partial
@@ -101,6 +102,13 @@ __device__ __forceinline__ int fix_block_exp(int e, int sc) { return max(e, max(
 // Bits of a block's values for order N (see the overflow bound above).
 __host__ __device__ constexpr int fix_bits(int N) { return N <= 6 ? 61 : 60; }
 
+// sg V in limbs, V < 2^61: the high one rounded to nearest, but kept below 2^31
+// (the low one is then up to 2^30).
+__device__ __forceinline__ fix2 fix_limbs(unsigned long long V, int sg) {
+  const unsigned h = min((unsigned)((V + (1ull << 29)) >> 30), 0x7fffffffu);
+  return {(int)h * sg, (int)((unsigned)V - (h << 30)) * sg};
+}
+
 // v in the limbs of a block of exponent E >= fix_exp(v): |v| 2^(B - 1 - (E -
 // 1023)) cut to an integer, both limbs with v's sign.
 template <int N>
@@ -112,8 +120,7 @@ __device__ __forceinline__ fix2 fix_of(double v, int E) {
   const unsigned s = (unsigned)E - ((hi >> 20) & 0x7ffu);
   unsigned long long V;
   asm("shr.u64 %0, %1, %2;" : "=l"(V) : "l"(M), "r"(s));   // clamps: 0 for s >= 64
-  const int sg = ((int)hi >> 31) | 1;
-  return {(int)(V >> 30) * sg, (int)((unsigned)V & 0x3fffffffu) * sg};
+  return fix_limbs(V, ((int)hi >> 31) | 1);
 }
 
 // 2^(60 - sc - sv) of a block of exponent E (NaN for a block that has none)
@@ -123,10 +130,10 @@ __device__ __forceinline__ double fix_unit(int E, int sc) {
   return __hiloint2double(min(E + 61 - fix_bits(N) - sc, 2046) << 20, 0);
 }
 
-// hi + mid 2^-30 of row a
+// hi + mid 2^-30 of row a, rounded
 template <int N>
 __device__ __forceinline__ long long fix_row(const FixRows& F, int a, const fix2 (&v)[N + 1]) {
-  long long hi = 0, mid = 0;
+  long long hi = 0, mid = 1ll << 29;
 #pragma unroll
   for (int l = 0; l <= N; ++l) {
     hi += (long long)F.ch[a][l] * v[l].h;
@@ -342,10 +349,6 @@ __device__ __forceinline__ unsigned long long fix_shr(unsigned long long m, unsi
   unsigned long long v;
   asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(s));   // clamps: 0 for s >= 64
   return v;
-}
-
-__device__ __forceinline__ fix2 fix_limbs(unsigned long long V, int sg) {
-  return {(int)(V >> 30) * sg, (int)((unsigned)V & 0x3fffffffu) * sg};
 }
 
 // a b in limbs of a block whose exponent fields of a and b add up to G at

@@ -21,9 +21,11 @@
 // it; the difference form of the FP64 chains is not needed.
 //
 // XG_FP64, a stage on the 128 x 128 x 16 order-4 box (17.0 M nodes): three line
-// kernels with FP64 chains 1.87 + 1.44 + 2.02 ms; tiles 1.57 + 1.41 ms (FP64
-// pipe 61 and 70 % busy, 38 and 28 FP64 instructions a node; 2,020 and 1,150
-// instructions a node in all).  33^3 nodes: 66 -> 27 us.
+// kernels with FP64 chains 1.87 + 1.44 + 2.02 ms; tiles 1.61 + 1.38 ms (FP64
+// pipe 60 and 72 % busy, 38 and 28 FP64 instructions a node; 2,100 and 1,200
+// instructions a node in all).  33^3 nodes: 66 -> 21 us.  At the full-size vortex,
+// where the parts of rho' cancel to 1e-3 and less, its tendency's error is 6e-14
+// (FP64 chains 7e-14).
 #pragma once
 
 #include <type_traits>
