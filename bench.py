@@ -79,8 +79,8 @@ def fp32_kernel_names(wl, contract=0, fused=False):
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # FP64 instructions (DFMA + DADD + DMUL) per node and launch of the mixed
 # path's kernels, from the --set full capture of the 64x64x16 order-4 case
-# (profiles/line_kernels_tc.md); the pipe issues 2 per clock per SM.
-DF64_FP64_INSTR_PER_NODE = {"k_df_line_x": 17.5, "k_df_tline_y": 14.0, "k_df_tline_z": 20.6}
+# (profiles/line_kernels_tc.md; the x pass: profiles/plane64.md); 2 issue per clock and SM.
+DF64_FP64_INSTR_PER_NODE = {"k_df_line_x": 11.9, "k_df_tline_y": 14.0, "k_df_tline_z": 20.6}
 FP64_PIPE_PEAK_GINSTR = 152 * 2 * 2.07e9 / 1e9
 
 
@@ -793,7 +793,7 @@ def batch_describe(wls):
 def batch_measure(xg, torch, dev, stream, world, local, K, Wm, sample_clocks, compare,
                   oracle_check, count=96):
     """The batched form on the 96-instance workload: autotune, then K steps
-    in one persistent launch timed with CUDA events; with ``compare`` also
+    in one call timed with CUDA events; with ``compare`` also
     the same instances stepped through single contexts (FP32, one launch
     sequence per instance) and in plain FP64."""
     wls = batch_workloads(count)
@@ -825,19 +825,22 @@ def batch_measure(xg, torch, dev, stream, world, local, K, Wm, sample_clocks, co
         out["dtype"] = "f32"
         out["ms_per_step"] = round(ms / K, 4)
         out["steps"] = K
-        out["launches_per_call"] = 1
+        # the LPT schedule launches each pass of each order, the others one kernel
+        lpt = tune.schedule == xg.XG_SCHED_LPT
+        out["launches_per_call"] = 2 * len(cfg["orders"]) * 3 * K if lpt else 1
         out["tuning"] = tune.as_dict()
         out["config"] = cfg
         peaks = json.load(open(PEAKS_FILE)) if os.path.exists(PEAKS_FILE) else {}
         hbm = float(peaks.get("hbm_gbs", 6800.0))
         achieved = BATCH_BYTES_PER_NODE * cfg["nodes"] * 3 * K / (ms / 1e3) / 1e9
-        out["roofline"] = {"kernel": "k_batch", "bound": "hbm", "achieved": round(achieved, 1),
+        out["roofline"] = {"kernel": "k_batch_plane + k_batch_z" if lpt else "k_batch", "bound": "hbm", "achieved": round(achieved, 1),
                            "peak": hbm, "unit": "GB/s", "frac": round(achieved / hbm, 4),
                            "traffic": (lambda b: None if b is None else round(b * cfg["nodes"] * 3 * K))(
                                traffic_per_launch("k_batch_per_node_stage")),
                            "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured copy)",
                            "bytes_per_node_stage": round(BATCH_BYTES_PER_NODE, 2),
-                           "launch": "one persistent launch of %d steps (%d stages)" % (K, 3 * K)}
+                           "launch": "%s of %d steps (%d stages)" % (
+                               "a launch per pass and order" if lpt else "one persistent launch", K, 3 * K)}
         if oracle_check:
             # one right-hand side of the whole batch, with the smallest
             # instance set to a seeded smooth random state (at the vortex
@@ -861,7 +864,7 @@ def batch_measure(xg, torch, dev, stream, world, local, K, Wm, sample_clocks, co
                 "instance": i, "nel": list(wl["nel"]), "N": wl["N"],
                 "rel_l2": [float("%.3e" % (np.linalg.norm(got[v] - ref[v]) /
                                            max(np.linalg.norm(ref[v]), 1e-300))) for v in range(5)],
-                "what": "one batched right-hand side (all 96 instances in one launch) of the "
+                "what": "one batched right-hand side (all 96 instances in one call) of the "
                         "smallest instance, at a seeded smooth random state plus its vortex, vs "
                         "the FP64 oracle, relative L2 per variable"}
     finally:
