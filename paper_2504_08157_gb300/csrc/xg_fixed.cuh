@@ -351,9 +351,18 @@ __device__ __forceinline__ unsigned long long fix_shr(unsigned long long m, unsi
   return v;
 }
 
-// a b in limbs of a block whose exponent fields of a and b add up to G at
-// most: |a b| 2^(B - 2 - (G - 2046)) cut to an integer (values below 2^-1022
-// count as zero).
+// Exponent field of a b on a scale of its own: the fields' sum, and one where the
+// significands' product reaches 2 (from their leading 32 bits; fix_limbs takes a
+// product that reaches it in the bits below).  ea, eb: the fields.
+__device__ __forceinline__ int fix_prod_top(double a, int ea, double b, int eb) {
+  const unsigned ah = (unsigned)__double2hiint(a), bh = (unsigned)__double2hiint(b);
+  const unsigned A1 = __funnelshift_l((unsigned)__double2loint(a), (ah & 0xfffffu) | 0x100000u, 11);
+  const unsigned B1 = __funnelshift_l((unsigned)__double2loint(b), (bh & 0xfffffu) | 0x100000u, 11);
+  return ea + eb + (int)(__umulhi(A1, B1) >> 31);
+}
+
+// a b in limbs of a block whose largest fix_prod_top is G: |a b| 2^(B - 1 - (G -
+// 2046)) cut to an integer (values below 2^-1022 count as zero).
 template <int N>
 __device__ __forceinline__ fix2 fix_prod(double a, double b, int G) {
   const unsigned ah = (unsigned)__double2hiint(a), al = (unsigned)__double2loint(a);
@@ -364,17 +373,17 @@ __device__ __forceinline__ fix2 fix_prod(double a, double b, int G) {
   const unsigned B1 = __funnelshift_l(bl, (bh & 0xfffffu) | 0x100000u, 11), B0 = bl << 11;
   unsigned long long P = (unsigned long long)A1 * B1 + __umulhi(A1, B0) + __umulhi(A0, B1);
   if (ea == 0 || eb == 0) P = 0;
-  return fix_limbs(fix_shr(P, (unsigned)(64 - fix_bits(N) + G) - (ea + eb)), ((int)(ah ^ bh) >> 31) | 1);
+  return fix_limbs(fix_shr(P, (unsigned)(63 - fix_bits(N) + G) - (ea + eb)), ((int)(ah ^ bh) >> 31) | 1);
 }
 
-// Block exponents usable with rows of scale sc (for fix_prod's sums of two
-// fields), and the exponent field of the unit 2^(60 - sc - sv) of its rows.
+// Block exponents usable with rows of scale sc (for fix_prod's largest
+// fix_prod_top), and the exponent field of the unit 2^(60 - sc - sv) of its rows.
 template <int N>
-__device__ __forceinline__ int fix_prod_exp(int G, int sc) { return max(G, 962 + fix_bits(N) + sc); }
+__device__ __forceinline__ int fix_prod_exp(int G, int sc) { return max(G, 963 + fix_bits(N) + sc); }
 template <int N>
 __device__ __forceinline__ int fix_field(int E, int sc) { return E + 61 - fix_bits(N) - sc; }
 template <int N>
-__device__ __forceinline__ int fix_prod_field(int G, int sc) { return G - 961 - fix_bits(N) - sc; }
+__device__ __forceinline__ int fix_prod_field(int G, int sc) { return G - 962 - fix_bits(N) - sc; }
 
 // r 2^(u - 1023) as an FP64 value, rounded to nearest, in integer operations
 // (I2F.F64 and the scaling product would cost two at the FP64 rate); u >= 1,
@@ -417,7 +426,7 @@ __device__ __forceinline__ void fix_flux_rows(const FixRows& F, const double (&m
   for (int l = 0; l <= N; ++l) {
     const int em = fix_exp_finite(m[l], b0);
     e0 = max(e0, em);
-    e4 = max(e4, em + fix_exp_finite(th[l], b4));
+    e4 = max(e4, fix_prod_top(m[l], em, th[l], fix_exp_finite(th[l], b4)));
   }
   b4 |= b0;
   fix2 v[N + 1];

@@ -234,8 +234,9 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
     if (gy >= ny) gy -= ny;
     xy_point(P, B, gx + (long long)nx * (gy + (long long)ny * z), z, i >= 0 && i < ox && j < oy, f);
     bool bad = false;
-    e[0] = max(fix_exp_finite(f.mu, bad), fix_exp_finite(f.mv, bad));
-    e[1] = e[0] + fix_exp_finite(f.th, bad);
+    const int eu = fix_exp_finite(f.mu, bad), ev = fix_exp_finite(f.mv, bad), et = fix_exp_finite(f.th, bad);
+    e[0] = max(eu, ev);
+    e[1] = max(fix_prod_top(f.mu, eu, f.th, et), fix_prod_top(f.mv, ev, f.th, et));
     if constexpr (!MIXED) {
       e[2] = max(max(fix_exp_finite(f.xx, bad), fix_exp_finite(f.xy, bad)), fix_exp_finite(f.yy, bad));
       e[3] = max(fix_exp_finite(f.xz, bad), fix_exp_finite(f.yz, bad));
@@ -571,7 +572,7 @@ __global__ void __launch_bounds__(z_tile_threads(N), z_tile_min_blocks(N))
 #pragma unroll
         for (int l = 0; l <= N; ++l) {
           t[l] = src[(NS + l) * kTileCols];
-          E = max(E, fix_exp_finite(a[l], b) + fix_exp_finite(t[l], b));
+          E = max(E, fix_prod_top(a[l], fix_exp_finite(a[l], b), t[l], fix_exp_finite(t[l], b)));
         }
         E = fix_prod_exp<N>(E, sc);
 #pragma unroll
