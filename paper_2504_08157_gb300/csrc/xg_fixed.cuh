@@ -6,17 +6,21 @@
 // with a constant matrix is cheaper in exact integer arithmetic:
 //   * the values of a block (an element segment, or a plane tile) are written
 //     as V = v 2^sv, |V| < 2^B, with one exponent for the block, B = 61 for
-//     orders up to 6 and 60 for 7 and 8: the largest value keeps B bits and
+//     orders up to 4 and 60 above: the largest value keeps B bits and
 //     every value down to 2^-8 (2^-7) of it all of its 53;
 //   * the matrix is written once per mesh as C = c 2^sc, from its long double
 //     entries, with sum_l |C_l| <= 2^60 over every assembled row (59 bits
-//     against FP64's 53); a row that sums to zero up to that rounding is made
-//     to sum to zero exactly, so constants have no derivative;
+//     against FP64's 53);
 //   * both are split into limbs, X = h 2^30 + l with |l| <= 2^29 (so that what
 //     is left out has no bias), and a product takes three IMAD.WIDE, hi += ch h
 //     and mid += ch l + cl h; the low product (below 2^-60 of sum |c| max |v|) is
-//     left out.  Nothing overflows: |hi| <= 2^61, |mid| <= 2^60 + (N + 1)
-//     2^(B - 2) <= 2^63;
+//     left out;
+//   * a row that sums to zero up to its entries' rounding is made to sum to
+//     zero in both limbs, which takes a few |cl| up to 2^30: then a constant
+//     has no derivative at all, as in the difference form (with the low limbs'
+//     sum left over it had one unit of r at some spacings).  Nothing overflows:
+//     |hi| <= 2^61 and, with sum |cl| <= 4/3 (N + 1) 2^29 where sum cl = 0,
+//     |mid| <= 2^60 + 4/3 (N + 1) 2^(B - 1) < 2^63;
 //   * r = hi + mid 2^-30, rounded, is one FP64 value again by one conversion, times
 //     2^(60 - sc - sv).
 // The sums of a block are exact up to those cuts, about 2^-59 of
@@ -74,12 +78,28 @@ inline void fix_rows(int N, const FixMatrix& c, int sc, FixRows* F) {
       sum += C[l];
       if (std::llabs(C[l]) > std::llabs(C[big])) big = l;
     }
-    // a row that sums to zero up to its entries' rounding sums to zero
-    if (std::llabs(sum) <= 8 * (N + 1)) C[big] -= sum;
+    const bool zero = std::llabs(sum) <= 8 * (N + 1);   // up to the entries' rounding
+    if (zero) C[big] -= sum;
+    long long high[kMaxOrder + 1], low[kMaxOrder + 1], over = 0;
     for (int l = 0; l <= N; ++l) {
-      const long long low = (long long)((unsigned long long)C[l] << 34) >> 34;   // signed 30 bits
-      F->cl[a][l] = (int)low;
-      F->ch[a][l] = (int)((C[l] - low) >> 30);
+      low[l] = (long long)((unsigned long long)C[l] << 34) >> 34;   // signed 30 bits
+      high[l] = (C[l] - low[l]) >> 30;
+      over += high[l];
+    }
+    // the high limbs to a sum of zero as well (|over| <= (N + 1) / 2: the low
+    // ones sum to -over 2^30), at the entries with the farthest low limbs
+    while (zero && over != 0) {
+      const int sg = over > 0 ? 1 : -1;
+      int far = 0;
+      for (int l = 1; l <= N; ++l)
+        if (sg * low[l] < sg * low[far]) far = l;
+      high[far] -= sg;
+      low[far] += (long long)sg << 30;
+      over -= sg;
+    }
+    for (int l = 0; l <= N; ++l) {
+      F->ch[a][l] = (int)high[l];
+      F->cl[a][l] = (int)low[l];
     }
   }
 }
@@ -100,7 +120,7 @@ constexpr int kFixNonfinite = 0x7ff;
 __device__ __forceinline__ int fix_block_exp(int e, int sc) { return max(e, max(128, sc + 2)); }
 
 // Bits of a block's values for order N (see the overflow bound above).
-__host__ __device__ constexpr int fix_bits(int N) { return N <= 6 ? 61 : 60; }
+__host__ __device__ constexpr int fix_bits(int N) { return N <= 4 ? 61 : 60; }
 
 // sg V in limbs, V < 2^61: the high one rounded to nearest, but kept below 2^31
 // (the low one is then up to 2^30).
