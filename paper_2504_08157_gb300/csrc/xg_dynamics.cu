@@ -74,16 +74,15 @@ __device__ __forceinline__ double line_apply(const LapParams& P, int d, const do
 // (xg_fixed.cuh): one thread per node with FP64 FMAs spent 3 (N + 1) (1 + 1/N)
 // of them a value, at the FP64 pipe's rate.  Grid of the plane pass: tiles, n_z,
 // 5 variables; out gets the x and y parts.  One Laplacian of the 64 x 64 x 16
-// order-4 box: 0.93-1.02 -> 0.22 + 0.12-0.16 ms; the plane pass is bound by
-// instruction issue (67 % busy, IMAD pipe 68 %), the z pass by the FP64 pipe
-// (3 instructions a value: conversion, scale-and-add, face sum).
+// order-4 box: 0.93-1.02 -> 0.27 + 0.12-0.16 ms; the plane pass is bound by
+// instruction issue (72 % busy, 350 instructions a value), the z pass by the FP64
+// pipe (3 instructions a value: conversion, scale-and-add, face sum).
 template <int N>
-__global__ void __launch_bounds__(kFixThreads) k_lap_plane(const LapParams P, const double* __restrict__ in,
+__global__ void __launch_bounds__(fix_plane_threads(N)) k_lap_plane(const LapParams P, const double* __restrict__ in,
                                                           double* __restrict__ out) {
   using L = FixPlane<N>;
-  __shared__ fix2 V[L::V];
-  __shared__ long long RA[2][L::RA], RB[2][L::RB];
-  __shared__ int emax;
+  __shared__ double V[L::V];
+  __shared__ FixPlaneRows<N> R;
   stage_kernel_begin();
   const int z = blockIdx.y, var = blockIdx.z;
   const int tilesx = (P.nseg[0] + L::E - 1) / L::E;
@@ -91,26 +90,16 @@ __global__ void __launch_bounds__(kFixThreads) k_lap_plane(const LapParams P, co
   const long long off = var * P.np + (long long)nx * ny * z;
   FixTile T;
   T.init<N>(P, blockIdx.x % tilesx, blockIdx.x / tilesx);
-  if (threadIdx.x == 0) emax = 0;
+  fix_plane_load<N, true, true>(in + off, T, nx, ny, V);
   __syncthreads();
-  double v[L::kLoads];
-  fix_plane_load<N, true, true>(in + off, T, nx, ny, v, &emax);
+  fix_plane_rows<N>(P.Kf[0], P.Kf[1], T, V, V, R);
   __syncthreads();
-  const int E = emax == kFixNonfinite ? emax : fix_block_exp(emax, P.Kf[0].sc);
-  if (E != kFixNonfinite) {
-    fix_plane_convert<N>(v, E, V);
-    __syncthreads();
-    fix_plane_rows<N, 0>(P.Kf[0], T, V, RA[0], RB[0]);
-    fix_plane_rows<N, 1>(P.Kf[1], T, V, RA[1], RB[1]);
-    __syncthreads();
-  }
-  const double unit = fix_unit<N>(E, P.Kf[0].sc);
   fix_plane_nodes<N>(T, [&](int i, int j) {
     const long long I = T.x0 + i + (long long)nx * (T.y0 + j);
-    if (E != kFixNonfinite) {
-      const long long r = fix_plane_node<N, 0>(T, RA[0], RB[0], i, j) + fix_plane_node<N, 1>(T, RA[1], RB[1], j, i);
-      out[off + I] = (double)r * unit;
-    } else {   // an infinity or NaN in the tile: FP64, node by node
+    const FixSum r = fix_add(fix_plane_x<N>(R, i, j), fix_plane_y<N>(T, R, i, j));
+    if (r.u < kFixBad) {
+      out[off + I] = fix_double(r);
+    } else {   // an infinity or NaN in a segment of the node: FP64
       double s = line_apply<N>(P, 0, in + off, (long long)nx * (T.y0 + j), 1, T.x0 + i);
       s += line_apply<N>(P, 1, in + off, T.x0 + i, nx, T.y0 + j);
       out[off + I] = s;
@@ -455,9 +444,9 @@ void launch_lap(const LapParams& P, const double* q, double* L1, const double* g
     const dim3 gp(((P.nseg[0] + TE - 1) / TE) * ((P.nseg[1] + TE - 1) / TE), P.n[2], 5);
     const int chunk = xg::fix_z_chunk(P.nseg[2], 5 * nxy, sms);
     const dim3 gz((unsigned)((nxy + 127) / 128), (P.nseg[2] + chunk - 1) / chunk, 5);
-    xg::launch_stage_kernel(xg::k_lap_plane<N>, gp, xg::kFixThreads, 0, st, P, q, L1);
+    xg::launch_stage_kernel(xg::k_lap_plane<N>, gp, xg::fix_plane_threads(N), 0, st, P, q, L1);
     xg::launch_stage_kernel(xg::k_lap_z<N, false>, gz, 128, 0, st, P, q, L1, nullptr, nullptr, chunk);
-    xg::launch_stage_kernel(xg::k_lap_plane<N>, gp, xg::kFixThreads, 0, st, P, L1, E);
+    xg::launch_stage_kernel(xg::k_lap_plane<N>, gp, xg::fix_plane_threads(N), 0, st, P, L1, E);
     xg::launch_stage_kernel(xg::k_lap_z<N, true>, gz, 128, 0, st, P, L1, E, q, gamma, chunk);
   } else {
     xg::launch_stage_kernel(xg::k_sponge_only, (unsigned)std::min<long long>((5 * P.np + 255) / 256, 65535), 256, 0, st, P.np, (int)nxy, q, gamma, E);

@@ -4,29 +4,30 @@
 // GB300 issues 1.9 FP64 FMAs per clock and SM but 60 IMAD.WIDE (32 x 32 -> 64
 // bits with a 64-bit addend; both measured), so a contraction of FP64 data
 // with a constant matrix is cheaper in exact integer arithmetic:
-//   * the values of a block (an element segment, or a plane tile) are written
-//     as V = v 2^sv, |V| < 2^B, with one exponent for the block, B = 61 for
-//     orders up to 4 and 60 above: the largest value keeps B bits and
-//     every value down to 2^-8 (2^-7) of it all of its 53;
+//   * the N + 1 values of an element segment are written as V = v 2^sv, |V| <
+//     2^B, B = 61 for orders up to 4 and 60 above, with one exponent for the
+//     segment: the largest value keeps B bits and every value down to 2^-8 (2^-7)
+//     of it all of its 53;
 //   * the matrix is written once per mesh as C = c 2^sc, from its long double
 //     entries, with sum_l |C_l| <= 2^60 over every assembled row (59 bits
 //     against FP64's 53);
-//   * both are split into limbs, X = h 2^30 + l with |l| <= 2^29 (so that what
-//     is left out has no bias), and a product takes three IMAD.WIDE, hi += ch h
-//     and mid += ch l + cl h; the low product (below 2^-60 of sum |c| max |v|) is
-//     left out;
+//   * both are split into limbs, X = h 2^30 + l, and a product takes three
+//     IMAD.WIDE, hi += ch h and mid += ch l + cl h; the low product (below 2^-58
+//     of sum |c| max |v|) is left out;
 //   * a row that sums to zero up to its entries' rounding is made to sum to
-//     zero in both limbs, which takes a few |cl| up to 2^30: then a constant
-//     has no derivative at all, as in the difference form (with the low limbs'
-//     sum left over it had one unit of r at some spacings).  Nothing overflows:
-//     |hi| <= 2^61 and, with sum |cl| <= 4/3 (N + 1) 2^29 where sum cl = 0,
-//     |mid| <= 2^60 + 4/3 (N + 1) 2^(B - 1) < 2^63;
+//     zero in both limbs, so that rows depend on the values' differences only:
+//     a constant has no derivative at all, as in the difference form, and what is
+//     left out has no bias.  That takes a few |cl| up to 2^30, with sum |cl| <=
+//     4/3 (N + 1) 2^29; nothing overflows: |hi| <= 2^61 and |mid| <= 2^60 +
+//     4/3 (N + 1) 2^(B - 1) < 2^63;
 //   * r = hi + mid 2^-30, rounded, is one FP64 value again by one conversion, times
 //     2^(60 - sc - sv).
-// The sums of a block are exact up to those cuts, about 2^-59 of
+// A segment's sums are exact up to those cuts, a few 2^-59 of its
 // sum |c| max |v|, where an FP64 FMA chain rounds at 2^-53 of its partial
-// sums.  A block with an infinity or NaN has no exponent; its callers take
-// the FP64 path or return NaN for the segment, as an FP64 chain would.
+// sums.  Sums over segments and directions are taken in the larger one's unit
+// (fix_add), so a node's error is one of the values in its own segments.  A
+// segment with an infinity or NaN has no exponent; its callers take the FP64
+// path or return NaN, as an FP64 chain would.
 #pragma once
 
 #include <cmath>
@@ -115,21 +116,20 @@ __device__ __forceinline__ int fix_exp(double v) { return (int)(((unsigned)__dou
 
 constexpr int kFixNonfinite = 0x7ff;
 
-// The exponent used for a block whose largest field is e, against rows of
-// scale sc: tiny blocks are cut at 2^-900 or so.
+// The exponent used for a segment whose largest field is e, against rows of
+// scale sc: tiny ones are cut at 2^-900 or so.
 __device__ __forceinline__ int fix_block_exp(int e, int sc) { return max(e, max(128, sc + 2)); }
 
-// Bits of a block's values for order N (see the overflow bound above).
+// Bits B of a segment's values (see the overflow bound above).
 __host__ __device__ constexpr int fix_bits(int N) { return N <= 4 ? 61 : 60; }
 
-// sg V in limbs, V < 2^61: the high one rounded to nearest, but kept below 2^31
-// (the low one is then up to 2^30).
+// sg V in limbs, V < 2^61: the low one cut, 0 .. 2^30 with v's sign.  (Rows
+// depend on differences, so the low limbs' mean does not bias them.)
 __device__ __forceinline__ fix2 fix_limbs(unsigned long long V, int sg) {
-  const unsigned h = min((unsigned)((V + (1ull << 29)) >> 30), 0x7fffffffu);
-  return {(int)h * sg, (int)((unsigned)V - (h << 30)) * sg};
+  return {(int)(V >> 30) * sg, (int)((unsigned)V & 0x3fffffffu) * sg};
 }
 
-// v in the limbs of a block of exponent E >= fix_exp(v): |v| 2^(B - 1 - (E -
+// v in the limbs of a segment of exponent E >= fix_exp(v): |v| 2^(B - 1 - (E -
 // 1023)) cut to an integer, both limbs with v's sign.
 template <int N>
 __device__ __forceinline__ fix2 fix_of(double v, int E) {
@@ -143,7 +143,7 @@ __device__ __forceinline__ fix2 fix_of(double v, int E) {
   return fix_limbs(V, ((int)hi >> 31) | 1);
 }
 
-// 2^(60 - sc - sv) of a block of exponent E (NaN for a block that has none)
+// 2^(60 - sc - sv) of a segment of exponent E (NaN for one that has none)
 template <int N>
 __device__ __forceinline__ double fix_unit(int E, int sc) {
   if (E == kFixNonfinite) return __hiloint2double(0x7ff80000, 0);
@@ -163,195 +163,6 @@ __device__ __forceinline__ long long fix_row(const FixRows& F, int a, const fix2
   return hi + (mid >> 30);
 }
 
-// ---------------------------------------------------------------- plane tiles
-// A CTA takes E x E elements of one level.  Its nodes' x and y rows need the
-// tile extended by the segment before it and its end face along each
-// direction (a cross); the extended tile is converted once, with one exponent,
-// into shared memory (two limbs a node), one thread takes a whole element
-// segment of a line -- the matrix then comes from the constant bank at fixed
-// offsets, and a segment's N + 1 values are read once for its N + 1 rows --
-// and leaves its rows as 64-bit integers, which the nodes add up exactly: rows
-// 0..N-1 in RA, row N, which belongs to the next segment's first node, in RB.
-__host__ __device__ constexpr int fix_plane_elems(int N) { return 32 / N; }
-constexpr int kFixThreads = 256;
-
-template <int N>
-struct FixPlane {
-  static constexpr int E = fix_plane_elems(N);
-  static constexpr int TS = E * N;            // <= 32: a warp takes a row of the tile, a lane a column
-  static constexpr int LO = TS + 1;           // owned extent (a wall's last node included)
-  static constexpr int LX = TS + N + 1;       // extended extent
-  static constexpr int PV = LX | 1;           // odd pitches: lanes along either axis hit distinct banks
-  static constexpr int PR = LO | 1;
-  static constexpr int V = LX * PV;           // 8-byte slots
-  static constexpr int RA = LO * PR;
-  static constexpr int RB = (E + 1) * LO;
-  static constexpr int kWarps = kFixThreads / 32;
-  static constexpr int kRows = (LX + kWarps - 1) / kWarps;                   // rows per warp
-  static constexpr int kSide = (LO * N + LX + kFixThreads - 1) / kFixThreads;    // the columns beside the tile's
-  static constexpr int kLoads = kRows + kSide;
-};
-
-// Extent of tile (bx, by) as PlaneTile (xg_plane_f32.cuh) for any line
-// parameters.
-struct FixTile {
-  int ekx, eky, x0, y0, ox, oy;
-  bool hxl, hyl;
-  template <int N, typename P>
-  __device__ __forceinline__ void init(const P& p, int bx, int by) {
-    constexpr int E = fix_plane_elems(N);
-    ekx = min(E, p.nseg[0] - bx * E);
-    eky = min(E, p.nseg[1] - by * E);
-    x0 = bx * E * N;
-    y0 = by * E * N;
-    ox = ekx * N + (!p.per[0] && bx * E + ekx == p.nseg[0] ? 1 : 0);
-    oy = eky * N + (!p.per[1] && by * E + eky == p.nseg[1] ? 1 : 0);
-    hxl = bx > 0 || p.per[0];
-    hyl = by > 0 || p.per[1];
-  }
-};
-
-// Slot k of this thread in the extended tile: row jj and column ii (both
-// offset by N); false where the thread has none.  The first kRows slots are
-// rows of the tile's own TS columns, one warp a row; the rest are the N columns
-// before them, of the owned rows, and the one after them, of every row (a
-// wall's last column has y segments of its own).
-template <int N>
-__device__ __forceinline__ bool fix_plane_slot(int k, int& jj, int& ii) {
-  using L = FixPlane<N>;
-  if (k < L::kRows) {
-    jj = (int)(threadIdx.x >> 5) + k * L::kWarps;
-    ii = N + (int)(threadIdx.x & 31);
-    return jj < L::LX && ii < N + L::TS;
-  }
-  const int t = (int)threadIdx.x + (k - L::kRows) * kFixThreads;
-  if (t < L::LO * N) {
-    const int r = t / N;
-    jj = N + r;
-    ii = t - r * N;
-    return true;
-  }
-  jj = t - L::LO * N;
-  ii = N + L::TS;
-  return jj < L::LX;
-}
-
-// Loads the cross of one variable f (a level's first node) into registers and
-// raises *emax to its largest exponent field.  X, Y: which directions' segments
-// are needed.
-template <int N, bool X, bool Y>
-__device__ __forceinline__ void fix_plane_load(const double* __restrict__ f, const FixTile& T, int nx, int ny,
-                                               double (&v)[FixPlane<N>::kLoads], int* emax) {
-  using L = FixPlane<N>;
-  int e = 0;
-#pragma unroll
-  for (int k = 0; k < L::kLoads; ++k) {
-    int jj, ii;
-    const bool has = fix_plane_slot<N>(k, jj, ii);
-    const int i = ii - N, j = jj - N;
-    // owned rows extended along x, owned columns extended along y
-    const bool inx = j >= 0 && j < T.oy && (i >= 0 || T.hxl) && i <= T.ekx * N;
-    const bool iny = i >= 0 && i < T.ox && (j >= 0 || T.hyl) && j <= T.eky * N;
-    v[k] = 0.0;
-    if (has && ((X && inx) || (Y && iny))) {
-      int gx = T.x0 + i, gy = T.y0 + j;
-      if (gx < 0) gx += nx;
-      if (gy < 0) gy += ny;
-      if (gx >= nx) gx -= nx;
-      if (gy >= ny) gy -= ny;
-      v[k] = f[gx + (long long)nx * gy];
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < L::kLoads; ++k) e = max(e, fix_exp(v[k]));
-  e = (int)__reduce_max_sync(0xffffffffu, (unsigned)e);
-  if ((threadIdx.x & 31) == 0) atomicMax(emax, e);
-}
-
-// The loaded values in limbs of a block of exponent E.
-template <int N>
-__device__ __forceinline__ void fix_plane_convert(const double (&v)[FixPlane<N>::kLoads], int E, fix2* V) {
-  using L = FixPlane<N>;
-#pragma unroll
-  for (int k = 0; k < L::kLoads; ++k) {
-    int jj, ii;
-    if (fix_plane_slot<N>(k, jj, ii)) V[jj * L::PV + ii] = fix_of<N>(v[k], E);
-  }
-}
-
-// Rows of every x segment (DIR 0) or y segment (DIR 1) of the tile: RA[j][i]
-// the row of node (i, j) in the segment that starts at or before it, RB[s][.]
-// row N of segment s - 1 (s = 0: the segment before the tile).
-template <int N, int DIR>
-__device__ __forceinline__ void fix_plane_rows(const FixRows& F, const FixTile& T, const fix2* V, long long* RA,
-                                               long long* RB) {
-  using L = FixPlane<N>;
-  const int ns = (DIR == 0 ? T.ekx : T.eky) + 1, no = DIR == 0 ? T.oy : T.ox;
-  const bool left = DIR == 0 ? T.hxl : T.hyl;
-  for (int t = threadIdx.x; t < ns * L::LO; t += kFixThreads) {
-    const int s = t / L::LO, o = t - s * L::LO;   // s - 1: the segment; o: the line
-    if (o >= no || (s == 0 && !left)) continue;
-    const fix2* p = DIR == 0 ? V + (o + N) * L::PV + s * N : V + s * N * L::PV + o + N;
-    fix2 v[N + 1];
-#pragma unroll
-    for (int l = 0; l <= N; ++l) v[l] = p[DIR == 0 ? l : l * L::PV];
-    RB[s * L::LO + o] = fix_row<N>(F, N, v);
-    if (s > 0) {
-#pragma unroll
-      for (int a = 0; a < N; ++a) {
-        const int g = (s - 1) * N + a;
-        RA[DIR == 0 ? o * L::PR + g : g * L::PR + o] = fix_row<N>(F, a, v);
-      }
-    }
-  }
-}
-
-// The assembled row of node g (0-based in the tile) on line o along DIR.
-template <int N, int DIR>
-__device__ __forceinline__ long long fix_plane_node(const FixTile& T, const long long* RA, const long long* RB,
-                                                    int g, int o) {
-  using L = FixPlane<N>;
-  const int s = g / N, ek = DIR == 0 ? T.ekx : T.eky;
-  if (s == ek) return 2 * RB[ek * L::LO + o];            // a wall's last node: its row twice
-  const long long r = RA[DIR == 0 ? o * L::PR + g : g * L::PR + o];
-  if (g != s * N) return r;
-  if (s > 0 || (DIR == 0 ? T.hxl : T.hyl)) return r + RB[s * L::LO + o];
-  return 2 * r;
-}
-
-// node(i, j) for every owned node of the tile: a warp takes a row, a lane a
-// column; a wall's last column (i = TS) goes to the threads of its own.
-template <int N, typename F>
-__device__ __forceinline__ void fix_plane_nodes(const FixTile& T, F node) {
-  using L = FixPlane<N>;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane < min(T.ox, L::TS)) {
-    for (int j = warp; j < T.oy; j += L::kWarps) node(lane, j);
-  }
-  if (T.ox > L::TS && (int)threadIdx.x < T.oy) node(L::TS, (int)threadIdx.x);
-}
-
-// One z segment's values (FP64, in registers) in limbs, with its own exponent.
-template <int N>
-__device__ __forceinline__ int fix_segment(const double (&v)[N + 1], int sc, fix2 (&f)[N + 1]) {
-  int e = fix_exp(v[0]);
-#pragma unroll
-  for (int l = 1; l <= N; ++l) e = max(e, fix_exp(v[l]));
-  const int E = e == kFixNonfinite ? e : fix_block_exp(e, sc);
-#pragma unroll
-  for (int l = 0; l <= N; ++l) f[l] = fix_of<N>(v[l], E);
-  return E;
-}
-
-// Segments per thread of a marching z pass: enough chunks to give every SM
-// 1,024 threads (a chunk start recomputes one segment's last row).
-inline int fix_z_chunk(int nseg, long long columns, int sms) {
-  long long chunks = (1024ll * sms + columns - 1) / columns;
-  if (chunks < 1) chunks = 1;
-  if (chunks > nseg) chunks = nseg;
-  return (int)((nseg + chunks - 1) / chunks);
-}
-
 // ---------------------------------------------------------------- fluxes
 // exponent field of v, 0 for an infinity or NaN
 __device__ __forceinline__ int fix_exp_finite(double v, bool& bad) {
@@ -361,10 +172,6 @@ __device__ __forceinline__ int fix_exp_finite(double v, bool& bad) {
   return b ? 0 : e;
 }
 
-__device__ __forceinline__ bool fix_bad(double v) { return fix_exp(v) == kFixNonfinite; }
-
-constexpr int kFixMark = (int)0x80000000;   // high limb of a value without an exponent: |h| < 2^31 for all others
-
 __device__ __forceinline__ unsigned long long fix_shr(unsigned long long m, unsigned s) {
   unsigned long long v;
   asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(s));   // clamps: 0 for s >= 64
@@ -372,7 +179,7 @@ __device__ __forceinline__ unsigned long long fix_shr(unsigned long long m, unsi
 }
 
 // Exponent field of a b on a scale of its own: the fields' sum, and one where the
-// significands' product reaches 2 (from their leading 32 bits; fix_limbs takes a
+// significands' product reaches 2 (from their leading 32 bits; fix_prod takes a
 // product that reaches it in the bits below).  ea, eb: the fields.
 __device__ __forceinline__ int fix_prod_top(double a, int ea, double b, int eb) {
   const unsigned ah = (unsigned)__double2hiint(a), bh = (unsigned)__double2hiint(b);
@@ -381,7 +188,7 @@ __device__ __forceinline__ int fix_prod_top(double a, int ea, double b, int eb) 
   return ea + eb + (int)(__umulhi(A1, B1) >> 31);
 }
 
-// a b in limbs of a block whose largest fix_prod_top is G: |a b| 2^(B - 1 - (G -
+// a b in limbs of a segment whose largest fix_prod_top is G: |a b| 2^(B - 1 - (G -
 // 2046)) cut to an integer (values below 2^-1022 count as zero).
 template <int N>
 __device__ __forceinline__ fix2 fix_prod(double a, double b, int G) {
@@ -393,10 +200,14 @@ __device__ __forceinline__ fix2 fix_prod(double a, double b, int G) {
   const unsigned B1 = __funnelshift_l(bl, (bh & 0xfffffu) | 0x100000u, 11), B0 = bl << 11;
   unsigned long long P = (unsigned long long)A1 * B1 + __umulhi(A1, B0) + __umulhi(A0, B1);
   if (ea == 0 || eb == 0) P = 0;
-  return fix_limbs(fix_shr(P, (unsigned)(63 - fix_bits(N) + G) - (ea + eb)), ((int)(ah ^ bh) >> 31) | 1);
+  const int sg = ((int)(ah ^ bh) >> 31) | 1;
+  const unsigned long long V = fix_shr(P, (unsigned)(63 - fix_bits(N) + G) - (ea + eb));
+  if (fix_bits(N) < 61) return fix_limbs(V, sg);
+  const unsigned h = min((unsigned)(V >> 30), 0x7fffffffu);   // V may reach 2^61
+  return {(int)h * sg, (int)((unsigned)V - (h << 30)) * sg};
 }
 
-// Block exponents usable with rows of scale sc (for fix_prod's largest
+// Exponents usable with rows of scale sc (for fix_prod's largest
 // fix_prod_top), and the exponent field of the unit 2^(60 - sc - sv) of its rows.
 template <int N>
 __device__ __forceinline__ int fix_prod_exp(int G, int sc) { return max(G, 963 + fix_bits(N) + sc); }
@@ -432,6 +243,321 @@ __device__ __forceinline__ double fix_out(long long r, int u) {
   if (MIXED) v = (double)r * __hiloint2double(min(u, 2046) << 20, 0);
   else fix_value(r, u, v);
   return v;
+}
+
+// ---------------------------------------------------------------- sums of rows
+// r 2^(u - 1023), |r| < 2^62: the rows of one segment share u, an exponent field.
+struct FixSum {
+  long long r;
+  int u;
+};
+
+constexpr int kFixBad = 0x4000;   // u of a segment that holds an infinity or NaN
+
+// a + b in the larger of the two units, the other rounded to it: the segments
+// keep the bits of their own values, whatever a neighbour or the other direction
+// holds.
+__device__ __forceinline__ FixSum fix_add(FixSum a, FixSum b) {
+  const bool swap = a.u < b.u;
+  const long long big = swap ? b.r : a.r, low = swap ? a.r : b.r;
+  const int d = min(abs(a.u - b.u), 62);
+  return {big + ((((low + low) >> d) + 1) >> 1), max(a.u, b.u)};
+}
+
+__device__ __forceinline__ FixSum fix_twice(FixSum a) { return {a.r + a.r, a.u}; }
+
+// Its FP64 value (u < kFixBad), in two FP64 operations.
+__device__ __forceinline__ double fix_double(FixSum a) {
+  return (double)a.r * __hiloint2double(min(a.u, 2046) << 20, 0);
+}
+
+// Its value for the form at hand (fix_out), NaN for a bad one.
+template <bool MIXED>
+__device__ __forceinline__ double fix_sum_out(FixSum a) {
+  return a.u >= kFixBad ? xg_nan(0.0) : fix_out<MIXED>(a.r, a.u);
+}
+
+// u, or 0 where all values are equal: the rows are zero, which is exact in any
+// unit, and must not cost the sums that they are added to any bits.
+template <int N>
+__device__ __forceinline__ int fix_unit_of(const fix2 (&v)[N + 1], int u) {
+  int differ = 0;
+#pragma unroll
+  for (int l = 1; l <= N; ++l) {
+    differ |= v[l].h ^ v[0].h;
+    differ |= v[l].l ^ v[0].l;
+  }
+  return differ != 0 ? u : 0;
+}
+
+// The values a of one segment, or the products t m, in limbs of an exponent of
+// their own; returns the u of their rows against a matrix of scale sc.
+template <int N>
+__device__ __forceinline__ int fix_values(const double (&a)[N + 1], int sc, fix2 (&v)[N + 1]) {
+  int e = fix_exp(a[0]);
+#pragma unroll
+  for (int l = 1; l <= N; ++l) e = max(e, fix_exp(a[l]));
+  const int E = fix_block_exp(e, sc);
+#pragma unroll
+  for (int l = 0; l <= N; ++l) v[l] = fix_of<N>(a[l], E);
+  return e == kFixNonfinite ? kFixBad : fix_unit_of<N>(v, fix_field<N>(E, sc));
+}
+
+template <int N>
+__device__ __forceinline__ int fix_products(const double* m, const double* t, int stride, int sc,
+                                            fix2 (&v)[N + 1]) {
+  bool bad = false;
+  int G = 0;
+#pragma unroll
+  for (int l = 0; l <= N; ++l) {
+    const double x = m[l * stride], y = t[l * stride];
+    G = max(G, fix_prod_top(x, fix_exp_finite(x, bad), y, fix_exp_finite(y, bad)));
+  }
+  G = fix_prod_exp<N>(G, sc);
+#pragma unroll
+  for (int l = 0; l <= N; ++l) v[l] = fix_prod<N>(t[l * stride], m[l * stride], G);
+  return bad ? kFixBad : fix_unit_of<N>(v, fix_prod_field<N>(G, sc));
+}
+
+// Rows of x segments, the segments of a line on consecutive lanes, so that a
+// first node's row is joined with row N of the segment before (left; a wall's
+// first and, where end, last node take theirs twice) without a barrier.  Called
+// by all lanes of a warp: act the lanes that have a segment, own those whose
+// rows are wanted; put(a, row) gets the nodes' rows.
+template <int N, typename Put>
+__device__ __forceinline__ void fix_x_rows(const FixRows& F, const fix2 (&v)[N + 1], int u, bool act, bool own,
+                                           bool left, bool end, Put put) {
+  FixSum last = {0, u}, before;
+  if (act) last.r = fix_row<N>(F, N, v);
+  before.r = __shfl_up_sync(0xffffffffu, last.r, 1);
+  before.u = __shfl_up_sync(0xffffffffu, last.u, 1);
+  if (!own) return;
+  const FixSum first = {fix_row<N>(F, 0, v), u};
+  put(0, left ? fix_add(first, before) : fix_twice(first));
+#pragma unroll
+  for (int a = 1; a < N; ++a) put(a, FixSum{fix_row<N>(F, a, v), u});
+  if (end) put(N, fix_twice(last));
+}
+
+// Slot of node i's unit among the 2 E + 1 of a line of E segments: a segment's
+// first node, which two segments meet in, has one of its own.
+template <int N>
+__device__ __forceinline__ int fix_unit_slot(int i) {
+  const int s = i / N;
+  return 2 * s + (i != s * N);
+}
+
+// ---------------------------------------------------------------- plane tiles
+// A CTA takes E x E elements of one level.  Its nodes' x and y rows need the
+// tile extended by the segment before it and its end face along each
+// direction (a cross), which is put into shared memory once; one thread takes a
+// whole element segment of a line -- the matrix then comes from the constant
+// bank at fixed offsets, and a segment's N + 1 values are read once for its
+// N + 1 rows -- converts its values with an exponent of their own and leaves its
+// rows as 64-bit integers, which the nodes add up (fix_add).  A warp takes the
+// x segments of 32 / (E + 1) lines, the one before the tile among them, or 32 y
+// segments.
+// (One exponent and one conversion a value for the whole tile, 0.234 against
+// 0.267 ms a Laplacian's pass over 5 x 4.3 M nodes, left a quiet segment the bits
+// that the loudest one of the tile had to spare.)
+__host__ __device__ constexpr int fix_plane_elems(int N) { return N == 1 ? 31 : (N == 2 ? 15 : 32 / N); }
+// (order 4: 21 tasks of a warp a tile, three rounds of seven)
+__host__ __device__ constexpr int fix_plane_threads(int N) { return N == 4 ? 224 : 256; }
+
+template <int N>
+struct FixPlane {
+  static constexpr int kThreads = fix_plane_threads(N);
+  static constexpr int E = fix_plane_elems(N);
+  static constexpr int TS = E * N;            // <= 32: a warp takes a row of the tile, a lane a column
+  static constexpr int LO = TS + 1;           // owned extent (a wall's last node included)
+  static constexpr int LX = TS + N + 1;       // extended extent
+  static constexpr int PV = LX | 1;           // odd pitches: lanes along either axis hit distinct banks
+  static constexpr int PR = LO | 1;
+  static constexpr int V = LX * PV;           // 8-byte slots
+  static constexpr int RX = LO * PR, UX = LO * (2 * E + 1);   // x rows (wall ends included) and units
+  static constexpr int RY = TS * PR, RB = (E + 1) * LO;       // y rows; rows N, and units, of segments -1..E-1
+  static constexpr int kWarps = kThreads / 32;
+  static constexpr int kRows = (LX + kWarps - 1) / kWarps;                   // rows per warp
+  static constexpr int kSide = (LO * N + LX + kThreads - 1) / kThreads;      // the columns beside the tile's
+};
+
+// Rows of a tile's segments.
+template <int N>
+struct FixPlaneRows {
+  using L = FixPlane<N>;
+  long long x[L::RX], y[L::RY], yn[L::RB];
+  int ux[L::UX], uy[L::RB];
+};
+
+// Extent of tile (bx, by) as PlaneTile (xg_plane_f32.cuh) for any line
+// parameters.
+struct FixTile {
+  int ekx, eky, x0, y0, ox, oy;
+  bool hxl, hyl;
+  template <int N, typename P>
+  __device__ __forceinline__ void init(const P& p, int bx, int by) {
+    constexpr int E = fix_plane_elems(N);
+    ekx = min(E, p.nseg[0] - bx * E);
+    eky = min(E, p.nseg[1] - by * E);
+    x0 = bx * E * N;
+    y0 = by * E * N;
+    ox = ekx * N + (!p.per[0] && bx * E + ekx == p.nseg[0] ? 1 : 0);
+    oy = eky * N + (!p.per[1] && by * E + eky == p.nseg[1] ? 1 : 0);
+    hxl = bx > 0 || p.per[0];
+    hyl = by > 0 || p.per[1];
+  }
+};
+
+// Loads the cross of one variable f (a level's first node) into V[j + N][i + N]:
+// a warp takes a row of the tile's own columns; the rest are the N columns before
+// them, of the owned rows, and the one after them, of every row (a wall's last
+// column has y segments of its own).  X, Y: which directions' segments are needed
+// (owned rows extended along x, owned columns along y).
+template <int N, bool X, bool Y>
+__device__ __forceinline__ void fix_plane_load(const double* __restrict__ f, const FixTile& T, int nx, int ny,
+                                               double* V) {
+  using L = FixPlane<N>;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int fx = T.ekx * N, fy = T.eky * N;
+  auto value = [&](int i, int j) -> double {
+    const bool inx = X && j >= 0 && j < T.oy && (i >= 0 || T.hxl) && i <= fx;
+    const bool iny = Y && i >= 0 && i < T.ox && (j >= 0 || T.hyl) && j <= fy;
+    if (!inx && !iny) return 0.0;
+    int gx = T.x0 + i, gy = T.y0 + j;
+    if (gx < 0) gx += nx;
+    if (gy < 0) gy += ny;
+    if (gx >= nx) gx -= nx;
+    if (gy >= ny) gy -= ny;
+    return f[gx + (long long)nx * gy];
+  };
+  double v[L::kRows], w[L::kSide];
+  const int gx = T.x0 + lane - (T.x0 + lane >= nx ? nx : 0);
+  const bool colx = X && lane < L::TS && lane <= fx, coly = Y && lane < L::TS && lane < T.ox;
+#pragma unroll
+  for (int k = 0; k < L::kRows; ++k) {
+    const int j = warp + k * L::kWarps - N;
+    int gy = T.y0 + j;
+    if (j < 0) gy += gy < 0 ? ny : 0;
+    else gy -= gy >= ny ? ny : 0;
+    v[k] = 0.0;
+    if ((colx && j >= 0 && j < T.oy) || (coly && (j >= 0 || T.hyl) && j <= fy)) v[k] = f[gx + (long long)nx * gy];
+  }
+#pragma unroll
+  for (int k = 0; k < L::kSide; ++k) {
+    const int t = (int)threadIdx.x + k * L::kThreads, r = t / N;
+    if (t < L::LO * N) w[k] = value(t - r * N - N, r);
+    else w[k] = value(L::TS, t - L::LO * N - N);
+  }
+#pragma unroll
+  for (int k = 0; k < L::kRows; ++k) {
+    const int jj = warp + k * L::kWarps;
+    if (lane < L::TS && jj < L::LX) V[jj * L::PV + N + lane] = v[k];
+  }
+#pragma unroll
+  for (int k = 0; k < L::kSide; ++k) {
+    const int t = (int)threadIdx.x + k * L::kThreads, r = t / N;
+    if (t < L::LO * N) V[(N + r) * L::PV + t - r * N] = w[k];
+    else if (t < L::LO * N + L::LX) V[(t - L::LO * N) * L::PV + N + L::TS] = w[k];
+  }
+}
+
+// Rows of every x segment of the tile's values Vx and y segment of Vy.
+template <int N>
+__device__ __forceinline__ void fix_plane_rows(const FixRows& FX, const FixRows& FY, const FixTile& T, const double* Vx,
+                                               const double* Vy, FixPlaneRows<N>& R) {
+  using L = FixPlane<N>;
+  constexpr int kLines = 32 / (L::E + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // y: a warp takes a segment of the tile's TS columns; the segments of a wall's
+  // last column are a task more
+  const int wx = (T.oy + kLines - 1) / kLines, y0 = T.hyl ? 0 : 1, wy = T.eky + 1 - y0 + (T.ox > L::TS ? 1 : 0);
+  for (int w = warp; w < wx + wy; w += L::kWarps) {
+    double a[N + 1];
+    fix2 v[N + 1];
+    if (w < wx) {
+      const int line = lane / (L::E + 1), s = lane - line * (L::E + 1) - 1, o = w * kLines + line;
+      const bool act = line < kLines && o < T.oy && s < T.ekx && (s >= 0 || T.hxl);
+      int u = 0;
+      if (act) {
+        const double* p = Vx + (o + N) * L::PV + (s + 1) * N;
+#pragma unroll
+        for (int l = 0; l <= N; ++l) a[l] = p[l];
+        u = fix_values<N>(a, FX.sc, v);
+      }
+      long long* r = R.x + o * L::PR + s * N;
+      int* ur = R.ux + o * (2 * L::E + 1) + 2 * s;
+      fix_x_rows<N>(FX, v, u, act, act && s >= 0, s > 0 || T.hxl, T.ox > T.ekx * N && s == T.ekx - 1,
+                    [&](int k, FixSum x) {
+                      r[k] = x.r;
+                      if (k < 2 || k == N) ur[k == N ? 2 : k] = x.u;
+                    });
+    } else {
+      const bool edge = w - wx + y0 > T.eky;
+      const int s = edge ? y0 + lane : w - wx + y0, o = edge ? L::TS : lane;   // s - 1: the segment
+      if (s > T.eky || o >= (edge ? T.ox : min(T.ox, L::TS))) continue;
+      const double* p = Vy + s * N * L::PV + o + N;
+#pragma unroll
+      for (int l = 0; l <= N; ++l) a[l] = p[l * L::PV];
+      R.uy[s * L::LO + o] = fix_values<N>(a, FY.sc, v);
+      R.yn[s * L::LO + o] = fix_row<N>(FY, N, v);
+      if (s > 0) {
+#pragma unroll
+        for (int k = 0; k < N; ++k) R.y[((s - 1) * N + k) * L::PR + o] = fix_row<N>(FY, k, v);
+      }
+    }
+  }
+}
+
+// The assembled x and y rows of the tile's node (i, j).
+template <int N>
+__device__ __forceinline__ FixSum fix_plane_x(const FixPlaneRows<N>& R, int i, int j) {
+  using L = FixPlane<N>;
+  return {R.x[j * L::PR + i], R.ux[j * (2 * L::E + 1) + fix_unit_slot<N>(i)]};
+}
+
+template <int N>
+__device__ __forceinline__ FixSum fix_plane_y(const FixTile& T, const FixPlaneRows<N>& R, int i, int j) {
+  using L = FixPlane<N>;
+  const int s = j / N;
+  const FixSum before = {R.yn[s * L::LO + i], R.uy[s * L::LO + i]};
+  if (s == T.eky) return fix_twice(before);              // a wall's last node: its row twice
+  const FixSum r = {R.y[j * L::PR + i], R.uy[(s + 1) * L::LO + i]};
+  if (j != s * N) return r;
+  return s > 0 || T.hyl ? fix_add(r, before) : fix_twice(r);
+}
+
+// node(i, j) for every owned node of the tile: a warp takes a row, a lane a
+// column; a wall's last column (i = TS) goes to the threads of its own.
+template <int N, typename F>
+__device__ __forceinline__ void fix_plane_nodes(const FixTile& T, F node) {
+  using L = FixPlane<N>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane < min(T.ox, L::TS)) {
+    for (int j = warp; j < T.oy; j += L::kWarps) node(lane, j);
+  }
+  if (T.ox > L::TS && (int)threadIdx.x < T.oy) node(L::TS, (int)threadIdx.x);
+}
+
+// ---------------------------------------------------------------- z lines
+// One z segment's values (FP64, in registers) in limbs, with its own exponent.
+template <int N>
+__device__ __forceinline__ int fix_segment(const double (&v)[N + 1], int sc, fix2 (&f)[N + 1]) {
+  int e = fix_exp(v[0]);
+#pragma unroll
+  for (int l = 1; l <= N; ++l) e = max(e, fix_exp(v[l]));
+  const int E = e == kFixNonfinite ? e : fix_block_exp(e, sc);
+#pragma unroll
+  for (int l = 0; l <= N; ++l) f[l] = fix_of<N>(v[l], E);
+  return E;
+}
+
+// Segments per thread of a marching z pass: enough chunks to give every SM
+// 1,024 threads (a chunk start recomputes one segment's last row).
+inline int fix_z_chunk(int nseg, long long columns, int sms) {
+  long long chunks = (1024ll * sms + columns - 1) / columns;
+  if (chunks < 1) chunks = 1;
+  if (chunks > nseg) chunks = nseg;
+  return (int)((nseg + chunks - 1) / chunks);
 }
 
 // Rows of the rho' and Theta' fluxes m and theta m of one segment, with an

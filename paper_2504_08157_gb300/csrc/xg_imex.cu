@@ -75,73 +75,45 @@ __device__ __forceinline__ double line_sum(const LineParams& P, int d, const dou
 // the z pass, blockIdx.z = 1 finishes rho u and rho v from Theta' (cpl = gamma
 // p0 / Theta0 per level).
 template <int N, bool PLAIN>
-__global__ void __launch_bounds__(kFixThreads) k_lin_plane(const LinParams Q, const double* __restrict__ v,
+__global__ void __launch_bounds__(fix_plane_threads(N)) k_lin_plane(const LinParams Q, const double* __restrict__ v,
                                                           const double* __restrict__ cpl, double c0, double c1,
                                                           double* __restrict__ out) {
   using L = FixPlane<N>;
-  __shared__ fix2 V[2][L::V];
-  __shared__ long long RA[2][L::RA], RB[2][L::RB];
-  __shared__ int emax;
+  __shared__ double V[2][L::V];
+  __shared__ FixPlaneRows<N> R;
   stage_kernel_begin();
   const LineParams& P = Q.P;
-  const int z = blockIdx.y, nx = P.n[0], ny = P.n[1], sc = Q.D[0].sc;
+  const int z = blockIdx.y, nx = P.n[0], ny = P.n[1];
   const int tilesx = (P.nseg[0] + L::E - 1) / L::E;
   const long long np = P.np, off = (long long)nx * ny * z;
   FixTile T;
   T.init<N>(P, blockIdx.x % tilesx, blockIdx.x / tilesx);
-  if (threadIdx.x == 0) emax = 0;
-  __syncthreads();
   const bool theta = blockIdx.z == 1;
   const double* fx = v + (theta ? 4 : 1) * np + off;
   const double* fy = v + (theta ? 4 : 2) * np + off;
-  const fix2* Vy = theta ? V[0] : V[1];
-  int E;
   if (theta) {
-    double a[L::kLoads];
-    fix_plane_load<N, true, true>(fx, T, nx, ny, a, &emax);
-    __syncthreads();
-    E = emax == kFixNonfinite ? emax : fix_block_exp(emax, sc);
-    if (E != kFixNonfinite) fix_plane_convert<N>(a, E, V[0]);
+    fix_plane_load<N, true, true>(fx, T, nx, ny, V[0]);
   } else {
-    // one exponent for both momenta: A is a sum of integers, exact where the
-    // two parts nearly cancel (a vortex)
-    double a[L::kLoads], b[L::kLoads];
-    fix_plane_load<N, true, false>(fx, T, nx, ny, a, &emax);
-    fix_plane_load<N, false, true>(fy, T, nx, ny, b, &emax);
-    __syncthreads();
-    E = emax == kFixNonfinite ? emax : fix_block_exp(emax, sc);
-    if (E != kFixNonfinite) {
-      fix_plane_convert<N>(a, E, V[0]);
-      fix_plane_convert<N>(b, E, V[1]);
-    }
+    fix_plane_load<N, true, false>(fx, T, nx, ny, V[0]);
+    fix_plane_load<N, false, true>(fy, T, nx, ny, V[1]);
   }
   __syncthreads();
-  if (E != kFixNonfinite) {
-    fix_plane_rows<N, 0>(Q.D[0], T, V[0], RA[0], RB[0]);
-    fix_plane_rows<N, 1>(Q.D[1], T, Vy, RA[1], RB[1]);
-    __syncthreads();
-  }
-  const double cp = theta ? cpl[z] : 1.0, unit = fix_unit<N>(E, sc) * cp;
+  fix_plane_rows<N>(Q.D[0], Q.D[1], T, V[0], theta ? V[0] : V[1], R);
+  __syncthreads();
+  const double cp = theta ? cpl[z] : 1.0;
   fix_plane_nodes<N>(T, [&](int i, int j) {
     const int gx = T.x0 + i, gy = T.y0 + j;
     const long long I = off + gx + (long long)nx * gy;
-    double dx, dy = 0.0;
-    if (E != kFixNonfinite) {
-      const long long rx = fix_plane_node<N, 0>(T, RA[0], RB[0], i, j), ry = fix_plane_node<N, 1>(T, RA[1], RB[1], j, i);
-      if (!theta) {
-        out[I] = (double)(rx + ry) * unit;
-        return;
-      }
-      dx = (double)rx * unit;
-      dy = (double)ry * unit;
-    } else {
-      dx = cp * line_sum<N>(P, 0, fx, (long long)nx * gy, 1, gx);
-      dy = cp * line_sum<N>(P, 1, fy, gx, nx, gy);
-      if (!theta) {
-        out[I] = dx + dy;
-        return;
-      }
+    const FixSum rx = fix_plane_x<N>(R, i, j), ry = fix_plane_y<N>(T, R, i, j);
+    double dx, dy;
+    if (!theta) {   // A as one sum: the two parts nearly cancel in a vortex
+      const FixSum r = fix_add(rx, ry);
+      out[I] = r.u < kFixBad ? fix_double(r)
+                             : line_sum<N>(P, 0, fx, (long long)nx * gy, 1, gx) + line_sum<N>(P, 1, fy, gx, nx, gy);
+      return;
     }
+    dx = cp * (rx.u < kFixBad ? fix_double(rx) : line_sum<N>(P, 0, fx, (long long)nx * gy, 1, gx));
+    dy = cp * (ry.u < kFixBad ? fix_double(ry) : line_sum<N>(P, 1, fy, gx, nx, gy));
     if (!P.per[0] && (gx == 0 || gx == nx - 1)) dx = 0.0;
     if (!P.per[1] && (gy == 0 || gy == ny - 1)) dy = 0.0;
     if (PLAIN) {
@@ -394,10 +366,10 @@ void launch_linear_n(xg_ctx* c, const Imex& X, const double* v, double c0, doubl
   const int chunk = xg::fix_z_chunk(P.nseg[2], nxy, c->sms);
   const dim3 gz((unsigned)((nxy + 127) / 128), (P.nseg[2] + chunk - 1) / chunk);
   if (c0 == 0.0 && c1 == 1.0) {
-    xg::launch_stage_kernel(xg::k_lin_plane<N, true>, gp, xg::kFixThreads, 0, st, X.lin, v, X.cpl, c0, c1, out);
+    xg::launch_stage_kernel(xg::k_lin_plane<N, true>, gp, xg::fix_plane_threads(N), 0, st, X.lin, v, X.cpl, c0, c1, out);
     xg::launch_stage_kernel(xg::k_lin_z<N, true>, gz, 128, 0, st, X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
   } else {
-    xg::launch_stage_kernel(xg::k_lin_plane<N, false>, gp, xg::kFixThreads, 0, st, X.lin, v, X.cpl, c0, c1, out);
+    xg::launch_stage_kernel(xg::k_lin_plane<N, false>, gp, xg::fix_plane_threads(N), 0, st, X.lin, v, X.cpl, c0, c1, out);
     xg::launch_stage_kernel(xg::k_lin_z<N, false>, gz, 128, 0, st, X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
   }
 }

@@ -9,16 +9,17 @@
 // those.  The kernel writes T (the x + y part) and W (w, p', theta), which the
 // z pass reads; v and the x part never leave the chip.
 //
-// Fixed point needs an exponent.  Every (x tile, y segment) has its own, per
-// group of fluxes that are summed together (rho' with Theta' apart, the two
-// horizontal momenta, the vertical one): the maximum over the segment's N + 1
-// lines, so it does not depend on which segments share a CTA, and a domain cut
-// into y-slabs gets the same bits as the whole.  x and y rows of a node are
-// then integers of one scale and are added exactly; a shared y face adds the
-// row N of the segment before it in the format of T (t0 + row N, the order in
-// which a partition face is completed).  The Theta' flux theta (rho u_d) is
-// formed as an integer product of 62 bits, so only theta's own rounding is in
-// it; the difference form of the FP64 chains is not needed.
+// Every element segment of a line has an exponent of its own, so its rows carry
+// the bits of its own values whatever the tile holds elsewhere, and no result
+// depends on the tiles: a domain cut into y-slabs gets the same bits as the
+// whole.  x and y rows of a node are integers, added in the larger one's unit
+// (fix_add); a shared y face adds the row N of the segment before it in the
+// format of T (t0 + row N, the order in which a partition face is completed).
+// The Theta' flux theta (rho u_d) is formed as an integer product of 62 bits, so
+// only theta's own rounding is in it; the difference form of the FP64 chains is
+// not needed.  (One exponent for an x tile and y segment, found by a reduction
+// over the block, took the same time, 0.413 against 0.404 ms for 4.3 M nodes, but
+// left values below 2^-8 of the tile's largest fewer bits than FP64 has.)
 //
 // XG_FP64, a stage on the 128 x 128 x 16 order-4 box (17.0 M nodes): three line
 // kernels with FP64 chains 1.87 + 1.44 + 2.02 ms; tiles 1.61 + 1.38 ms (FP64
@@ -57,22 +58,24 @@ __host__ __device__ constexpr int z_tile_segments(int N) { return N >= 8 ? 1 : 8
 __host__ __device__ constexpr int z_tile_threads(int N) { return kTileCols * (z_tile_segments(N) * N + 1); }
 __host__ __device__ constexpr int z_tile_min_blocks(int N) { return 1152 / z_tile_threads(N); }
 
-// Element rows of a tile: about 8 nodes, so that the N + 1 columns before and
-// after a tile and its closing line are a quarter of its nodes.
+// Elements of a tile along x, whose segments and the one before them share a
+// warp; element rows: about 8 nodes, so that the N + 1 columns before and after a
+// tile and its closing line are a quarter of its nodes.
+__host__ __device__ constexpr int xy_elems_x(int N) { return fix_plane_elems(N); }
 __host__ __device__ constexpr int xy_elems_y(int N) { return N == 1 ? 9 : (N == 3 ? 3 : (N >= 5 ? 1 : 8 / N)); }
 
 template <int N>
 struct XYTile {
-  static constexpr int EX = 32 / N, EY = xy_elems_y(N);
+  static constexpr int EX = xy_elems_x(N), EY = xy_elems_y(N);
   static constexpr int TX = EX * N, TY = EY * N;
   static constexpr int CX = TX == 32 ? N + 1 : N;       // columns beside the 32 that a warp's lanes take
   static constexpr int PX = (N + TX + 1) | 1;           // V: columns -N .. TX
-  static constexpr int PR = TX | 1;                     // x rows
   static constexpr int LY = TY + 1, LX = TX + 1;
-  static constexpr int V = EY * (N + 1) * PX;           // one flux
-  static constexpr int RX = LY * PR, RNX = LY * (EX + 1);
+  static constexpr int PR = LX | 1;                     // x rows, a wall's last node included
+  static constexpr int V = LY * PX;                     // one value
+  static constexpr int RX = LY * PR, UX = LY * (2 * EX + 1);
   static constexpr int RY = TY * LX, RNY = EY * LX;
-  static constexpr size_t bytes = 8 * (size_t)(9 * V + 5 * (RX + RNX + RY + RNY));
+  static constexpr size_t bytes = 8 * (size_t)(8 * V + 5 * (RX + RY + RNY)) + 4 * 5 * (size_t)(UX + RNY);
   static constexpr int side_warps(int ey) { return ((ey * N + 1) * CX + 31) / 32; }
   static constexpr int threads(int ey) { return 32 * (ey * N + 1 + side_warps(ey)); }
 };
@@ -172,13 +175,12 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
   using M = typename XYTypes<Params>::M;
   constexpr bool MIXED = XYTypes<Params>::mixed;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fix2* V = reinterpret_cast<fix2*>(smem_raw);
-  long long* RX = reinterpret_cast<long long*>(V + 9 * L::V);
-  long long* RNX = RX + 5 * L::RX;
-  long long* RY = RNX + 5 * L::RNX;
+  double* V = reinterpret_cast<double*>(smem_raw);    // rho u, rho v, theta, then the momentum's fluxes
+  long long* RX = reinterpret_cast<long long*>(V + 8 * L::V);
+  long long* RY = RX + 5 * L::RX;
   long long* RNY = RY + 5 * L::RY;
-  __shared__ int Es[4][L::EY];
-  __shared__ int nonfinite;
+  int* UX = reinterpret_cast<int*>(RNY + 5 * L::RNY);   // units of the x rows and the y segments
+  int* UY = UX + 5 * L::UX;
 
   const LineParams& G = XYTypes<Params>::line(P);
   const int nx = G.n[0], ny = G.n[1];
@@ -197,10 +199,7 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
   const int warps = blockDim.x >> 5;
   const int lines = ey * N + 1;                            // warps that take a line each
 
-  if (threadIdx.x < 4 * L::EY) (&Es[0][0])[threadIdx.x] = 0;
-  if (threadIdx.x == 0) nonfinite = 0;
   stage_kernel_begin();
-  __syncthreads();
 
   // this thread's node (i, j) of the tile: a warp takes a line, the warps
   // after them the N columns before the tile and its 33rd
@@ -220,155 +219,101 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
   const int sj = j < fy ? j / N : eky - 1, aj = j - sj * N;
   const bool closes = aj == 0 && sj > 0 && inside;
 
-  // exponents: of rho u and rho v, of theta's products with them, and (FP64
-  // form) of the horizontal momenta's fluxes and the vertical one's
-  constexpr int kE = MIXED ? 2 : 4;
-  XYFlux<M> f;
-  int e[kE];
-#pragma unroll
-  for (int k = 0; k < kE; ++k) e[k] = 0;
   if (need) {
+    XYFlux<M> f;
     int gx = x0 + i, gy = y0 + j;
     if (gx < 0) gx += nx;
     if (gx >= nx) gx -= nx;
     if (gy >= ny) gy -= ny;
     xy_point(P, B, gx + (long long)nx * (gy + (long long)ny * z), z, i >= 0 && i < ox && j < oy, f);
-    bool bad = false;
-    const int eu = fix_exp_finite(f.mu, bad), ev = fix_exp_finite(f.mv, bad), et = fix_exp_finite(f.th, bad);
-    e[0] = max(eu, ev);
-    e[1] = max(fix_prod_top(f.mu, eu, f.th, et), fix_prod_top(f.mv, ev, f.th, et));
-    if constexpr (!MIXED) {
-      e[2] = max(max(fix_exp_finite(f.xx, bad), fix_exp_finite(f.xy, bad)), fix_exp_finite(f.yy, bad));
-      e[3] = max(fix_exp_finite(f.xz, bad), fix_exp_finite(f.yz, bad));
-    }
-    if (bad) nonfinite = 1;
-  }
-  if (warp < lines) {
-    // a line that closes segment sj - 1 counts for it by its `inside` columns
-    // alone; only the closing column of an inner tile can be among the lanes
-    // without being inside
-    const bool two = aj == 0 && sj > 0 && j <= fy, differ = two && ox <= 31;
-#pragma unroll
-    for (int k = 0; k < kE; ++k) {
-      const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)e[k]);
-      const int mc = differ ? (int)__reduce_max_sync(0xffffffffu, inside ? (unsigned)e[k] : 0u) : m;
-      if (lane == k && j <= fy) {
-        atomicMax(&Es[k][sj], m);
-        if (two) atomicMax(&Es[k][sj - 1], mc);
-      }
-    }
-  } else {
-    for (int s = 0; s < eky; ++s) {
-      const bool in = need && (s == sj || (closes && s == sj - 1));
-#pragma unroll
-      for (int k = 0; k < kE; ++k) {
-        const int m = (int)__reduce_max_sync(0xffffffffu, in ? (unsigned)e[k] : 0u);
-        if (lane == k) atomicMax(&Es[k][s], m);
-      }
-    }
-  }
-  __syncthreads();
-
-  const int sc = P.F[0].sc;
-  if (need) {
-    auto put = [&](int s, int a) {
-      fix2* v = V + (s * (N + 1) + a) * L::PX + i + N;
-      const int E0 = fix_block_exp(Es[0][s], sc), E4 = fix_prod_exp<N>(Es[1][s], sc);
-      v[0] = fix_of<N>(f.mu, E0);
-      v[L::V] = fix_of<N>(f.mv, E0);
-      v[2 * L::V] = fix_prod<N>(f.th, f.mu, E4);
-      v[3 * L::V] = fix_prod<N>(f.th, f.mv, E4);
-      if constexpr (MIXED) {
-        df* p = reinterpret_cast<df*>(v);
-        p[4 * L::V] = f.xx;
-        p[5 * L::V] = f.xy;
-        p[6 * L::V] = f.xz;
-        p[7 * L::V] = f.yy;
-        p[8 * L::V] = f.yz;
-      } else {
-        const int E1 = fix_block_exp(Es[2][s], sc), E3 = fix_block_exp(Es[3][s], sc);
-        v[4 * L::V] = fix_of<N>(f.xx, E1);
-        v[5 * L::V] = fix_of<N>(f.xy, E1);
-        v[6 * L::V] = fix_of<N>(f.xz, E3);
-        v[7 * L::V] = fix_of<N>(f.yy, E1);
-        v[8 * L::V] = fix_of<N>(f.yz, E3);
-      }
-      if (nonfinite) {
-        const fix2 mark = {kFixMark, 0};
-        const bool bth = fix_bad(f.th);
-        if (fix_bad(f.mu)) v[0] = mark;
-        if (fix_bad(f.mv)) v[L::V] = mark;
-        if (fix_bad(f.mu) || bth) v[2 * L::V] = mark;
-        if (fix_bad(f.mv) || bth) v[3 * L::V] = mark;
-        if constexpr (!MIXED) {
-          if (fix_bad(f.xx)) v[4 * L::V] = mark;
-          if (fix_bad(f.xy)) v[5 * L::V] = mark;
-          if (fix_bad(f.xz)) v[6 * L::V] = mark;
-          if (fix_bad(f.yy)) v[7 * L::V] = mark;
-          if (fix_bad(f.yz)) v[8 * L::V] = mark;
-        }
-      }
-    };
-    put(sj, aj);
-    if (closes) put(sj - 1, N);
+    double* v = V + j * L::PX + i + N;
+    v[0] = f.mu;
+    v[L::V] = f.mv;
+    v[2 * L::V] = f.th;
+    M* p = reinterpret_cast<M*>(v);
+    p[3 * L::V] = f.xx;
+    p[4 * L::V] = f.xy;
+    p[5 * L::V] = f.xz;
+    p[6 * L::V] = f.yy;
+    p[7 * L::V] = f.yz;
   }
   __syncthreads();
 
   // one thread per segment, variable and direction; a warp's tasks are of one
-  // kind.  fluxes of variable c along x: mu, xx, xy, xz, theta mu; along y:
-  // mv, xy, yy, yz, theta mv
-  constexpr unsigned kFx = 0x26540u, kFy = 0x38751u;
-  // row A .. B - 1 of the segment at p (stride sp) in direction D to r (stride
-  // sr), row N to rn; mixed momentum in double-float, the rest in fixed point
-  auto rows = [&](auto dir, int c, const fix2* p, int sp, long long* r, int sr, long long* rn, bool all) {
-    constexpr int D = decltype(dir)::value;
-    if (MIXED && c != 0 && c != 4) {
-      if constexpr (MIXED) {
-        df v[N + 1];
+  // kind.  Values of variable c along x: rho u, xx, xy, xz, rho u (and theta);
+  // along y: rho v, xy, yy, yz, rho v.  Mixed momentum in double-float, the rest
+  // in fixed point.
+  constexpr unsigned kFx = 0x05430u, kFy = 0x17641u;
+  auto limbs = [&](int c, const double* p, int at, int sp, int sc, fix2 (&v)[N + 1]) -> int {
+    if (c == 4) return fix_products<N>(p, V + 2 * L::V + at, sp, sc, v);
+    double a[N + 1];
 #pragma unroll
-        for (int l = 0; l <= N; ++l) v[l] = reinterpret_cast<const df*>(p)[l * sp];
-        if (all) {
+    for (int l = 0; l <= N; ++l) a[l] = p[l * sp];
+    return fix_values<N>(a, sc, v);
+  };
+  constexpr int kLines = 32 / (L::EX + 1);                // x: the segment before the tile and its own EX
+  const int cy = ox > L::TX ? L::LX : L::TX;              // columns of the y tasks
+  const int wx = (oyx + kLines - 1) / kLines, wy = (eky * cy + 31) / 32;
+  for (int w = warp; w < 5 * (wx + wy); w += warps) {
+    if (w < 5 * wx) {
+      const int c = w / wx, line = lane / (L::EX + 1), s = lane - line * (L::EX + 1) - 1;
+      const int o = (w - c * wx) * kLines + line;
+      const bool act = line < kLines && o < oyx && s < ekx && (s >= 0 || hxl), own = act && s >= 0;
+      const bool left = s > 0 || hxl, end = endx && s == ekx - 1;
+      const int at = o * L::PX + (s + 1) * N;
+      const double* p = V + ((kFx >> (4 * c)) & 15u) * L::V + at;
+      long long* r = RX + c * L::RX + o * L::PR + s * N;
+      if (MIXED && c != 0 && c != 4) {
+        if constexpr (MIXED) {
+          df v[N + 1], last = {0.0f, 0.0f}, before;
+          if (act) {
 #pragma unroll
-          for (int a = 0; a < N; ++a) reinterpret_cast<df*>(r)[a * sr] = df_row<N, D>(P.D, a, v);
+            for (int l = 0; l <= N; ++l) v[l] = reinterpret_cast<const df*>(p)[l];
+            last = df_row<N, 0>(P.D, N, v);
+          }
+          before.h = __shfl_up_sync(0xffffffffu, last.h, 1);
+          before.l = __shfl_up_sync(0xffffffffu, last.l, 1);
+          if (own) {
+            df* q = reinterpret_cast<df*>(r);
+            const df first = df_row<N, 0>(P.D, 0, v);
+            q[0] = left ? df_add(first, before) : df_scale2(first, 2.0f);
+#pragma unroll
+            for (int a = 1; a < N; ++a) q[a] = df_row<N, 0>(P.D, a, v);
+            if (end) q[N] = df_scale2(last, 2.0f);
+          }
         }
-        *reinterpret_cast<df*>(rn) = df_row<N, D>(P.D, N, v);
+      } else {
+        fix2 v[N + 1];
+        int u = 0;
+        if (act) u = limbs(c, p, at, 1, P.F[0].sc, v);
+        int* ur = UX + c * L::UX + o * (2 * L::EX + 1) + 2 * s;
+        fix_x_rows<N>(P.F[0], v, u, act, own, left, end, [&](int a, FixSum x) {
+          r[a] = x.r;
+          if (a < 2 || a == N) ur[a == N ? 2 : a] = x.u;
+        });
       }
     } else {
-      fix2 v[N + 1];
-#pragma unroll
-      for (int l = 0; l <= N; ++l) v[l] = p[l * sp];
-      if (all) {
-#pragma unroll
-        for (int a = 0; a < N; ++a) r[a * sr] = fix_row<N>(P.F[D], a, v);
-      }
-      *rn = fix_row<N>(P.F[D], N, v);
-    }
-  };
-  const int cy = ox > L::TX ? L::LX : L::TX;              // columns of the y tasks
-  const int wx = (oyx * L::EX + 31) / 32, wy = (eky * cy + 31) / 32;
-  const int wl = hxl ? (oyx + 31) / 32 : 0;
-  for (int w = warp; w < 5 * (wx + wy + wl); w += warps) {
-    if (w < 5 * wx) {
-      const int c = w / wx, t = (w - c * wx) * 32 + lane;
-      const int o = t / L::EX, s = t - o * L::EX;
-      if (o < oyx && s < ekx) {
-        const int so = o < fy ? o / N : eky - 1;
-        rows(std::integral_constant<int, 0>(), c,
-             V + ((kFx >> (4 * c)) & 15u) * L::V + (so * (N + 1) + o - so * N) * L::PX + N + s * N, 1,
-             RX + c * L::RX + o * L::PR + s * N, 1, RNX + c * L::RNX + o * (L::EX + 1) + s + 1, true);
-      }
-    } else if (w < 5 * (wx + wy)) {
       const int c = (w - 5 * wx) / wy, t = (w - 5 * wx - c * wy) * 32 + lane;
       const int s = ox > L::TX ? t / L::LX : t / L::TX, k = t - s * cy;
-      if (s < eky && k < ox)
-        rows(std::integral_constant<int, 1>(), c, V + ((kFy >> (4 * c)) & 15u) * L::V + s * (N + 1) * L::PX + N + k,
-             L::PX, RY + c * L::RY + s * N * L::LX + k, L::LX, RNY + c * L::RNY + s * L::LX + k, true);
-    } else {   // row N of the x segment before the tile
-      const int c = (w - 5 * (wx + wy)) / wl, o = (w - 5 * (wx + wy) - c * wl) * 32 + lane;
-      if (o < oyx) {
-        const int so = o < fy ? o / N : eky - 1;
-        rows(std::integral_constant<int, 0>(), c, V + ((kFx >> (4 * c)) & 15u) * L::V + (so * (N + 1) + o - so * N) * L::PX,
-             1, nullptr, 1, RNX + c * L::RNX + o * (L::EX + 1), false);
+      if (s >= eky || k >= ox) continue;
+      const int at = s * N * L::PX + N + k;
+      const double* p = V + ((kFy >> (4 * c)) & 15u) * L::V + at;
+      long long *r = RY + c * L::RY + s * N * L::LX + k, *rn = RNY + c * L::RNY + s * L::LX + k;
+      if (MIXED && c != 0 && c != 4) {
+        if constexpr (MIXED) {
+          df v[N + 1];
+#pragma unroll
+          for (int l = 0; l <= N; ++l) v[l] = reinterpret_cast<const df*>(p)[l * L::PX];
+#pragma unroll
+          for (int a = 0; a < N; ++a) reinterpret_cast<df*>(r)[a * L::LX] = df_row<N, 1>(P.D, a, v);
+          *reinterpret_cast<df*>(rn) = df_row<N, 1>(P.D, N, v);
+        }
+      } else {
+        fix2 v[N + 1];
+        UY[c * L::RNY + s * L::LX + k] = limbs(c, p, at, L::PX, P.F[1].sc, v);
+#pragma unroll
+        for (int a = 0; a < N; ++a) r[a * L::LX] = fix_row<N>(P.F[1], a, v);
+        *rn = fix_row<N>(P.F[1], N, v);
       }
     }
   }
@@ -391,53 +336,28 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
       fat = ((long long)next * G.n[2] + z) * nx + x0 + i;
     }
   }
-  const int si = i / N;
   const bool wraps = j == 0 && hyl && gridDim.y == 1;     // one tile around: its own closing row
   const int sl = wraps ? eky - 1 : sj - 1;                // the y segment that ends at this line
   const long long I = x0 + i + (long long)nx * (y0 + j + (long long)ny * z);
-  auto marked = [&](const fix2* p, int stride) {
-    bool m = false;
-    for (int l = 0; l <= N; ++l) m |= p[l * stride].h == kFixMark;
-    return m;
-  };
   // a variable in fixed point
   auto node = [&](int c) {
-    const fix2* vy = V + ((kFy >> (4 * c)) & 15u) * L::V + N + i;
-    const int k = c == 0 ? 0 : (c == 4 ? 1 : (c == 3 ? 3 : 2));
-    auto field = [&](int s) {
-      return c == 4 ? fix_prod_field<N>(fix_prod_exp<N>(Es[k][s], sc), sc) : fix_field<N>(fix_block_exp(Es[k][s], sc), sc);
+    auto end_row = [&](int s) -> FixSum {
+      return {RNY[c * L::RNY + s * L::LX + i], UY[c * L::RNY + s * L::LX + i]};
     };
     if (closing) {
-      double r = fix_out<MIXED>(RNY[c * L::RNY + (eky - 1) * L::LX + i], field(eky - 1));
-      if (nonfinite && marked(vy + (eky - 1) * (N + 1) * L::PX, L::PX)) r = xg_nan(0.0);
-      faces[c * fstride + fat] = r;
+      faces[c * fstride + fat] = fix_sum_out<MIXED>(end_row(eky - 1));
       return;
     }
-    long long r;
-    const long long* rn = RNX + c * L::RNX + j * (L::EX + 1);
-    if (i == fx) {
-      r = 2 * rn[ekx];                                    // a wall's last node: its row twice
-    } else {
-      r = RX[c * L::RX + j * L::PR + i];
-      if (i == si * N) r += (si > 0 || hxl) ? rn[si] : r;
-    }
+    const FixSum rx = {RX[c * L::RX + j * L::PR + i], UX[c * L::UX + j * (2 * L::EX + 1) + fix_unit_slot<N>(i)]};
+    FixSum ry;
     if (j == fy) {
-      r += 2 * RNY[c * L::RNY + (eky - 1) * L::LX + i];
+      ry = fix_twice(end_row(eky - 1));                   // a wall's last node: its row twice
     } else {
-      const long long t = RY[c * L::RY + j * L::LX + i];
-      r += t;
-      if (j == 0 && !hyl && !open_lo) r += t;
+      ry = {RY[c * L::RY + j * L::LX + i], UY[c * L::RNY + sj * L::LX + i]};
+      if (j == 0 && !hyl && !open_lo) ry = fix_twice(ry);
     }
-    double v = fix_out<MIXED>(r, field(sj));
-    if (closes || wraps) v = v + fix_out<MIXED>(RNY[c * L::RNY + sl * L::LX + i], field(sl));
-    if (nonfinite) {
-      const fix2* vx = V + ((kFx >> (4 * c)) & 15u) * L::V + (sj * (N + 1) + aj) * L::PX + N;
-      bool m = marked(vy + sj * (N + 1) * L::PX, L::PX);
-      if (closes || wraps) m |= marked(vy + sl * (N + 1) * L::PX, L::PX);
-      if (i < fx) m |= marked(vx + si * N, 1);
-      if (i == si * N && (si > 0 || hxl)) m |= marked(vx + (si - 1) * N, 1);
-      if (m) v = xg_nan(0.0);
-    }
+    double v = fix_sum_out<MIXED>(fix_add(rx, ry));
+    if (closes || wraps) v = v + fix_sum_out<MIXED>(end_row(sl));
     B.T[c * np + I] = v;
   };
   node(0);
@@ -448,7 +368,6 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
     node(3);
   } else {
     const df* RXm = reinterpret_cast<const df*>(RX);
-    const df* RNXm = reinterpret_cast<const df*>(RNX);
     const df* RYm = reinterpret_cast<const df*>(RY);
     const df* RNYm = reinterpret_cast<const df*>(RNY);
 #pragma unroll
@@ -457,14 +376,7 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
         reinterpret_cast<df*>(faces)[c * fstride + fat] = RNYm[c * L::RNY + (eky - 1) * L::LX + i];
         continue;
       }
-      df r;
-      const df* rn = RNXm + c * L::RNX + j * (L::EX + 1);
-      if (i == fx) {
-        r = df_scale2(rn[ekx], 2.0f);
-      } else {
-        r = RXm[c * L::RX + j * L::PR + i];
-        if (i == si * N) r = (si > 0 || hxl) ? df_add(r, rn[si]) : df_scale2(r, 2.0f);
-      }
+      df r = RXm[c * L::RX + j * L::PR + i];
       if (j == fy) {
         r = df_add(r, df_scale2(RNYm[c * L::RNY + (eky - 1) * L::LX + i], 2.0f));
       } else {
@@ -627,7 +539,7 @@ __global__ void __launch_bounds__(z_tile_threads(N), z_tile_min_blocks(N))
 // Element rows of the x-y tiles of a mesh: the most, EY, unless fewer give the
 // chip blocks that it would lack.
 inline int xy_tile_rows(int N, const int (&nseg)[3], int levels, int sms) {
-  const int most = xy_elems_y(N), ex = 32 / N;
+  const int most = xy_elems_y(N), ex = xy_elems_x(N);
   const long long columns = (long long)((nseg[0] + ex - 1) / ex) * levels;
   int ey = most;
   while (ey > 1 && columns * ((nseg[1] + ey - 1) / ey) < 3ll * sms) --ey;
