@@ -34,7 +34,7 @@ struct LapParams {
   int n[3], nseg[3], per[3];
   long long np;
   double Km[3][kMaxOrder + 1][kMaxOrder + 1];
-  FixRows Kf[3];   // Km in fixed point; x and y share their scale
+  FixRows Kf[3];   // Km in fixed point
 };
 
 template <int N>
@@ -536,23 +536,20 @@ xg_status xg_set_dynamics(xg_ctx* c, const xg_dynamics* dyn) {
   long double D[xg::kMaxOrder + 1][xg::kMaxOrder + 1], w[xg::kMaxOrder + 1];
   xg::lgl_derivative(N, D);
   xg::lgl_weights(N, w);
-  xg::FixMatrix Kl[3];
-  double most[3];
   for (int d = 0; d < 3; ++d) {
+    xg::FixMatrix Kl;
     const long double s = -(long double)nu[d] * (2.0L / h[d]) * (2.0L / h[d]);
     for (int a = 0; a <= N; ++a) {
       const long double wa = (a == 0 || a == N) ? 2.0L * w[0] : w[a];
       for (int l = 0; l <= N; ++l) {
         long double K = 0.0L;
         for (int k = 0; k <= N; ++k) K += w[k] * D[k][a] * D[k][l];
-        Kl[d][a][l] = s * K / wa;
-        P->Km[d][a][l] = (double)Kl[d][a][l];
+        Kl[a][l] = s * K / wa;
+        P->Km[d][a][l] = (double)Kl[a][l];
       }
     }
-    most[d] = xg::fix_row_sum(N, Kl[d]);
+    xg::fix_rows(N, Kl, &P->Kf[d]);
   }
-  for (int d = 0; d < 3; ++d)   // x and y sums are added as integers: one scale
-    xg::fix_rows(N, Kl[d], xg::fix_scale_of(d < 2 ? std::max(most[0], most[1]) : most[2]), &P->Kf[d]);
   cudaError_t e = cudaSuccess;
   const size_t vec = sizeof(double) * 5 * (size_t)c->np;
   if (!c->dyn_L1) e = cudaMalloc((void**)&c->dyn_L1, vec);

@@ -59,16 +59,14 @@ inline double fix_row_sum(int N, const FixMatrix& c) {
   return std::fmax(most, face);
 }
 
-// sc for matrices whose largest row sum is `most` (directions that are summed
-// as integers share it); ldexp of zero rows is harmless.
-inline int fix_scale_of(double most) {
+// c in fixed point, on a scale of its own: sums of rows of two matrices are taken
+// in the larger one's unit (fix_add), and a direction of wide spacing, whose
+// matrix is small, keeps its bits beside one of narrow spacing.
+inline void fix_rows(int N, const FixMatrix& c, FixRows* F) {
+  const double most = fix_row_sum(N, c);
   int e = 0;
   if (most > 0.0 && std::isfinite(most)) std::frexp(most, &e);
-  return 60 - e;
-}
-
-inline void fix_rows(int N, const FixMatrix& c, int sc, FixRows* F) {
-  F->sc = sc;
+  const int sc = F->sc = 60 - e;
   for (int a = 0; a <= kMaxOrder; ++a)
     for (int l = 0; l <= kMaxOrder; ++l) F->ch[a][l] = F->cl[a][l] = 0;
   for (int a = 0; a <= N; ++a) {

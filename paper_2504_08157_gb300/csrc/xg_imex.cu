@@ -669,19 +669,7 @@ cudaError_t prepare(xg_ctx* c, int m, cudaStream_t st) {
     X->m = m;
     X->n = n;
     X->lin.P = c->P;
-    const int N = c->d.order;
-    long double D[xg::kMaxOrder + 1][xg::kMaxOrder + 1];
-    xg::FixMatrix Dl[3];
-    double most[3];
-    xg::lgl_derivative(N, D);
-    for (int d = 0; d < 3; ++d) {   // -(2/h) D, rows 0 and N halved
-      const long double h = ((long double)c->d.hi[d] - c->d.lo[d]) / c->d.nel[d];
-      for (int a = 0; a <= N; ++a)
-        for (int l = 0; l <= N; ++l) Dl[d][a][l] = -(2.0L / h) * (a == 0 || a == N ? 0.5L : 1.0L) * D[a][l];
-      most[d] = xg::fix_row_sum(N, Dl[d]);
-    }
-    for (int d = 0; d < 3; ++d)     // x and y sums are added as integers: one scale
-      xg::fix_rows(N, Dl[d], xg::fix_scale_of(d < 2 ? std::max(most[0], most[1]) : most[2]), &X->lin.D[d]);
+    xg::fill_fix_params(&c->d, X->lin.D);
     X->hpart.resize((size_t)xg::kDotBlocksMax * 5 * xg::kDotBatch);
     int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->dev);

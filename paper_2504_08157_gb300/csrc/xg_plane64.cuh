@@ -39,8 +39,7 @@
 
 namespace xg {
 
-// FP64 launch constants with the fixed-point matrices of the three directions
-// (x and y share their scale).
+// FP64 launch constants with the fixed-point matrices of the three directions.
 struct F64Params {
   LineParams P64;
   FixRows F[3];

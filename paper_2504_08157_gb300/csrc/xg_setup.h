@@ -177,16 +177,13 @@ inline void fill_fix_params(const xg_mesh_desc* d, FixRows (&F)[3]) {
   const int N = d->order;
   long double D[kMaxOrder + 1][kMaxOrder + 1];
   lgl_derivative(N, D);
-  FixMatrix M[3];
+  FixMatrix M;
   for (int k = 0; k < 3; ++k) {
     const long double h = ((long double)d->hi[k] - d->lo[k]) / d->nel[k];
     for (int a = 0; a <= N; ++a)
-      for (int l = 0; l <= N; ++l) M[k][a][l] = -(2.0L / h) * ((a == 0 || a == N) ? 0.5L : 1.0L) * D[a][l];
+      for (int l = 0; l <= N; ++l) M[a][l] = -(2.0L / h) * ((a == 0 || a == N) ? 0.5L : 1.0L) * D[a][l];
+    fix_rows(N, M, &F[k]);
   }
-  const int sxy = fix_scale_of(std::fmax(fix_row_sum(N, M[0]), fix_row_sum(N, M[1])));
-  fix_rows(N, M[0], sxy, &F[0]);
-  fix_rows(N, M[1], sxy, &F[1]);
-  fix_rows(N, M[2], fix_scale_of(fix_row_sum(N, M[2])), &F[2]);
 }
 
 // A double split into a double-float pair (host).

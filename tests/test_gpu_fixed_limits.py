@@ -50,10 +50,12 @@ TOL = 16 * 2.0 ** -53
 
 
 class Lines:
-    """Assembled 1-D operators of a box in extended precision."""
+    """Assembled 1-D operators of a box in extended precision.  Along the
+    direction ``uniform`` the box's fields do not vary, and nothing is allowed
+    for it."""
 
-    def __init__(self, wl):
-        self.wl, self.N = wl, wl["N"]
+    def __init__(self, wl, uniform=None):
+        self.wl, self.N, self.uniform = wl, wl["N"], uniform
         self.n = [wl["N"] * e + (0 if p else 1) for e, p in zip(wl["nel"], wl["periodic"])]
         x = lgl.lgl_points_extended(self.N)
         self.D, self.w = lgl.derivative_matrix(x), lgl.lgl_weights(self.N, x)
@@ -67,6 +69,8 @@ class Lines:
 
     def rows(self, M, f, d):
         """(sum of the node's rows of M along d, R max |f| over its segments)."""
+        if d == self.uniform:
+            return np.zeros_like(f), np.zeros_like(f)
         f = np.moveaxis(f, 2 - d, -1)
         N, nel, per = self.N, self.wl["nel"][d], self.wl["periodic"][d]
         out, top = np.zeros_like(f), np.zeros_like(f)
@@ -139,11 +143,11 @@ def _beyond(got, ref, top):
     return float((np.abs(got - ref) / (TOL * top + np.longdouble(1e-300))).max())
 
 
-def _check(wl, device):
+def _check(wl, device, uniform=None):
     """Tendency, linear operator and hyper-diffusion of wl's state, node by
     node; the mixed form's rho' and Theta' too."""
     import torch
-    ref, (_, phys, _) = Lines(wl), oracle_of(wl)
+    ref, (_, phys, _) = Lines(wl, uniform), oracle_of(wl)
     L, top = ref.rhs(wl["q"], phys)
     worst = {}
     for prec, vs in ((0, range(5)), (2, (0, 4))):
@@ -184,3 +188,24 @@ def test_quiet_nodes_keep_their_digits(cuda_device, N, per, fall):
     k = np.arange(wl["q"].shape[1])
     wl["q"] = wl["q"] * s[k % n[0] if fall == 0 else k // n[0] % n[1]]
     _check(wl, cuda_device)
+
+
+@pytest.mark.parametrize("uniform", [True, False])
+@pytest.mark.parametrize("narrow,ratio", [(0, 1e3), (1, 1e3), (0, 1e5), (1, 1e5), (2, 1e5)])
+@pytest.mark.parametrize("N", [2, 4, 5, 7])
+def test_spacings_of_different_size(cuda_device, N, narrow, ratio, uniform):
+    """One direction's spacing 1e3 and 1e5 times smaller than the others': the
+    wide directions' derivatives keep FP64's precision, which shows where the
+    state does not vary along the narrow one."""
+    nel, h = (4, 3, 2), [2000.0, 2000.0, 2000.0]
+    h[narrow] /= ratio
+    per = (True, True, False)
+    wl = W.box(nel, N, (0.0, 0.0, 0.0), tuple(n * d for n, d in zip(nel, h)), per, f=1.0e-4, seed=19)
+    wl["S_theta"] = None
+    if uniform:
+        if narrow == 2:
+            pytest.skip("the reference state varies along z")
+        n = [N * e + (0 if p else 1) for e, p in zip(nel, per)]
+        q = wl["q"].reshape([5] + n[::-1])
+        wl["q"] = np.ascontiguousarray(np.broadcast_to(q.take([1], axis=3 - narrow), q.shape)).reshape(5, -1)
+    _check(wl, cuda_device, narrow if uniform else None)
