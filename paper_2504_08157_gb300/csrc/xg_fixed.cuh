@@ -536,7 +536,77 @@ __device__ __forceinline__ void fix_plane_nodes(const FixTile& T, F node) {
   if (T.ox > L::TS && (int)threadIdx.x < T.oy) node(L::TS, (int)threadIdx.x);
 }
 
+// ---------------------------------------------------------------- nodes
+// The assembled row of one node along one line, by one thread: the same segments,
+// units and sums as the tiles', bit for bit, at a conversion per value and node.
+// It serves levels that leave most of a tile empty.  R: the line's matrix in shared
+// memory (fix_stage_rows).
+template <int N>
+struct FixTable {
+  int2 c[N + 1][N + 1];
+  int sc;
+};
+
+template <int N>
+__device__ __forceinline__ void fix_stage_rows(const FixRows& F, FixTable<N>& R) {
+  for (int k = threadIdx.x; k < (N + 1) * (N + 1); k += blockDim.x) {
+    const int a = k / (N + 1), l = k - a * (N + 1);
+    R.c[a][l] = make_int2(F.ch[a][l], F.cl[a][l]);
+  }
+  if (threadIdx.x == 0) R.sc = F.sc;
+}
+
+template <int N>
+__device__ __forceinline__ FixSum fix_line_node(const FixTable<N>& R, const double* __restrict__ f, long long base,
+                                                long long sd, int g, int nd, int nseg, bool per) {
+  const int s = min(g / N, nseg - 1), a = g - s * N;
+  auto row = [&](int seg, int k) -> FixSum {
+    double x[N + 1];
+#pragma unroll
+    for (int l = 0; l <= N; ++l) {
+      const int at = seg * N + l;
+      x[l] = f[base + sd * (at >= nd ? at - nd : at)];
+    }
+    fix2 v[N + 1];
+    const int u = fix_values<N>(x, R.sc, v);
+    long long hi = 0, mid = 1ll << 29;
+#pragma unroll
+    for (int l = 0; l <= N; ++l) {
+      const int2 c = R.c[k][l];
+      hi += (long long)c.x * v[l].h;
+      mid += (long long)c.x * v[l].l;
+      mid += (long long)c.y * v[l].h;
+    }
+    return {hi + (mid >> 30), u};
+  };
+  const FixSum r = row(s, a);
+  if (a == N) return fix_twice(r);
+  if (a != 0) return r;
+  return s > 0 || per ? fix_add(r, row(s > 0 ? s - 1 : nseg - 1, N)) : fix_twice(r);
+}
+
+// Whether the tiles take the x and y sums of a level: where it fills an (N + 1)th
+// of them (order 1: nine tenths) and a third of their width, which a warp's lanes
+// are.  Two Laplacians over 1 M nodes, tiles against nodes: order 4, levels of 4 x 8
+// nodes 1.68 / 0.45 ms, 4 x 128 1.06 / 0.45, 8 x 32 0.58 / 0.45, 32 x 8 0.37 /
+// 0.45, 32 x 128 0.25 / 0.45.
+inline bool fix_plane_pays(int N, int nx, int ny, int nelx, int nely) {
+  const int E = fix_plane_elems(N);
+  const long long width = (long long)((nelx + E - 1) / E) * E * N, height = (long long)((nely + E - 1) / E) * E * N;
+  if (N == 1) return 10ll * nx * ny >= 9 * width * height;
+  return (long long)(N + 1) * nx * ny >= width * height && 3ll * nx >= width;
+}
+
 // ---------------------------------------------------------------- z lines
+// A block of a marching z pass takes 128 columns of one chunk, or all columns of
+// several chunks where there are few.
+constexpr int kFixZThreads = 128;
+inline int fix_z_columns(long long nxy) {
+  int c = kFixZThreads;
+  while (c > 1 && c / 2 >= nxy) c /= 2;
+  return c;
+}
+
 // One z segment's values (FP64, in registers) in limbs, with its own exponent.
 template <int N>
 __device__ __forceinline__ int fix_segment(const double (&v)[N + 1], int sc, fix2 (&f)[N + 1]) {

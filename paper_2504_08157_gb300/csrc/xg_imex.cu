@@ -62,6 +62,34 @@ __device__ __forceinline__ double line_sum(const LineParams& P, int d, const dou
   return a == 0 || a == N ? acc + acc : acc;
 }
 
+// The plane pass's result at node (gx, gy) of a level (its first node: off; fx and
+// fy the level's fields) from the x and y rows: A, or rho u and rho v.
+template <int N, bool PLAIN>
+__device__ __forceinline__ void lin_plane_node(const LineParams& P, const double* __restrict__ v, const double* fx,
+                                               const double* fy, bool theta, double cp, double c0, double c1,
+                                               long long off, int gx, int gy, FixSum rx, FixSum ry,
+                                               double* __restrict__ out) {
+  const int nx = P.n[0], ny = P.n[1];
+  const long long np = P.np, I = off + gx + (long long)nx * gy;
+  if (!theta) {   // A as one sum: the two parts nearly cancel in a vortex
+    const FixSum r = fix_add(rx, ry);
+    out[I] = r.u < kFixBad ? fix_double(r)
+                           : line_sum<N>(P, 0, fx, (long long)nx * gy, 1, gx) + line_sum<N>(P, 1, fy, gx, nx, gy);
+    return;
+  }
+  double dx = cp * (rx.u < kFixBad ? fix_double(rx) : line_sum<N>(P, 0, fx, (long long)nx * gy, 1, gx));
+  double dy = cp * (ry.u < kFixBad ? fix_double(ry) : line_sum<N>(P, 1, fy, gx, nx, gy));
+  if (!P.per[0] && (gx == 0 || gx == nx - 1)) dx = 0.0;
+  if (!P.per[1] && (gy == 0 || gy == ny - 1)) dy = 0.0;
+  if (PLAIN) {
+    out[np + I] = dx;
+    out[2 * np + I] = dy;
+  } else {
+    out[np + I] = fma(c1, dx, c0 * v[np + I]);
+    out[2 * np + I] = fma(c1, dy, c0 * v[2 * np + I]);
+  }
+}
+
 // out = c0 v + c1 L(v) (out = L(v) for c0 = 0, c1 = 1) in two passes with the
 // line sums in 64-bit fixed point (xg_fixed.cuh).  One thread per node with
 // FP64 FMAs spent 7 (N + 1) (1 + 1/N) of them a node and ran at the FP64
@@ -102,28 +130,35 @@ __global__ void __launch_bounds__(fix_plane_threads(N)) k_lin_plane(const LinPar
   __syncthreads();
   const double cp = theta ? cpl[z] : 1.0;
   fix_plane_nodes<N>(T, [&](int i, int j) {
-    const int gx = T.x0 + i, gy = T.y0 + j;
-    const long long I = off + gx + (long long)nx * gy;
-    const FixSum rx = fix_plane_x<N>(R, i, j), ry = fix_plane_y<N>(T, R, i, j);
-    double dx, dy;
-    if (!theta) {   // A as one sum: the two parts nearly cancel in a vortex
-      const FixSum r = fix_add(rx, ry);
-      out[I] = r.u < kFixBad ? fix_double(r)
-                             : line_sum<N>(P, 0, fx, (long long)nx * gy, 1, gx) + line_sum<N>(P, 1, fy, gx, nx, gy);
-      return;
-    }
-    dx = cp * (rx.u < kFixBad ? fix_double(rx) : line_sum<N>(P, 0, fx, (long long)nx * gy, 1, gx));
-    dy = cp * (ry.u < kFixBad ? fix_double(ry) : line_sum<N>(P, 1, fy, gx, nx, gy));
-    if (!P.per[0] && (gx == 0 || gx == nx - 1)) dx = 0.0;
-    if (!P.per[1] && (gy == 0 || gy == ny - 1)) dy = 0.0;
-    if (PLAIN) {
-      out[np + I] = dx;
-      out[2 * np + I] = dy;
-    } else {
-      out[np + I] = fma(c1, dx, c0 * v[np + I]);
-      out[2 * np + I] = fma(c1, dy, c0 * v[2 * np + I]);
-    }
+    lin_plane_node<N, PLAIN>(P, v, fx, fy, theta, cp, c0, c1, off, T.x0 + i, T.y0 + j, fix_plane_x<N>(R, i, j),
+                             fix_plane_y<N>(T, R, i, j), out);
   });
+}
+
+// The same with a thread a node (blockIdx.z as the plane pass), for levels that
+// fill no tile.
+template <int N, bool PLAIN>
+__global__ void __launch_bounds__(128) k_lin_nodes(const LinParams Q, const double* __restrict__ v,
+                                                  const double* __restrict__ cpl, double c0, double c1,
+                                                  double* __restrict__ out) {
+  __shared__ FixTable<N> R[2];
+  stage_kernel_begin();
+  fix_stage_rows<N>(Q.D[0], R[0]);
+  fix_stage_rows<N>(Q.D[1], R[1]);
+  __syncthreads();
+  const LineParams& P = Q.P;
+  const long long np = P.np, I = blockIdx.x * 128ll + threadIdx.x;
+  if (I >= np) return;
+  const int nx = P.n[0], ny = P.n[1];
+  const long long line = I / nx;
+  const int gx = (int)(I - line * nx), z = (int)(line / ny), gy = (int)(line - (long long)z * ny);
+  const bool theta = blockIdx.z == 1;
+  const long long off = (long long)nx * ny * z;
+  const double* fx = v + (theta ? 4 : 1) * np + off;
+  const double* fy = v + (theta ? 4 : 2) * np + off;
+  lin_plane_node<N, PLAIN>(P, v, fx, fy, theta, theta ? cpl[z] : 1.0, c0, c1, off, gx, gy,
+                           fix_line_node<N>(R[0], fx, (long long)nx * gy, 1, gx, nx, P.nseg[0], P.per[0]),
+                           fix_line_node<N>(R[1], fy, gx, nx, gy, ny, P.nseg[1], P.per[1]), out);
 }
 
 // z pass: one thread per column, marching the segments of its chunk
@@ -138,9 +173,9 @@ __global__ void __launch_bounds__(128) k_lin_z(const LinParams Q, const double* 
   const FixRows& D = Q.D[2];
   const long long np = P.np, nxy = (long long)P.n[0] * P.n[1];
   const long long col = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (col >= nxy) return;
   const int nz = P.n[2], nseg = P.nseg[2];
-  const int s0 = blockIdx.y * chunk, s1 = min(nseg, s0 + chunk);
+  const int s0 = (blockIdx.y * blockDim.y + threadIdx.y) * chunk, s1 = min(nseg, s0 + chunk);
+  if (col >= nxy || s0 >= nseg) return;
   const double* __restrict__ rw = v + 3 * np + col;
   const double* __restrict__ th = v + 4 * np + col;
   auto lev = [&](int g) -> int { return g == nz ? 0 : g; };
@@ -234,6 +269,51 @@ __global__ void __launch_bounds__(128) k_lin_z(const LinParams Q, const double* 
     const double A = out[col + nxy * g], rp = v[col + nxy * g];
     put(g, rp, fma(2.0, carry[0], A), fma(2.0, carry[1], th0[g] * A), 0.0);
   }
+}
+
+// Order 1, where a row is a difference and a factor: a thread a node takes all
+// directions in FP64 (1 M nodes 0.059 ms at any shape; two passes in fixed point
+// 0.085 where the tiles are full).
+template <bool PLAIN>
+__global__ void __launch_bounds__(128) k_lin_linear(const LinParams Q, const double* __restrict__ v,
+                                                   const double* __restrict__ cpl, const double* __restrict__ th0,
+                                                   double c0, double c1, double* __restrict__ out) {
+  stage_kernel_begin();
+  const LineParams& P = Q.P;
+  const long long np = P.np, I = blockIdx.x * 128ll + threadIdx.x;
+  if (I >= np) return;
+  const int nx = P.n[0], ny = P.n[1], nz = P.n[2];
+  const long long line = I / nx, nxy = (long long)nx * ny;
+  const int z = (int)(line / ny), gy = (int)(line - (long long)z * ny), gx = (int)(I - line * nx);
+  // the row of a field whose value at the node is c, and next to it at(step)
+  auto row = [&](int d, int g, double c, auto at) -> double {
+    const int n = P.n[d];
+    const bool right = g < n - 1 || P.per[d], left = g > 0 || P.per[d];
+    double r = c, l = c;
+    if (right) r = at(g < n - 1 ? 1 : 1 - n);
+    if (left) l = at(g > 0 ? -1 : n - 1);
+    const double k = P.Dm[d][0][1];                  // = -Dm[1][0]; a wall's node: its row twice
+    return (right && left ? k : k + k) * (r - l);
+  };
+  auto field = [&](int d, int g, const double* f, long long sd) -> double {
+    return row(d, g, f[I], [&](int k) -> double { return f[I + sd * k]; });
+  };
+  const double* w = v + 3 * np;
+  const double* t = v + 4 * np;
+  const double A = field(0, gx, v + np, 1) + field(1, gy, v + 2 * np, nx);
+  const double cp = cpl[z], th = th0[z];
+  double L[5];
+  L[0] = A + field(2, z, w, nxy);
+  L[1] = cp * field(0, gx, t, 1);
+  L[2] = cp * field(1, gy, t, nx);
+  L[3] = row(2, z, cp * t[I], [&](int k) -> double { return cpl[z + k] * t[I + nxy * k]; });
+  L[3] = fma(-P.g, v[I], L[3]);
+  L[4] = fma(th, A, row(2, z, th * w[I], [&](int k) -> double { return th0[z + k] * w[I + nxy * k]; }));
+  if (!P.per[0] && (gx == 0 || gx == nx - 1)) L[1] = 0.0;
+  if (!P.per[1] && (gy == 0 || gy == ny - 1)) L[2] = 0.0;
+  if (!P.per[2] && (z == 0 || z == nz - 1)) L[3] = 0.0;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) out[k * np + I] = PLAIN ? L[k] : fma(c1, L[k], c0 * v[k * np + I]);
 }
 
 struct Comb {
@@ -357,37 +437,48 @@ struct Imex {
   long long reorth = 0;        // Arnoldi steps that took a second Gram-Schmidt pass
 };
 
-template <int N>
+template <int N, bool PLAIN>
 void launch_linear_n(xg_ctx* c, const Imex& X, const double* v, double c0, double c1, double* out, cudaStream_t st) {
-  constexpr int E = xg::fix_plane_elems(N);
   const LineParams& P = X.lin.P;
   const long long nxy = (long long)P.n[0] * P.n[1];
-  const dim3 gp(((P.nseg[0] + E - 1) / E) * ((P.nseg[1] + E - 1) / E), P.n[2], 2);
-  const int chunk = xg::fix_z_chunk(P.nseg[2], nxy, c->sms);
-  const dim3 gz((unsigned)((nxy + 127) / 128), (P.nseg[2] + chunk - 1) / chunk);
-  if (c0 == 0.0 && c1 == 1.0) {
-    xg::launch_stage_kernel(xg::k_lin_plane<N, true>, gp, xg::fix_plane_threads(N), 0, st, X.lin, v, X.cpl, c0, c1, out);
-    xg::launch_stage_kernel(xg::k_lin_z<N, true>, gz, 128, 0, st, X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
+  const dim3 gn((unsigned)((P.np + 127) / 128), 1, N == 1 ? 1 : 2);
+  if constexpr (N == 1) {
+    xg::launch_stage_kernel(xg::k_lin_linear<PLAIN>, gn, 128, 0, st, X.lin, v, X.cpl, X.th0, c0, c1, out);
   } else {
-    xg::launch_stage_kernel(xg::k_lin_plane<N, false>, gp, xg::fix_plane_threads(N), 0, st, X.lin, v, X.cpl, c0, c1, out);
-    xg::launch_stage_kernel(xg::k_lin_z<N, false>, gz, 128, 0, st, X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
+    constexpr int E = xg::fix_plane_elems(N);
+    const dim3 gp(((P.nseg[0] + E - 1) / E) * ((P.nseg[1] + E - 1) / E), P.n[2], 2);
+    const int chunk = xg::fix_z_chunk(P.nseg[2], nxy, c->sms);
+    const int cols = xg::fix_z_columns(nxy), par = xg::kFixZThreads / cols;
+    const dim3 bz(cols, par), gz((unsigned)((nxy + cols - 1) / cols), ((P.nseg[2] + chunk - 1) / chunk + par - 1) / par);
+    if (xg::fix_plane_pays(N, P.n[0], P.n[1], P.nseg[0], P.nseg[1]))
+      xg::launch_stage_kernel(xg::k_lin_plane<N, PLAIN>, gp, xg::fix_plane_threads(N), 0, st, X.lin, v, X.cpl, c0, c1, out);
+    else
+      xg::launch_stage_kernel(xg::k_lin_nodes<N, PLAIN>, gn, 128, 0, st, X.lin, v, X.cpl, c0, c1, out);
+    xg::launch_stage_kernel(xg::k_lin_z<N, PLAIN>, gz, bz, 0, st, X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);
   }
+}
+
+template <bool PLAIN>
+cudaError_t launch_linear_as(xg_ctx* c, const Imex& X, const double* v, double c0, double c1, double* out,
+                             cudaStream_t st) {
+  switch (c->d.order) {
+    case 1: launch_linear_n<1, PLAIN>(c, X, v, c0, c1, out, st); break;
+    case 2: launch_linear_n<2, PLAIN>(c, X, v, c0, c1, out, st); break;
+    case 3: launch_linear_n<3, PLAIN>(c, X, v, c0, c1, out, st); break;
+    case 4: launch_linear_n<4, PLAIN>(c, X, v, c0, c1, out, st); break;
+    case 5: launch_linear_n<5, PLAIN>(c, X, v, c0, c1, out, st); break;
+    case 6: launch_linear_n<6, PLAIN>(c, X, v, c0, c1, out, st); break;
+    case 7: launch_linear_n<7, PLAIN>(c, X, v, c0, c1, out, st); break;
+    case 8: launch_linear_n<8, PLAIN>(c, X, v, c0, c1, out, st); break;
+    default: return cudaErrorInvalidValue;
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t launch_linear(xg_ctx* c, const Imex& X, const double* v, double c0, double c1, double* out,
                           cudaStream_t st) {
-  switch (c->d.order) {
-    case 1: launch_linear_n<1>(c, X, v, c0, c1, out, st); break;
-    case 2: launch_linear_n<2>(c, X, v, c0, c1, out, st); break;
-    case 3: launch_linear_n<3>(c, X, v, c0, c1, out, st); break;
-    case 4: launch_linear_n<4>(c, X, v, c0, c1, out, st); break;
-    case 5: launch_linear_n<5>(c, X, v, c0, c1, out, st); break;
-    case 6: launch_linear_n<6>(c, X, v, c0, c1, out, st); break;
-    case 7: launch_linear_n<7>(c, X, v, c0, c1, out, st); break;
-    case 8: launch_linear_n<8>(c, X, v, c0, c1, out, st); break;
-    default: return cudaErrorInvalidValue;
-  }
-  return cudaGetLastError();
+  return c0 == 0.0 && c1 == 1.0 ? launch_linear_as<true>(c, X, v, c0, c1, out, st)
+                                : launch_linear_as<false>(c, X, v, c0, c1, out, st);
 }
 
 cudaError_t comb(const std::vector<std::pair<double, const double*>>& terms, double* out, long long n,
