@@ -190,14 +190,19 @@ struct InterpNode {
 // intermediates stay in L2.  A thread of the z and y passes walks along the
 // interpolated axis, so that the fine values that consecutive coarse nodes share
 // come from L1: one coarse node a thread read five values from L2 for each.
+// Blocks are as wide as the lines are (interp_width), with several planes or lines
+// where these are short, and a small plane's walk along z is cut into slices
+// (blockIdx.y): one element of 5 x 5 fine columns by 2,000 along z, five variables,
+// 13.7 -> 0.18 ms a call.
 template <int NP>
 __global__ void __launch_bounds__(256) k_interp_z(const double* __restrict__ in, double* __restrict__ out,
                                                   const InterpAxis A, long long plane, int p0, int np) {
+  const int lo = (int)((long long)np * blockIdx.y / gridDim.y), hi = (int)((long long)np * (blockIdx.y + 1) / gridDim.y);
   for (long long i = blockIdx.x * 256ll + threadIdx.x; i < plane; i += gridDim.x * 256ll) {
-    int v = p0 / A.n_out, c = p0 - v * A.n_out;
+    int v = (p0 + lo) / A.n_out, c = p0 + lo - v * A.n_out;
     const double* f = in + (long long)v * A.n_in * plane + i;
-    double* o = out + i;
-    for (int p = 0; p < np; ++p) {
+    double* o = out + lo * plane + i;
+    for (int p = lo; p < hi; ++p) {
       InterpNode<NP> n;
       n.load(A, c);
       *o = n.value([&](int k) { return f[k * plane]; });
@@ -213,11 +218,13 @@ __global__ void __launch_bounds__(256) k_interp_z(const double* __restrict__ in,
 constexpr int kInterpRows = 16;   // coarse lines a thread of the y pass walks
 template <int NP>
 __global__ void __launch_bounds__(128) k_interp_y(const double* __restrict__ in, double* __restrict__ out,
-                                                  const InterpAxis A, int nx) {
-  const double* f = in + (long long)blockIdx.z * A.n_in * nx;
-  double* o = out + (long long)blockIdx.z * A.n_out * nx;
+                                                  const InterpAxis A, int nx, int np) {
+  const int p = blockIdx.z * blockDim.y + threadIdx.y;
+  if (p >= np) return;
+  const double* f = in + (long long)p * A.n_in * nx;
+  double* o = out + (long long)p * A.n_out * nx;
   for (int c0 = blockIdx.y * kInterpRows; c0 < A.n_out; c0 += gridDim.y * kInterpRows)
-    for (int i = blockIdx.x * 128 + threadIdx.x; i < nx; i += gridDim.x * 128)
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nx; i += gridDim.x * blockDim.x)
       for (int c = c0; c < min(c0 + kInterpRows, A.n_out); ++c) {
         InterpNode<NP> n;
         n.load(A, c);
@@ -229,12 +236,19 @@ __global__ void __launch_bounds__(128) k_interp_y(const double* __restrict__ in,
 template <int NP>
 __global__ void __launch_bounds__(128) k_interp_x(const double* __restrict__ in, double* __restrict__ out,
                                                   const InterpAxis A, long long lines) {
-  const int c = blockIdx.x * 128 + threadIdx.x;
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= A.n_out) return;
   InterpNode<NP> n;
   n.load(A, c);
-  for (long long j = blockIdx.y; j < lines; j += gridDim.y)
+  for (long long j = (long long)blockIdx.y * blockDim.y + threadIdx.y; j < lines; j += (long long)gridDim.y * blockDim.y)
     out[j * A.n_out + c] = n.value([&](int k) { return in[j * A.n_in + k]; });
+}
+
+// Threads along a line of n nodes in a block of 128.
+inline int interp_width(int n) {
+  int w = 128;
+  while (w > 1 && w / 2 >= n) w /= 2;
+  return w;
 }
 
 // The passes of one chunk of n planes.
@@ -244,12 +258,15 @@ cudaError_t interp_chunk(const double* src, double* t1, double* t2, double* dst,
   const int nx = A[0].n_in, nyf = A[1].n_in, nyc = A[1].n_out;
   const long long plane = (long long)nx * nyf;
   const unsigned bz = (unsigned)std::min<long long>((plane + 255) / 256, 1 << 20);
-  k_interp_z<NP><<<bz, 256, 0, st>>>(src, t1, A[2], plane, p0, (int)n);
+  const unsigned slices = std::min(n, (1024u + bz - 1) / bz);   // about 2^18 threads
+  k_interp_z<NP><<<dim3(bz, slices), 256, 0, st>>>(src, t1, A[2], plane, p0, (int)n);
+  const int wy = interp_width(nx), ry = 128 / wy;
   const unsigned by = (unsigned)std::min((nyc + kInterpRows - 1) / kInterpRows, 65535);
-  k_interp_y<NP><<<dim3((unsigned)((nx + 127) / 128), by, n), 128, 0, st>>>(t1, t2, A[1], nx);
+  k_interp_y<NP><<<dim3((unsigned)((nx + wy - 1) / wy), by, (n + ry - 1) / ry), dim3(wy, ry), 0, st>>>(t1, t2, A[1], nx, (int)n);
+  const int wx = interp_width(A[0].n_out), rx = 128 / wx;
   const long long lines = (long long)nyc * n;
-  k_interp_x<NP><<<dim3((unsigned)((A[0].n_out + 127) / 128), (unsigned)std::min<long long>((lines + 3) / 4, 65535)),
-                   128, 0, st>>>(t2, dst, A[0], lines);
+  k_interp_x<NP><<<dim3((unsigned)((A[0].n_out + wx - 1) / wx), (unsigned)std::min<long long>((lines + 4 * rx - 1) / (4 * rx), 65535)),
+                   dim3(wx, rx), 0, st>>>(t2, dst, A[0], lines);
   return cudaGetLastError();
 }
 

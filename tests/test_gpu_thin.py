@@ -66,3 +66,25 @@ def test_operators_on_thin_boxes(cuda_device, N, nel, per):
     wl = _box(nel, N, per)
     wl["S_theta"] = None
     check_nodes(wl, cuda_device)
+
+
+@pytest.mark.parametrize("shape", sorted(THIN))
+def test_restriction_cost_on_thin_boxes(cuda_device, shape):
+    """A fine node of a thin box costs at most six times one of a full box (the
+    axes' tables are host work by the node of an axis, and the call waits)."""
+    import time
+    import torch
+    from paper_2504_08157_gb300 import xg
+    t = {}
+    for nel in (THIN[shape], FULL):
+        wl = _box(nel)
+        with GpuContext(wl) as g, GpuContext(_box(nel, 2)) as c:
+            src = torch.from_numpy(wl["q"]).to(cuda_device)
+            dst = torch.empty((5, c.np), dtype=torch.float64, device=cuda_device)
+            best = float("inf")
+            for _ in range(8):
+                a = time.perf_counter()
+                xg.xg_restrict(g.ctx, c.ctx, src, dst)
+                best = min(best, time.perf_counter() - a)
+            t[nel] = best / g.np
+    assert t[THIN[shape]] <= 6.0 * t[FULL], (t[THIN[shape]] * 1e9, t[FULL] * 1e9)
