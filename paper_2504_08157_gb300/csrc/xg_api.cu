@@ -165,8 +165,8 @@ __global__ void k_from_f32(const float* __restrict__ in, double* __restrict__ ou
 
 namespace {
 
-constexpr int kDiagBlocks = 608;    // 4 per SM
 constexpr int kDiagThreads = 256;
+int diag_blocks(const xg_ctx* c) { return 4 * c->sms; }
 
 // Per-block FP64 sums of M_I q_v,I (v = 0..4), M_I = Wx(gx) Wy(gy) Wz(gz)
 // with the Jacobian folded into Wx, in a fixed order: a warp takes whole rows
@@ -211,10 +211,10 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(const R* __restri
 }
 
 // one warp per variable
-__global__ void k_diag_final(const double* __restrict__ partial, double* __restrict__ out) {
+__global__ void k_diag_final(const double* __restrict__ partial, int blocks, double* __restrict__ out) {
   const int v = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double s = 0.0;
-  for (int b = lane; b < kDiagBlocks; b += 32) s += partial[b * 5 + v];
+  for (int b = lane; b < blocks; b += 32) s += partial[b * 5 + v];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
   if (lane == 0) out[v] = s;
@@ -634,7 +634,7 @@ xg_status xg_mesh_create(const xg_mesh_desc* d, xg_ctx** out) {
     e = cudaMalloc((void**)&c->Fy, sizeof(double) * 5 * (size_t)c->nty * (size_t)n[2] * (size_t)n[0]);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hflag, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->wasm, sizeof(double) * (size_t)(n[0] + n[1] + n[2]));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&c->partial, sizeof(double) * 5 * kDiagBlocks);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&c->partial, sizeof(double) * 5 * (size_t)diag_blocks(c));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hdiag, sizeof(double) * 5);
   if (e == cudaSuccess) {
     // assembled 1-D LGL weights per direction (Eq. 8-9 on the uniform box):
@@ -1159,14 +1159,15 @@ xg_status xg_diagnostics(xg_ctx* c, double out[5], void* stream) {
   if (c->failed) return XG_ERR_CUDA;
   if (!c->has_state) return XG_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
+  const int blocks = diag_blocks(c);
   if (c->f32)
-    k_diag_partial<float><<<kDiagBlocks, kDiagThreads, 0, st>>>((const float*)c->A, c->wasm, c->n[0],
-                                                                c->n[1], c->n[2], c->np, c->partial);
+    k_diag_partial<float><<<blocks, kDiagThreads, 0, st>>>((const float*)c->A, c->wasm, c->n[0], c->n[1], c->n[2],
+                                                           c->np, c->partial);
   else
-    k_diag_partial<double><<<kDiagBlocks, kDiagThreads, 0, st>>>(c->A, c->wasm, c->n[0], c->n[1],
-                                                                 c->n[2], c->np, c->partial);
+    k_diag_partial<double><<<blocks, kDiagThreads, 0, st>>>(c->A, c->wasm, c->n[0], c->n[1], c->n[2], c->np,
+                                                            c->partial);
   XG_CUDA(c, cudaGetLastError());
-  k_diag_final<<<1, 160, 0, st>>>(c->partial, c->T);   // T is free between stages
+  k_diag_final<<<1, 160, 0, st>>>(c->partial, blocks, c->T);   // T is free between stages
   XG_CUDA(c, cudaGetLastError());
   XG_CUDA(c, cudaMemcpyAsync(c->hdiag, c->T, sizeof(double) * 5, cudaMemcpyDeviceToHost, st));
   XG_CUDA(c, cudaStreamSynchronize(st));

@@ -57,7 +57,7 @@ struct xg_ctx {
   double* base = nullptr;  // [4][nz] (double-float pairs for XG_DF64 and XG_FP32)
   double* base64 = nullptr;  // [4][nz] the same table in FP64
   double* wasm = nullptr;  // assembled 1-D mass weights: [n_x + n_y + n_z], J folded into x
-  double* partial = nullptr;  // [kDiagBlocks][5] per-block conservation sums
+  double* partial = nullptr;  // [4 per SM][5] per-block conservation sums
   double* hdiag = nullptr;    // pinned [5]
   int* flag = nullptr;
   int* hflag = nullptr;  // pinned
