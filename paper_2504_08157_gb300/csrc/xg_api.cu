@@ -169,11 +169,13 @@ constexpr int kDiagThreads = 256;
 int diag_blocks(const xg_ctx* c) { return 4 * c->sms; }
 
 // Per-block FP64 sums of M_I q_v,I (v = 0..4), M_I = Wx(gx) Wy(gy) Wz(gz)
-// with the Jacobian folded into Wx, in a fixed order: a warp takes whole rows
+// with the Jacobian folded into Wx, in a fixed order.  A warp takes whole rows
 // (its lanes along x), so that a value costs one FP64 FMA with Wx and a row
 // one with Wy Wz, and no index is divided; the FP64 pipe then bounds it beside
-// the reads.  128 x 128 x 16 order-4 box, FP64: 0.274 -> 0.176 ms.
-template <typename R>
+// the reads.  128 x 128 x 16 order-4 box, FP64: 0.274 -> 0.176 ms.  FLAT, where
+// rows are shorter than a warp or fewer than the warps: a thread a node, with
+// its weight and index of its own (rows of 4 nodes, 0.64 M: 0.47 -> 0.09 ms).
+template <typename R, bool FLAT>
 __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(const R* __restrict__ q,
                                                                const double* __restrict__ wasm, int nx, int ny,
                                                                int nz, long long np, double* __restrict__ partial) {
@@ -181,20 +183,30 @@ __global__ void __launch_bounds__(kDiagThreads) k_diag_partial(const R* __restri
   __shared__ double red[5][kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double acc[5] = {0, 0, 0, 0, 0};
-  const long long nrows = (long long)ny * nz;
-  for (long long r = (long long)blockIdx.x * kWarps + warp; r < nrows; r += (long long)gridDim.x * kWarps) {
-    const int gz = (int)(r / ny), gy = (int)(r - (long long)gz * ny);
-    const R* row = q + r * nx;
-    double ar[5] = {0, 0, 0, 0, 0};
-#pragma unroll 2
-    for (int x = lane; x < nx; x += 32) {
-      const double w = wasm[x];
+  if (FLAT) {   // np < 2^32
+    for (long long I = (long long)blockIdx.x * kDiagThreads + threadIdx.x; I < np;
+         I += (long long)gridDim.x * kDiagThreads) {
+      const unsigned r = (unsigned)I / (unsigned)nx, gz = r / (unsigned)ny;
+      const double m = wasm[(unsigned)I - r * nx] * (wasm[nx + r - gz * ny] * wasm[nx + ny + gz]);
 #pragma unroll
-      for (int v = 0; v < 5; ++v) ar[v] = fma(w, xg::to_double(row[v * np + x]), ar[v]);
+      for (int v = 0; v < 5; ++v) acc[v] = fma(m, xg::to_double(q[v * np + I]), acc[v]);
     }
-    const double wyz = wasm[nx + gy] * wasm[nx + ny + gz];
+  } else {
+    const long long nrows = (long long)ny * nz;
+    for (long long r = (long long)blockIdx.x * kWarps + warp; r < nrows; r += (long long)gridDim.x * kWarps) {
+      const int gz = (int)(r / ny), gy = (int)(r - (long long)gz * ny);
+      const R* row = q + r * nx;
+      double ar[5] = {0, 0, 0, 0, 0};
+#pragma unroll 2
+      for (int x = lane; x < nx; x += 32) {
+        const double w = wasm[x];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) acc[v] = fma(wyz, ar[v], acc[v]);
+        for (int v = 0; v < 5; ++v) ar[v] = fma(w, xg::to_double(row[v * np + x]), ar[v]);
+      }
+      const double wyz = wasm[nx + gy] * wasm[nx + ny + gz];
+#pragma unroll
+      for (int v = 0; v < 5; ++v) acc[v] = fma(wyz, ar[v], acc[v]);
+    }
   }
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
@@ -1160,12 +1172,13 @@ xg_status xg_diagnostics(xg_ctx* c, double out[5], void* stream) {
   if (!c->has_state) return XG_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const int blocks = diag_blocks(c);
-  if (c->f32)
-    k_diag_partial<float><<<blocks, kDiagThreads, 0, st>>>((const float*)c->A, c->wasm, c->n[0], c->n[1], c->n[2],
-                                                           c->np, c->partial);
-  else
-    k_diag_partial<double><<<blocks, kDiagThreads, 0, st>>>(c->A, c->wasm, c->n[0], c->n[1], c->n[2], c->np,
-                                                            c->partial);
+  const bool flat = (c->n[0] < 32 || (long long)c->n[1] * c->n[2] < (long long)blocks * (kDiagThreads / 32)) &&
+                    c->np < (1ll << 32);
+  auto sums = [&](auto kernel, auto q) {
+    kernel<<<blocks, kDiagThreads, 0, st>>>(q, c->wasm, c->n[0], c->n[1], c->n[2], c->np, c->partial);
+  };
+  if (c->f32) sums(flat ? k_diag_partial<float, true> : k_diag_partial<float, false>, (const float*)c->A);
+  else sums(flat ? k_diag_partial<double, true> : k_diag_partial<double, false>, (const double*)c->A);
   XG_CUDA(c, cudaGetLastError());
   k_diag_final<<<1, 160, 0, st>>>(c->partial, blocks, c->T);   // T is free between stages
   XG_CUDA(c, cudaGetLastError());

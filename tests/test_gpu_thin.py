@@ -5,8 +5,9 @@ on rows or on columns must not leave most of the chip idle on them."""
 import pytest
 
 from inputs import workloads as W
+from oracle import euler as E
 
-from helpers import GpuContext
+from helpers import GpuContext, oracle_of
 from test_gpu_fixed_limits import _check as check_nodes
 
 pytestmark = pytest.mark.gpu
@@ -88,3 +89,23 @@ def test_restriction_cost_on_thin_boxes(cuda_device, shape):
                 best = min(best, time.perf_counter() - a)
             t[nel] = best / g.np
     assert t[THIN[shape]] <= 6.0 * t[FULL], (t[THIN[shape]] * 1e9, t[FULL] * 1e9)
+
+
+# (a call's own work, launches and waits, is most of it at 50,000 nodes)
+WIDE = {"column": (1, 1, 15600), "pencil": (1, 16000, 4), "sheet": (1, 250, 250)}
+
+
+@pytest.mark.parametrize("shape", sorted(WIDE))
+def test_conservation_sums_cost_on_thin_boxes(cuda_device, shape):
+    """A node of a thin box of a million costs at most twice one of a full box."""
+    import numpy as np
+    t = {}
+    for nel in (WIDE[shape], (32, 32, 15)):
+        wl = _box(nel)
+        with GpuContext(wl) as g:
+            t[nel] = _time(lambda: g.xg.xg_diagnostics(g.ctx)) / g.np
+            sums = np.array(g.xg.xg_diagnostics(g.ctx))
+            m, _, _ = oracle_of(wl)
+        M = E.mass(m)
+        assert np.all(np.abs(sums - (M * wl["q"]).sum(axis=1)) <= 1e-13 * (M * np.abs(wl["q"])).sum(axis=1))
+    assert t[WIDE[shape]] <= 2.0 * t[(32, 32, 15)], t
