@@ -277,18 +277,21 @@ __device__ __forceinline__ double rsqrt_newton(double x) {
 // far from under- and overflow, where rsqrt_newton is good to an ulp or two
 __device__ __forceinline__ bool rsqrt_range(double x) { return x > 1.0e-280 && x < 1.0e280; }
 
-// sum of the block's values of v over its warps, in warp order (thread 0)
-__device__ __forceinline__ double block_sum(double v, double* red) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = red[0];
-#pragma unroll
-  for (int k = 1; k < kRiWarps; ++k) t += red[k];
-  return t;
+// A sum with what its roundings left out (Knuth's TwoSum): the last steps of a
+// centroid's sums, over warps and chunks, where positions of both signs cancel.
+// In FP64 alone they put it off by up to eight times as much as the lanes' own
+// sums do.
+struct Sum2 {
+  double h, l;
+};
+
+__device__ __forceinline__ Sum2 sum2(Sum2 a, Sum2 b) {
+  const double s = a.h + b.h, t = s - a.h;
+  return {s, (a.l + b.l) + ((a.h - (s - t)) + (b.h - t))};
 }
+
+// (an infinity leaves no remainder)
+__device__ __forceinline__ double value_of(Sum2 a) { return a.l == a.l ? a.h + a.l : a.h; }
 
 // grid (chunks, n_z): |u|, |u| x and |u| y over a chunk of a level's rows
 template <typename R>
@@ -297,8 +300,8 @@ __global__ void __launch_bounds__(kRiThreads) k_ri_centroid(const R* __restrict_
                                                            const double* __restrict__ px,
                                                            const double* __restrict__ py, int nx,
                                                            int ny, long long np,
-                                                           double* __restrict__ part) {
-  __shared__ double red[kRiWarps];
+                                                           Sum2* __restrict__ part) {
+  __shared__ double red[3][kRiWarps];
   const int gz = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int y0 = (int)((long long)ny * blockIdx.x / gridDim.x), y1 = (int)((long long)ny * (blockIdx.x + 1) / gridDim.x);
   const double r0 = rho0[gz];
@@ -323,27 +326,39 @@ __global__ void __launch_bounds__(kRiThreads) k_ri_centroid(const R* __restrict_
     s += sr;
     sy = fma(sr, py[y], sy);
   }
-  double* out = part + 3 * (blockIdx.x + (long long)gridDim.x * gz);
-  const double a = block_sum(s, red), b = block_sum(sx, red), c = block_sum(sy, red);
-  if (threadIdx.x == 0) {
-    out[0] = a;
-    out[1] = b;
-    out[2] = c;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s += __shfl_down_sync(0xffffffffu, s, o);
+    sx += __shfl_down_sync(0xffffffffu, sx, o);
+    sy += __shfl_down_sync(0xffffffffu, sy, o);
+  }
+  if (lane == 0) {
+    red[0][warp] = s;
+    red[1][warp] = sx;
+    red[2][warp] = sy;
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) {
+    Sum2 t = {red[threadIdx.x][0], 0.0};
+#pragma unroll
+    for (int k = 1; k < kRiWarps; ++k) t = sum2(t, {red[threadIdx.x][k], 0.0});
+    part[3 * (blockIdx.x + (long long)gridDim.x * gz) + threadIdx.x] = t;
   }
 }
 
-// The centroid of level gz from its chunks' sums, in chunk order.
-__device__ __forceinline__ void level_centroid(const double* __restrict__ part, int chunks, int gz, double cx0,
-                                               double cy0, double& cx, double& cy) {
-  double s = 0.0, sx = 0.0, sy = 0.0;
-  for (int k = 0; k < chunks; ++k) {
-    const double* p = part + 3 * (k + (long long)chunks * gz);
-    s += p[0];
-    sx += p[1];
-    sy += p[2];
+// The centroid of level gz from its chunks' sums, in chunk order, to c2; called by
+// a whole block.
+__device__ __forceinline__ void level_centroid(const Sum2* __restrict__ part, int chunks, int gz, double cx0,
+                                               double cy0, double (&c2)[2]) {
+  __shared__ double sums[3];
+  if (threadIdx.x < 3) {
+    Sum2 t = {0.0, 0.0};
+    for (int k = 0; k < chunks; ++k) t = sum2(t, part[3 * (k + (long long)chunks * gz) + threadIdx.x]);
+    sums[threadIdx.x] = value_of(t);
   }
-  cx = s > 0.0 ? sx / s : cx0;
-  cy = s > 0.0 ? sy / s : cy0;
+  __syncthreads();
+  if (threadIdx.x < 2) c2[threadIdx.x] = sums[0] > 0.0 ? sums[1 + threadIdx.x] / sums[0] : (threadIdx.x == 0 ? cx0 : cy0);
+  __syncthreads();
 }
 
 // grid (chunks, n_z): tangential-speed sums and node counts per strip over a
@@ -354,7 +369,7 @@ __global__ void __launch_bounds__(kRiThreads) k_ri_strip(const R* __restrict__ q
                                                         const double* __restrict__ rho0,
                                                         const double* __restrict__ px,
                                                         const double* __restrict__ py, int nx, int ny,
-                                                        long long np, const double* __restrict__ cpart,
+                                                        long long np, const Sum2* __restrict__ cpart,
                                                         double cx0, double cy0, int nstrips, double eps,
                                                         double* __restrict__ cent,
                                                         double* __restrict__ part, int* __restrict__ cntp) {
@@ -367,14 +382,8 @@ __global__ void __launch_bounds__(kRiThreads) k_ri_strip(const R* __restrict__ q
     bins[k] = 0.0;
     cnts[k] = 0;
   }
-  if (threadIdx.x == 0) {
-    level_centroid(cpart, gridDim.x, gz, cx0, cy0, c2[0], c2[1]);
-    if (blockIdx.x == 0) {
-      cent[2 * gz] = c2[0];
-      cent[2 * gz + 1] = c2[1];
-    }
-  }
-  __syncthreads();
+  level_centroid(cpart, gridDim.x, gz, cx0, cy0, c2);
+  if (threadIdx.x < 2 && blockIdx.x == 0) cent[2 * gz + threadIdx.x] = c2[threadIdx.x];
   const double cx = c2[0], cy = c2[1], r0 = rho0[gz];
   const float ieps = (float)(1.0 / eps);
   double* wb = bins + warp * nstrips;
@@ -694,7 +703,7 @@ xg_status xg_ri_velocity(xg_ctx* c, int nstrips, double* u_ri, double* centroid,
   // one buffer: positions, results (centroids, then means), chunk sums and
   // counts
   const size_t nres = 2 * (size_t)nz + (size_t)nz * nstrips;
-  const size_t nd = (size_t)nx + ny + nres + (size_t)nz * chunks * (3 + nstrips);
+  const size_t nd = (size_t)nx + ny + nres + (size_t)nz * chunks * (6 + nstrips);
   const size_t bytes = sizeof(double) * nd + sizeof(int) * (size_t)nz * chunks * nstrips;
   cudaError_t e = cudaSuccess;
   if (c->ri_bytes < bytes) {   // kept by the context: every call waits for its own work
@@ -710,8 +719,8 @@ xg_status xg_ri_velocity(xg_ctx* c, int nstrips, double* u_ri, double* centroid,
     pos = axis_positions(c, 0);
     const std::vector<double> ay = axis_positions(c, 1);
     pos.insert(pos.end(), ay.begin(), ay.end());
-    double *px = buf, *py = px + nx, *cent = py + ny, *mn = cent + 2 * nz, *cpart = cent + nres,
-           *part = cpart + 3 * (size_t)nz * chunks;
+    double *px = buf, *py = px + nx, *cent = py + ny, *mn = cent + 2 * nz, *part = cent + nres + 6 * (size_t)nz * chunks;
+    xg::Sum2* cpart = reinterpret_cast<xg::Sum2*>(cent + nres);
     int* cntp = reinterpret_cast<int*>(buf + nd);
     const double cx0 = 0.5 * (c->d.lo[0] + c->d.hi[0]), cy0 = 0.5 * (c->d.lo[1] + c->d.hi[1]);
     const double R = 0.5 * std::min(c->d.hi[0] - c->d.lo[0], c->d.hi[1] - c->d.lo[1]);
