@@ -317,11 +317,23 @@ __device__ __forceinline__ int fix_products(const double* m, const double* t, in
   return bad ? kFixBad : fix_unit_of<N>(v, fix_prod_field<N>(G, sc));
 }
 
-// Rows of x segments, the segments of a line on consecutive lanes, so that a
-// first node's row is joined with row N of the segment before (left; a wall's
-// first and, where end, last node take theirs twice) without a barrier.  Called
-// by all lanes of a warp: act the lanes that have a segment, own those whose
-// rows are wanted; put(a, row) gets the nodes' rows.
+// x segments of a tile's lines, each line's E and the one before the tile, go to
+// lanes in line order, 31 to a warp: a warp's lane 0 repeats the last one of the warp
+// before.  Each lane so finds the segment before its own on the lane before it.
+constexpr int kFixLanes = 31;
+__host__ __device__ constexpr int fix_x_tasks(int lines, int E) { return (lines * (E + 1) + kFixLanes - 1) / kFixLanes; }
+template <int E>
+__device__ __forceinline__ void fix_x_slot(int task, int lane, int& line, int& s) {
+  const int f = task * kFixLanes + lane - 1;   // -1: none
+  line = f < 0 ? 1 << 30 : f / (E + 1);
+  s = f - (f < 0 ? 0 : line * (E + 1)) - 1;    // -1: the segment before the tile
+}
+
+// Rows of x segments on the lanes of fix_x_slot, so that a first node's row is
+// joined with row N of the segment before (left; a wall's first and, where end,
+// last node take theirs twice) without a barrier.  Called by all lanes of a warp:
+// act the lanes that have a segment, own those whose rows are wanted; put(a, row)
+// gets the nodes' rows.
 template <int N, typename Put>
 __device__ __forceinline__ void fix_x_rows(const FixRows& F, const fix2 (&v)[N + 1], int u, bool act, bool own,
                                            bool left, bool end, Put put) {
@@ -352,14 +364,13 @@ __device__ __forceinline__ int fix_unit_slot(int i) {
 // whole element segment of a line -- the matrix then comes from the constant
 // bank at fixed offsets, and a segment's N + 1 values are read once for its
 // N + 1 rows -- converts its values with an exponent of their own and leaves its
-// rows as 64-bit integers, which the nodes add up (fix_add).  A warp takes the
-// x segments of 32 / (E + 1) lines, the one before the tile among them, or 32 y
-// segments.
+// rows as 64-bit integers, which the nodes add up (fix_add).  A warp takes 31 x
+// segments or a y segment of every column.
 // (One exponent and one conversion a value for the whole tile, 0.234 against
 // 0.267 ms a Laplacian's pass over 5 x 4.3 M nodes, left a quiet segment the bits
 // that the loudest one of the tile had to spare.)
-__host__ __device__ constexpr int fix_plane_elems(int N) { return N == 1 ? 31 : (N == 2 ? 15 : 32 / N); }
-// (order 4: 21 tasks of a warp a tile, three rounds of seven)
+__host__ __device__ constexpr int fix_plane_elems(int N) { return 32 / N; }
+// (order 4: 20 tasks of a warp a tile, three rounds of seven)
 __host__ __device__ constexpr int fix_plane_threads(int N) { return N == 4 ? 224 : 256; }
 
 template <int N>
@@ -464,17 +475,18 @@ template <int N>
 __device__ __forceinline__ void fix_plane_rows(const FixRows& FX, const FixRows& FY, const FixTile& T, const double* Vx,
                                                const double* Vy, FixPlaneRows<N>& R) {
   using L = FixPlane<N>;
-  constexpr int kLines = 32 / (L::E + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // y: a warp takes a segment of the tile's TS columns; the segments of a wall's
-  // last column are a task more
-  const int wx = (T.oy + kLines - 1) / kLines, y0 = T.hyl ? 0 : 1, wy = T.eky + 1 - y0 + (T.ox > L::TS ? 1 : 0);
+  // y: a warp takes a segment of the tile's TS columns, or up to 32 segments of a
+  // wall's last column
+  const int wx = fix_x_tasks(T.oy, L::E), y0 = T.hyl ? 0 : 1, ns = T.eky + 1 - y0;
+  const int wy = ns + (T.ox > L::TS ? (ns + 31) / 32 : 0);
   for (int w = warp; w < wx + wy; w += L::kWarps) {
     double a[N + 1];
     fix2 v[N + 1];
     if (w < wx) {
-      const int line = lane / (L::E + 1), s = lane - line * (L::E + 1) - 1, o = w * kLines + line;
-      const bool act = line < kLines && o < T.oy && s < T.ekx && (s >= 0 || T.hxl);
+      int o, s;
+      fix_x_slot<L::E>(w, lane, o, s);
+      const bool act = o < T.oy && s < T.ekx && (s >= 0 || T.hxl);
       int u = 0;
       if (act) {
         const double* p = Vx + (o + N) * L::PV + (s + 1) * N;
@@ -484,14 +496,14 @@ __device__ __forceinline__ void fix_plane_rows(const FixRows& FX, const FixRows&
       }
       long long* r = R.x + o * L::PR + s * N;
       int* ur = R.ux + o * (2 * L::E + 1) + 2 * s;
-      fix_x_rows<N>(FX, v, u, act, act && s >= 0, s > 0 || T.hxl, T.ox > T.ekx * N && s == T.ekx - 1,
+      fix_x_rows<N>(FX, v, u, act, act && s >= 0 && lane > 0, s > 0 || T.hxl, T.ox > T.ekx * N && s == T.ekx - 1,
                     [&](int k, FixSum x) {
                       r[k] = x.r;
                       if (k < 2 || k == N) ur[k == N ? 2 : k] = x.u;
                     });
     } else {
-      const bool edge = w - wx + y0 > T.eky;
-      const int s = edge ? y0 + lane : w - wx + y0, o = edge ? L::TS : lane;   // s - 1: the segment
+      const bool edge = w - wx >= ns;
+      const int s = y0 + (edge ? 32 * (w - wx - ns) + lane : w - wx), o = edge ? L::TS : lane;   // s - 1: the segment
       if (s > T.eky || o >= (edge ? T.ox : min(T.ox, L::TS))) continue;
       const double* p = Vy + s * N * L::PV + o + N;
 #pragma unroll

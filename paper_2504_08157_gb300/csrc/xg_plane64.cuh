@@ -57,9 +57,8 @@ __host__ __device__ constexpr int z_tile_segments(int N) { return N >= 8 ? 1 : 8
 __host__ __device__ constexpr int z_tile_threads(int N) { return kTileCols * (z_tile_segments(N) * N + 1); }
 __host__ __device__ constexpr int z_tile_min_blocks(int N) { return 1152 / z_tile_threads(N); }
 
-// Elements of a tile along x, whose segments and the one before them share a
-// warp; element rows: about 8 nodes, so that the N + 1 columns before and after a
-// tile and its closing line are a quarter of its nodes.
+// Elements of a tile along x; element rows: about 8 nodes, so that the N + 1
+// columns before and after a tile and its closing line are a quarter of its nodes.
 __host__ __device__ constexpr int xy_elems_x(int N) { return fix_plane_elems(N); }
 __host__ __device__ constexpr int xy_elems_y(int N) { return N == 1 ? 9 : (N == 3 ? 3 : (N >= 5 ? 1 : 8 / N)); }
 
@@ -250,14 +249,14 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
     for (int l = 0; l <= N; ++l) a[l] = p[l * sp];
     return fix_values<N>(a, sc, v);
   };
-  constexpr int kLines = 32 / (L::EX + 1);                // x: the segment before the tile and its own EX
   const int cy = ox > L::TX ? L::LX : L::TX;              // columns of the y tasks
-  const int wx = (oyx + kLines - 1) / kLines, wy = (eky * cy + 31) / 32;
+  const int wx = fix_x_tasks(oyx, L::EX), wy = (eky * cy + 31) / 32;
   for (int w = warp; w < 5 * (wx + wy); w += warps) {
     if (w < 5 * wx) {
-      const int c = w / wx, line = lane / (L::EX + 1), s = lane - line * (L::EX + 1) - 1;
-      const int o = (w - c * wx) * kLines + line;
-      const bool act = line < kLines && o < oyx && s < ekx && (s >= 0 || hxl), own = act && s >= 0;
+      const int c = w / wx;
+      int o, s;
+      fix_x_slot<L::EX>(w - c * wx, lane, o, s);
+      const bool act = o < oyx && s < ekx && (s >= 0 || hxl), own = act && s >= 0 && lane > 0;
       const bool left = s > 0 || hxl, end = endx && s == ekx - 1;
       const int at = o * L::PX + (s + 1) * N;
       const double* p = V + ((kFx >> (4 * c)) & 15u) * L::V + at;
