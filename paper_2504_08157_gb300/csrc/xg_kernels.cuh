@@ -148,9 +148,12 @@ __device__ __forceinline__ double drow_from(const LineParams& P, int a, const do
   return acc;
 }
 
+// (the first product rounded by itself: at order 1, where it is the whole row,
+// the compiler would fuse it with the sum it is added to, and a face between two
+// tiles or slabs, which hand the row on, would differ from one inside a tile)
 template <int N, int D>
 __device__ __forceinline__ double drow_N(const LineParams& P, const double (&d)[N + 1]) {
-  double acc = P.Dm[D][N][1] * d[1];
+  double acc = __dmul_rn(P.Dm[D][N][1], d[1]);
 #pragma unroll
   for (int l = 2; l <= N; ++l) acc = fma(P.Dm[D][N][l], d[l], acc);
   return acc;
