@@ -546,11 +546,17 @@ inline int xy_tile_rows(int N, const int (&nseg)[3], int levels, int sms) {
 
 // Whether the mixed form takes the x-y tiles instead of the x and y line
 // kernels.  The tiles do the pointwise work 1.4 times and the rho' and Theta'
-// rows without the FP64 pipe; the lines need a second launch and an x line's
-// segments to fill a CTA.  Measured a stage, tiles against lines: order 7, 4.1 M
-// nodes 0.94 / 1.20 ms; order 5 0.80 / 0.78; order 4, 17 M nodes 2.69 / 2.26;
-// order 4, 33^3 nodes 22 / 29 us.  The rule leaves n_y out, so that a y-slab of
-// a domain takes the path of the whole.
-inline bool df_uses_plane(int N, const int (&n)[3]) { return N > kDfLineOrder || (long long)n[0] * n[2] <= 4096; }
+// rows without the FP64 pipe; a short x line fills only part of its CTA.  So the
+// line lies at a length, one for each order.  A right-hand side of 3 M nodes,
+// tiles over lines, is 0.75 / 0.97 / 1.05 at 32, 64 and 80 nodes (order 2), 0.91 /
+// 0.90 / 1.15 at 33, 48 and 63 (order 3), 0.63 / 0.89 / 1.03 / 1.11 at 32, 64, 96
+// and 128 (order 4), 0.45 / 0.90 / 1.12 / 1.22 at 30, 80, 95 and 125 (order 5), and
+// 1.0 or more at order 1.  Boxes of few nodes would gain from the tiles beyond it
+// (order 4, 128 nodes: 0.83 at 30,000 nodes, equal at 300,000), but the rule leaves
+// n_y out, so that a y-slab of a domain takes the path of the whole.
+inline bool df_uses_plane(int N, const int (&n)[3]) {
+  constexpr int kMost[kDfLineOrder + 1] = {0, 0, 64, 48, 96, 90};
+  return N > kDfLineOrder || n[0] <= kMost[N];
+}
 
 }  // namespace xg

@@ -1,5 +1,5 @@
-"""GPU checks of the mixed form's line kernels on boxes that only long x lines
-reach: slabs against their domain, bit for bit."""
+"""GPU checks of the mixed form's two sets of x and y kernels: which one a box
+takes, and the line kernels on slabs against their domain, bit for bit."""
 
 import numpy as np
 import pytest
@@ -28,6 +28,24 @@ def _takes_lines(g):
     _, launches = g.xg.xg_kernel_times(g.ctx)
     g.xg.xg_profile(g.ctx, False)
     return launches[1] > 0
+
+
+# the longest x line of each order that the tiles take (0: none)
+LONGEST = {1: 0, 2: 64, 3: 48, 4: 96, 5: 90}
+
+
+@pytest.mark.parametrize("ny,nz", [(1, 1), (2, 7), (60, 1)])
+@pytest.mark.parametrize("N", range(1, 6))
+def test_path_by_the_length_of_x_lines_alone(cuda_device, N, ny, nz):
+    """Beyond the crossover a box takes the lines however few levels it has: the
+    tiles cost more there once n_y fills the chip, and a slab must take the path
+    of its domain whatever its n_y."""
+    most = LONGEST[N] // N
+    for nx, lines in ((most, False), (most + 1, True), (max(most + 1, 200 // N), True)):
+        if nx == 0:
+            continue
+        with GpuContext(_box((nx, ny, nz), N, (True, True, False)), precision=DF64) as g:
+            assert _takes_lines(g) == lines, nx
 
 
 @pytest.mark.parametrize("per_y", [True, False])
