@@ -642,7 +642,11 @@ xg_status xg_mesh_create(const xg_mesh_desc* d, xg_ctx** out) {
     }
   }
   e = cudaMalloc((void**)&c->flag, sizeof(int));
-  if (e == cudaSuccess && !c->f32)
+  // the y tiles' rows go to W's first row, which the x-y tiles leave free, where
+  // they fit it (all but meshes whose tiles are cut to few element rows, and those
+  // that need v there)
+  if (!c->f32 && 5ll * c->nty <= n[1] && (!c->dfm || c->df_plane)) c->Fy = c->W;
+  else if (e == cudaSuccess && !c->f32)
     e = cudaMalloc((void**)&c->Fy, sizeof(double) * 5 * (size_t)c->nty * (size_t)n[2] * (size_t)n[0]);
   if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hflag, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc((void**)&c->wasm, sizeof(double) * (size_t)(n[0] + n[1] + n[2]));
@@ -1199,9 +1203,9 @@ void xg_destroy(xg_ctx* c) {
   cudaFree(c->Bq);
   cudaFree(c->Cq);
   cudaFree(c->Dq);
-  cudaFree(c->W);
   cudaFree(c->T);
-  cudaFree(c->Fy);
+  if (c->Fy != c->W) cudaFree(c->Fy);
+  cudaFree(c->W);
   cudaFree(c->S);
   cudaFree(c->base);
   cudaFree(c->base64);

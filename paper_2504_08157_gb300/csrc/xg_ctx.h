@@ -52,7 +52,7 @@ struct xg_ctx {
   double* Dq = nullptr;  // q^{n+1}; swapped with A after every step
   double* W = nullptr;   // [4][np] primitives: w, p', theta in rows 1..3 (FP32: v, w, p' in [3][np])
   double* T = nullptr;   // [5][np] partial tendency
-  double* Fy = nullptr;  // FP64 states: [5][y tiles][nz][nx] y-face rows between the x-y and z passes
+  double* Fy = nullptr;  // FP64 states: [5][y tiles][nz][nx] y-face rows between the x-y and z passes (W's row 0, or its own)
   double* S = nullptr;   // [np] heating
   double* base = nullptr;  // [4][nz] (double-float pairs for XG_DF64 and XG_FP32)
   double* base64 = nullptr;  // [4][nz] the same table in FP64
