@@ -20,8 +20,10 @@
  * take tiles according to the schedule and meet at a grid barrier between
  * passes.  Each barrier wait is bounded: a CTA that waits longer than the spin
  * limit records XG_ERR_TIMEOUT and every CTA leaves the launch at its next
- * barrier.  Either way the call's launches are captured once per step count
- * into a CUDA graph and replayed.
+ * barrier.  Either way the launches are captured into CUDA graphs and replayed:
+ * the cooperative launch once per step count, the launches of XG_SCHED_LPT eight
+ * steps at a time, so that neither their number nor their size grows with the
+ * number of steps.
  *
  * Schedules (tile-to-CTA assignment):
  *   XG_SCHED_ROUND_ROBIN  tile t of a pass goes to CTA t mod G (tiles in

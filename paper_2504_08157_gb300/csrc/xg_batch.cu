@@ -344,6 +344,8 @@ namespace {
 
 constexpr size_t kSyncBytes = 128;   // bar @0, err @4, flag @8, ctr @16 (2 x 4 x 8 bytes)
 constexpr long long kSpinLimit = 20000000;   // ~2 s of 100 ns polls
+constexpr int kGraphSteps = 8;               // steps of a graph of launches (even)
+constexpr size_t kGraphsKept = 16;
 
 xg_status batch_fail(xg_batch* b, cudaError_t e, const char* where) {
   fprintf(stderr, "xg_batch: %s: %s\n", where, cudaGetErrorString(e));
@@ -491,8 +493,7 @@ cudaError_t launch(xg_batch* b, const BRun& R, cudaStream_t st) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaError_t e = cudaMemsetAsync(b->dsync, 0, kSyncBytes, st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
   if (R.schedule == XG_SCHED_LPT && !R.selftest) {
     const int one = b->tune.ctas_per_sm == 1;
     e = cudaEventRecord(b->fork, st);
@@ -513,7 +514,8 @@ cudaError_t launch(xg_batch* b, const BRun& R, cudaStream_t st) {
     }
     return e;
   }
-  return cudaLaunchKernelEx(&cfg, xg::k_batch, R);
+  e = cudaMemsetAsync(b->dsync, 0, kSyncBytes, st);
+  return e == cudaSuccess ? cudaLaunchKernelEx(&cfg, xg::k_batch, R) : e;
 }
 
 // Refresh the instance records (buffer roles, dt) on `st`.
@@ -537,38 +539,52 @@ xg_status upload_instances(xg_batch* b, const double* dt, cudaStream_t st) {
   return XG_OK;
 }
 
-// One persistent launch (through a cached graph when possible); waits for
-// it and returns the status it recorded.
-xg_status run(xg_batch* b, int nstages, int rhs_only, cudaStream_t st, bool timed, float* ms) {
+// The graph of nstages stages, captured at its first use; null where capturing is
+// not possible.
+cudaGraphExec_t graph_of(xg_batch* b, int nstages, int rhs_only) {
+  if (!b->graph_ok) return nullptr;
+  const auto key = std::make_pair(nstages, rhs_only);
+  const auto it = b->graphs.find(key);
+  if (it != b->graphs.end()) return it->second;
+  if (b->graphs.size() >= kGraphsKept) drop_graphs(b);
   const BRun R = make_run(b, nstages, rhs_only, 0, kSpinLimit);
+  cudaGraph_t g = nullptr;
   cudaGraphExec_t exec = nullptr;
-  if (b->graph_ok) {
-    auto key = std::make_pair(nstages, rhs_only);
-    auto it = b->graphs.find(key);
-    if (it != b->graphs.end()) {
-      exec = it->second;
-    } else {
-      cudaGraph_t g = nullptr;
-      cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
-      cudaError_t e2 = cudaSuccess;
-      if (e == cudaSuccess) {
-        e2 = launch(b, R, b->cap);
-        e = cudaStreamEndCapture(b->cap, &g);
-      }
-      if (e == cudaSuccess && e2 == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
-      if (g) cudaGraphDestroy(g);
-      if (e != cudaSuccess || e2 != cudaSuccess) {
-        cudaGetLastError();
-        exec = nullptr;
-        b->graph_ok = false;   // launch directly from now on
-      } else {
-        b->graphs[key] = exec;
-      }
-    }
+  cudaError_t e = cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal);
+  cudaError_t e2 = cudaSuccess;
+  if (e == cudaSuccess) {
+    e2 = launch(b, R, b->cap);
+    e = cudaStreamEndCapture(b->cap, &g);
   }
+  if (e == cudaSuccess && e2 == cudaSuccess) e = cudaGraphInstantiate(&exec, g, 0);
+  if (g) cudaGraphDestroy(g);
+  if (e != cudaSuccess || e2 != cudaSuccess) {
+    cudaGetLastError();
+    b->graph_ok = false;   // launch directly from now on
+    return nullptr;
+  }
+  b->graphs[key] = exec;
+  return exec;
+}
+
+// The launches of nstages stages (through cached graphs when possible); waits for
+// them and returns the status they recorded.  XG_SCHED_LPT launches six kernels a
+// step and order, so its graphs hold kGraphSteps steps at most -- an even number,
+// after which q^n is where it was -- and a long call replays them: a graph of the
+// whole call took host and driver memory and time by the step, 24,000 kernel nodes
+// for 1,000 steps of four orders, kept for every step count.
+xg_status run(xg_batch* b, int nstages, int rhs_only, cudaStream_t st, bool timed, float* ms) {
+  const bool lpt = b->tune.schedule == XG_SCHED_LPT;
+  const int period = lpt && !rhs_only ? 3 * kGraphSteps : nstages;
+  if (lpt) XB_CUDA(b, cudaMemsetAsync(b->dsync, 0, kSyncBytes, st));
   if (timed) XB_CUDA(b, cudaEventRecord(b->ev[0], st));
-  if (exec) XB_CUDA(b, cudaGraphLaunch(exec, st));
-  else XB_CUDA(b, launch(b, R, st));
+  for (int done = 0; done < nstages;) {
+    const int part = std::min(period, nstages - done);
+    const cudaGraphExec_t exec = graph_of(b, part, rhs_only);
+    if (exec) XB_CUDA(b, cudaGraphLaunch(exec, st));
+    else XB_CUDA(b, launch(b, make_run(b, part, rhs_only, 0, kSpinLimit), st));
+    done += part;
+  }
   if (timed) XB_CUDA(b, cudaEventRecord(b->ev[1], st));
   XB_CUDA(b, cudaMemcpyAsync(b->hsync, b->dsync + 4, 2 * sizeof(int), cudaMemcpyDeviceToHost, st));
   XB_CUDA(b, cudaStreamSynchronize(st));
