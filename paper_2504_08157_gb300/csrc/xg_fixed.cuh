@@ -370,8 +370,10 @@ __device__ __forceinline__ int fix_unit_slot(int i) {
 // 0.267 ms a Laplacian's pass over 5 x 4.3 M nodes, left a quiet segment the bits
 // that the loudest one of the tile had to spare.)
 __host__ __device__ constexpr int fix_plane_elems(int N) { return 32 / N; }
-// (order 4: 20 tasks of a warp a tile, three rounds of seven)
-__host__ __device__ constexpr int fix_plane_threads(int N) { return N == 4 ? 224 : 256; }
+// (Seven warps, six at order 8, whose tiles have few and long tasks: two Laplacians
+// over 4.3 M nodes at order 4 0.841 ms with seven, 0.854 with eight, 0.879 with ten;
+// over 5.7 M at order 8 0.915 with six, 0.983 with seven, 1.081 with eight.)
+__host__ __device__ constexpr int fix_plane_threads(int N) { return N == 8 ? 192 : 224; }
 
 template <int N>
 struct FixPlane {
