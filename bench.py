@@ -67,6 +67,16 @@ PLANE_KERNEL_OF = {1: "k_f_plane_xy_tc", 2: "k_f_plane_xy_h16"}
 COLUMN_NAMES = ("k_f_column", "-", "-")
 
 
+# a mixed context whose box takes the x-y tiles (short x lines, or an order above
+# the line kernels'): the y slot has no launches
+DF64_TILE_NAMES = ("k_plane_xy_mixed", "-", "k_df_tline_z")
+
+
+def df64_kernel_names(launches):
+    """The kernels behind the mixed form's timing slots, from their launch counts."""
+    return KERNEL_NAMES[2] if launches[1] else DF64_TILE_NAMES
+
+
 def fp32_kernel_names(wl, contract=0, fused=False):
     """The kernels behind the FP32 form's timing slots on workload wl."""
     if contract:
@@ -488,6 +498,7 @@ KERNEL_VALUES_PER_NODE = {"k_line_x": 14, "k_line_y": 16, "k_line_z": _Z_VALUES,
                           # the mixed path's y pass also writes, and its z pass reads, the rows of
                           # the y faces (5 values at one plane in N = 4, the bench order)
                           "k_df_line_x": 14, "k_df_tline_y": 16 + 5 / 4, "k_df_tline_z": _Z_VALUES + 5 / 4,
+                          "k_plane_xy_mixed": 13 + 5 / 8,   # the FP64 tiles' values in mixed arithmetic
                           "k_f_plane_xy": 13, "k_f_plane_xy_tc": 13, "k_f_plane_xy_h16": 13,
                           "k_f_tline": _Z_VALUES - 1, "k_f_column": 5 + 1 + 5 * 2 / 3 + 5}
 # The method's own traffic per node and stage: q and S in,
@@ -549,6 +560,8 @@ def run_xg(args, world, rank, local):
             xg.xg_set_fused(ctx, 1)
         knames = fp32_kernel_names(wl, contract, args.fused)
     ms_max, kms, klaunch, clk = timed_steps(xg, torch, ctx, dt, K, Wm, stream, world, local, True)
+    if prec == xg.XG_DF64:
+        knames = df64_kernel_names(klaunch)
     value = gdof(ms_max, K)
 
     # roofline: the method's algorithmic bytes per unique node and RK stage
@@ -588,7 +601,7 @@ def run_xg(args, world, rank, local):
         roof["alu"] = {"kernel": kname, "achieved": round(fach, 4), "peak": round(FP64_PEAK_TFLOPS, 4),
                        "unit": "TFLOP/s", "frac": round(fach / FP64_PEAK_TFLOPS, 4),
                        "peak_source": "FP64 derived: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz"}
-    if prec == xg.XG_DF64 and wl["N"] == 4:
+    if prec == xg.XG_DF64 and wl["N"] == 4 and knames == KERNEL_NAMES[2]:
         # the pipe that binds this path: FP64 instructions over the stage and per kernel
         inst = sum(DF64_FP64_INSTR_PER_NODE.values()) * cfg["nodes"]
         per_k = {n: round(DF64_FP64_INSTR_PER_NODE[n] * cfg["nodes"] / (per_launch[n] / 1e3) / 1e9
@@ -648,8 +661,9 @@ def run_xg(args, world, rank, local):
             xg.xg_set_contraction(c2, contract)
         if p == xg.XG_FP32 and fused:
             xg.xg_set_fused(c2, 1)
-        names = fp32_kernel_names(wl, contract, fused) if p == xg.XG_FP32 else KERNEL_NAMES[p]
         msp, kmsp, klp, _ = timed_steps(xg, torch, c2, dt, Kp, 3, stream, world, local, False)
+        names = fp32_kernel_names(wl, contract, fused) if p == xg.XG_FP32 else \
+            df64_kernel_names(klp) if p == xg.XG_DF64 else KERNEL_NAMES[p]
         xg.xg_destroy(c2)
         return {"value": round(gdof(msp, Kp), 4), "unit": "GDOF/s", "dtype": dtype,
                 "ms_per_step": round(msp / Kp, 4), "steps": Kp,
