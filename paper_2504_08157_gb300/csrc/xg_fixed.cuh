@@ -199,10 +199,9 @@ __device__ __forceinline__ fix2 fix_prod(double a, double b, int G) {
   unsigned long long P = (unsigned long long)A1 * B1 + __umulhi(A1, B0) + __umulhi(A0, B1);
   if (ea == 0 || eb == 0) P = 0;
   const int sg = ((int)(ah ^ bh) >> 31) | 1;
-  const unsigned long long V = fix_shr(P, (unsigned)(63 - fix_bits(N) + G) - (ea + eb));
-  if (fix_bits(N) < 61) return fix_limbs(V, sg);
-  const unsigned h = min((unsigned)(V >> 30), 0x7fffffffu);   // V may reach 2^61
-  return {(int)h * sg, (int)((unsigned)V - (h << 30)) * sg};
+  unsigned long long V = fix_shr(P, (unsigned)(63 - fix_bits(N) + G) - (ea + eb));
+  if (fix_bits(N) == 61) V = min(V, (1ull << 61) - 1);   // (see fix_prod_top; h stays below 2^31)
+  return fix_limbs(V, sg);
 }
 
 // Exponents usable with rows of scale sc (for fix_prod's largest
