@@ -1,8 +1,9 @@
 /*
- * xg_batch.h -- batched persistent form of the explicit CG Euler path of
- * xg.h: many independent limited-area instances, each its own mesh (own
- * element counts and polynomial order), own reference state, vortex and
- * heating, advanced together by ONE persistent kernel launch per call.
+ * xg_batch.h -- batched form of the explicit CG Euler path of xg.h: many
+ * independent limited-area instances, each its own mesh (own element counts
+ * and polynomial order), own reference state, vortex and heating, advanced
+ * together: by launches that each hold the tiles of all instances of an order,
+ * or by one persistent kernel launch per call.
  *
  * The paper runs one simulator per GPU (Sec. 4, Sec. 5); it notes the model
  * can hold several independent simulation objects, which is what a batch

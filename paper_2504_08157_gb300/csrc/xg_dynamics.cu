@@ -74,9 +74,10 @@ __device__ __forceinline__ double line_apply(const LapParams& P, int d, const do
 // (xg_fixed.cuh): one thread per node with FP64 FMAs spent 3 (N + 1) (1 + 1/N)
 // of them a value, at the FP64 pipe's rate.  Grid of the plane pass: tiles, n_z,
 // 5 variables; out gets the x and y parts.  One Laplacian of the 64 x 64 x 16
-// order-4 box: 0.93-1.02 -> 0.27 + 0.12-0.16 ms; the plane pass is bound by
-// instruction issue (72 % busy, 350 instructions a value), the z pass by the FP64
-// pipe (3 instructions a value: conversion, scale-and-add, face sum).
+// order-4 box: 0.93-1.02 -> 0.25 + 0.13-0.17 ms; the plane pass is bound by
+// instruction issue (2.9 a clock of 4, 340 instructions a value), the z pass by the
+// FP64 pipe (79 % busy, 3 to 4 instructions a value: conversion, scale-and-add, face
+// sum).
 template <int N>
 __global__ void __launch_bounds__(fix_plane_threads(N)) k_lap_plane(const LapParams P, const double* __restrict__ in,
                                                           double* __restrict__ out) {

@@ -366,7 +366,7 @@ __device__ __forceinline__ int fix_unit_slot(int i) {
 // rows as 64-bit integers, which the nodes add up (fix_add).  A warp takes 31 x
 // segments or a y segment of every column.
 // (One exponent and one conversion a value for the whole tile, 0.234 against
-// 0.267 ms a Laplacian's pass over 5 x 4.3 M nodes, left a quiet segment the bits
+// 0.253 ms a Laplacian's pass over 5 x 4.3 M nodes, left a quiet segment the bits
 // that the loudest one of the tile had to spare.)
 __host__ __device__ constexpr int fix_plane_elems(int N) { return 32 / N; }
 // (Seven warps, six at order 8, whose tiles have few and long tasks: two Laplacians

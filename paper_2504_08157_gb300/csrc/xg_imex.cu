@@ -95,8 +95,8 @@ __device__ __forceinline__ void lin_plane_node(const LineParams& P, const double
 // FP64 FMAs spent 7 (N + 1) (1 + 1/N) of them a node and ran at the FP64
 // pipe's rate, 8 times the time of the bytes.  Here the FP64 pipe is left with the
 // conversions of the sums and the assembly, about 20 instructions a node.
-// 80 x 80 x 24 order-5 box: 2.39 -> 0.61 + 0.51 ms (issue-bound; FP64 pipe 71 %
-// busy in the z pass).
+// A quarter of the 80 x 80 x 24 order-5 box, which took 2.39 ms so: 0.16 + 0.15 ms (2.7
+// instructions a clock in the plane pass, the FP64 pipe 83 % busy in the z pass).
 //
 // Plane pass: x and y sums over the tiles of a level (blockIdx.x), level
 // blockIdx.y; blockIdx.z = 0 puts A = dx(rho u) + dy(rho v) into out[0] for

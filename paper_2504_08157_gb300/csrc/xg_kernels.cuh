@@ -124,6 +124,8 @@ __device__ __forceinline__ bool is_nonfinite(double v) {
 }
 
 // ---------------------------------------------------------------- difference form
+// (the y and z passes of the mixed lines; contractions in fixed point depend on
+// differences by themselves, xg_fixed.cuh)
 // The rho' and Theta' tendencies are residuals of cancelling flux
 // derivatives where the flow is nearly non-divergent (in a vortex the x and
 // y parts nearly cancel), so their rounding must stay far below the size of

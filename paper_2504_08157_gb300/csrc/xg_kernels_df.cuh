@@ -1,6 +1,7 @@
-// xg_kernels_df.cuh -- the FP64-accurate fast path (XG_DF64): the line
-// kernels of xg_kernels.cuh with the work split between the FP64 and the
-// FP32 pipes.
+// xg_kernels_df.cuh -- the FP64-accurate fast path (XG_DF64): line kernels with
+// the work split between the FP64 and the FP32 pipes (boxes of short x lines and
+// orders above kDfLineOrder take the x-y tiles of xg_plane64.cuh for the x and y
+// passes).
 //
 // GB300 runs 2 FP64 FMAs per clock per SM against 128 FP32 FMAs.  The state
 // stays in FP64 (every [5][Np] array holds doubles, the ABI's own format), and

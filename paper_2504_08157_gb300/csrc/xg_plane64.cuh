@@ -22,8 +22,8 @@
 // left values below 2^-8 of the tile's largest fewer bits than FP64 has.)
 //
 // XG_FP64, a stage on the 128 x 128 x 16 order-4 box (17.0 M nodes): three line
-// kernels with FP64 chains 1.87 + 1.44 + 2.02 ms; tiles 1.61 + 1.38 ms (FP64
-// pipe 60 and 72 % busy, 38 and 28 FP64 instructions a node; 2,100 and 1,200
+// kernels with FP64 chains 1.87 + 1.44 + 2.02 ms; tiles 1.57 + 1.39 ms (FP64
+// pipe 63 and 73 % busy with 37 and 38 instructions a node; 2,180 and 1,220
 // instructions a node in all).  33^3 nodes: 66 -> 21 us.  At the full-size vortex,
 // where the parts of rho' cancel to 1e-3 and less, its tendency's error is 6e-14
 // (FP64 chains 7e-14).
