@@ -87,10 +87,10 @@ def fp32_kernel_names(wl, contract=0, fused=False):
 # FP64 peak derived from unit counts and clock: 152 SMs x 2 DFMA/clk/SM x
 # 2 flop x 2.07 GHz (maximum SM clock).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# FP64 instructions (DFMA + DADD + DMUL) per node and launch of the mixed
-# path's kernels, from the --set full capture of the 64x64x16 order-4 case
-# (profiles/line_kernels_tc.md; the x pass: profiles/plane64.md); 2 issue per clock and SM.
-DF64_FP64_INSTR_PER_NODE = {"k_df_line_x": 11.9, "k_df_tline_y": 14.0, "k_df_tline_z": 20.6}
+# Instructions of the FP64 pipe per node and launch of the mixed path's kernels
+# (arithmetic, comparisons and conversions), from the capture of the 64x64x16
+# order-4 case (profiles/stage_kernels.md); 2 issue per clock and SM.
+DF64_FP64_INSTR_PER_NODE = {"k_df_line_x": 12.0, "k_df_tline_y": 14.0, "k_df_tline_z": 26.3}
 FP64_PIPE_PEAK_GINSTR = 152 * 2 * 2.07e9 / 1e9
 
 
