@@ -78,8 +78,8 @@ __device__ __forceinline__ double line_apply(const LapParams& P, int d, const do
 // instruction issue (2.9 a clock of 4, 340 instructions a value), the z pass by the
 // FP64 pipe (79 % busy, 3 to 4 instructions a value: conversion, scale-and-add, face
 // sum).
-template <int N>
-__global__ void __launch_bounds__(fix_plane_threads(N)) k_lap_plane(const LapParams P, const double* __restrict__ in,
+template <int N, int W>
+__global__ void __launch_bounds__(32 * W) k_lap_plane(const LapParams P, const double* __restrict__ in,
                                                           double* __restrict__ out) {
   using L = FixPlane<N>;
   __shared__ double V[L::V];
@@ -91,11 +91,11 @@ __global__ void __launch_bounds__(fix_plane_threads(N)) k_lap_plane(const LapPar
   const long long off = var * P.np + (long long)nx * ny * z;
   FixTile T;
   T.init<N>(P, blockIdx.x % tilesx, blockIdx.x / tilesx);
-  fix_plane_load<N, true, true>(in + off, T, nx, ny, V);
+  fix_plane_load<N, W, true, true>(in + off, T, nx, ny, V);
   __syncthreads();
-  fix_plane_rows<N>(P.Kf[0], P.Kf[1], T, V, V, R);
+  fix_plane_rows<N, W>(P.Kf[0], P.Kf[1], T, V, V, R);
   __syncthreads();
-  fix_plane_nodes<N>(T, [&](int i, int j) {
+  fix_plane_nodes<N, W>(T, [&](int i, int j) {
     const long long I = T.x0 + i + (long long)nx * (T.y0 + j);
     const FixSum r = fix_add(fix_plane_x<N>(R, i, j), fix_plane_y<N>(T, R, i, j));
     if (r.u < kFixBad) {
@@ -524,14 +524,18 @@ void launch_lap(const LapParams& P, const double* q, double* L1, const double* g
   const int cols = xg::fix_z_columns(nxy), par = xg::kFixZThreads / cols;
   const dim3 bz(cols, par), gz((unsigned)((nxy + cols - 1) / cols), ((P.nseg[2] + chunk - 1) / chunk + par - 1) / par, 5);
   const bool tiles = xg::fix_plane_pays(N, P.n[0], P.n[1], P.nseg[0], P.nseg[1]);
+  const bool wide = xg::fix_plane_wide((long long)gp.x * gp.y * gp.z, sms);
   if (N == 1 && !tiles) {
     xg::launch_stage_kernel(xg::k_lap_linear<false>, gn, 128, 0, st, P, q, L1, nullptr, nullptr);
     xg::launch_stage_kernel(xg::k_lap_linear<true>, gn, 128, 0, st, P, L1, E, q, gamma);
     return;
   }
   auto plane = [&](const double* in, double* out) {
-    if (tiles) {
-      xg::launch_stage_kernel(xg::k_lap_plane<N>, gp, xg::fix_plane_threads(N), 0, st, P, in, out);
+    constexpr int W = xg::fix_plane_warps(N), WW = xg::kFixWideWarps;
+    if (tiles && wide) {
+      xg::launch_stage_kernel(xg::k_lap_plane<N, WW>, gp, 32 * WW, 0, st, P, in, out);
+    } else if (tiles) {
+      xg::launch_stage_kernel(xg::k_lap_plane<N, W>, gp, 32 * W, 0, st, P, in, out);
     } else {
       if constexpr (N > 1) xg::launch_stage_kernel(xg::k_lap_nodes<N>, gn, 128, 0, st, P, in, out);
     }

@@ -316,16 +316,25 @@ __device__ __forceinline__ int fix_products(const double* m, const double* t, in
   return bad ? kFixBad : fix_unit_of<N>(v, fix_prod_field<N>(G, sc));
 }
 
-// x segments of a tile's lines, each line's E and the one before the tile, go to
+// x segments of a tile's lines, n of each line and the one before the tile, go to
 // lanes in line order, 31 to a warp: a warp's lane 0 repeats the last one of the warp
-// before.  Each lane so finds the segment before its own on the lane before it.
+// before.  Each lane so finds the segment before its own on the lane before it.  n is a
+// full tile's number, a constant; small launches, where a tile's time counts, take the
+// tile's own (dynamics on 20 x 40 x 45 nodes 193 -> 180 us; on full tiles it costs 1 %).
 constexpr int kFixLanes = 31;
-__host__ __device__ constexpr int fix_x_tasks(int lines, int E) { return (lines * (E + 1) + kFixLanes - 1) / kFixLanes; }
+__host__ __device__ constexpr int fix_x_tasks(int lines, int n) { return (lines * (n + 1) + kFixLanes - 1) / kFixLanes; }
+// 2^16 / (n + 1) rounded up: f fix_x_div(n) >> 16 = floor(f / (n + 1)) for -1 <= f < 1300
+__device__ __forceinline__ int fix_x_div(int n) { return (int)__fdividef(65536.0f, (float)(n + 1)) + 1; }
+__device__ __forceinline__ void fix_x_slot(int task, int lane, int n, int div, int& line, int& s) {
+  const int f = task * kFixLanes + lane - 1;   // -1: none (line -1)
+  line = (f * div) >> 16;
+  s = f - line * (n + 1) - 1;                  // -1: the segment before the tile
+}
 template <int E>
 __device__ __forceinline__ void fix_x_slot(int task, int lane, int& line, int& s) {
-  const int f = task * kFixLanes + lane - 1;   // -1: none
+  const int f = task * kFixLanes + lane - 1;
   line = f < 0 ? 1 << 30 : f / (E + 1);
-  s = f - (f < 0 ? 0 : line * (E + 1)) - 1;    // -1: the segment before the tile
+  s = f - (f < 0 ? 0 : line * (E + 1)) - 1;
 }
 
 // Rows of x segments on the lanes of fix_x_slot, so that a first node's row is
@@ -369,14 +378,17 @@ __device__ __forceinline__ int fix_unit_slot(int i) {
 // 0.253 ms a Laplacian's pass over 5 x 4.3 M nodes, left a quiet segment the bits
 // that the loudest one of the tile had to spare.)
 __host__ __device__ constexpr int fix_plane_elems(int N) { return 32 / N; }
-// (Seven warps, six at order 8, whose tiles have few and long tasks: two Laplacians
-// over 4.3 M nodes at order 4 0.841 ms with seven, 0.854 with eight, 0.879 with ten;
-// over 5.7 M at order 8 0.915 with six, 0.983 with seven, 1.081 with eight.)
-__host__ __device__ constexpr int fix_plane_threads(int N) { return N == 8 ? 192 : 224; }
+// Warps of a tile's block: seven, six at order 8, whose tiles have few and long
+// tasks (two Laplacians over 4.3 M nodes at order 4 0.841 ms with seven, 0.854 with
+// eight, 0.879 with ten; over 5.7 M at order 8 0.915 with six, 0.983 with seven).
+// Twelve where a launch has fewer blocks than fit the chip at once, and a tile's
+// own time counts.
+__host__ __device__ constexpr int fix_plane_warps(int N) { return N == 8 ? 6 : 7; }
+constexpr int kFixWideWarps = 12;
+inline bool fix_plane_wide(long long blocks, int sms) { return blocks <= 3ll * sms; }
 
 template <int N>
 struct FixPlane {
-  static constexpr int kThreads = fix_plane_threads(N);
   static constexpr int E = fix_plane_elems(N);
   static constexpr int TS = E * N;            // <= 32: a warp takes a row of the tile, a lane a column
   static constexpr int LO = TS + 1;           // owned extent (a wall's last node included)
@@ -386,9 +398,6 @@ struct FixPlane {
   static constexpr int V = LX * PV;           // 8-byte slots
   static constexpr int RX = LO * PR, UX = LO * (2 * E + 1);   // x rows (wall ends included) and units
   static constexpr int RY = TS * PR, RB = (E + 1) * LO;       // y rows; rows N, and units, of segments -1..E-1
-  static constexpr int kWarps = kThreads / 32;
-  static constexpr int kRows = (LX + kWarps - 1) / kWarps;                   // rows per warp
-  static constexpr int kSide = (LO * N + LX + kThreads - 1) / kThreads;      // the columns beside the tile's
 };
 
 // Rows of a tile's segments.
@@ -423,10 +432,12 @@ struct FixTile {
 // them, of the owned rows, and the one after them, of every row (a wall's last
 // column has y segments of its own).  X, Y: which directions' segments are needed
 // (owned rows extended along x, owned columns along y).
-template <int N, bool X, bool Y>
+template <int N, int W, bool X, bool Y>
 __device__ __forceinline__ void fix_plane_load(const double* __restrict__ f, const FixTile& T, int nx, int ny,
                                                double* V) {
   using L = FixPlane<N>;
+  constexpr int kRows = (L::LX + W - 1) / W;                           // rows of a warp
+  constexpr int kSide = (L::LO * N + L::LX + 32 * W - 1) / (32 * W);   // columns beside the tile's of a thread
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int fx = T.ekx * N, fy = T.eky * N;
   auto value = [&](int i, int j) -> double {
@@ -440,12 +451,12 @@ __device__ __forceinline__ void fix_plane_load(const double* __restrict__ f, con
     if (gy >= ny) gy -= ny;
     return f[gx + (long long)nx * gy];
   };
-  double v[L::kRows], w[L::kSide];
+  double v[kRows], w[kSide];
   const int gx = T.x0 + lane - (T.x0 + lane >= nx ? nx : 0);
   const bool colx = X && lane < L::TS && lane <= fx, coly = Y && lane < L::TS && lane < T.ox;
 #pragma unroll
-  for (int k = 0; k < L::kRows; ++k) {
-    const int j = warp + k * L::kWarps - N;
+  for (int k = 0; k < kRows; ++k) {
+    const int j = warp + k * W - N;
     int gy = T.y0 + j;
     if (j < 0) gy += gy < 0 ? ny : 0;
     else gy -= gy >= ny ? ny : 0;
@@ -453,41 +464,44 @@ __device__ __forceinline__ void fix_plane_load(const double* __restrict__ f, con
     if ((colx && j >= 0 && j < T.oy) || (coly && (j >= 0 || T.hyl) && j <= fy)) v[k] = f[gx + (long long)nx * gy];
   }
 #pragma unroll
-  for (int k = 0; k < L::kSide; ++k) {
-    const int t = (int)threadIdx.x + k * L::kThreads, r = t / N;
+  for (int k = 0; k < kSide; ++k) {
+    const int t = (int)threadIdx.x + k * 32 * W, r = t / N;
     if (t < L::LO * N) w[k] = value(t - r * N - N, r);
     else w[k] = value(L::TS, t - L::LO * N - N);
   }
 #pragma unroll
-  for (int k = 0; k < L::kRows; ++k) {
-    const int jj = warp + k * L::kWarps;
+  for (int k = 0; k < kRows; ++k) {
+    const int jj = warp + k * W;
     if (lane < L::TS && jj < L::LX) V[jj * L::PV + N + lane] = v[k];
   }
 #pragma unroll
-  for (int k = 0; k < L::kSide; ++k) {
-    const int t = (int)threadIdx.x + k * L::kThreads, r = t / N;
+  for (int k = 0; k < kSide; ++k) {
+    const int t = (int)threadIdx.x + k * 32 * W, r = t / N;
     if (t < L::LO * N) V[(N + r) * L::PV + t - r * N] = w[k];
     else if (t < L::LO * N + L::LX) V[(t - L::LO * N) * L::PV + N + L::TS] = w[k];
   }
 }
 
 // Rows of every x segment of the tile's values Vx and y segment of Vy.
-template <int N>
+template <int N, int W>
 __device__ __forceinline__ void fix_plane_rows(const FixRows& FX, const FixRows& FY, const FixTile& T, const double* Vx,
                                                const double* Vy, FixPlaneRows<N>& R) {
   using L = FixPlane<N>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // y: a warp takes a segment of the tile's TS columns, or up to 32 segments of a
   // wall's last column
-  const int wx = fix_x_tasks(T.oy, L::E), y0 = T.hyl ? 0 : 1, ns = T.eky + 1 - y0;
+  constexpr bool kOwn = W == kFixWideWarps;   // the tile's own number of x segments
+  const int div = kOwn ? fix_x_div(T.ekx) : 0;
+  const int wx = fix_x_tasks(T.oy, kOwn ? T.ekx : L::E), y0 = T.hyl ? 0 : 1, ns = T.eky + 1 - y0;
   const int wy = ns + (T.ox > L::TS ? (ns + 31) / 32 : 0);
-  for (int w = warp; w < wx + wy; w += L::kWarps) {
+  for (int w = warp; w < wx + wy; w += W) {
     double a[N + 1];
     fix2 v[N + 1];
     if (w < wx) {
       int o, s;
-      fix_x_slot<L::E>(w, lane, o, s);
-      const bool act = o < T.oy && s < T.ekx && (s >= 0 || T.hxl);
+      if (kOwn) fix_x_slot(w, lane, T.ekx, div, o, s);
+      else fix_x_slot<L::E>(w, lane, o, s);
+      const bool act = o >= 0 && o < T.oy && s < T.ekx && (s >= 0 || T.hxl);
       int u = 0;
       if (act) {
         const double* p = Vx + (o + N) * L::PV + (s + 1) * N;
@@ -539,12 +553,12 @@ __device__ __forceinline__ FixSum fix_plane_y(const FixTile& T, const FixPlaneRo
 
 // node(i, j) for every owned node of the tile: a warp takes a row, a lane a
 // column; a wall's last column (i = TS) goes to the threads of its own.
-template <int N, typename F>
+template <int N, int W, typename F>
 __device__ __forceinline__ void fix_plane_nodes(const FixTile& T, F node) {
   using L = FixPlane<N>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (lane < min(T.ox, L::TS)) {
-    for (int j = warp; j < T.oy; j += L::kWarps) node(lane, j);
+    for (int j = warp; j < T.oy; j += W) node(lane, j);
   }
   if (T.ox > L::TS && (int)threadIdx.x < T.oy) node(L::TS, (int)threadIdx.x);
 }

@@ -102,10 +102,10 @@ __device__ __forceinline__ void lin_plane_node(const LineParams& P, const double
 // blockIdx.y; blockIdx.z = 0 puts A = dx(rho u) + dy(rho v) into out[0] for
 // the z pass, blockIdx.z = 1 finishes rho u and rho v from Theta' (cpl = gamma
 // p0 / Theta0 per level).
-template <int N, bool PLAIN>
-__global__ void __launch_bounds__(fix_plane_threads(N)) k_lin_plane(const LinParams Q, const double* __restrict__ v,
-                                                          const double* __restrict__ cpl, double c0, double c1,
-                                                          double* __restrict__ out) {
+template <int N, bool PLAIN, int W>
+__global__ void __launch_bounds__(32 * W) k_lin_plane(const LinParams Q, const double* __restrict__ v,
+                                                      const double* __restrict__ cpl, double c0, double c1,
+                                                      double* __restrict__ out) {
   using L = FixPlane<N>;
   __shared__ double V[2][L::V];
   __shared__ FixPlaneRows<N> R;
@@ -120,16 +120,16 @@ __global__ void __launch_bounds__(fix_plane_threads(N)) k_lin_plane(const LinPar
   const double* fx = v + (theta ? 4 : 1) * np + off;
   const double* fy = v + (theta ? 4 : 2) * np + off;
   if (theta) {
-    fix_plane_load<N, true, true>(fx, T, nx, ny, V[0]);
+    fix_plane_load<N, W, true, true>(fx, T, nx, ny, V[0]);
   } else {
-    fix_plane_load<N, true, false>(fx, T, nx, ny, V[0]);
-    fix_plane_load<N, false, true>(fy, T, nx, ny, V[1]);
+    fix_plane_load<N, W, true, false>(fx, T, nx, ny, V[0]);
+    fix_plane_load<N, W, false, true>(fy, T, nx, ny, V[1]);
   }
   __syncthreads();
-  fix_plane_rows<N>(Q.D[0], Q.D[1], T, V[0], theta ? V[0] : V[1], R);
+  fix_plane_rows<N, W>(Q.D[0], Q.D[1], T, V[0], theta ? V[0] : V[1], R);
   __syncthreads();
   const double cp = theta ? cpl[z] : 1.0;
-  fix_plane_nodes<N>(T, [&](int i, int j) {
+  fix_plane_nodes<N, W>(T, [&](int i, int j) {
     lin_plane_node<N, PLAIN>(P, v, fx, fy, theta, cp, c0, c1, off, T.x0 + i, T.y0 + j, fix_plane_x<N>(R, i, j),
                              fix_plane_y<N>(T, R, i, j), out);
   });
@@ -450,8 +450,12 @@ void launch_linear_n(xg_ctx* c, const Imex& X, const double* v, double c0, doubl
     const int chunk = xg::fix_z_chunk(P.nseg[2], nxy, c->sms);
     const int cols = xg::fix_z_columns(nxy), par = xg::kFixZThreads / cols;
     const dim3 bz(cols, par), gz((unsigned)((nxy + cols - 1) / cols), ((P.nseg[2] + chunk - 1) / chunk + par - 1) / par);
-    if (xg::fix_plane_pays(N, P.n[0], P.n[1], P.nseg[0], P.nseg[1]))
-      xg::launch_stage_kernel(xg::k_lin_plane<N, PLAIN>, gp, xg::fix_plane_threads(N), 0, st, X.lin, v, X.cpl, c0, c1, out);
+    constexpr int W = xg::fix_plane_warps(N), WW = xg::kFixWideWarps;
+    const bool tiles = xg::fix_plane_pays(N, P.n[0], P.n[1], P.nseg[0], P.nseg[1]);
+    if (tiles && xg::fix_plane_wide((long long)gp.x * gp.y * gp.z, c->sms))
+      xg::launch_stage_kernel(xg::k_lin_plane<N, PLAIN, WW>, gp, 32 * WW, 0, st, X.lin, v, X.cpl, c0, c1, out);
+    else if (tiles)
+      xg::launch_stage_kernel(xg::k_lin_plane<N, PLAIN, W>, gp, 32 * W, 0, st, X.lin, v, X.cpl, c0, c1, out);
     else
       xg::launch_stage_kernel(xg::k_lin_nodes<N, PLAIN>, gn, 128, 0, st, X.lin, v, X.cpl, c0, c1, out);
     xg::launch_stage_kernel(xg::k_lin_z<N, PLAIN>, gz, bz, 0, st, X.lin, v, X.cpl, X.th0, c0, c1, out, chunk);

@@ -250,13 +250,16 @@ __global__ void __launch_bounds__(XYTile<N>::threads(XYTile<N>::EY), 1088 / XYTi
     return fix_values<N>(a, sc, v);
   };
   const int cy = ox > L::TX ? L::LX : L::TX;              // columns of the y tasks
-  const int wx = fix_x_tasks(oyx, L::EX), wy = (eky * cy + 31) / 32;
+  const bool low = L::EY > 1 && ey < L::EY;               // a small launch: a tile's time counts
+  const int div = low ? fix_x_div(ekx) : 0;
+  const int wx = fix_x_tasks(oyx, low ? ekx : L::EX), wy = (eky * cy + 31) / 32;
   for (int w = warp; w < 5 * (wx + wy); w += warps) {
     if (w < 5 * wx) {
       const int c = w / wx;
       int o, s;
-      fix_x_slot<L::EX>(w - c * wx, lane, o, s);
-      const bool act = o < oyx && s < ekx && (s >= 0 || hxl), own = act && s >= 0 && lane > 0;
+      if (low) fix_x_slot(w - c * wx, lane, ekx, div, o, s);
+      else fix_x_slot<L::EX>(w - c * wx, lane, o, s);
+      const bool act = o >= 0 && o < oyx && s < ekx && (s >= 0 || hxl), own = act && s >= 0 && lane > 0;
       const bool left = s > 0 || hxl, end = endx && s == ekx - 1;
       const int at = o * L::PX + (s + 1) * N;
       const double* p = V + ((kFx >> (4 * c)) & 15u) * L::V + at;
