@@ -630,7 +630,7 @@ xg_status xg_mesh_create(const xg_mesh_desc* d, xg_ctx** out) {
   }
   if (c->f32) xg::fill_f32_params(c->P, &c->Pf);
   c->tile_ey = xg::xy_tile_rows(d->order, d->nel, n[2], sms);
-  c->df_plane = xg::df_uses_plane(d->order, geo.n);
+  c->df_plane = xg::df_uses_plane(d->order, d->nel[0]);
   const int ey = c->dfm && !c->df_plane ? xg::df_tile_segments(d->order, 1) : c->tile_ey;
   c->fy = ey * d->order;
   // (y tiles of the line kernels hand their row N on by way of Fy also where

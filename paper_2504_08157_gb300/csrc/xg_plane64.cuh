@@ -549,17 +549,18 @@ inline int xy_tile_rows(int N, const int (&nseg)[3], int levels, int sms) {
 
 // Whether the mixed form takes the x-y tiles instead of the x and y line
 // kernels.  The tiles do the pointwise work 1.4 times and the rho' and Theta'
-// rows without the FP64 pipe; a short x line fills only part of its CTA.  So the
-// line lies at a length, one for each order.  A right-hand side of 3 M nodes,
-// tiles over lines, is 0.75 / 0.97 / 1.05 at 32, 64 and 80 nodes (order 2), 0.91 /
-// 0.90 / 1.15 at 33, 48 and 63 (order 3), 0.63 / 0.89 / 1.03 / 1.11 at 32, 64, 96
+// rows without the FP64 pipe; a short x line fills only part of its CTA, and a tile
+// that is not full costs almost as much as one that is.  So the line lies at a number of
+// elements for each order, two tiles' (three at orders 4 and 5).  A right-hand side of
+// 3 M nodes, tiles over lines, is 0.75 / 0.97 / 1.05 at 32, 64 and 80 nodes (order 2),
+// 0.91 / 0.90 / 1.15 at 33, 48 and 63 (order 3), 0.63 / 0.89 / 1.03 / 1.11 at 32, 64, 96
 // and 128 (order 4), 0.45 / 0.90 / 1.12 / 1.22 at 30, 80, 95 and 125 (order 5), and
 // 1.0 or more at order 1.  Boxes of few nodes would gain from the tiles beyond it
 // (order 4, 128 nodes: 0.83 at 30,000 nodes, equal at 300,000), but the rule leaves
 // n_y out, so that a y-slab of a domain takes the path of the whole.
-inline bool df_uses_plane(int N, const int (&n)[3]) {
-  constexpr int kMost[kDfLineOrder + 1] = {0, 0, 64, 48, 96, 90};
-  return N > kDfLineOrder || n[0] <= kMost[N];
+inline bool df_uses_plane(int N, int nelx) {
+  constexpr int kMost[kDfLineOrder + 1] = {0, 0, 32, 20, 24, 18};
+  return N > kDfLineOrder || nelx <= kMost[N];
 }
 
 }  // namespace xg

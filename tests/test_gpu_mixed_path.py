@@ -34,7 +34,7 @@ def _takes_lines(g):
 
 
 # the longest x line of each order that the tiles take (0: none)
-LONGEST = {1: 0, 2: 64, 3: 48, 4: 96, 5: 90}
+LONGEST = {1: 0, 2: 64, 3: 60, 4: 96, 5: 90}
 
 
 @pytest.mark.parametrize("ny,nz", [(1, 1), (2, 7), (60, 1)])
@@ -72,7 +72,7 @@ ENDS = [(False, False, False), (True, True, False), (False, True, True), (True, 
 
 
 @pytest.mark.parametrize("per", ENDS)
-@pytest.mark.parametrize("N,nel", [(1, (20, 7, 1)), (1, (140, 1, 1)), (2, (33, 9, 1)), (2, (133, 1, 1)), (3, (17, 7, 1)),
+@pytest.mark.parametrize("N,nel", [(1, (20, 7, 1)), (1, (140, 1, 1)), (2, (33, 9, 1)), (2, (133, 1, 1)), (3, (21, 7, 1)),
                                    (3, (130, 1, 1)), (4, (25, 1, 1)), (4, (25, 5, 2)), (4, (130, 2, 1)), (5, (19, 1, 1)),
                                    (5, (19, 3, 1))])
 def test_line_kernels_match_extended_precision(cuda_device, N, nel, per):
