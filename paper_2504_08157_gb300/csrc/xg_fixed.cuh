@@ -66,7 +66,8 @@ inline void fix_rows(int N, const FixMatrix& c, FixRows* F) {
   const double most = fix_row_sum(N, c);
   int e = 0;
   if (most > 0.0 && std::isfinite(most)) std::frexp(most, &e);
-  const int sc = F->sc = 60 - e;
+  // (a matrix of zeros: a unit so small that its rows never set that of a sum)
+  const int sc = F->sc = most == 0.0 ? 1000 : 60 - e;
   for (int a = 0; a <= kMaxOrder; ++a)
     for (int l = 0; l <= kMaxOrder; ++l) F->ch[a][l] = F->cl[a][l] = 0;
   for (int a = 0; a <= N; ++a) {

@@ -209,3 +209,24 @@ def test_spacings_of_different_size(cuda_device, N, narrow, ratio, uniform):
         q = wl["q"].reshape([5] + n[::-1])
         wl["q"] = np.ascontiguousarray(np.broadcast_to(q.take([1], axis=3 - narrow), q.shape)).reshape(5, -1)
     _check(wl, cuda_device, narrow if uniform else None)
+
+
+@pytest.mark.parametrize("off", [(0,), (1,), (2,), (0, 1), (1, 2), (0, 2)])
+@pytest.mark.parametrize("N,nel", [(4, (9, 9, 2)), (5, (7, 6, 2)), (4, (1, 6, 5)), (1, (33, 32, 2))])
+def test_diffusion_off_in_some_directions(cuda_device, N, nel, off):
+    """A direction without diffusion takes nothing from the others' rows, weak
+    diffusion's included (its matrix is small against one)."""
+    import torch
+    wl = W.box(nel, N, (0.0, 0.0, 0.0), (9.0e4 * nel[0], 8.0e4 * nel[1], 7.0e3 * nel[2]), (True, False, False), seed=43)
+    c = [0.0 if d in off else 1e-18 for d in range(3)]     # the axes are in the order of their spacing
+    ref = Lines(wl)
+    with GpuContext(wl) as g:
+        g.xg.xg_set_dynamics(g.ctx, tuple(c), 0.5, 0.0, 0.0)
+        out = torch.empty((5, g.np), dtype=torch.float64, device=cuda_device)
+        g.xg.xg_dynamics_tendency(g.ctx, out)
+        got = out.cpu().numpy()
+    nu = [np.sqrt(np.longdouble(a)) * (h / N) ** 2 / np.sqrt(np.longdouble(0.5)) for a, h in zip(c, ref.h)]
+    for v in range(5):
+        first, t1 = ref.laplacian(ref.field(wl["q"][v]), nu)
+        second, t2 = ref.laplacian(first, nu)
+        assert _beyond(got[v], -second, t2 + ref.laplacian(t1, nu)[1]) <= 1.0
